@@ -124,7 +124,11 @@ typedef struct {
     int m2l_rotation;        /* S|R translations for few right-hand sides: 0 dense p^2 x p^2
                                 matrices, 1 rotation form (rotate to the translation axis, coaxial
                                 translation, rotate back; ~3.3 p^3 instead of p^4 operations),
-                                -1 automatic: rotation form for p >= 9 [-1]                      */
+                                -1 automatic: FP64 S|R on the tensor cores in exact 8-bit digits
+                                where p is even in 4..10 and the digit images (32 to 43 bytes per matrix
+                                value) take at most an eighth of the free device memory, for any
+                                number of right-hand sides; otherwise, and for the remaining
+                                translations, rotation form for p >= 9 [-1]                     */
     int profile_phases;      /* non-zero: record CUDA events around the matvec phases so that
                                 fmbem_last_matvec_times can report them [0]                       */
     int near_cache;          /* near-field kernel scalars g, c of every (target, source, domain)

@@ -60,6 +60,7 @@ static void free_all(fmbem *h) {
         if (e) { cudaEventDestroy(e); e = nullptr; }
     for (auto &st : h->io_stream)
         if (st) { cudaStreamDestroy(st); st = nullptr; }
+    if (h->oz_err_host) { cudaFreeHost(h->oz_err_host); h->oz_err_host = nullptr; }
     h->io_buf = nullptr;  // freed with the allocations above
     h->io_bytes = 0;
 }

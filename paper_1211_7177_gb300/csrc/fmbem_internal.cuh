@@ -176,6 +176,7 @@ struct fmbem {
     int16_t *chunk_off = nullptr;
     std::vector<int64_t> h_chunk_first;                   // [lmax+2] first chunk of each level
     std::vector<int64_t> h_pair_first;                    // [lmax+2] first CSR position of each level
+    std::vector<int32_t> h_group_beg;                     // [(lmax-1) 316 + 1] first pair_e entry of (level >= 2, offset)
     void *ybuf = nullptr;                                 // per-pair M2L results
     size_t ybuf_bytes = 0;
 
@@ -194,6 +195,16 @@ struct fmbem {
     void *Aofs = nullptr;  // S|R bf16 hi/lo images for the offset-stationary few-column M2L (BF16x3)
     void *chunk_pairs = nullptr;  // int2 [chunks][32]: (source box, CSR position) of each chunk's pairs
     int *tc_err = nullptr;
+    // FP64 M2L on the tensor cores (m2l_oz.cu): digit images of the S|R matrices, their row exponents,
+    // the degrees' balancing exponents, the expansions' digits (scratch), and a host-visible copy of
+    // the time-out flag (the FP64 products do not wait for the device)
+    void *oz_img = nullptr;
+    int *oz_er = nullptr, *oz_bal = nullptr;
+    void *oz_pairs = nullptr;        // int2 [n_ff]: (source box, CSR position) in pair_e order
+    int32_t *oz_group = nullptr;     // device copy of h_group_beg
+    void *oz_dig = nullptr;
+    size_t oz_dig_bytes = 0;
+    int *oz_err_host = nullptr;
     bool m2l_rotation = false;
     int n_tlen = 0;
     int8_t *rot_tidx = nullptr;  // [316] index of the offset's length among the distinct lengths
@@ -355,6 +366,12 @@ void build_ofs_tables(fmbem *h, cudaStream_t s);
 void split_expansions_bf16(fmbem *h, float *C, int64_t nr, cudaStream_t s);
 int64_t ofs_y_dom(const fmbem *h, int64_t nr);
 void run_m2l_ofs(fmbem *h, const float *C, float *Y, int64_t nr, cudaStream_t s, int l0, int l1, int reserve_sms);
+bool m2l_oz_supported(const fmbem *h);
+void build_oz_tables(fmbem *h, cudaStream_t s);
+int64_t oz_y_dom(const fmbem *h, int W);
+size_t oz_digit_bytes(const fmbem *h, int W);
+void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s);
+void check_oz_err(fmbem *h, cudaStream_t s);
 void pack_rot_tables(fmbem *h, cudaStream_t s);
 void pack_rot_tables_mm(fmbem *h, cudaStream_t s);
 void build_rot_mm_lists(fmbem *h, cudaStream_t s);

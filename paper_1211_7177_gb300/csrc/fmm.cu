@@ -921,7 +921,8 @@ template <typename R>
 __global__ void k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, int p2, int64_t nbox, int col0, int ncol,
                              int ct, const int32_t *parent, const uint64_t *key, const int32_t *ff_start,
                              const cx<R> *Tll, const cx<R> *Y, int64_t e_first, cx<R> *D, const cx<R> *Yll,
-                             const int32_t *ll_entry, int64_t ll_first, int64_t y_dstride, int64_t yll_dstride) {
+                             const int32_t *ll_entry, int64_t ll_first, int64_t y_dstride, int64_t yll_dstride,
+                             const int *err) {
     const int d = d0 + (int)blockIdx.y;  // domain: one grid row per domain, each with its own Y blocks
     Y += (int64_t)blockIdx.y * y_dstride;
     if (Yll) Yll += (int64_t)blockIdx.y * yll_dstride;
@@ -973,6 +974,7 @@ __global__ void k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, i
             a3 += y[3 * st];
         }
         for (; e < e1; ++e, y += st) a0 += y[0];
+        if (err && *err) a0.re = a0.im = (R)NAN;  // the pair results are incomplete (a wait ran out)
         D[(((int64_t)d * nbox + g) * 3 * nr + col0 + c) * p2 + r] = (a0 + a1) + (a2 + a3);
     }
 }
@@ -3014,6 +3016,35 @@ static size_t ofs_ybuf_need(const fmbem *h, int64_t nr) {
     return sizeof(float) * (size_t)(h->Jf + 1) * (ofs_y_dom(h, nr) + (size_t)ne * 3 * nr * 2 * h->p2);
 }
 
+// FP64 M2L on the tensor cores (m2l_oz.cu): columns per window.  All levels' pair results of a window
+// are kept (its products run in one launch), so the window is narrowed until they take at most 8 GB;
+// at most as many columns as the per-target reduction has threads for, in whole right-hand sides.
+// 0: not used (its images were not built, or the caller asked for a translation form).
+static int oz_window(const fmbem *h, int64_t nr) {
+    if (h->oz_img == nullptr) return 0;
+    const int rows_pad = ((h->p2 + 31) / 32) * 32;
+    int64_t most = std::min<int64_t>(48, 3 * (1024 / rows_pad));
+    if (h->R_D64 != nullptr) most = std::min<int64_t>(most, 24);  // L2L in rotation form beside it
+    const int64_t per_col = (int64_t)sizeof(c64) * (h->Jf + 1) * std::max<int64_t>(h->n_ff, 1) * h->p2;
+    most = std::max<int64_t>(3, std::min(most, (int64_t(8) << 30) / per_col) / 3 * 3);
+    const int64_t windows = (3 * nr + most - 1) / most, W = 3 * ((nr + windows - 1) / windows);
+    // its row and result indices are 32-bit
+    if ((h->Jf + 1) * h->nbox * W >= INT32_MAX || h->n_ff * W >= INT32_MAX) return 0;
+    return (int)W;
+}
+// bytes of a window's pair results, then one level's rotation-form L2L entries
+static size_t oz_ybuf_need(const fmbem *h, int W) {
+    int64_t ne = 0;
+    for (int l = 2; l <= h->lmax; ++l)
+        if (!h->h_rmm_first.empty()) ne = std::max(ne, h->h_rmm_first[l + 1] - h->h_rmm_first[l]);
+    return sizeof(c64) * (size_t)(h->Jf + 1) * (size_t)(std::max<int64_t>(h->n_ff, 1) + ne) * (size_t)W * h->p2;
+}
+// the scratch of a window exists
+static bool oz_ready(const fmbem *h, int W) {
+    return W > 0 && h->oz_dig != nullptr && h->oz_dig_bytes >= oz_digit_bytes(h, W) && h->ybuf != nullptr &&
+           h->ybuf_bytes >= oz_ybuf_need(h, W);
+}
+
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_results = true) {
     const size_t cb = sizeof(c64);
     if (h->scratch_rhs < nr) {
@@ -3027,8 +3058,17 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
     // one column window of the FP64 rotation form for more columns); sized by the columns of
     // this call, so that a few-column call after a many-column one still takes the chunked path
     const bool many = rot_many_path(h, nr, precision == FMBEM_FP64);
-    if (pair_results && (3 * nr <= 24 || many)) {
-        size_t need = ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb);
+    const int ozw = precision == FMBEM_FP64 && pair_results ? oz_window(h, nr) : 0;
+    if (ozw > 0 && h->oz_dig_bytes < oz_digit_bytes(h, ozw)) {
+        if (h->oz_dig) dev_free(h, h->oz_dig);
+        h->oz_dig = nullptr;
+        h->oz_dig_bytes = 0;
+        h->oz_dig = dev_alloc(h, oz_digit_bytes(h, ozw));
+        h->oz_dig_bytes = oz_digit_bytes(h, ozw);
+    }
+    if (pair_results && (3 * nr <= 24 || many || ozw > 0)) {
+        size_t need = 3 * nr <= 24 || many ? ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb) : 0;
+        if (ozw > 0) need = std::max(need, oz_ybuf_need(h, ozw));
         if (precision == FMBEM_BF16X3 && h->Aofs != nullptr && 3 * nr <= 24) need = std::max(need, ofs_ybuf_need(h, nr));
         if (h->ybuf == nullptr || h->ybuf_bytes < need) {
             if (h->ybuf) dev_free(h, h->ybuf);
@@ -3170,7 +3210,10 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
     constexpr int MAXC = 24;
     // FP64 with more than MAXC columns and rotation tables: the rotation form in column windows
     const bool rot_many = rot_many_path(h, nr, !f32);
-    const int ncol = rot_many ? rot_many_cols(h) : (int)std::min<int64_t>(3 * nr, MAXC);
+    // FP64 on the tensor cores, any number of columns in windows
+    const int ozw = f32 ? 0 : oz_window(h, nr);
+    const bool oz = oz_ready(h, ozw);
+    const int ncol = oz ? ozw : rot_many ? rot_many_cols(h) : (int)std::min<int64_t>(3 * nr, MAXC);
     const size_t tbytes = sizeof(cx<R>) * p2 * p2;
     const size_t budget = 200 * 1024;
     auto xs_bytes = [&](int c) { return sizeof(cx<R>) * c * MAXC * p2; };
@@ -3189,10 +3232,10 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
     // rotation form of the chunked S|R (when its tables were built)
     const int pp = h->p;
     const RotLaunch rl = rot_launch<R>(h, ncol, budget);
-    const bool chunked =
-        (3 * nr <= MAXC ? pc >= 1 && smc <= budget
+    const bool chunked = oz ||
+        ((3 * nr <= MAXC ? pc >= 1 && smc <= budget
                         : rot_many && rl.ok && h->ybuf_bytes >= ybuf_need(h, ncol, sizeof(cx<R>))) &&
-        h->ybuf != nullptr && rows_pad <= max_thr;
+         h->ybuf != nullptr && rows_pad <= max_thr);
     const bool use_rot = chunked && rl.ok;
     if (tensor_mode && f32 && h->Atc != nullptr && 3 * nr >= 48) {
         run_m2l_tc(h, (float *)C, (float *)D, nr, s, tensor_mode == 2, c_split);
@@ -3229,18 +3272,21 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
             }
         }
         const int64_t y_dom = ofs ? ofs_y_dom(h, nr) / 2 : 0;  // in complex values
+        const bool all_levels = ofs || oz;  // every level's products in one launch before the loop
         // per level and column window, all domains in one launch each (grid rows): domain d's pair
         // results at Y + d * ystr, its rotation-form L2L entries after every domain's pair results
-        for (int l = 2; l <= lmax; ++l) {
-            const LevelInfo &Lv = h->lev[l];
-            const int64_t c0 = h->h_chunk_first[l], nch = h->h_chunk_first[l + 1] - c0;
-            const int64_t nchild = h->h_rmm_first.empty() ? 0 : h->h_rmm_first[l + 1] - h->h_rmm_first[l];
-            for (int col0 = 0; col0 < 3 * nr; col0 += ncol) {
-                const int nc = (int)std::min<int64_t>(ncol, 3 * nr - col0);
-                const int64_t e_first = ofs ? 0 : h->h_pair_first[l];
-                const int64_t ystr = ofs ? y_dom : (h->h_pair_first[l + 1] - e_first) * nc * p2;
+        for (int col0 = 0; col0 < 3 * nr; col0 += ncol) {
+            const int nc = (int)std::min<int64_t>(ncol, 3 * nr - col0);
+            if constexpr (sizeof(R) == 8)
+                if (oz) run_m2l_oz(h, C, Y, nr, col0, nc, s);
+            for (int l = 2; l <= lmax; ++l) {
+                const LevelInfo &Lv = h->lev[l];
+                const int64_t c0 = h->h_chunk_first[l], nch = h->h_chunk_first[l + 1] - c0;
+                const int64_t nchild = h->h_rmm_first.empty() ? 0 : h->h_rmm_first[l + 1] - h->h_rmm_first[l];
+                const int64_t e_first = all_levels ? 0 : h->h_pair_first[l];
+                const int64_t ystr = ofs ? y_dom : oz ? oz_y_dom(h, nc) / 2 : (h->h_pair_first[l + 1] - e_first) * nc * p2;
                 const dim3 grid((unsigned)nch, (unsigned)(J + 1));
-                if (nch > 0 && !ofs) {  // (the offset-stationary products ran above)
+                if (nch > 0 && !all_levels) {  // (the tensor-core products ran above)
                     if (use_rot)
                         launch_rot<R>(rl, nch, s, c0, l, lmax, J + 1, nr, pp, h->nbox, col0, nc, h->chunk_beg,
                                       h->chunk_cnt, h->chunk_off, h->pair_e, h->ff_src, h->rot_tidx, h->n_tlen, RD, RP,
@@ -3278,7 +3324,7 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                 const int ct = (nc + L2L_CPT - 1) / L2L_CPT;
                 k_l2l_reduce<R><<<dim3((unsigned)Lv.n, (unsigned)(J + 1)), rows_pad * ct, sizeof(cx<R>) * nc * p2, sr>>>(
                     Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, h->box_parent, h->box_key, h->ff_start, Tll, Y,
-                    e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str);
+                    e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
                 CKL("k_l2l_reduce");
             }
         }
@@ -3565,6 +3611,7 @@ static void check_fp32_only(const fmbem *h, int precision) {
 
 void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaStream_t s) {
     check_fp32_only(h, precision);
+    check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
     const DomainConsts *dc = (const DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
@@ -3579,6 +3626,7 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
 
 void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaStream_t s) {
     check_fp32_only(h, precision);
+    check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
     static_assert(sizeof(DomainConsts) == 3 * sizeof(c64), "layout");
     DomainConsts *dc = (DomainConsts *)h->dcons;
@@ -3650,18 +3698,24 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     unsigned char *base = (unsigned char *)static_scratch_address();
     // run the regular passes on pointers into the static array; the handle's own scratch
     // pointers are restored afterwards, so fmbem_matvec is unaffected
-    void *sv_dens = h->dens, *sv_C = h->Cexp, *sv_D = h->Dexp, *sv_y = h->ybuf;
+    void *sv_dens = h->dens, *sv_C = h->Cexp, *sv_D = h->Dexp, *sv_y = h->ybuf, *sv_dig = h->oz_dig;
+    const size_t sv_yb = h->ybuf_bytes;
+    auto restore = [&] {
+        h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y; h->ybuf_bytes = sv_yb; h->oz_dig = sv_dig;
+    };
     h->dens = base;
     h->Cexp = base + b_dens;
     h->Dexp = base + b_dens + b_exp;
     h->ybuf = b_y ? base + b_dens + 2 * b_exp : nullptr;
+    h->ybuf_bytes = b_y;
+    h->oz_dig = nullptr;  // no digits in the static array: the FP64 pipe's translations
     try {
         matvec_impl<R>(h, x, y, nr, s, (const DomainConsts *)h->dcons);
     } catch (...) {
-        h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y;
+        restore();
         throw;
     }
-    h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y;
+    restore();
 }
 
 void run_matvec_noalloc(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaStream_t s) {

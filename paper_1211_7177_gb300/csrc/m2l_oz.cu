@@ -1,0 +1,655 @@
+// m2l_oz.cu -- the FP64 M2L (S|R part of Eq. 2.21) on the GB300 tensor cores.
+//
+// GB300 runs FP64 at about 1/60 of its FP32 rate, and the double-precision M2L on the FP64 pipe was
+// bound by it (the folded rotation form 88 % busy at p = 10, the dense many-column form at p = 8).
+// Here each double is cut into OZ_S = 8 signed 8-bit digits (the error-free transformation of Ozaki,
+// Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication", 2012), every digit is
+// an exact bf16, and the products of digits are summed exactly: a digit product is at most 2^14 units,
+// so that the sums over K = 2 p^2 <= 200 stay below the 24 bits that FP32 tensor memory holds.
+//
+//   S|R[R][K] 2^(s_K - er_R) = sum_i T_i[R][K] 2^(-7 - 8 i),   C[K][col] 2^(-s_K - ec_col) likewise,
+//   Y[R][col] = 2^(er_R + ec_col) sum_{d = 0..7} sum_{i + j = d} T_i C_j   (d > 7 is below 2^-64).
+//
+// s_K (one power of two per degree, domain and level) balances the matrices, whose entries grow like
+// double factorials of the degrees while the expansions shrink; er (per matrix row) and ec (per source
+// column) bring the largest entries to [1/2, 1).  The diagonals d = 0..4 have a tensor-memory accumulator
+// each (exact); d = 5..7 share one, whose FP32 rounding is below 2^-60.  The six sums are added without
+// error in FP32 pairs and rounded once to a double.  Measured on pair results against quad
+// precision (rms relative error, torus of 3840 nodes): p = 8 8e-17 and p = 10 3e-16, where the FP64 sums
+// of the dense form have 5e-16 and the rotation form 1e-8 (a seven-digit form had 6e-16 and 1.5e-15).
+//
+// The FF pairs of one level and offset share a matrix; their columns (W per pair) follow one another
+// and are cut into tiles of OZ_N = 80, the N of the MMAs (six accumulators of 80 columns fill tensor
+// memory); the matrix rows are its M = 128 (one row tile for p <= 8, two for p = 10).  The results go to
+// Y[pair][column], which k_l2l_reduce sums per target.
+#include <algorithm>
+#include <string>
+
+#include "fmbem_internal.cuh"
+#include "tc_ptx.cuh"
+
+namespace {
+
+constexpr int OZ_S = 8;      // digits per double
+constexpr int OZ_N = 80;     // pair columns per tile
+constexpr int OZ_ACC = 6;    // accumulators: d = 0, 1, 2, 3, 4 and 5..7
+constexpr int OZ_SLOTS = 4;  // operand ring: one K block of 16 each
+constexpr int OZ_FILL = 3;   // producer warps
+constexpr int OZ_EPI = 16;   // epilogue warps
+constexpr int OZ_NONFINITE = 1 << 20;  // exponent marking a column or row with an Inf or a NaN
+constexpr uint32_t OZ_A_BYTES = OZ_S * TC_M * 32u, OZ_B_BYTES = OZ_S * OZ_N * 32u;
+constexpr uint32_t OZ_SLOT_BYTES = OZ_A_BYTES + OZ_B_BYTES;
+constexpr int OZ_ROW = OZ_S * 32;  // bytes of a source column's digits in one K block
+constexpr int OZ_MAX_LEVELS = 12;
+constexpr int OZ_THREADS = 32 * (OZ_FILL + 1 + OZ_EPI);
+static_assert(OZ_SLOTS == 4 && OZ_FILL == 3 && OZ_EPI == 16 && OZ_ACC * OZ_N <= 512 && OZ_S == 8,
+              "ring arithmetic, tensor-memory lanes of the epilogue warps, tensor memory, digit arithmetic");
+
+// byte offset of the 16-byte chunk c (0, 1) of a row in the 32-byte-swizzled K-major layout
+__host__ __device__ __forceinline__ uint32_t sw32_chunk(int row, int c) {
+    return (uint32_t)(row * 32 + ((c ^ (row >> 2)) & 1) * 16);
+}
+// shared-memory matrix descriptor, K-major, 32-byte swizzle: 8-row groups 256 bytes apart
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(256 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)6 << 61;
+    return d;
+}
+
+struct OzLevels {  // first box of each level (levels 2..lmax), for the level of a box
+    int lmax;
+    int64_t off[OZ_MAX_LEVELS + 2];
+};
+
+// exponent e with |x| < 2^e for the larger of two doubles (zero: very small; Inf, NaN: OZ_NONFINITE)
+__device__ __forceinline__ int oz_exp2(double a, double b) {
+    const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+    const int e = max(ea, eb);
+    if (e == 0x7ff) return OZ_NONFINITE;
+    if (e == 0) return a == 0.0 && b == 0.0 ? -OZ_NONFINITE : -1022;
+    return e - 1022;
+}
+
+// the digits of x 2^shift (|x 2^shift| < 1), each as the bf16 bits of digit 2^(-7 - 8 i)
+__device__ __forceinline__ void oz_digits(double x, int shift, uint16_t *out) {
+    long long m = __double2ll_rn(ldexp(x, shift + 8 * OZ_S - 1));
+#pragma unroll
+    for (int i = OZ_S - 1; i >= 0; --i) {
+        const int dgt = i > 0 ? (int)(int8_t)(m & 0xff) : (int)m;
+        if (i > 0) m = (m - dgt) >> 8;
+        const float f = (float)dgt * __int_as_float((127 - 7 - 8 * i) << 23);
+        out[i] = (uint16_t)(__float_as_uint(f) >> 16);  // at most 8 significant bits: exact
+    }
+}
+
+// s_K per (domain, level) and degree n: minus half the exponent of the largest entry between
+// coefficients of degree n, over all 316 offsets, less n / 4 (expansions of surface nodes shrink a
+// little faster with the degree than that; measured 1.3 to 2 times more exact than without); grid
+// (matrix sets, degree)
+__global__ void k_oz_balance(const c64 *T, int p, int lmax, int *bal) {
+    const int set = blockIdx.x, n = blockIdx.y, p2 = p * p;
+    const int d = set / (lmax - 1), l = 2 + set % (lmax - 1), w = 2 * n + 1;
+    const c64 *M = T + m2l_matrix(d, l, 0, lmax) * p2 * p2;
+    int e = -OZ_NONFINITE;
+    for (int i = threadIdx.x; i < 316 * w * w; i += blockDim.x) {
+        const int o = i / (w * w), c = n * n + (i / w) % w, r = n * n + i % w;
+        const c64 t = M[((int64_t)o * p2 + c) * p2 + r];
+        const int x = oz_exp2(t.re, t.im);
+        if (x < OZ_NONFINITE) e = max(e, x);
+    }
+    __shared__ int best;
+    if (threadIdx.x == 0) best = -OZ_NONFINITE;
+    __syncthreads();
+    atomicMax(&best, e);
+    __syncthreads();
+    if (threadIdx.x == 0) bal[set * p + n] = best > -OZ_NONFINITE ? -(best >> 1) - n / 4 : 0;
+}
+
+__device__ __forceinline__ int oz_degree(int q) {
+    int n = 0;
+    while ((n + 1) * (n + 1) <= q) ++n;
+    return n;
+}
+
+// digit images of the S|R matrices: block per matrix; per (row tile, K block) eight digit blocks of
+// 128 rows x 16 K in the 32-byte-swizzled K-major layout, real-form rows 2r + a as in m2l_tc.cu
+__global__ void __launch_bounds__(256) k_oz_images(const c64 *T, int p, int lmax, int mt, int kblocks, const int *bal,
+                                                   unsigned char *img, int *er) {
+    const int64_t mat = blockIdx.x;
+    const int set = (int)(mat / 316), o = (int)(mat % 316), p2 = p * p;
+    const int d = set / (lmax - 1), l = 2 + set % (lmax - 1);
+    const c64 *M = T + m2l_matrix(d, l, o, lmax) * p2 * p2;
+    __shared__ int s_er[400], s_bal[400];
+    for (int c = threadIdx.x; c < p2; c += blockDim.x) s_bal[c] = bal[set * p + oz_degree(c)];
+    __syncthreads();
+    for (int r = threadIdx.x; r < p2; r += blockDim.x) {
+        int e = -OZ_NONFINITE;
+        for (int c = 0; c < p2; ++c) {
+            const c64 t = M[(int64_t)c * p2 + r];
+            const int x = oz_exp2(t.re, t.im);
+            e = max(e, x == OZ_NONFINITE ? x : x + s_bal[c]);
+        }
+        if (e < -OZ_NONFINITE / 2) e = 0;
+        if (e > OZ_NONFINITE / 2) e = OZ_NONFINITE;
+        s_er[r] = e;
+        er[mat * p2 + r] = e;
+    }
+    __syncthreads();
+    unsigned char *out = img + mat * (int64_t)mt * kblocks * OZ_A_BYTES;
+    const int chunks = kblocks * 2;  // 16-byte chunks (eight K values) of a row
+    for (int i = threadIdx.x; i < mt * TC_M * chunks; i += blockDim.x) {
+        const int R = i / chunks, ch = i % chunks, kb = ch >> 1, r = R >> 1, a = R & 1;
+        uint16_t w[OZ_S][8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = ch * 4 + j;
+            c64 t = {0.0, 0.0};
+            int sh = 0;
+            if (r < p2 && c < p2 && s_er[r] != OZ_NONFINITE) {
+                t = M[(int64_t)c * p2 + r];
+                sh = s_bal[c] - s_er[r];
+            }
+            uint16_t u[OZ_S], v[OZ_S];
+            oz_digits(a == 0 ? t.re : t.im, sh, u);    // [[Re, -Im], [Im, Re]]
+            oz_digits(a == 0 ? -t.im : t.re, sh, v);
+#pragma unroll
+            for (int k = 0; k < OZ_S; ++k) {
+                w[k][2 * j] = u[k];
+                w[k][2 * j + 1] = v[k];
+            }
+        }
+        unsigned char *blk = out + ((int64_t)(R / TC_M) * kblocks + kb) * OZ_A_BYTES;
+        const uint32_t at = sw32_chunk(R % TC_M, ch & 1);
+#pragma unroll
+        for (int k = 0; k < OZ_S; ++k)
+            *reinterpret_cast<uint4 *>(blk + k * (TC_M * 32) + at) =
+                make_uint4(w[k][0] | (uint32_t)w[k][1] << 16, w[k][2] | (uint32_t)w[k][3] << 16,
+                           w[k][4] | (uint32_t)w[k][5] << 16, w[k][6] | (uint32_t)w[k][7] << 16);
+    }
+}
+
+// digits of the multipole expansions, columns col0 .. col0 + W - 1 of every box of levels >= 2: a warp
+// per (domain, box, column) row; row (d nbox + box) W + c holds per K block eight digit rows of 32
+// bytes, and ec its exponent
+__global__ void __launch_bounds__(256) k_oz_split(const c64 *C, const OzLevels L, int64_t nbox, int64_t ncols, int col0,
+                                                  int W, int ndom, int p, int kblocks, const int *bal, unsigned char *out,
+                                                  int *ec) {
+    const int lane = threadIdx.x & 31, p2 = p * p;
+    const int64_t nb = nbox - L.off[2];
+    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= (int64_t)ndom * nb * W) return;
+    const int c = (int)(i % W);
+    const int64_t b = L.off[2] + (i / W) % nb;
+    const int d = (int)(i / W / nb);
+    int l = 2;
+    while (l < L.lmax && L.off[l + 1] <= b) ++l;
+    const int *s = bal + (d * (L.lmax - 1) + l - 2) * p;
+    const c64 *x = C + (((int64_t)d * nbox + b) * ncols + col0 + c) * p2;
+    constexpr int Q = 4;  // p^2 <= 100 coefficients over 32 lanes
+    c64 v[Q];
+    int sc[Q], e = -OZ_NONFINITE;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const int q = lane + 32 * k;
+        v[k] = q < p2 ? x[q] : c64{0.0, 0.0};
+        sc[k] = q < p2 ? s[oz_degree(q)] : 0;
+        const int y = oz_exp2(v[k].re, v[k].im);
+        e = max(e, abs(y) == OZ_NONFINITE ? y : y - sc[k]);
+    }
+    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    const bool bad = e > OZ_NONFINITE / 2;
+    if (e < -OZ_NONFINITE / 2 || bad) e = 0;
+    const int64_t row = ((int64_t)d * nbox + b) * W + c;
+    if (lane == 0) ec[row] = bad ? OZ_NONFINITE : e;
+    unsigned char *o = out + row * (int64_t)kblocks * OZ_ROW;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const int q = lane + 32 * k;
+        if (q >= kblocks * 8) break;
+        uint16_t a[OZ_S], b2[OZ_S];
+        oz_digits(bad ? 0.0 : v[k].re, -sc[k] - e, a);
+        oz_digits(bad ? 0.0 : v[k].im, -sc[k] - e, b2);
+        unsigned char *w = o + (q >> 3) * OZ_ROW + (q & 7) * 4;
+#pragma unroll
+        for (int j = 0; j < OZ_S; ++j) *reinterpret_cast<uint32_t *>(w + j * 32) = a[j] | (uint32_t)b2[j] << 16;
+    }
+}
+
+struct OzP {
+    int64_t nbox, y_dom;
+    int W, p2, kblocks;  // columns per pair of this window, K blocks of 16
+    int lmax, ndom, mt, ngroup;
+};
+__host__ __device__ __forceinline__ int oz_tiles(int64_t pairs, int W) { return (int)((pairs * W + OZ_N - 1) / OZ_N); }
+
+// unit v of a launch (row tile fastest, so that concurrent CTAs share source digits, then the tiles of
+// a group, which share a matrix): domain, row tile, group (level, offset) and its columns
+struct OzTile {
+    int d, mt, g, n;     // n columns of the tile
+    int64_t pair0;       // first pair (pair_e position) of the group
+    int col0;            // first column within the group
+};
+__device__ __forceinline__ OzTile oz_tile(const OzP &P, int v, int ntile, const int *first, const int32_t *group) {
+    OzTile t;
+    t.mt = v % P.mt;
+    v /= P.mt;
+    t.d = v / ntile;
+    v -= t.d * ntile;
+    int lo = 0, hi = P.ngroup;  // the group with first[g] <= v < first[g + 1]
+    while (hi - lo > 1) {
+        const int m = (lo + hi) >> 1;
+        if (first[m] <= v) lo = m;
+        else hi = m;
+    }
+    t.g = lo;
+    t.pair0 = group[lo];
+    t.col0 = (v - first[lo]) * OZ_N;
+    t.n = (int)min((int64_t)OZ_N, (int64_t)(group[lo + 1] - t.pair0) * P.W - t.col0);
+    return t;
+}
+
+// 2^k (s + w + r) as a double by FP32 and integer operations: an FP64 addition keeps a quarter of the SM
+// busy for 64 cycles here, and with two of them per result the sums took longer than the MMAs.  The three
+// floats become a head h, a tail g of at most half its ulp and a rest e2, and g and e2 are added to the
+// bits of h's double in quarters of its last place (within 0.8 of which the result is).  FP64 where the
+// sum nearly cancels, and where k is out of the doubles' range (OZ_NONFINITE and beyond: an Inf or a NaN).
+__device__ __noinline__ double oz_compose_far(float s, float w, float r, int k) {
+    if (k > OZ_NONFINITE / 2) return __longlong_as_double(0x7ff8000000000000ll);
+    return ldexp(((double)s + (double)w) + (double)r, k);
+}
+__device__ __forceinline__ float oz_two_sum(float a, float b, float &err) {
+    const float s = a + b, t = s - a;
+    err = (a - (s - t)) + (b - t);
+    return s;
+}
+__device__ __forceinline__ double oz_compose(float s, float w, float r, int k) {
+    float e1, e2, g;
+    const float h1 = oz_two_sum(s, w, e1), t = oz_two_sum(e1, r, e2), h = oz_two_sum(h1, t, g);
+    if (!(fabsf(e2) <= fabsf(h) * 5.8207661e-11f) || abs(k) > 800) return oz_compose_far(s, w, r, k);  // 2^-34
+    const int b = __float_as_int(h), eh = (b >> 23) & 0xff, bg = __float_as_int(g), eg = (bg >> 23) & 0xff;
+    // |g| in quarters of 2^(exponent of h - 52): 24 bits times 2^7, shifted right by eh - eg - 24 >= 0
+    int q = (int)(((uint32_t)(bg & 0x7fffff) | 0x800000u) << 7 >> min(max(eh - eg - 24, 0), 31));
+    if (eg == 0) q = 0;
+    const float quarter = __int_as_float(min(127 + 54 + 127 - eh, 254) << 23);
+    int x = __float_as_int(__fmaf_rn(e2, quarter, 12582912.f)) - 0x4b400000;  // |e2| is below 2^21 quarters
+    if (b < 0) x = -x;
+    x += (b ^ bg) < 0 ? -q : q;
+    // below a power of two the last place is half as large
+    const int add = (b & 0x7fffff) == 0 && x < 0 ? (x + 1) >> 1 : (x + 2) >> 2;
+    const long long mag = ((long long)(((b & 0x7fffffff) >> 3) + ((896 + k) << 20)) << 32 | (uint32_t)(b << 29)) + add;
+    return eh == 0 ? 0.0 : __longlong_as_double(mag | (long long)(b & 0x80000000) << 32);
+}
+
+// Persistent, one CTA per SM (20 warps, five to a scheduler).  Warps 0-2 fill the ring, each every third K
+// block of the CTA's sequence of tiles (the digit image by bulk copy, the gathered source digits by 16-byte
+// cp.async), the pairs of their next tile already on the way; warp 3 issues the MMAs; warps 4-19 empty the
+// accumulators (three floats per result in registers), free tensor memory for the next tile, and then
+// compose the doubles and store them beside that tile's MMAs (eight epilogue warps with twice the columns,
+// and twice the unrolled code, took longer over it than the MMAs).
+__global__ void __launch_bounds__(OZ_THREADS, 1)
+    k_m2l_oz(const OzP P, const int32_t *__restrict__ group, const int2 *__restrict__ pairs,
+             const unsigned char *__restrict__ Cdig, const int *__restrict__ ec, const unsigned char *__restrict__ img,
+             const int *__restrict__ er, double *Y, int *err, int *err_host) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ uint64_t full[OZ_SLOTS], empty[OZ_SLOTS], done, tfree, fin;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_abort;
+    __shared__ int rowid[OZ_FILL][OZ_N];  // per producer warp: digit row of each pair column (-1: none)
+    __shared__ int s_part[OZ_THREADS / 32];
+    __shared__ int first[(OZ_MAX_LEVELS - 2) * 316 + 1];  // tiles before each group
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    auto give_up = [&] {
+        atomicExch(err, 1);
+        *(volatile int *)err_host = 1;
+        s_abort = 1;
+    };
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < OZ_SLOTS; ++s) {
+            mbar_init(&full[s], 33);  // the filling warp's 32 lanes + the bulk copy's expect_tx
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&done, 1);
+        mbar_init(&tfree, 32 * OZ_EPI);
+        mbar_init(&fin, 1);
+        s_abort = *(volatile int *)err;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512)
+                     : "memory");
+    {  // prefix sum of the groups' tiles
+        const int per = (P.ngroup + OZ_THREADS - 1) / OZ_THREADS, g0 = min(threadIdx.x * per, P.ngroup);
+        const int g1 = min(g0 + per, P.ngroup);
+        int sum = 0;
+        for (int g = g0; g < g1; ++g) sum += oz_tiles(group[g + 1] - group[g], P.W);
+        int inc = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) s_part[warp] = inc;
+        __syncthreads();
+        int at = inc - sum;
+        for (int w = 0; w < warp; ++w) at += s_part[w];
+        for (int g = g0; g < g1; ++g) {
+            first[g] = at;
+            at += oz_tiles(group[g + 1] - group[g], P.W);
+        }
+        if (g0 < g1 && g1 == P.ngroup) first[P.ngroup] = at;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    const int ntile = first[P.ngroup], nunit = ntile * P.ndom * P.mt;
+
+    if (warp < OZ_FILL) {
+        // ------------------------------------------------------------------ producers
+        // source boxes of a tile's columns lane, lane + 32, lane + 64
+        auto sources = [&](const OzTile &t, int *src) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int m = lane + 32 * k;
+                src[k] = m < t.n ? pairs[t.pair0 + (t.col0 + m) / P.W].x : -1;
+            }
+        };
+        int src[3];
+        OzTile t;
+        if ((int)blockIdx.x < nunit) {
+            t = oz_tile(P, blockIdx.x, ntile, first, group);
+            sources(t, src);
+        }
+        int u = 0, turn = 0, last = -1;  // K blocks of the CTA's sequence, u mod OZ_FILL, this warp's last
+        bool stop = false;
+        for (int v = blockIdx.x; v < nunit && !stop; v += gridDim.x) {
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int m = lane + 32 * k, c = (t.col0 + m) % P.W;
+                if (m < OZ_N)
+                    rowid[warp][m] = src[k] >= 0 ? (int)(((int64_t)t.d * P.nbox + src[k]) * P.W + c) : -1;
+            }
+            __syncwarp();
+            const OzTile cur = t;
+            if (v + (int)gridDim.x < nunit) {
+                t = oz_tile(P, v + gridDim.x, ntile, first, group);
+                sources(t, src);
+            }
+            const int n_pad = (cur.n + 15) & ~15;
+            const int64_t mat = (int64_t)cur.d * (P.lmax - 1) * 316 + cur.g;
+            const unsigned char *A = img + (mat * P.mt + cur.mt) * P.kblocks * (int64_t)OZ_A_BYTES;
+            for (int kb = 0; kb < P.kblocks; ++kb, ++u, turn = turn == OZ_FILL - 1 ? 0 : turn + 1) {
+                if (turn != warp) continue;
+                const int slot = u & 3;
+                const uint32_t sA = sbase + (uint32_t)slot * OZ_SLOT_BYTES, sB = sA + OZ_A_BYTES;
+                bool ok = u < OZ_SLOTS || mbar_wait(&empty[slot], (uint32_t)((u >> 2) - 1) & 1u);
+                ok = __all_sync(0xffffffffu, ok && !s_abort);
+                if (!ok) {
+                    if (lane == 0) give_up();
+                    stop = true;
+                    break;
+                }
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(&full[slot], OZ_A_BYTES);
+                    bulk_load(sA, A + (int64_t)kb * OZ_A_BYTES, OZ_A_BYTES, &full[slot]);
+                }
+                // a column's 256 bytes of digits: 16 lanes each, eight columns a lane in one go
+                const int part = lane & 15, dg = part >> 1, ch = part & 1;
+                const unsigned char *src0 = Cdig + (int64_t)kb * OZ_ROW + part * 16;
+                const uint32_t dst0 = sB + (uint32_t)dg * (OZ_N * 32u), stride = (uint32_t)P.kblocks * OZ_ROW;
+                for (int m0 = lane >> 4; m0 < n_pad; m0 += 16) {
+                    int row[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) row[k] = rowid[warp][m0 + 2 * k];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + sw32_chunk(m0 + 2 * k, ch)),
+                                     "l"(src0 + (uint64_t)(uint32_t)max(row[k], 0) * stride), "r"(row[k] >= 0 ? 16 : 0)
+                                     : "memory");
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[slot])) : "memory");
+                last = u;
+            }
+        }
+        // after an abort: wait (bounded) for this warp's last bulk copy
+        if (lane == 0 && s_abort && last >= 0 && !mbar_wait(&full[last & 3], (uint32_t)(last >> 2) & 1u)) give_up();
+    } else if (warp == OZ_FILL) {
+        // ------------------------------------------------------------------ MMA issuer
+        // the whole warp runs the loop, so that descriptors stay in uniform registers (issued by one
+        // divergent lane, an MMA cost 95 cycles, twice its operands' shared-memory reads); one elected
+        // lane issues
+        uint32_t leader;
+        asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
+        bool ok = true;
+        int u = 0, nt = 0;
+        for (int v = blockIdx.x; v < nunit && ok && !s_abort; v += gridDim.x) {
+            const OzTile t = oz_tile(P, v, ntile, first, group);
+            const uint32_t idesc = idesc_bf16((t.n + 15) & ~15);
+            if (nt > 0) ok = __all_sync(0xffffffffu, mbar_wait(&tfree, (uint32_t)(nt - 1) & 1u));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int kb = 0; kb < P.kblocks; ++kb, ++u) {
+                const int s = u & 3;
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)(u >> 2) & 1u));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t sA = sbase + (uint32_t)s * OZ_SLOT_BYTES;
+                const uint64_t da = smem_desc_sw32(sA), db = smem_desc_sw32(sA + OZ_A_BYTES);
+                // a digit of the matrix against every digit it meets, held in the collector after the
+                // first; the smallest products first, so that the shared accumulator loses least
+#pragma unroll
+                for (int i = 0; i < OZ_S; ++i)
+#pragma unroll
+                    for (int j = OZ_S - 1 - i; j >= 0; --j) {
+                        const int dd = i + j;
+                        const uint32_t acc = tmem + (uint32_t)((dd < OZ_ACC ? dd : OZ_ACC - 1) * OZ_N);
+                        const bool head = i == 0 && (dd < OZ_ACC - 1 || dd == OZ_S - 1);
+                        const uint64_t a = da + (uint64_t)((i * (TC_M * 32)) >> 4), b = db + (uint64_t)((j * (OZ_N * 32)) >> 4);
+                        const uint32_t add = head && kb == 0 ? 0u : 1u;
+                        if (i == OZ_S - 1) mma_bf16_if<0>(leader, acc, a, b, idesc, add);
+                        else if (j == OZ_S - 1 - i) mma_bf16_if<1>(leader, acc, a, b, idesc, add);
+                        else if (j > 0) mma_bf16_if<2>(leader, acc, a, b, idesc, add);
+                        else mma_bf16_if<3>(leader, acc, a, b, idesc, add);
+                    }
+                if (leader) mma_commit(&empty[s]);
+                __syncwarp();
+            }
+            if (ok && leader) mma_commit(&done);
+            __syncwarp();
+            ++nt;
+        }
+        if (leader) {  // arrives once every MMA issued above has completed
+            if (nt > 0) mma_commit(&fin);
+            else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&fin)) : "memory");
+            if (!ok) give_up();
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------------ epilogue warps 4..19
+        // warp: accumulator lanes 32 (warp mod 4) .., columns 16 b + 4 sub + j (b < NG, j < 4)
+        const int quarter = warp & 3, sub = (warp - 4) >> 2;
+        constexpr int NG = OZ_N / 16;
+        int nt = 0;
+        for (int v = blockIdx.x; v < nunit; v += gridDim.x) {
+            const OzTile t = oz_tile(P, v, ntile, first, group);
+            const int64_t mat = (int64_t)t.d * (P.lmax - 1) * 316 + t.g;
+            const int R = t.mt * TC_M + quarter * 32 + lane;
+            const bool rows = t.mt * TC_M + quarter * 32 < 2 * P.p2, row_ok = R < 2 * P.p2;
+            const int eR = row_ok ? er[mat * P.p2 + (R >> 1)] : 0;
+            // lane i knows column i of this warp's 20: its row of Y and its exponent
+            const int m = 16 * (lane >> 2) + 4 * sub + (lane & 3);
+            int yr = -1, ex = 0;
+            if (m < t.n && lane < 4 * NG) {
+                const int2 pr = pairs[t.pair0 + (t.col0 + m) / P.W];
+                const int c = (t.col0 + m) % P.W;
+                yr = pr.y * P.W + c;
+                ex = ec[((int64_t)t.d * P.nbox + pr.x) * P.W + c];
+            }
+            bool ok = !s_abort && mbar_wait(&done, (uint32_t)nt & 1u);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) {
+                if (lane == 0) give_up();
+                break;
+            }
+            ++nt;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int ng = rows ? (t.n - 4 * sub + 15) / 16 : 0;  // this warp's column groups in use
+            float hi[4 * NG], mi[4 * NG], lo[4 * NG];
+#pragma unroll
+            for (int b = 0; b < NG; ++b) {
+                if (b < ng) {
+                    uint32_t a[OZ_ACC][4];
+#pragma unroll
+                    for (int k = 0; k < OZ_ACC; ++k) {
+                        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(k * OZ_N + 16 * b + 4 * sub);
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(a[k][0]), "=r"(a[k][1]), "=r"(a[k][2]), "=r"(a[k][3])
+                                     : "r"(ta));
+                    }
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float d0 = __uint_as_float(a[0][j]), d1 = __uint_as_float(a[1][j]);
+                        const float d3 = __uint_as_float(a[3][j]);
+                        const float s = d0 + d1, sb = s - d0;                         // s + e = d0 + d1
+                        const float e = (d0 - (s - sb)) + (d1 - sb);
+                        const float l = e + __uint_as_float(a[2][j]);                 // exact: within 24 bits
+                        const float m = l + d3, mb = m - l;                           // m + .. = l + d3
+                        const float x = ((l - (m - mb)) + (d3 - mb)) + __uint_as_float(a[4][j]);  // exact
+                        const float w = m + x, wb = w - m;                            // w + .. = m + x
+                        hi[4 * b + j] = s;
+                        mi[4 * b + j] = w;
+                        lo[4 * b + j] = ((m - (w - wb)) + (x - wb)) + __uint_as_float(a[5][j]);
+                    }
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tfree)) : "memory");
+            double *Yd = Y + (int64_t)t.d * P.y_dom + R;
+#pragma unroll
+            for (int b = 0; b < NG; ++b) {
+                if (b < ng) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int i = 4 * b + j;
+                        const int o = __shfl_sync(0xffffffffu, yr, i);
+                        const int k = __shfl_sync(0xffffffffu, ex, i) + eR;
+                        const double x = oz_compose(hi[i], mi[i], lo[i], k);
+                        if (row_ok && o >= 0) Yd[(int64_t)o * (2 * P.p2)] = x;
+                    }
+                }
+            }
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    if (threadIdx.x == 0 && !mbar_wait(&fin, 0)) give_up();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+}
+
+__global__ void k_oz_pairs(int64_t n, const int32_t *pair_e, const int32_t *ff_src, int2 *out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < n) out[i] = make_int2(ff_src[pair_e[i]], pair_e[i]);
+}
+
+int oz_kblocks(int p2) { return (2 * p2 + 15) / 16; }
+int oz_mt(int p2) { return (2 * p2 + TC_M - 1) / TC_M; }
+
+}  // namespace
+
+// even p in 4..10: K = 2 p^2 <= 200 keeps the digit sums exact, and a K block of 16 ends at a whole
+// coefficient
+bool m2l_oz_supported(const fmbem *h) {
+    return h->p >= 4 && h->p <= 10 && h->p % 2 == 0 && h->lmax >= 2 && h->lmax < OZ_MAX_LEVELS && !h->opt.fp32_only;
+}
+
+// digit images of every S|R matrix of levels 2..l_max; not built when they would take more than an
+// eighth of the free device memory (the FP64 pipe's kernels then remain)
+void build_oz_tables(fmbem *h, cudaStream_t s) {
+    const int p2 = h->p2, kb = oz_kblocks(p2), mt = oz_mt(p2), sets = (h->Jf + 1) * (h->lmax - 1);
+    const int64_t nmat = (int64_t)sets * 316, bytes = nmat * mt * kb * (int64_t)OZ_A_BYTES;
+    size_t free_b = 0, total_b = 0;
+    CK(cudaMemGetInfo(&free_b, &total_b));
+    if (h->n_ff <= 0 || h->tc_err == nullptr || (size_t)bytes > free_b / 8) return;
+    h->oz_group = (int32_t *)dev_alloc(h, sizeof(int32_t) * h->h_group_beg.size());
+    CK(cudaMemcpyAsync(h->oz_group, h->h_group_beg.data(), sizeof(int32_t) * h->h_group_beg.size(), cudaMemcpyHostToDevice, s));
+    h->oz_pairs = dev_alloc(h, sizeof(int2) * h->n_ff);
+    k_oz_pairs<<<(unsigned)((h->n_ff + 255) / 256), 256, 0, s>>>(h->n_ff, h->pair_e, h->ff_src, (int2 *)h->oz_pairs);
+    CKL("k_oz_pairs");
+    h->oz_bal = (int *)dev_alloc(h, sizeof(int) * sets * h->p);
+    h->oz_er = (int *)dev_alloc(h, sizeof(int) * nmat * p2);
+    h->oz_img = dev_alloc(h, bytes);
+    CK(cudaHostAlloc((void **)&h->oz_err_host, sizeof(int), cudaHostAllocMapped));
+    *h->oz_err_host = 0;
+    k_oz_balance<<<dim3((unsigned)sets, (unsigned)h->p), 256, 0, s>>>(h->T_m2l64, h->p, h->lmax, h->oz_bal);
+    CKL("k_oz_balance");
+    k_oz_images<<<(unsigned)nmat, 256, 0, s>>>(h->T_m2l64, h->p, h->lmax, mt, kb, h->oz_bal, (unsigned char *)h->oz_img,
+                                               h->oz_er);
+    CKL("k_oz_images");
+}
+
+// doubles of Y per domain for a window of W columns, and bytes of the window's digits and exponents
+int64_t oz_y_dom(const fmbem *h, int W) { return h->n_ff * W * 2 * h->p2; }
+size_t oz_digit_bytes(const fmbem *h, int W) {
+    const size_t rows = (size_t)(h->Jf + 1) * h->nbox * W;
+    return rows * oz_kblocks(h->p2) * OZ_ROW + rows * sizeof(int);
+}
+
+// the S|R products of every level and domain for columns col0 .. col0 + W - 1 of C (3 n_rhs columns)
+// into Y[d][CSR position][W][p^2] (domains oz_y_dom apart)
+void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s) {
+    if (h->n_ff <= 0) return;
+    const int p2 = h->p2, kb = oz_kblocks(p2), ndom = h->Jf + 1;
+    OzLevels L{};
+    L.lmax = h->lmax;
+    for (int l = 2; l <= h->lmax; ++l) L.off[l] = h->lev[l].off;
+    L.off[h->lmax + 1] = h->nbox;
+    const int64_t rows = (int64_t)ndom * (h->nbox - L.off[2]) * W;
+    unsigned char *dig = (unsigned char *)h->oz_dig;
+    int *ec = (int *)(dig + (size_t)ndom * h->nbox * W * kb * OZ_ROW);
+    k_oz_split<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(C, L, h->nbox, 3 * nr, col0, W, ndom, h->p, kb, h->oz_bal, dig, ec);
+    CKL("k_oz_split");
+    OzP P{};
+    P.nbox = h->nbox;
+    P.W = W;
+    P.p2 = p2;
+    P.kblocks = kb;
+    P.lmax = h->lmax;
+    P.ndom = ndom;
+    P.mt = oz_mt(p2);
+    P.ngroup = (h->lmax - 1) * 316;
+    P.y_dom = oz_y_dom(h, W);
+    int64_t tiles = 0;
+    for (int g = 0; g < P.ngroup; ++g) tiles += oz_tiles(h->h_group_beg[g + 1] - h->h_group_beg[g], W);
+    const size_t smem = OZ_SLOTS * (size_t)OZ_SLOT_BYTES + 1024;
+    CK(cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int dev = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    // an odd grid: a CTA then alternates between the row tiles, of which the second is the shorter
+    const int64_t grid = std::min<int64_t>(tiles * ndom * P.mt, (nsm - 1) | 1);
+    if (grid <= 0) return;
+    k_m2l_oz<<<(unsigned)grid, OZ_THREADS, smem, s>>>(P, h->oz_group, (const int2 *)h->oz_pairs, dig, ec,
+                                                      (const unsigned char *)h->oz_img, h->oz_er, (double *)Y, h->tc_err,
+                                                      h->oz_err_host);
+    CKL("k_m2l_oz");
+}
+
+// a wait of the FP64 tensor-core M2L that ran out on an earlier product of this handle
+void check_oz_err(fmbem *h, cudaStream_t s) {
+    if (h->oz_err_host == nullptr || *(volatile int *)h->oz_err_host == 0) return;
+    *(volatile int *)h->oz_err_host = 0;
+    CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
+    throw fmbem_error{FMBEM_ERR_DEVICE_TIMEOUT, "tensor-core M2L (FP64): an mbarrier wait timed out"};
+}

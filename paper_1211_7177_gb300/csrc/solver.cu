@@ -627,6 +627,7 @@ fmbem_status run_solve(fmbem *h, const c64 *b, c64 *x, int64_t nr, double tol, i
             its = itot;
         }
         CK(cudaStreamSynchronize(s));
+        check_oz_err(h, s);
     } catch (...) {
         dev_free(h, W.partial);
         dev_free(h, W.dres);

@@ -614,6 +614,8 @@ void build_tables(fmbem *h, cudaStream_t s) {
     if (m2l_tc_supported(h) && !h->opt.fp32_only) build_tc_tables(h, s);
     // bf16 S|R images for the offset-stationary few-column tensor-core M2L (BF16x3)
     if (m2l_ofs_supported(h) && !h->opt.fp32_only) build_ofs_tables(h, s);
+    // digit images for the FP64 tensor-core M2L; an explicit m2l_rotation keeps the form it names
+    if (m2l_oz_supported(h) && h->opt.m2l_rotation == -1) build_oz_tables(h, s);
     if (h->opt.fp32_only) {  // single-precision tables only: the FP64 bases and matrices go
         CK(cudaStreamSynchronize(s));
         for (c64 **q : {&h->T_m2l64, &h->T_mm64, &h->T_ll64, &h->B_p2m64, &h->B_l2p64, &h->B_l2pg64}) {

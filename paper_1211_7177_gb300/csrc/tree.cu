@@ -777,13 +777,17 @@ void build_tree(fmbem *h, cudaStream_t s) {
         std::vector<int32_t> hb(316), hbeg(316);
         std::vector<int32_t> cbeg, ccnt;
         std::vector<int16_t> coff;
+        h->h_group_beg.clear();
         h->h_chunk_first.assign(lmax + 2, 0);
         h->h_pair_first.assign(lmax + 2, 0);
         for (int l = 0; l <= lmax + 1; ++l) h->h_pair_first[l] = l <= lmax ? hs[h->lev[l].off] : hs[tot];
         for (int l = 0; l <= lmax; ++l) {
             h->h_chunk_first[l] = (int64_t)cbeg.size();
             const int64_t e0 = hs[h->lev[l].off], e1 = hs[h->lev[l].off + h->lev[l].n];
-            if (e1 <= e0) continue;
+            if (e1 <= e0) {
+                if (l >= 2) h->h_group_beg.insert(h->h_group_beg.end(), 316, (int32_t)e0);
+                continue;
+            }
             CK(cudaMemsetAsync(ocnt, 0, sizeof(int32_t) * 316, s));
             k_count_offsets<<<nblk(e1 - e0, TB), TB, 0, s>>>(e0, e1, h->ff_off, ocnt);
             CKL("k_count_offsets");
@@ -792,6 +796,7 @@ void build_tree(fmbem *h, cudaStream_t s) {
             int32_t acc = (int32_t)e0;
             for (int o = 0; o < 316; ++o) {
                 hbeg[o] = acc;
+                h->h_group_beg.push_back(acc);
                 for (int32_t c = 0; c < hb[o]; c += M2L_CHUNK) {
                     cbeg.push_back(acc + c);
                     ccnt.push_back(std::min(M2L_CHUNK, hb[o] - c));
@@ -804,6 +809,7 @@ void build_tree(fmbem *h, cudaStream_t s) {
             CKL("k_fill_offsets");
         }
         h->h_chunk_first[lmax + 1] = (int64_t)cbeg.size();
+        h->h_group_beg.push_back(hs[tot]);
         const size_t nc = std::max<size_t>(cbeg.size(), 1);
         h->chunk_beg = (int32_t *)dev_alloc(h, sizeof(int32_t) * nc);
         h->chunk_cnt = (int32_t *)dev_alloc(h, sizeof(int32_t) * nc);
