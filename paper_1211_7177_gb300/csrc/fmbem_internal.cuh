@@ -152,6 +152,11 @@ struct fmbem {
     int4 *near_items = nullptr;  // warp work items of the near field (leaf, target offset, tg, nsl)
     int n_near_items = 0;
     int *near_next = nullptr;    // unit counter of the persistent near-field kernels, reset per launch
+    int4 *near_ditems = nullptr;  // items of the double-precision near field (k_near_d): leaf, target offset, tg, nsl
+    int n_near_ditems = 0;
+    int64_t near_tiles_max = 0;   // 32-source tiles of the longest source list
+    c64 *near_am = nullptr, *near_part = nullptr;  // its per-source vectors and partial sums (scratch)
+    size_t near_am_bytes = 0, near_part_bytes = 0;
     int4 *near_groups = nullptr;  // target groups of the lane-per-RHS near field (leaf, target offset, count, -):
                                   // n_near_groups in leaf order, then the same sorted by pair work
     int n_near_groups = 0;

@@ -35,7 +35,7 @@ struct DomainConsts {  // per domain, device array
 template <typename R>
 __device__ __forceinline__ void prep_body(int64_t N, int64_t nr, const c64 *x, const int32_t *perm, const double *nrm,
                                           const double *w, const int32_t *dom, const DomainConsts *dc, cx<R> *dens,
-                                          int64_t bx, int64_t by, cx<R> *sj = nullptr) {
+                                          int64_t bx, int64_t by, cx<R> *sj = nullptr, cx<R> *am = nullptr) {
     int64_t i = bx * (int64_t)blockDim.x + threadIdx.x;
     int64_t r = by;
     if (i >= N) return;
@@ -59,11 +59,20 @@ __device__ __forceinline__ void prep_body(int64_t N, int64_t nr, const c64 *x, c
         d1[3 + q] = gw * Psi[q];
     }
     if (sj) sj[r * N + i] = wi * tn;  // v_1 - v_0 = s n (see k_near_ws)
+    if (am) {  // n . v_0, v_0 x n and s (see k_near_d)
+        cx<R> *o = am + (r * N + i) * 5;
+        const cx<R> v[3] = {wi * Phi[0], wi * Phi[1], wi * Phi[2]};
+        o[0] = n[0] * v[0] + n[1] * v[1] + n[2] * v[2];
+        o[1] = n[2] * v[1] - n[1] * v[2];
+        o[2] = n[0] * v[2] - n[2] * v[0];
+        o[3] = n[1] * v[0] - n[0] * v[1];
+        o[4] = wi * tn;
+    }
 }
 template <typename R>
 __global__ void k_prep(int64_t N, int64_t nr, const c64 *x, const int32_t *perm, const double *nrm, const double *w,
-                       const int32_t *dom, const DomainConsts *dc, cx<R> *dens, cx<R> *sj) {
-    prep_body<R>(N, nr, x, perm, nrm, w, dom, dc, dens, blockIdx.x, blockIdx.y, sj);
+                       const int32_t *dom, const DomainConsts *dc, cx<R> *dens, cx<R> *sj, cx<R> *am) {
+    prep_body<R>(N, nr, x, perm, nrm, w, dom, dc, dens, blockIdx.x, blockIdx.y, sj, am);
 }
 
 // The single-precision densities straight into the node-major layout below (k_dens_node_major's
@@ -1776,6 +1785,192 @@ __global__ void __launch_bounds__(32 * NW_WARPS, 4) k_near_w(
     }
 }
 
+// The near field in double precision, any number of right-hand sides, both sides of every pair in one
+// pass.  Bound by the FP64 pipe (a warp instruction keeps a quarter of an SM busy for 64 cycles), so what
+// counts is FP64 instructions per pair, idle lanes and SMs without work:
+//   - with a = n.v_0 and m = v_0 x n per source (k_prep), the bracket is U = a r + r x m, 18 operations;
+//     the two sides are tied as in k_near_ws (v_1 = v_0 + s n, q_1 = -gamma_j q_0); with the cached pair
+//     scalars g, c of both wavenumbers a pair takes 75 operations (84 with w = n x r formed per pair);
+//   - a warp owns tg targets of a leaf x nsl = 32 / tg source slices, the tg that leaves least lanes idle;
+//   - the sources of an item are split over nsp units where there are fewer items than warps to fill the
+//     chip; the partial sums go to part[split][r][node][6] and k_near_finish adds them in order, with the
+//     far field and the self block.
+// A block per leaf before: 2562 nodes 1159 us (56 leaves on 152 SMs), 163842 nodes 16.7 ms.
+constexpr int ND_WARPS = 4;
+struct NearDTile {  // 32 sources: position and scatterer, a and m, s and q
+    V4<double> pos[32];
+    double2 am[4][32], s[32], q[3][32];
+};
+template <bool CACHED>
+__global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_d(
+    const int32_t *__restrict__ leaf_box, const int4 *__restrict__ items, int n_items, int n_units, int nsp,
+    int *next_unit, int64_t N, int64_t nr, const int32_t *__restrict__ nbeg, const int32_t *__restrict__ nend,
+    const int32_t *__restrict__ nbr_start, const int32_t *__restrict__ nbr_idx, const double *__restrict__ pos,
+    const int32_t *__restrict__ dom, const c64 *__restrict__ dens, const c64 *__restrict__ am, const DomainConsts *dc,
+    const int64_t *__restrict__ cache_base, const V4<double> *__restrict__ cache, c64 *part, bool side1) {
+    __shared__ NearDTile tiles[ND_WARPS];
+    __shared__ int rng_beg[ND_WARPS][32], rng_cum[ND_WARPS][33];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    NearDTile &T = tiles[warp];
+    int *rb_ = rng_beg[warp], *rc_ = rng_cum[warp];
+    for (;;) {
+        int unit = 0;
+        if (lane == 0) unit = atomicAdd(next_unit, 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        // (item, right-hand side, split), items with the most work first
+        const int item_id = unit / (int)(nr * nsp), rem = unit - item_id * (int)(nr * nsp);
+        const int64_t r = rem / nsp;
+        const int sp = rem - (int)r * nsp;
+        __syncwarp();  // the previous unit's shared-memory reads are done
+        const int4 it = items[item_id];
+        const int leaf = it.x, tg = it.z, nsl = it.w;
+        const int64_t g = leaf_box[leaf];
+        const int nb0 = nbr_start[leaf], nnb = nbr_start[leaf + 1] - nb0;
+        {
+            int beg = 0, cnt = 0;
+            if (lane < nnb) {
+                const int b = nbr_idx[nb0 + lane];
+                beg = nbeg[b];
+                cnt = nend[b] - beg;
+            }
+            int incl = cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane < nnb) { rb_[lane] = beg; rc_[lane] = incl - cnt; }
+            if (lane == nnb - 1) rc_[nnb] = incl;
+        }
+        __syncwarp();
+        const int nsrc = rc_[nnb], ntile = (nsrc + 31) / 32;
+        const int tile0 = (int)((int64_t)sp * ntile / nsp), tile1 = (int)((int64_t)(sp + 1) * ntile / nsp);
+        const int ti = lane % tg, sl = lane / tg;
+        const bool busy = sl < nsl;
+        const int t0 = nbeg[g], NT = nend[g] - t0, a = t0 + it.y + ti;
+        const double ax = pos[3 * a], ay = pos[3 * a + 1], az = pos[3 * a + 2];
+        const int adom = side1 ? dom[a] : -1;
+        const c64 k0 = dc[0].k, kj = dc[max(adom, 0)].k;
+        const V4<double> *cs = CACHED ? cache + 2 * cache_base[leaf] + (it.y + ti) : nullptr;
+        const c64 *d0 = dens + r * N * 6, *amr = am + r * N * 5;
+        c64 acc0[3], acc1[3], bq[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc0[c] = acc1[c] = bq[c] = {0, 0};
+        for (int t = tile0; t < tile1; ++t) {
+            const int e0 = t * 32;
+            __syncwarp();  // the tile before is no longer read
+            if (e0 + lane < nsrc) {
+                const int q = source_range(rc_, nnb, e0 + lane);
+                const int64_t i = rb_[q] + (e0 + lane - rc_[q]);
+                T.pos[lane] = V4<double>{pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], (double)dom[i]};
+                const double2 *A = reinterpret_cast<const double2 *>(amr + 5 * i);
+                const double2 *Q = reinterpret_cast<const double2 *>(d0 + 6 * i);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) T.am[c][lane] = A[c];
+                T.s[lane] = A[4];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) T.q[c][lane] = Q[3 + c];
+            }
+            __syncwarp();
+            const int ns = busy ? min(32, nsrc - e0) : 0;
+            for (int u = sl; u < ns; u += nsl) {
+                const V4<double> p = T.pos[u];
+                const double rx = p.x - ax, ry = p.y - ay, rz = p.z - az;
+                c64 g0, c0, g1, c1;
+                const bool same = p.w == (double)adom;
+                if (CACHED) {
+                    const V4<double> v0 = cs[(int64_t)(e0 + u) * NT];
+                    g0 = {v0.x, v0.y};
+                    c0 = {v0.z, v0.w};
+                    if (same) {
+                        const V4<double> v1 = cs[((int64_t)nsrc + e0 + u) * NT];
+                        g1 = {v1.x, v1.y};
+                        c1 = {v1.z, v1.w};
+                    }
+                } else {
+                    const double R2 = rx * rx + ry * ry + rz * rz;
+                    const double inv = R2 > 0.0 ? rsqrt_(R2) : 0.0, Rr = R2 * inv;  // the node itself drops out
+                    pair_scalars<double>(inv, Rr, k0, g0, c0);
+                    if (same) pair_scalars<double>(inv, Rr, kj, g1, c1);
+                }
+                const double2 A = T.am[0][u], m0 = T.am[1][u], m1 = T.am[2][u], m2 = T.am[3][u];
+                // U = a r + r x m
+                c64 U[3] = {{fma(A.x, rx, fma(ry, m2.x, -rz * m1.x)), fma(A.y, rx, fma(ry, m2.y, -rz * m1.y))},
+                            {fma(A.x, ry, fma(rz, m0.x, -rx * m2.x)), fma(A.y, ry, fma(rz, m0.y, -rx * m2.y))},
+                            {fma(A.x, rz, fma(rx, m1.x, -ry * m0.x)), fma(A.y, rz, fma(rx, m1.y, -ry * m0.y))}};
+                const c64 mc = {-c0.re, -c0.im};
+                c64 q[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    q[c] = {T.q[c][u].x, T.q[c][u].y};
+                    cfma(acc0[c], mc, U[c]);
+                    cfma(acc0[c], g0, q[c]);
+                }
+                if (same) {
+                    const double2 s = T.s[u];
+                    U[0] = {fma(s.x, rx, U[0].re), fma(s.y, rx, U[0].im)};
+                    U[1] = {fma(s.x, ry, U[1].re), fma(s.y, ry, U[1].im)};
+                    U[2] = {fma(s.x, rz, U[2].re), fma(s.y, rz, U[2].im)};
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        cfma(acc1[c], c1, U[c]);
+                        cfma(bq[c], g1, q[c]);
+                    }
+                }
+            }
+        }
+        if (side1) {
+            const c64 mg = dc[adom].gamma;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cfma(acc1[c], c64{-mg.re, -mg.im}, bq[c]);
+        }
+        // sum the slices of each target in order, through the tile's shared memory
+        c64 *S = reinterpret_cast<c64 *>(&T);  // [6][32]
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            S[c * 32 + lane] = acc0[c];
+            S[(3 + c) * 32 + lane] = acc1[c];
+        }
+        __syncwarp();
+        for (int o = lane; o < tg * 6; o += 32) {
+            const int tt = o / 6, row = o - tt * 6;
+            c64 v = S[row * 32 + tt];
+            for (int k = 1; k < nsl; ++k) v += S[row * 32 + k * tg + tt];
+            part[(((int64_t)sp * nr + r) * N + t0 + it.y + tt) * 6 + row] = v;
+        }
+    }
+}
+
+// the rows of k_near_d: partial sums in split order, the far field (L2P) of the row's domain and the row
+// of the self block; thread per (node, row), grid (.., right-hand side)
+__global__ void __launch_bounds__(192) k_near_finish(int64_t N, int64_t nr, int nsp, int p2, int64_t nbox,
+                                                     const int32_t *__restrict__ node_leaf, const int32_t *__restrict__ dom,
+                                                     const int32_t *__restrict__ perm, const c64 *__restrict__ Bl2p,
+                                                     const c64 *__restrict__ D, const c64 *__restrict__ Mself,
+                                                     const c64 *__restrict__ x, const c64 *__restrict__ part, c64 *y) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (i >= N * 6) return;
+    const int64_t a = i / 6;
+    const int row = (int)(i - a * 6), sd = row / 3, c = row % 3;
+    c64 v = part[(r * N + a) * 6 + row];
+    for (int s = 1; s < nsp; ++s) v += part[((s * nr + r) * N + a) * 6 + row];
+    const int d = sd == 0 ? 0 : dom[a];
+    const c64 *Dl = D + (((int64_t)d * nbox + node_leaf[a]) * 3 * nr + 3 * r + c) * p2, *B = Bl2p + ((int64_t)sd * N + a) * p2;
+    c64 w = {0, 0};
+    int q = 0;
+    for (; q + 1 < p2; q += 2) {  // two chains
+        cfma(v, Dl[q], B[q]);
+        cfma(w, Dl[q + 1], B[q + 1]);
+    }
+    if (q < p2) cfma(v, Dl[q], B[q]);
+    v += w;
+    const int64_t u = perm[a];
+    const c64 *M = Mself + 36 * u + 6 * row, *xa = x + (r * N + u) * 6;
+    for (int cc = 0; cc < 6; ++cc) cfma(v, M[cc], xa[cc]);
+    y[(r * N + u) * 6 + row] = v;
+}
+
 // Steps 4-5 for one to three right-hand sides in single precision, both sides of every pair in
 // one pass.  One warp owns one unit: an item of near_work_items (tg targets of one leaf over nsl
 // source slices) and one right-hand side.  The densities of k_prep tie the two sides together:
@@ -2887,6 +3082,39 @@ void near_work_items(fmbem *h, cudaStream_t s) {
     h->near_items = (int4 *)dev_alloc(h, sizeof(int4) * items.size());
     h->near_next = (int *)dev_alloc(h, sizeof(int));
     CK(cudaMemcpyAsync(h->near_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s));
+    // items of k_near_d: tg targets x nsl = floor(32 / tg) slices, the tg of least lane time
+    // ceil(nt / tg) / nsl (from 4: fewer targets reload the sources too often), most work first
+    {
+        std::vector<int4> ditems;
+        std::vector<int64_t> dcost;
+        for (int64_t leaf = 0; leaf < nl; ++leaf) {
+            const int nt = ne[leaf] - nb[leaf];
+            if (nt <= 0) continue;
+            int tg = std::min(nt, 32);
+            double best = 1e30;
+            for (int k = std::min(nt, 32); k >= std::min(nt, 4); --k) {
+                const double c = (double)((nt + k - 1) / k) / (32 / k);
+                if (c < best - 1e-12) { best = c; tg = k; }
+            }
+            int64_t nsrc = 0;
+            for (int q = ns[leaf]; q < ns[leaf + 1]; ++q) nsrc += neA[ni[q]] - nbA[ni[q]];
+            for (int t = 0; t < nt; t += tg) {
+                const int cnt = std::min(tg, nt - t);
+                ditems.push_back(int4{(int)leaf, t, cnt, 32 / cnt});
+                dcost.push_back((nsrc + 32 / cnt - 1) / (32 / cnt));
+            }
+            h->near_tiles_max = std::max<int64_t>(h->near_tiles_max, (nsrc + 31) / 32);
+        }
+        std::vector<int> dorder(ditems.size());
+        for (size_t k = 0; k < dorder.size(); ++k) dorder[k] = (int)k;
+        std::stable_sort(dorder.begin(), dorder.end(), [&](int u, int v) { return dcost[u] > dcost[v]; });
+        std::vector<int4> dsorted(ditems.size());
+        for (size_t k = 0; k < dorder.size(); ++k) dsorted[k] = ditems[dorder[k]];
+        h->n_near_ditems = (int)ditems.size();
+        h->near_ditems = (int4 *)dev_alloc(h, sizeof(int4) * std::max<size_t>(ditems.size(), 1));
+        CK(cudaMemcpyAsync(h->near_ditems, dsorted.data(), sizeof(int4) * dsorted.size(), cudaMemcpyHostToDevice, s));
+        CK(cudaStreamSynchronize(s));
+    }
     // target groups of at most NR_TT targets per leaf for k_near_r, near-equal sizes: in leaf
     // (Morton) order, so that concurrent units share sources in L2, and again with the most pair
     // work first, for the last slab
@@ -3043,6 +3271,32 @@ static size_t oz_ybuf_need(const fmbem *h, int W) {
 static bool oz_ready(const fmbem *h, int W) {
     return W > 0 && h->oz_dig != nullptr && h->oz_dig_bytes >= oz_digit_bytes(h, W) && h->ybuf != nullptr &&
            h->ybuf_bytes >= oz_ybuf_need(h, W);
+}
+
+// source splits per item of k_near_d: about eight units for each of the 608 warp schedulers, no more than
+// the longest source list has tiles, eight at most (the partial sums' buffer)
+static int near_d_splits(const fmbem *h, int64_t nr) {
+    const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_ditems * nr);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({8, h->near_tiles_max, (8 * 608 + units - 1) / units}));
+}
+// the near field's partial sums (rows complex values of a node and right-hand side; units of rb
+// right-hand sides), and per-source vectors of the FP64 forward product
+static void ensure_near_scratch(fmbem *h, int64_t nr, int rb, int rows, bool am) {
+    const size_t npart = sizeof(c64) * rows * h->N * nr * near_d_splits(h, (nr + rb - 1) / rb), nam = sizeof(c64) * 5 * h->N * nr;
+    if (h->near_part_bytes < npart) {
+        if (h->near_part) dev_free(h, h->near_part);
+        h->near_part = nullptr;
+        h->near_part_bytes = 0;
+        h->near_part = (c64 *)dev_alloc(h, npart);
+        h->near_part_bytes = npart;
+    }
+    if (am && h->near_am_bytes < nam) {
+        if (h->near_am) dev_free(h, h->near_am);
+        h->near_am = nullptr;
+        h->near_am_bytes = 0;
+        h->near_am = (c64 *)dev_alloc(h, nam);
+        h->near_am_bytes = nam;
+    }
 }
 
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_results = true) {
@@ -3412,7 +3666,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
         CKL("k_prep_node_major");
     } else {
         k_prep<R><<<dim3(nblk(N, 128), (unsigned)nr), 128, 0, s>>>(N, nr, x, h->perm, h->nrm, h->w, h->dom, dc, dens,
-                                                                    sj);
+                                                                    sj, f32 ? nullptr : (cx<R> *)h->near_am);
         CKL("k_prep");
         if (densT != nullptr) {
             k_dens_node_major<<<dim3((unsigned)((N + 15) / 16), (unsigned)(nrT / 32)), 256, 0, s>>>(
@@ -3528,7 +3782,27 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                 h->nbox, (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y, !h->ibc);
             CKL("k_near_ws");
         }
-    } else if (nr >= 4) {
+    } else if (h->near_am != nullptr) {
+        const int nsp = near_d_splits(h, nr);
+        const int64_t units = (int64_t)h->n_near_ditems * nr * nsp;
+        if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
+        auto launch_d = [&](auto kern) {
+            int per_sm = 0;
+            CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * ND_WARPS, 0));
+            const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((units + ND_WARPS - 1) / ND_WARPS,
+                                                                        (int64_t)std::max(per_sm, 1) * nsm));
+            CK(cudaMemsetAsync(h->near_next, 0, sizeof(int), s));
+            kern<<<(unsigned)grid, 32 * ND_WARPS, 0, s>>>(
+                h->leaf_box, h->near_ditems, h->n_near_ditems, (int)units, nsp, h->near_next, N, nr, h->box_nbeg,
+                h->box_nend, h->nbr_start, h->nbr_idx, h->pos, h->dom, dens, h->near_am, dc, h->near_base,
+                (const V4<double> *)h->near_cache64, h->near_part, !h->ibc);
+            CKL("k_near_d");
+        };
+        if (h->near_cache64) launch_d(k_near_d<true>);
+        else launch_d(k_near_d<false>);
+        k_near_finish<<<dim3(nblk(6 * N, 192), (unsigned)nr), 192, 0, s>>>(N, nr, nsp, p2, h->nbox, h->node_leaf, h->dom, h->perm,
+                                                                          Bl2p, D, h->Mself, x, h->near_part, y);
+    } else if (nr >= 4) {  // the allocation-free product
         constexpr int RBLK = 2;
         const size_t smn = sizeof(NearSmemRB<R, RBLK>);
         CK(cudaFuncSetAttribute(k_near_rb<R, false, RBLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smn));
@@ -3628,6 +3902,7 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
+    if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, 1, 6, true);
     static_assert(sizeof(DomainConsts) == 3 * sizeof(c64), "layout");
     DomainConsts *dc = (DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
@@ -3699,16 +3974,19 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     // run the regular passes on pointers into the static array; the handle's own scratch
     // pointers are restored afterwards, so fmbem_matvec is unaffected
     void *sv_dens = h->dens, *sv_C = h->Cexp, *sv_D = h->Dexp, *sv_y = h->ybuf, *sv_dig = h->oz_dig;
+    c64 *sv_am = h->near_am;
     const size_t sv_yb = h->ybuf_bytes;
     auto restore = [&] {
         h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y; h->ybuf_bytes = sv_yb; h->oz_dig = sv_dig;
+        h->near_am = sv_am;
     };
     h->dens = base;
     h->Cexp = base + b_dens;
     h->Dexp = base + b_dens + b_exp;
     h->ybuf = b_y ? base + b_dens + 2 * b_exp : nullptr;
     h->ybuf_bytes = b_y;
-    h->oz_dig = nullptr;  // no digits in the static array: the FP64 pipe's translations
+    h->oz_dig = nullptr;  // no digits in the static array: the FP64 pipe's translations,
+    h->near_am = nullptr;  // and no partial sums: the near field by a block per leaf
     try {
         matvec_impl<R>(h, x, y, nr, s, (const DomainConsts *)h->dcons);
     } catch (...) {
