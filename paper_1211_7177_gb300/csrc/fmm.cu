@@ -2593,209 +2593,255 @@ __global__ void k_p2m_adj(const int32_t *leaf_box, int64_t N, int64_t nr, int p2
     }
 }
 
-template <typename R>
-struct AdjTile {
-    V4<R> pa[128];      // position (high part) and scatterer id
-    V4<R> pb[128];      // position low part (double-float only)
-    cx<R> xv[3][128];   // the side's monopole strengths
+// The transposed near field by warps, both sides of every pair in one pass (the units, slices and splits of
+// k_near_d).  With w = r x n, r = s_a - s_b and n the target's normal, the three gradient terms of u above
+// are, per source and side, +-c B(x), B(x) = x x w - (n.r) x (the target sees -n on the background side), so
+// a pair keeps 3 + 3 sums per side instead of the 3 + 9 of phi and grad phi, and geometry, w and, in single
+// precision, the pair scalars of RB right-hand sides are formed once.  Partial sums (u near, phi near of both
+// sides) go to part[split][r][node][12]; k_near_adj_finish adds them, the far field and the self block.
+// A block per leaf, right-hand side and side before, L2P by one thread per target: 17026 nodes x 3 RHS in
+// single precision 915 us, 10242 nodes in double 2865 us.
+template <typename R, int RB>
+struct AdjTile {  // 32 sources: position (high part) and scatterer, low part, x of both sides
+    V4<R> pa[32], pb[32];
+    V2<R> x[RB][2][3][32];
 };
-template <typename R>
-union AdjSmem {
-    AdjTile<R> tile;
-    cx<R> red[12][128];  // per source slice: phi (3) and grad phi (9)
-};
-
-// near field, L2P (value and gradient), assembly and the transposed self block for one leaf;
-// threads split as (target, source slice) like k_near, both domains one after the other; grid
-// (leaf, right-hand side)
-template <typename R, bool DOUBLE_FLOAT>
-__global__ void __launch_bounds__(128) k_near_adj(const int32_t *leaf_box, int64_t N, int64_t nr, int p2, int64_t nbox,
-                                                  const int32_t *nbeg, const int32_t *nend, const int32_t *nbr_start,
-                                                  const int32_t *nbr_idx, const R *pos_hi, const R *pos_lo,
-                                                  const double *nrm, const double *w, const int32_t *dom,
-                                                  const int32_t *perm, const cx<R> *dens, const DomainConsts *dc,
-                                                  const cx<R> *Bl2p, const cx<R> *Bl2pg, const cx<R> *D,
-                                                  const c64 *Mself, const c64 *x, c64 *y, const int64_t *cache_base,
-                                                  const V4<R> *cache) {
-    __shared__ AdjSmem<R> S;
-    __shared__ int rng_beg[32], rng_cum[33];
-    AdjTile<R> &T = S.tile;
-    const int64_t g = leaf_box[blockIdx.x];
-    const int nb0 = nbr_start[blockIdx.x], nnb = nbr_start[blockIdx.x + 1] - nb0;
-    if (threadIdx.x == 0) {
-        int cum = 0;
-        for (int q = 0; q < nnb; ++q) {
-            const int b = nbr_idx[nb0 + q];
-            rng_beg[q] = nbeg[b];
-            rng_cum[q] = cum;
-            cum += nend[b] - nbeg[b];
+template <typename R, bool CACHED, int RB>
+__global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
+    const int32_t *__restrict__ leaf_box, const int4 *__restrict__ items, int n_items, int n_units, int nsp, int nrb,
+    int *next_unit, int64_t N, int64_t nr, const int32_t *__restrict__ nbeg, const int32_t *__restrict__ nend,
+    const int32_t *__restrict__ nbr_start, const int32_t *__restrict__ nbr_idx, const R *__restrict__ pos_hi,
+    const R *__restrict__ pos_lo, const double *__restrict__ nrm, const int32_t *__restrict__ dom,
+    const cx<R> *__restrict__ dens, const DomainConsts *dc, const int64_t *__restrict__ cache_base,
+    const V4<R> *__restrict__ cache, cx<R> *part) {
+    constexpr bool LO = sizeof(R) == 4;  // double-float positions
+    __shared__ AdjTile<R, RB> tiles[ND_WARPS];
+    __shared__ int rng_beg[ND_WARPS][32], rng_cum[ND_WARPS][33];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    AdjTile<R, RB> &T = tiles[warp];
+    int *rb_ = rng_beg[warp], *rc_ = rng_cum[warp];
+    for (;;) {
+        int unit = 0;
+        if (lane == 0) unit = atomicAdd(next_unit, 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= n_units) break;
+        const int item_id = unit / (nrb * nsp), rem = unit - item_id * (nrb * nsp);
+        const int rblk = rem / nsp, sp = rem - rblk * nsp;
+        const int64_t r0 = (int64_t)rblk * RB;
+        __syncwarp();  // the previous unit's shared-memory reads are done
+        const int4 it = items[item_id];
+        const int leaf = it.x, tg = it.z, nsl = it.w;
+        const int64_t g = leaf_box[leaf];
+        const int nb0 = nbr_start[leaf], nnb = nbr_start[leaf + 1] - nb0;
+        {
+            int beg = 0, cnt = 0;
+            if (lane < nnb) {
+                const int b = nbr_idx[nb0 + lane];
+                beg = nbeg[b];
+                cnt = nend[b] - beg;
+            }
+            int incl = cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane < nnb) { rb_[lane] = beg; rc_[lane] = incl - cnt; }
+            if (lane == nnb - 1) rc_[nnb] = incl;
         }
-        rng_cum[nnb] = cum;
-    }
-    __syncthreads();
-    const int nsrc = rng_cum[nnb];
-    const int t0 = nbeg[g], t1 = nend[g], NT = t1 - t0;
-    for (int64_t r = blockIdx.y; r < nr; r += gridDim.y) {  // right-hand sides across the grid
-        for (int tb = t0; tb < t1; tb += 128) {
-            const int nt = min(128, t1 - tb);
-            const int nsl = 128 / nt;
-            const int tg = threadIdx.x % nt, slice = threadIdx.x / nt;
-            const bool active = slice < nsl;
-            const int a = tb + tg;
-            const R ax = pos_hi[3 * a], ay = pos_hi[3 * a + 1], az = pos_hi[3 * a + 2];
-            R alx = 0, aly = 0, alz = 0;
-            if (DOUBLE_FLOAT) { alx = pos_lo[3 * a]; aly = pos_lo[3 * a + 1]; alz = pos_lo[3 * a + 2]; }
-            const int adom = dom[a];
-            const R adom_r = (R)adom;
-            const V4<R> *cs0 = cache ? cache + 2 * cache_base[blockIdx.x] + (tb - t0 + tg) : nullptr;
-            c64 yacc[6] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
-            for (int side = 0; side < 2; ++side) {
-                const int d = side == 0 ? 0 : adom;
-                const cx<R> k = to<R>(dc[d].k);
-                cx<R> phi[3], gphi[3][3];  // gphi[k][c] = d phi_c / d s_k
+        __syncwarp();
+        const int nsrc = rc_[nnb], ntile = (nsrc + 31) / 32;
+        const int tile0 = (int)((int64_t)sp * ntile / nsp), tile1 = (int)((int64_t)(sp + 1) * ntile / nsp);
+        const int ti = lane % tg, sl = lane / tg;
+        const bool busy = sl < nsl;
+        const int t0 = nbeg[g], NT = nend[g] - t0, a = t0 + it.y + ti;
+        const R ax = pos_hi[3 * a], ay = pos_hi[3 * a + 1], az = pos_hi[3 * a + 2];
+        const R lx = LO ? pos_lo[3 * a] : (R)0, ly = LO ? pos_lo[3 * a + 1] : (R)0, lz = LO ? pos_lo[3 * a + 2] : (R)0;
+        const R nx = (R)nrm[3 * a], ny = (R)nrm[3 * a + 1], nz = (R)nrm[3 * a + 2];
+        const int adom = dom[a];
+        const cx<R> k0 = to<R>(dc[0].k), kj = to<R>(dc[adom].k);
+        const V4<R> *cs = CACHED ? cache + 2 * cache_base[leaf] + (it.y + ti) : nullptr;
+        cx<R> u[RB][2][3], phi[RB][2][3];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    phi[c] = {0, 0};
+        for (int rr = 0; rr < RB; ++rr)
 #pragma unroll
-                    for (int kk = 0; kk < 3; ++kk) gphi[kk][c] = {0, 0};
-                }
-                for (int s0 = 0; s0 < nsrc; s0 += 128) {
-                    __syncthreads();
-                    {
-                        const int e = s0 + threadIdx.x;
-                        if (e < nsrc) {
-                            const int q = source_range(rng_cum, nnb, e);
-                            const int i = rng_beg[q] + (e - rng_cum[q]);
-                            T.pa[threadIdx.x] = V4<R>{pos_hi[3 * i], pos_hi[3 * i + 1], pos_hi[3 * i + 2], (R)dom[i]};
-                            R lo[3] = {0, 0, 0};
-                            if (DOUBLE_FLOAT) { lo[0] = pos_lo[3 * i]; lo[1] = pos_lo[3 * i + 1]; lo[2] = pos_lo[3 * i + 2]; }
-                            T.pb[threadIdx.x] = V4<R>{lo[0], lo[1], lo[2], 0};
-                            const cx<R> *dn = dens + ((side * nr + r) * N + i) * 6;
-                            for (int c = 0; c < 3; ++c) T.xv[c][threadIdx.x] = dn[c];
-                        }
+            for (int sd = 0; sd < 2; ++sd)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) u[rr][sd][c] = phi[rr][sd][c] = {0, 0};
+        for (int t = tile0; t < tile1; ++t) {
+            const int e0 = t * 32;
+            __syncwarp();  // the tile before is no longer read
+            if (e0 + lane < nsrc) {
+                const int q = source_range(rc_, nnb, e0 + lane);
+                const int64_t i = rb_[q] + (e0 + lane - rc_[q]);
+                T.pa[lane] = V4<R>{pos_hi[3 * i], pos_hi[3 * i + 1], pos_hi[3 * i + 2], (R)dom[i]};
+                if (LO) T.pb[lane] = V4<R>{pos_lo[3 * i], pos_lo[3 * i + 1], pos_lo[3 * i + 2], 0};
+#pragma unroll
+                for (int rr = 0; rr < RB; ++rr)
+#pragma unroll
+                    for (int sd = 0; sd < 2; ++sd) {
+                        const cx<R> *dn = dens + ((sd * nr + min(r0 + rr, nr - 1)) * N + i) * 6;
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) T.x[rr][sd][c][lane] = V2<R>{dn[c].re, dn[c].im};
                     }
-                    __syncthreads();
-                    const int ns = min(128, nsrc - s0);
-                    if (active)
-                        for (int u = slice; u < ns; u += nsl) {
-                            const V4<R> pa = T.pa[u];
-                            if (side == 1 && pa.w != adom_r) continue;  // scatterer d sums over its own nodes
-                            const V4<R> pb = T.pb[u];
-                            R rx = pa.x - ax, ry = pa.y - ay, rz = pa.z - az;
-                            if (DOUBLE_FLOAT) { rx += pb.x - alx; ry += pb.y - aly; rz += pb.z - alz; }
-                            cx<R> gs, cs;
-                            if (cs0) {
-                                const V4<R> sv = cs0[((int64_t)side * nsrc + s0 + u) * NT];
-                                gs = {sv.x, sv.y};
-                                cs = {sv.z, sv.w};
-                            } else {
-                                const R R2 = rx * rx + ry * ry + rz * rz;
-                                const R inv = R2 > (R)0 ? rsqrt_(R2) : (R)0;  // the node itself drops out
-                                pair_scalars<R>(inv, R2 * inv, k, gs, cs);
-                            }
-                            // grad phi at the target: c (s_target - s_source) = -c r
-                            const cx<R> cr[3] = {-rx * cs, -ry * cs, -rz * cs};
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) {
-                                const cx<R> xc = T.xv[c][u];
-                                cfma(phi[c], gs, xc);
-#pragma unroll
-                                for (int kk = 0; kk < 3; ++kk) cfma(gphi[kk][c], cr[kk], xc);
-                            }
-                        }
+            }
+            __syncwarp();
+            const int ns = busy ? min(32, nsrc - e0) : 0;
+            for (int s = sl; s < ns; s += nsl) {
+                const V4<R> p = T.pa[s];
+                R rx = p.x - ax, ry = p.y - ay, rz = p.z - az;
+                if (LO) {
+                    const V4<R> pl = T.pb[s];
+                    rx += pl.x - lx;
+                    ry += pl.y - ly;
+                    rz += pl.z - lz;
                 }
-                // sum the source slices in a fixed order
-                __syncthreads();
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    S.red[c][threadIdx.x] = phi[c];
-#pragma unroll
-                    for (int kk = 0; kk < 3; ++kk) S.red[3 + 3 * kk + c][threadIdx.x] = gphi[kk][c];
-                }
-                __syncthreads();
-                if (threadIdx.x < nt) {
-                    c64 ph[3], gp[3][3];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        cx<R> v = S.red[c][threadIdx.x];
-                        for (int sl = 1; sl < nsl; ++sl) v += S.red[c][sl * nt + threadIdx.x];
-                        ph[c] = c64{(double)v.re, (double)v.im};
-#pragma unroll
-                        for (int kk = 0; kk < 3; ++kk) {
-                            cx<R> t = S.red[3 + 3 * kk + c][threadIdx.x];
-                            for (int sl = 1; sl < nsl; ++sl) t += S.red[3 + 3 * kk + c][sl * nt + threadIdx.x];
-                            gp[kk][c] = c64{(double)t.re, (double)t.im};
-                        }
+                const bool same = p.w == (R)adom;
+                cx<R> gs[2], c2[2];
+                if (CACHED) {
+                    const V4<R> v0 = cs[(int64_t)(e0 + s) * NT];
+                    gs[0] = {v0.x, v0.y};
+                    c2[0] = {v0.z, v0.w};
+                    if (same) {
+                        const V4<R> v1 = cs[((int64_t)nsrc + e0 + s) * NT];
+                        gs[1] = {v1.x, v1.y};
+                        c2[1] = {v1.z, v1.w};
                     }
-                    // far field: L2P of phi and grad phi from the leaf's local expansions
-                    const cx<R> *Dl = D + (((int64_t)d * nbox + g) * 3 * nr + 3 * r) * p2;
-                    const cx<R> *B = Bl2p + ((int64_t)side * N + a) * p2;
-                    const cx<R> *G = Bl2pg + ((int64_t)side * N + a) * 3 * p2;
-                    cx<R> fp[3] = {{0, 0}, {0, 0}, {0, 0}}, fg[3][3];
+                } else {
+                    const R R2 = rx * rx + ry * ry + rz * rz;
+                    const R inv = R2 > (R)0 ? rsqrt_(R2) : (R)0, Rr = R2 * inv;  // the node itself drops out
+                    pair_scalars<R>(inv, Rr, k0, gs[0], c2[0]);
+                    if (same) pair_scalars<R>(inv, Rr, kj, gs[1], c2[1]);
+                }
+                const R wx = ry * nz - rz * ny, wy = rz * nx - rx * nz, wz = rx * ny - ry * nx;
+                const R nr_ = nx * rx + ny * ry + nz * rz;
+                const cx<R> m0 = {-c2[0].re, -c2[0].im};
 #pragma unroll
-                    for (int c = 0; c < 3; ++c)
+                for (int rr = 0; rr < RB; ++rr)
 #pragma unroll
-                        for (int kk = 0; kk < 3; ++kk) fg[kk][c] = {0, 0};
-                    for (int q = 0; q < p2; ++q) {
-                        const cx<R> b = B[q], gx = G[q], gy = G[p2 + q], gz = G[2 * p2 + q];
+                    for (int sd = 0; sd < 2; ++sd) {
+                        if (sd == 1 && !same) continue;
+                        const V2<R> x0 = T.x[rr][sd][0][s], x1 = T.x[rr][sd][1][s], x2 = T.x[rr][sd][2][s];
+                        const cx<R> X[3] = {{x0.x, x0.y}, {x1.x, x1.y}, {x2.x, x2.y}};
+                        const cx<R> B[3] = {wz * X[1] - wy * X[2] - nr_ * X[0], wx * X[2] - wz * X[0] - nr_ * X[1],
+                                            wy * X[0] - wx * X[1] - nr_ * X[2]};
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            const cx<R> dq = Dl[c * p2 + q];
-                            cfma(fp[c], dq, b);
-                            cfma(fg[0][c], dq, gx);
-                            cfma(fg[1][c], dq, gy);
-                            cfma(fg[2][c], dq, gz);
+                            cfma(u[rr][sd][c], sd == 0 ? m0 : c2[1], B[c]);
+                            cfma(phi[rr][sd][c], gs[sd], X[c]);
                         }
                     }
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        ph[c] += c64{(double)fp[c].re, (double)fp[c].im};
-#pragma unroll
-                        for (int kk = 0; kk < 3; ++kk) gp[kk][c] += c64{(double)fg[kk][c].re, (double)fg[kk][c].im};
-                    }
-                    // assembly in double precision
-                    const double sg = side == 0 ? -1.0 : 1.0;
-                    const double nb[3] = {nrm[3 * a], nrm[3 * a + 1], nrm[3 * a + 2]};
-                    const double np_[3] = {sg * nb[0], sg * nb[1], sg * nb[2]};
-                    const c64 div = gp[0][0] + gp[1][1] + gp[2][2];
-                    c64 u[3];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        c64 v = np_[c] * div;
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) v -= np_[i] * gp[c][i];
-#pragma unroll
-                        for (int kk = 0; kk < 3; ++kk) v += np_[kk] * gp[kk][c];
-                        u[c] = v;
-                    }
-                    if (side == 1) {  // T_j u = u + t_j n (n.u), n the scatterer normal
-                        const c64 nu = nb[0] * u[0] + nb[1] * u[1] + nb[2] * u[2];
-                        const c64 tn = dc[d].t * nu;
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) u[c] += nb[c] * tn;
-                    }
-                    const double wa = w[a];
-                    const c64 sig = side == 0 ? c64{-1.0, 0.0} : dc[d].gamma;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        yacc[c] += wa * u[c];
-                        yacc[3 + c] += (sig * ph[c]) * wa;
-                    }
-                }
             }
-            if (threadIdx.x < nt) {  // transposed self block, stored in user order
-                const int64_t uu = perm[a];
-                const c64 *M = Mself + 36 * uu;
-                const c64 *xa = x + (r * N + uu) * 6;
-                c64 *ya = y + (r * N + uu) * 6;
+        }
+        // sum the slices of each target in order, through the tile's shared memory
+        cx<R> *S = reinterpret_cast<cx<R> *>(&T);
+        static_assert(sizeof(AdjTile<R, RB>) >= 6 * 32 * sizeof(cx<R>), "slice sums");
+        constexpr int HALF = sizeof(AdjTile<R, RB>) >= 12 * 32 * sizeof(cx<R>) ? 12 : 6;  // rows at a time
 #pragma unroll
-                for (int pc = 0; pc < 6; ++pc) {
-                    c64 acc = yacc[pc];
-                    for (int q = 0; q < 6; ++q) cfma(acc, M[q * 6 + pc], xa[q]);
-                    ya[pc] = acc;
+        for (int rr = 0; rr < RB; ++rr) {
+            if (r0 + rr >= nr) break;
+#pragma unroll
+            for (int h0 = 0; h0 < 12; h0 += HALF) {
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < HALF; ++j) {
+                    const int row = h0 + j, sd = row / 6, c = row % 3;
+                    S[j * 32 + lane] = row % 6 < 3 ? u[rr][sd][c] : phi[rr][sd][c];
+                }
+                __syncwarp();
+                for (int o = lane; o < tg * HALF; o += 32) {
+                    const int tt = o / HALF, j = o - tt * HALF;
+                    cx<R> v = S[j * 32 + tt];
+                    for (int k = 1; k < nsl; ++k) v += S[j * 32 + k * tg + tt];
+                    part[(((int64_t)sp * nr + r0 + rr) * N + t0 + it.y + tt) * 12 + h0 + j] = v;
                 }
             }
         }
+    }
+}
+
+// assembly of k_near_adj's partial sums: eight lanes per (node, right-hand side), four per side; each sums a
+// quarter of the far field (L2P of phi and grad phi) of its side's domain, then in double precision
+// u far + u near, T_d, the weights, and the transposed self block, a row of which each of six lanes takes
+template <typename R>
+__global__ void __launch_bounds__(128) k_near_adj_finish(
+    int64_t N, int64_t nr, int nsp, int p2, int64_t nbox, const int32_t *__restrict__ node_leaf,
+    const double *__restrict__ nrm, const double *__restrict__ w, const int32_t *__restrict__ dom,
+    const int32_t *__restrict__ perm, const DomainConsts *dc, const cx<R> *__restrict__ Bl2p,
+    const cx<R> *__restrict__ Bl2pg, const cx<R> *__restrict__ D, const c64 *__restrict__ Mself,
+    const c64 *__restrict__ x, const cx<R> *__restrict__ part, c64 *y) {
+    const int64_t a_ = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3, r = blockIdx.y;
+    const int64_t a = min(a_, N - 1);  // whole groups of eight lanes stay for the shuffles
+    const int l8 = threadIdx.x & 7, side = l8 >> 2, qpart = l8 & 3;
+    const int d = side == 0 ? 0 : dom[a];
+    cx<R> fp[3], fg[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        fp[c] = {0, 0};
+#pragma unroll
+        for (int kk = 0; kk < 3; ++kk) fg[kk][c] = {0, 0};
+    }
+    const cx<R> *Dl = D + (((int64_t)d * nbox + node_leaf[a]) * 3 * nr + 3 * r) * p2;
+    const cx<R> *B = Bl2p + ((int64_t)side * N + a) * p2, *G = Bl2pg + ((int64_t)side * N + a) * 3 * p2;
+    for (int q = qpart; q < p2; q += 4) {
+        const cx<R> b = B[q], gx = G[q], gy = G[p2 + q], gz = G[2 * p2 + q];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cx<R> dq = Dl[c * p2 + q];
+            cfma(fp[c], dq, b);
+            cfma(fg[0][c], dq, gx);
+            cfma(fg[1][c], dq, gy);
+            cfma(fg[2][c], dq, gz);
+        }
+    }
+    // the far u of this quarter (linear in grad phi), then phi and u summed over the quarters
+    const R sg = side == 0 ? (R)-1 : (R)1;
+    const R n1[3] = {sg * (R)nrm[3 * a], sg * (R)nrm[3 * a + 1], sg * (R)nrm[3 * a + 2]};
+    const cx<R> div = fg[0][0] + fg[1][1] + fg[2][2];
+    c64 u[3], ph[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        cx<R> v = n1[c] * div;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v += n1[i] * (fg[i][c] - fg[c][i]);
+#pragma unroll
+        for (int o = 2; o > 0; o >>= 1) {
+            v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+            v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+            fp[c].re += __shfl_xor_sync(0xffffffffu, fp[c].re, o);
+            fp[c].im += __shfl_xor_sync(0xffffffffu, fp[c].im, o);
+        }
+        u[c] = {(double)v.re, (double)v.im};
+        ph[c] = {(double)fp[c].re, (double)fp[c].im};
+    }
+    for (int s = 0; s < nsp; ++s) {
+        const cx<R> *P = part + ((s * nr + r) * N + a) * 12 + 6 * side;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            u[c] += c64{(double)P[c].re, (double)P[c].im};
+            ph[c] += c64{(double)P[3 + c].re, (double)P[3 + c].im};
+        }
+    }
+    if (side == 1) {  // T_j u = u + t_j n (n.u), n the scatterer normal
+        const double nb[3] = {nrm[3 * a], nrm[3 * a + 1], nrm[3 * a + 2]};
+        const c64 tn = dc[d].t * (nb[0] * u[0] + nb[1] * u[1] + nb[2] * u[2]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] += nb[c] * tn;
+    }
+    const double wa = w[a];
+    const c64 sig = side == 0 ? c64{-1.0, 0.0} : dc[d].gamma;
+    c64 acc = {0, 0};  // row l8 of the result (l8 < 6)
+#pragma unroll
+    for (int row = 0; row < 6; ++row) {
+        c64 v = row < 3 ? wa * u[row % 3] : (sig * ph[row % 3]) * wa;
+        v.re += __shfl_xor_sync(0xffffffffu, v.re, 4);  // the other side
+        v.im += __shfl_xor_sync(0xffffffffu, v.im, 4);
+        if (row == l8) acc = v;
+    }
+    if (l8 < 6 && a_ < N) {
+        const int64_t uu = perm[a];
+        const c64 *M = Mself + 36 * uu, *xa = x + (r * N + uu) * 6;
+        for (int q = 0; q < 6; ++q) cfma(acc, M[q * 6 + l8], xa[q]);
+        y[(r * N + uu) * 6 + l8] = acc;
     }
 }
 
@@ -3849,17 +3895,36 @@ static void adjoint_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_
     downward_pass<R>(h, nr, s, tensor_mode);
     const R *ph = f32 ? (const R *)h->pos_hi : (const R *)h->pos;
     const R *pl = f32 ? (const R *)h->pos_lo : nullptr;
-    const V4<R> *cache = f32 ? nullptr : (const V4<R> *)h->near_cache64;
-    if constexpr (sizeof(R) == 4)
-        k_near_adj<R, true><<<dim3((unsigned)h->n_leaves, (unsigned)std::min<int64_t>(nr, 65535)), 128, 0, s>>>(h->leaf_box, N, nr, p2, h->nbox, h->box_nbeg, h->box_nend,
-                                                          h->nbr_start, h->nbr_idx, ph, pl, h->nrm, h->w, h->dom,
-                                                          h->perm, dens, dc, Bl2p, Bl2pg, D, h->Mself, x, y,
-                                                          h->near_base, cache);
-    else
-        k_near_adj<R, false><<<dim3((unsigned)h->n_leaves, (unsigned)std::min<int64_t>(nr, 65535)), 128, 0, s>>>(h->leaf_box, N, nr, p2, h->nbox, h->box_nbeg, h->box_nend,
-                                                           h->nbr_start, h->nbr_idx, ph, pl, h->nrm, h->w, h->dom,
-                                                           h->perm, dens, dc, Bl2p, Bl2pg, D, h->Mself, x, y,
-                                                           h->near_base, cache);
+    int dev = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    auto launch_adj = [&](auto kern, int rb) {
+        const int64_t nrb = (nr + rb - 1) / rb;
+        const int nsp = near_d_splits(h, nrb);
+        const int64_t units = (int64_t)h->n_near_ditems * nrb * nsp;
+        if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
+        int per_sm = 0;
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * ND_WARPS, 0));
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((units + ND_WARPS - 1) / ND_WARPS,
+                                                                    (int64_t)std::max(per_sm, 1) * nsm));
+        CK(cudaMemsetAsync(h->near_next, 0, sizeof(int), s));
+        kern<<<(unsigned)grid, 32 * ND_WARPS, 0, s>>>(
+            h->leaf_box, h->near_ditems, h->n_near_ditems, (int)units, nsp, (int)nrb, h->near_next, N, nr, h->box_nbeg,
+            h->box_nend, h->nbr_start, h->nbr_idx, ph, pl, h->nrm, h->dom, dens, dc, h->near_base,
+            f32 ? nullptr : (const V4<R> *)h->near_cache64, (cx<R> *)h->near_part);
+        CKL("k_near_adj");
+        k_near_adj_finish<R><<<dim3(nblk(8 * N, 128), (unsigned)nr), 128, 0, s>>>(
+            N, nr, nsp, p2, h->nbox, h->node_leaf, h->nrm, h->w, h->dom, h->perm, dc, Bl2p, Bl2pg, D, h->Mself, x,
+            (const cx<R> *)h->near_part, y);
+    };
+    if constexpr (sizeof(R) == 4) {  // three right-hand sides share the pair scalars
+        if (nr == 1) launch_adj(k_near_adj<R, false, 1>, 1);
+        else launch_adj(k_near_adj<R, false, 3>, 3);
+    } else if (h->near_cache64) {
+        launch_adj(k_near_adj<R, true, 1>, 1);
+    } else {
+        launch_adj(k_near_adj<R, false, 1>, 1);
+    }
     CKL("k_near_adj");
     apply_near_singular(h, x, y, nr, s, true);  // transposed near-singular pair corrections (option)
 }
@@ -3887,6 +3952,7 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
+    ensure_near_scratch(h, nr, precision == FMBEM_FP64 || nr == 1 ? 1 : 3, 12, false);
     const DomainConsts *dc = (const DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
         adjoint_impl<float>(h, x, y, nr, s, dc, precision == FMBEM_TF32 ? 1 : 2);

@@ -51,3 +51,21 @@ def test_oracle_near_only():
     y = h.matvec(torch.from_numpy(x).cuda()).cpu().numpy()
     yo = o.matvec(x)
     assert np.linalg.norm(y - yo) < 1e-5 * np.linalg.norm(yo)
+
+
+# the transposed near field by warps (k_near_adj): b . (A x) = x . (A^T b) with the forward product, in double
+# precision to the rounding of their sums (as above, over the terms' sum), in single to 2^-24 of ~1000 terms
+@pytest.mark.parametrize("name,opt", [("1", {}), ("3", {}), ("2", dict(leaf_size=1, max_level=3)), ("3", dict(near_cache=0)),
+                                      ("two", {}), ("two", dict(near_cache=0)), ("ring", dict(adaptive=1, leaf_size=20)),
+                                      ("2", dict(node_mode=fm.NODES_CENTROID)), ("3", dict(boundary=fm.IMPEDANCE))])
+@pytest.mark.parametrize("n_rhs", [1, 2, 3, 4])
+@pytest.mark.parametrize("precision,tol", [(fm.FP64, 1e-12), (fm.FP32, 1e-5)])
+def test_adjoint_identity(name, opt, n_rhs, precision, tol):
+    V, F, D = mesh(name)
+    h = fm.FMBEM(V, F, D, [1.0, -5 + 0.2j, 2.25][: D.max() + 1], [1.0, 1.3, 1.0][: D.max() + 1], 1.7, p=4, m2l_rotation=0,
+                 **opt)
+    x, b = (torch.from_numpy(fi.random_complex((n_rhs, h.N, 6), seed=s)).cuda() for s in (1, 2))
+    y, z = h.matvec(x, precision=precision), h.adjoint_matvec(b, precision=precision)
+    for r in range(n_rhs):
+        assert abs(complex((b[r] * y[r]).sum() - (x[r] * z[r]).sum())) <= tol * float((b[r] * y[r]).abs().sum())
+    assert torch.equal(z, h.adjoint_matvec(b, precision=precision))
