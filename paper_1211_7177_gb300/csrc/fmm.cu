@@ -2002,7 +2002,7 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
     int64_t nr, const int32_t *nbeg, const int32_t *nend, const int32_t *nbr_start, const int32_t *nbr_idx,
     const float4 *__restrict__ rec, const cx<float> *dens, const cx<float> *sjump, const DomainConsts *dc,
     const int32_t *perm, int p2, int64_t nbox, const cx<float> *__restrict__ Bl2p, const cx<float> *__restrict__ D,
-    const c64 *__restrict__ Mself, const c64 *__restrict__ x, c64 *y, bool side1) {
+    const c64 *__restrict__ Mself, const c64 *__restrict__ x, c64 *y, bool side1, int nsp, cx<float> *part) {
     __shared__ SideTile tiles[NS_WARPS][2];
     __shared__ int rng_beg[NS_WARPS][32], rng_cum[NS_WARPS][33];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2013,8 +2013,9 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
         if (lane == 0) unit = atomicAdd(next_unit, 1);
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= n_units) break;
-        const int64_t r = unit / n_items;
-        const int item_id = unit - (int)r * n_items;
+        const int rs = unit / n_items, sp = rs % nsp;  // (right-hand side, source split)
+        const int64_t r = rs / nsp;
+        const int item_id = unit - rs * n_items;
         __syncwarp();  // the previous unit's shared-memory reads are done
         const int4 it = items[item_id];
         const int leaf = it.x, tg = it.z, nsl = it.w;
@@ -2063,9 +2064,10 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
         cx<float> acc0[3], acc1[3], bq[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc0[c] = acc1[c] = bq[c] = {0, 0};
-        const int ntile = (nsrc + NS_TS - 1) / NS_TS;
-        stage(T[0], 0);
-        for (int t = 0; t < ntile; ++t) {
+        const int nall = (nsrc + NS_TS - 1) / NS_TS;  // this split's tiles tile0 .. ntile - 1
+        const int tile0 = (int)((int64_t)sp * nall / nsp), ntile = (int)((int64_t)(sp + 1) * nall / nsp);
+        if (tile0 < ntile) stage(T[tile0 & 1], tile0 * NS_TS);
+        for (int t = tile0; t < ntile; ++t) {
             if (t + 1 < ntile) stage(T[(t + 1) & 1], (t + 1) * NS_TS);
             else cp_async_commit();  // an empty group keeps "all but the newest group done" meaning tile t
             cp_async_wait1();
@@ -2144,8 +2146,10 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
                 }
             }
         };
-        l2p(0, acc0);
-        if (side1) l2p(1, acc1);
+        if (sp == 0) {
+            l2p(0, acc0);
+            if (side1) l2p(1, acc1);
+        }
         // sum the slices of each target: lane ti + tg * sl, fixed tree over sl
         for (int off = nsl >> 1; off >= 1; off >>= 1) {
 #pragma unroll
@@ -2167,6 +2171,11 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
             for (int c = 0; c < 3; ++c) { Ys[ti * 6 + c] = acc0[c]; Ys[ti * 6 + 3 + c] = acc1[c]; }
         }
         __syncwarp();
+        if (nsp > 1) {  // a split's sums: k_near_sum adds them and the self block
+            for (int o = lane; o < tg * 6; o += 32)
+                part[(((int64_t)sp * nr + r) * N + nbeg[g] + it.y) * 6 + o] = Ys[o];
+            continue;
+        }
         const int nrow = side1 ? 6 : 3;
         for (int o = lane; o < tg * nrow; o += 32) {
             const int t = o / nrow, row = o - t * nrow, side = row / 3, c = row - 3 * side;
@@ -2182,6 +2191,28 @@ __global__ void __launch_bounds__(32 * NS_WARPS, 6) k_near_ws(
             y[(r * N + u) * 6 + row] = v;
         }
     }
+}
+
+// the rows of a split k_near_ws: the splits' sums in order and the row of the self block in double
+// precision; thread per (node, row), grid (.., right-hand side)
+__global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp, int nrow, const int32_t *__restrict__ perm,
+                                                  const cx<float> *__restrict__ part, const c64 *__restrict__ Mself,
+                                                  const c64 *__restrict__ x, c64 *y) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (i >= N * 6) return;
+    const int64_t a = i / 6;
+    const int row = (int)(i - a * 6);
+    if (row >= nrow) return;
+    cx<float> f = part[(r * N + a) * 6 + row];
+    for (int s = 1; s < nsp; ++s) f += part[((s * nr + r) * N + a) * 6 + row];
+    const int64_t u = perm[a];
+    const c64 *M = Mself + 36 * u + 6 * row, *xa = x + (r * N + u) * 6;
+    c64 v = {(double)f.re, (double)f.im};
+    cfma(v, M[0], xa[0]);
+    cfma(v, M[1], xa[1]);
+    cfma(v, M[2], xa[2]);
+    cfma(v, M[3 + row % 3], xa[3 + row % 3]);
+    y[(r * N + u) * 6 + row] = v;
 }
 
 // Steps 4-5 for 32 or more right-hand sides in single precision, one lane per right-hand side,
@@ -3325,10 +3356,17 @@ static int near_d_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_ditems * nr);
     return (int)std::max<int64_t>(1, std::min<int64_t>({8, h->near_tiles_max, (8 * 608 + units - 1) / units}));
 }
-// the near field's partial sums (rows complex values of a node and right-hand side; units of rb
-// right-hand sides), and per-source vectors of the FP64 forward product
-static void ensure_near_scratch(fmbem *h, int64_t nr, int rb, int rows, bool am) {
-    const size_t npart = sizeof(c64) * rows * h->N * nr * near_d_splits(h, (nr + rb - 1) / rb), nam = sizeof(c64) * 5 * h->N * nr;
+// and per item of k_near_ws (single precision, 1-3 right-hand sides): about two units for each of the 24
+// warps an SM holds.  A unit is latency-bound (a pair takes about 400 cycles of its warp), so with one unit
+// per item 10242 nodes (1450 units) took 215 us, ten times the arithmetic's time
+static int near_ws_splits(const fmbem *h, int64_t nr) {
+    const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_items * nr);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({8, h->near_tiles_max, (2 * 24 * 152 + units - 1) / units}));
+}
+// the near field's partial sums (rows complex values of a node, right-hand side and split), and per-source
+// vectors of the FP64 forward product
+static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, int rows, bool am) {
+    const size_t npart = sizeof(c64) * rows * h->N * nr * nsp, nam = sizeof(c64) * 5 * h->N * nr;
     if (h->near_part_bytes < npart) {
         if (h->near_part) dev_free(h, h->near_part);
         h->near_part = nullptr;
@@ -3816,7 +3854,9 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
             else if (rest > 0) launch_w(k_near_w<4>, 4, sizeof(WarpTile<4>), 32 * nblk);
         } else {  // few right-hand sides: both sides of a pair in one pass, one unit per item and RHS
             if (h->near_items == nullptr) throw fmbem_error{FMBEM_ERR_CUDA, "near-field work items were not built"};
-            const int64_t units = (int64_t)h->n_near_items * nr;
+            const int nsp = h->near_part != nullptr ? near_ws_splits(h, nr) : 1;
+            const int64_t units = (int64_t)h->n_near_items * nr * nsp;
+            if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
             int per_sm = 0;
             CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_near_ws, 32 * NS_WARPS, 0));
             const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((units + NS_WARPS - 1) / NS_WARPS,
@@ -3825,8 +3865,12 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
             k_near_ws<<<(unsigned)grid, 32 * NS_WARPS, 0, s>>>(
                 h->leaf_box, h->near_items, h->n_near_items, (int)units, h->near_next, N, nr, h->box_nbeg, h->box_nend,
                 h->nbr_start, h->nbr_idx, h->src_rec, (const cx<float> *)dens, (const cx<float> *)sj, dc, h->perm, p2,
-                h->nbox, (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y, !h->ibc);
+                h->nbox, (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y, !h->ibc, nsp,
+                (cx<float> *)h->near_part);
             CKL("k_near_ws");
+            if (nsp > 1)
+                k_near_sum<<<dim3(nblk(6 * N, 192), (unsigned)nr), 192, 0, s>>>(
+                    N, nr, nsp, h->ibc ? 3 : 6, h->perm, (const cx<float> *)h->near_part, h->Mself, x, y);
         }
     } else if (h->near_am != nullptr) {
         const int nsp = near_d_splits(h, nr);
@@ -3952,7 +3996,7 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
-    ensure_near_scratch(h, nr, precision == FMBEM_FP64 || nr == 1 ? 1 : 3, 12, false);
+    ensure_near_scratch(h, nr, near_d_splits(h, precision == FMBEM_FP64 || nr == 1 ? nr : (nr + 2) / 3), 12, false);
     const DomainConsts *dc = (const DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
         adjoint_impl<float>(h, x, y, nr, s, dc, precision == FMBEM_TF32 ? 1 : 2);
@@ -3968,7 +4012,8 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
-    if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, 1, 6, true);
+    if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6, true);
+    else if (nr < 4) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
     static_assert(sizeof(DomainConsts) == 3 * sizeof(c64), "layout");
     DomainConsts *dc = (DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
@@ -4040,11 +4085,12 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     // run the regular passes on pointers into the static array; the handle's own scratch
     // pointers are restored afterwards, so fmbem_matvec is unaffected
     void *sv_dens = h->dens, *sv_C = h->Cexp, *sv_D = h->Dexp, *sv_y = h->ybuf, *sv_dig = h->oz_dig;
-    c64 *sv_am = h->near_am;
+    c64 *sv_am = h->near_am, *sv_part = h->near_part;
     const size_t sv_yb = h->ybuf_bytes;
     auto restore = [&] {
         h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y; h->ybuf_bytes = sv_yb; h->oz_dig = sv_dig;
         h->near_am = sv_am;
+        h->near_part = sv_part;
     };
     h->dens = base;
     h->Cexp = base + b_dens;
@@ -4052,7 +4098,7 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     h->ybuf = b_y ? base + b_dens + 2 * b_exp : nullptr;
     h->ybuf_bytes = b_y;
     h->oz_dig = nullptr;  // no digits in the static array: the FP64 pipe's translations,
-    h->near_am = nullptr;  // and no partial sums: the near field by a block per leaf
+    h->near_am = h->near_part = nullptr;  // and no partial sums: a block per leaf (FP64), whole items (FP32)
     try {
         matvec_impl<R>(h, x, y, nr, s, (const DomainConsts *)h->dcons);
     } catch (...) {
