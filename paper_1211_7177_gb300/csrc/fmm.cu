@@ -197,12 +197,69 @@ __device__ __forceinline__ void p2m_body(int64_t g, int64_t N, int64_t nr, int p
     if (q < p2)
         for (int c = 0; c < 3; ++c) C[(((int64_t)d * nbox + g) * 3 * nr + 3 * r + c) * p2 + q] = acc[c];
 }
-template <typename R>
-__global__ void k_p2m(const int32_t *leaf_box, int64_t N, int64_t nr, int p2, int64_t nbox, const int32_t *nbeg,
-                      const int32_t *nend, const int32_t *dom, const double *nrm, const cx<R> *dens, const cx<R> *Bp2m,
-                      cx<R> *C) {
-    p2m_body<R>(leaf_box[blockIdx.x], N, nr, p2, nbox, nbeg, nend, dom, nrm, dens, Bp2m, C, blockIdx.x, blockIdx.y,
-                blockIdx.z);
+// The same for one to three right-hand sides with the nodes of a leaf dealt to NG groups of rows_pad
+// threads and the groups' sums added in order through shared memory: with one group a block kept two warps
+// busy, and 56 leaves took as long as one of them (FP64, 2562 nodes: 137 us).
+constexpr int P2M_GROUPS = 4;
+template <typename R, int NG>
+__global__ void k_p2m(const int32_t *leaf_box, int64_t N, int64_t nr, int p2, int rows_pad, int64_t nbox,
+                      const int32_t *nbeg, const int32_t *nend, const int32_t *dom, const double *nrm, const cx<R> *dens,
+                      const cx<R> *Bp2m, cx<R> *C) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cx<R>(*W)[4][3] = reinterpret_cast<cx<R>(*)[4][3]>(smem_raw);  // [P2M_WN]; then the groups' sums
+    const int64_t g = leaf_box[blockIdx.x], r = blockIdx.z;
+    const int d = blockIdx.y, side = d == 0 ? 0 : 1;
+    const R sg = d == 0 ? (R)-1 : (R)1;
+    const int i0 = nbeg[g], i1 = nend[g];
+    const int q = NG == 1 ? threadIdx.x : threadIdx.x % rows_pad, grp = NG == 1 ? 0 : threadIdx.x / rows_pad;
+    cx<R> acc[3] = {{0, 0}, {0, 0}, {0, 0}};
+    for (int ib = i0; ib < i1; ib += P2M_WN) {
+        const int nk = min(P2M_WN, i1 - ib);
+        __syncthreads();
+        for (int e = threadIdx.x; e < 3 * nk; e += blockDim.x) {
+            const int il = e / 3, c = e - 3 * il, i = ib + il;
+            if (d > 0 && dom[i] != d) {
+                for (int k = 0; k < 4; ++k) W[il][k][c] = {0, 0};
+                continue;
+            }
+            const cx<R> *dn = dens + ((side * nr + r) * N + i) * 6;
+            const cx<R> v[3] = {dn[0], dn[1], dn[2]};
+            const R n[3] = {sg * (R)nrm[3 * i], sg * (R)nrm[3 * i + 1], sg * (R)nrm[3 * i + 2]};
+            const cx<R> nv = n[0] * v[0] + n[1] * v[1] + n[2] * v[2];
+            W[il][0][c] = dn[3 + c];
+            const cx<R> vc = c == 0 ? v[0] : (c == 1 ? v[1] : v[2]);  // selects, not a local-memory index
+            const R nc = c == 0 ? n[0] : (c == 1 ? n[1] : n[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                cx<R> t = n[k] * vc - nc * v[k];
+                if (k == c) t += nv;
+                W[il][1 + k][c] = t;
+            }
+        }
+        __syncthreads();
+        if (q < p2)
+            for (int il = grp; il < nk; il += NG) {
+                const cx<R> *B = Bp2m + ((int64_t)side * N + ib + il) * 4 * p2;
+                const cx<R> b[4] = {B[q], B[p2 + q], B[2 * p2 + q], B[3 * p2 + q]};
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) cfma(acc[c], W[il][k][c], b[k]);
+            }
+    }
+    cx<R> *S = reinterpret_cast<cx<R> *>(smem_raw);  // [group][3][rows_pad]
+    if (NG > 1) {
+        __syncthreads();
+        if (grp > 0)
+            for (int c = 0; c < 3; ++c) S[((grp - 1) * 3 + c) * rows_pad + q] = acc[c];
+        __syncthreads();
+    }
+    if (grp == 0 && q < p2)
+        for (int c = 0; c < 3; ++c) {
+            cx<R> v = acc[c];
+            for (int k = 1; k < NG; ++k) v += S[((k - 1) * 3 + c) * rows_pad + q];
+            C[(((int64_t)d * nbox + g) * 3 * nr + 3 * r + c) * p2 + q] = v;
+        }
 }
 
 // P2M for blocks of RB right-hand sides: the basis values of a (node, coefficient) are read once
@@ -924,11 +981,16 @@ __global__ void __launch_bounds__(32 * ROTC_WARPS) k_m2l_rot_cols(
 }
 
 // D(l,q) = R|R D(parent) + sum of the target's M2L pair results (Eq. 2.21), columns col0..col0+ncol.
-// Threads: rows_pad x ct column groups; a thread owns columns cid * L2L_CPT .. + L2L_CPT - 1.
+// Threads: rows_pad x ct column groups x NG pair groups; a thread owns columns cid * L2L_CPT .. + L2L_CPT - 1
+// and, with few columns, a quarter of the pairs (and of the dense R|R's inputs), the quarters added in order
+// through shared memory: a box has up to 189 pairs, whose results one thread read one after the other (FP64,
+// 642 nodes: 32 us for one level of 56 boxes).
 constexpr int L2L_CPT = 3;
-template <typename R>
-__global__ void k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, int p2, int64_t nbox, int col0, int ncol,
-                             int ct, const int32_t *parent, const uint64_t *key, const int32_t *ff_start,
+constexpr int L2L_GROUPS = 4;
+template <typename R, int NG>
+__global__ void __launch_bounds__(1024)
+    k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, int p2, int64_t nbox, int col0, int ncol, int ct,
+                             int rows_pad, const int32_t *parent, const uint64_t *key, const int32_t *ff_start,
                              const cx<R> *Tll, const cx<R> *Y, int64_t e_first, cx<R> *D, const cx<R> *Yll,
                              const int32_t *ll_entry, int64_t ll_first, int64_t y_dstride, int64_t yll_dstride,
                              const int *err) {
@@ -938,8 +1000,8 @@ __global__ void k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, i
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<R> *X = reinterpret_cast<cx<R> *>(smem_raw);
     const int64_t g = off + blockIdx.x;
-    const int rows_pad = blockDim.x / ct;
-    const int r = threadIdx.x % rows_pad, cid = threadIdx.x / rows_pad;
+    const int nt = rows_pad * ct, grp = NG == 1 ? 0 : threadIdx.x / nt;
+    const int r = threadIdx.x % rows_pad, cid = (NG == 1 ? threadIdx.x : threadIdx.x % nt) / rows_pad;
     const cx<R> *T = nullptr;
     if (l >= 3 && Yll == nullptr) {
         const int64_t P = parent[g];
@@ -948,44 +1010,63 @@ __global__ void k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, i
         T = Tll + oct_matrix(d, l, (int)(key[g] & 7), lmax) * p2 * p2;
         __syncthreads();
     }
-    if (r >= p2) return;
-    const int e0 = ff_start[g], e1 = ff_start[g + 1];
     // this thread's columns c0 .. c0 + L2L_CPT - 1: one read of T per row k feeds all of them
     const int c0 = cid * L2L_CPT;
-    cx<R> lp[L2L_CPT];
+    cx<R> sum[L2L_CPT];
 #pragma unroll
-    for (int j = 0; j < L2L_CPT; ++j) lp[j] = {0, 0};
-    if (T)
-        for (int k = 0; k < p2; ++k) {
-            const cx<R> t = T[(int64_t)k * p2 + r];
+    for (int j = 0; j < L2L_CPT; ++j) sum[j] = {0, 0};
+    if (r < p2) {
+        const int f0 = ff_start[g], cnt = ff_start[g + 1] - f0;
+        const int e0 = f0 + grp * cnt / NG, e1 = f0 + (grp + 1) * cnt / NG;
+        if (T)
+            for (int k = grp; k < p2; k += NG) {
+                const cx<R> t = T[(int64_t)k * p2 + r];
+#pragma unroll
+                for (int j = 0; j < L2L_CPT; ++j)
+                    if (c0 + j < ncol) cfma(sum[j], t, X[(c0 + j) * p2 + k]);
+            }
+        if (l >= 3 && Yll != nullptr && grp == 0) {  // R|R already applied in rotation form, per child entry
+            const cx<R> *yl = Yll + ((int64_t)(ll_entry[g] - ll_first) * ncol) * p2 + r;
 #pragma unroll
             for (int j = 0; j < L2L_CPT; ++j)
-                if (c0 + j < ncol) cfma(lp[j], t, X[(c0 + j) * p2 + k]);
+                if (c0 + j < ncol) sum[j] = yl[(c0 + j) * p2];
         }
-    if (l >= 3 && Yll != nullptr) {  // R|R already applied in rotation form, per child entry
-        const cx<R> *yl = Yll + ((int64_t)(ll_entry[g] - ll_first) * ncol) * p2 + r;
 #pragma unroll
-        for (int j = 0; j < L2L_CPT; ++j)
-            if (c0 + j < ncol) lp[j] = yl[(c0 + j) * p2];
-    }
-#pragma unroll
-    for (int j = 0; j < L2L_CPT; ++j) {
-        const int c = c0 + j;
-        if (c >= ncol) break;
-        cx<R> a0 = lp[j], a1 = {0, 0}, a2 = {0, 0}, a3 = {0, 0};
-        const cx<R> *y = Y + ((e0 - e_first) * ncol + c) * p2 + r;
-        const int64_t st = (int64_t)ncol * p2;
-        int e = e0;
-        for (; e + 4 <= e1; e += 4, y += 4 * st) {
-            a0 += y[0];
-            a1 += y[st];
-            a2 += y[2 * st];
-            a3 += y[3 * st];
+        for (int j = 0; j < L2L_CPT; ++j) {
+            const int c = c0 + j;
+            if (c >= ncol) break;
+            cx<R> a0 = sum[j], a1 = {0, 0}, a2 = {0, 0}, a3 = {0, 0};
+            const cx<R> *y = Y + ((e0 - e_first) * ncol + c) * p2 + r;
+            const int64_t st = (int64_t)ncol * p2;
+            int e = e0;
+            for (; e + 4 <= e1; e += 4, y += 4 * st) {
+                a0 += y[0];
+                a1 += y[st];
+                a2 += y[2 * st];
+                a3 += y[3 * st];
+            }
+            for (; e < e1; ++e, y += st) a0 += y[0];
+            sum[j] = (a0 + a1) + (a2 + a3);
         }
-        for (; e < e1; ++e, y += st) a0 += y[0];
-        if (err && *err) a0.re = a0.im = (R)NAN;  // the pair results are incomplete (a wait ran out)
-        D[(((int64_t)d * nbox + g) * 3 * nr + col0 + c) * p2 + r] = (a0 + a1) + (a2 + a3);
     }
+    if (NG > 1) {
+        cx<R> *S = X + (T ? ncol * p2 : 0);  // [group][L2L_CPT][rows_pad ct]
+        if (grp > 0)
+#pragma unroll
+            for (int j = 0; j < L2L_CPT; ++j) S[((grp - 1) * L2L_CPT + j) * nt + threadIdx.x % nt] = sum[j];
+        __syncthreads();
+        if (grp == 0)
+#pragma unroll
+            for (int j = 0; j < L2L_CPT; ++j)
+                for (int k = 1; k < NG; ++k) sum[j] += S[((k - 1) * L2L_CPT + j) * nt + threadIdx.x];
+    }
+    if (grp == 0 && r < p2)
+#pragma unroll
+        for (int j = 0; j < L2L_CPT; ++j) {
+            if (c0 + j >= ncol) break;
+            if (err && *err) sum[j].re = sum[j].im = (R)NAN;  // the pair results are incomplete (a wait ran out)
+            D[(((int64_t)d * nbox + g) * 3 * nr + col0 + c0 + j) * p2 + r] = sum[j];
+        }
 }
 
 // Rotation-form M2M: the parent's multipole is the sum of its children's translated expansions,
@@ -1942,33 +2023,34 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_d(
     }
 }
 
-// the rows of k_near_d: partial sums in split order, the far field (L2P) of the row's domain and the row
-// of the self block; thread per (node, row), grid (.., right-hand side)
+// the rows of k_near_d: the far field (L2P) of the row's domain, partial sums in split order and the row of
+// the self block; four lanes per (node, row), each a quarter of L2P's coefficients (its loads follow one
+// another); grid (.., right-hand side)
 __global__ void __launch_bounds__(192) k_near_finish(int64_t N, int64_t nr, int nsp, int p2, int64_t nbox,
                                                      const int32_t *__restrict__ node_leaf, const int32_t *__restrict__ dom,
                                                      const int32_t *__restrict__ perm, const c64 *__restrict__ Bl2p,
                                                      const c64 *__restrict__ D, const c64 *__restrict__ Mself,
                                                      const c64 *__restrict__ x, const c64 *__restrict__ part, c64 *y) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, r = blockIdx.y;
-    if (i >= N * 6) return;
-    const int64_t a = i / 6;
-    const int row = (int)(i - a * 6), sd = row / 3, c = row % 3;
-    c64 v = part[(r * N + a) * 6 + row];
-    for (int s = 1; s < nsp; ++s) v += part[((s * nr + r) * N + a) * 6 + row];
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 2, r = blockIdx.y;
+    const int l4 = threadIdx.x & 3;
+    const int64_t a = min(i / 6, N - 1);  // whole groups of four lanes stay for the shuffles
+    const int row = (int)(i % 6), sd = row / 3, c = row % 3;
     const int d = sd == 0 ? 0 : dom[a];
     const c64 *Dl = D + (((int64_t)d * nbox + node_leaf[a]) * 3 * nr + 3 * r + c) * p2, *B = Bl2p + ((int64_t)sd * N + a) * p2;
-    c64 w = {0, 0};
-    int q = 0;
-    for (; q + 1 < p2; q += 2) {  // two chains
-        cfma(v, Dl[q], B[q]);
-        cfma(w, Dl[q + 1], B[q + 1]);
-    }
-    if (q < p2) cfma(v, Dl[q], B[q]);
-    v += w;
+    c64 v = {0, 0};
+#pragma unroll 4
+    for (int q = l4; q < p2; q += 4) cfma(v, Dl[q], B[q]);
     const int64_t u = perm[a];
     const c64 *M = Mself + 36 * u + 6 * row, *xa = x + (r * N + u) * 6;
-    for (int cc = 0; cc < 6; ++cc) cfma(v, M[cc], xa[cc]);
-    y[(r * N + u) * 6 + row] = v;
+    for (int cc = l4; cc < 6; cc += 4) cfma(v, M[cc], xa[cc]);
+    if (l4 == 0)
+        for (int s = 0; s < nsp; ++s) v += part[((s * nr + r) * N + a) * 6 + row];
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+        v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
+        v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
+    }
+    if (l4 == 0 && i < N * 6) y[(r * N + u) * 6 + row] = v;
 }
 
 // Steps 4-5 for one to three right-hand sides in single precision, both sides of every pair in
@@ -3224,9 +3306,14 @@ void near_work_items(fmbem *h, cudaStream_t s) {
 }
 
 // The child boxes of every level l >= 3 for the rotation-form M2M and L2L: entries grouped by
-// octant (the child-parent direction), in chunks of at most M2L_CHUNK that share it; each chunk
+// octant (the child-parent direction), in chunks that share it; each chunk
 // carries the far-field offset code of the same direction for M2M (child to parent, offset
 // (4o-2) per axis) and for L2L (parent to child, the opposite one).
+// A chunk is ten children, one pass of k_m2l_rot_cols (32 columns), where a level has few boxes (200 boxes
+// in chunks of 32 were 28 blocks of four passes, FP64 237 us a level, now 66), and M2L_CHUNK otherwise: the
+// rotation factors are loaded less often, which counts where BF16x3 runs these launches on eight SMs beside
+// its M2L (163842 nodes, M2M + downward pass: 712 boxes in chunks of ten 1.53 ms, of 30 1.48, of 32 1.466).
+constexpr int RMM_FEW = 400;
 void build_rot_mm_lists(fmbem *h, cudaStream_t s) {
     const int lmax = h->lmax;
     std::vector<uint64_t> key(h->nbox);
@@ -3247,10 +3334,11 @@ void build_rot_mm_lists(fmbem *h, cudaStream_t s) {
             const int ox = (o >> 2) & 1, oy = (o >> 1) & 1, oz = o & 1;  // Morton bit order x, y, z
             const int16_t mm = (int16_t)m2l_offset_code(4 * ox - 2, 4 * oy - 2, 4 * oz - 2);
             const int16_t ll = (int16_t)m2l_offset_code(2 - 4 * ox, 2 - 4 * oy, 2 - 4 * oz);
-            int in_chunk = M2L_CHUNK;
+            const int chunk = Lv.n < RMM_FEW ? 10 : M2L_CHUNK;
+            int in_chunk = chunk;
             for (int64_t g = Lv.off; g < Lv.off + Lv.n; ++g) {
                 if ((int)(key[g] & 7) != o) continue;
-                if (in_chunk == M2L_CHUNK) {
+                if (in_chunk == chunk) {
                     cbeg.push_back((int32_t)child.size());
                     ccnt.push_back(0);
                     cmm.push_back(mm);
@@ -3350,18 +3438,20 @@ static bool oz_ready(const fmbem *h, int W) {
            h->ybuf_bytes >= oz_ybuf_need(h, W);
 }
 
-// source splits per item of k_near_d: about eight units for each of the 608 warp schedulers, no more than
-// the longest source list has tiles, eight at most (the partial sums' buffer)
+// source splits per item of k_near_d: about sixteen units for each of the 608 warp schedulers, no more than
+// the longest source list has tiles, 32 at most (the partial sums' buffer).  The four warps of a scheduler
+// share its FP64 pipe and end together, so with five units each some got eight (2562 nodes: 520-930 us with
+// at most eight splits)
 static int near_d_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_ditems * nr);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({8, h->near_tiles_max, (8 * 608 + units - 1) / units}));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({32, h->near_tiles_max, (16 * 608 + units - 1) / units}));
 }
-// and per item of k_near_ws (single precision, 1-3 right-hand sides): about two units for each of the 24
+// and per item of k_near_ws (single precision, 1-3 right-hand sides): about four units for each of the 24
 // warps an SM holds.  A unit is latency-bound (a pair takes about 400 cycles of its warp), so with one unit
 // per item 10242 nodes (1450 units) took 215 us, ten times the arithmetic's time
 static int near_ws_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_items * nr);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({8, h->near_tiles_max, (2 * 24 * 152 + units - 1) / units}));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * 152 + units - 1) / units}));
 }
 // the near field's partial sums (rows complex values of a node, right-hand side and split), and per-source
 // vectors of the FP64 forward product
@@ -3660,9 +3750,20 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                 }
                 cudaStream_t sr = overlap && l < lmax ? h->aux_stream : s;  // this level's reduction
                 const int ct = (nc + L2L_CPT - 1) / L2L_CPT;
-                k_l2l_reduce<R><<<dim3((unsigned)Lv.n, (unsigned)(J + 1)), rows_pad * ct, sizeof(cx<R>) * nc * p2, sr>>>(
-                    Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, h->box_parent, h->box_key, h->ff_start, Tll, Y,
-                    e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
+                // pair groups where the boxes do not fill the chip (3384 boxes in two domains, FP64: 690 us with
+                // one group, 1016 with four), and none on the few SMs that the BF16x3 overlap leaves
+                const bool one = Lv.n * (J + 1) >= 512 || (overlap && l < lmax) || rows_pad * ct * L2L_GROUPS > 512;
+                const size_t smr = sizeof(cx<R>) * ((l >= 3 && Yll == nullptr ? (size_t)nc * p2 : 0) +
+                                                    (one ? 0 : (size_t)(L2L_GROUPS - 1) * L2L_CPT * rows_pad * ct));
+                const dim3 rgrid((unsigned)Lv.n, (unsigned)(J + 1));
+                if (one)
+                    k_l2l_reduce<R, 1><<<rgrid, rows_pad * ct, smr, sr>>>(
+                        Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent, h->box_key, h->ff_start,
+                        Tll, Y, e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
+                else
+                    k_l2l_reduce<R, L2L_GROUPS><<<rgrid, rows_pad * ct * L2L_GROUPS, smr, sr>>>(
+                        Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent, h->box_key, h->ff_start,
+                        Tll, Y, e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
                 CKL("k_l2l_reduce");
             }
         }
@@ -3728,6 +3829,9 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     const cx<R> *Bl2p = f32 ? (const cx<R> *)h->B_l2p32 : (const cx<R> *)h->B_l2p64;
     const bool timing = h->profile && h->ev[0] != nullptr;
     if (timing) CK(cudaEventRecord(h->ev[0], s));
+    int dev = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
 
     // single precision with 32 or more right-hand sides: a node-major copy of the background
     // densities and the normal jumps for k_near_r in the half of the density buffer that double
@@ -3773,9 +3877,19 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     } else if (nr >= 4)
         k_p2m_rb<R, P2M_RB><<<dim3((unsigned)h->n_leaves, J + 1, (unsigned)((nr + P2M_RB - 1) / P2M_RB)), tbc, 0, s>>>(
             h->leaf_box, N, nr, p2, h->nbox, h->box_nbeg, h->box_nend, h->dom, h->nrm, dens, Bp2m, C);
-    else  // one thread per coefficient
-        k_p2m<R><<<dim3((unsigned)h->n_leaves, J + 1, (unsigned)nr), ((p2 + 31) / 32) * 32, 0, s>>>(
-            h->leaf_box, N, nr, p2, h->nbox, h->box_nbeg, h->box_nend, h->dom, h->nrm, dens, Bp2m, C);
+    else {  // threads per (coefficient, group of nodes)
+        const int rows_pad = ((p2 + 31) / 32) * 32;
+        // one group where the blocks fill the chip (163842 nodes, FP32: 202 us; four groups 229)
+        const bool one = (int64_t)h->n_leaves * (J + 1) * nr >= 8 * nsm || rows_pad > 128;
+        const dim3 grid((unsigned)h->n_leaves, J + 1, (unsigned)nr);
+        const size_t smp = sizeof(cx<R>) * (size_t)std::max(P2M_WN * 12, one ? 0 : (P2M_GROUPS - 1) * 3 * rows_pad);
+        if (one)
+            k_p2m<R, 1><<<grid, rows_pad, smp, s>>>(h->leaf_box, N, nr, p2, rows_pad, h->nbox, h->box_nbeg, h->box_nend,
+                                                    h->dom, h->nrm, dens, Bp2m, C);
+        else
+            k_p2m<R, P2M_GROUPS><<<grid, rows_pad * P2M_GROUPS, smp, s>>>(h->leaf_box, N, nr, p2, rows_pad, h->nbox, h->box_nbeg,
+                                                                          h->box_nend, h->dom, h->nrm, dens, Bp2m, C);
+    }
     CKL("k_p2m");
     if (timing) CK(cudaEventRecord(h->ev[1], s));
     if (tc_up) run_m2m_tc(h, (float *)C, nr, s, tc_p2m);
@@ -3786,12 +3900,8 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     const R *ph = f32 ? (const R *)h->pos_hi : (const R *)h->pos;
     const R *pl = f32 ? (const R *)h->pos_lo : nullptr;
     const R *nn = f32 ? (const R *)h->nrm_f : (const R *)h->nrm;
-    // near field: in single precision the warp-independent kernel with blocks of RB right-hand
-    // sides (the pair scalars are shared by the block); for fewer than 4 right-hand sides, and in
-    // double precision, the block-cooperative kernels (more threads per leaf, FP64 pipe busier)
-    int dev = 0, nsm = 0;
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    // near field: kernels of independent warps; blocks of right-hand sides share the pair scalars in single
+    // precision, the cache holds them in double
     // the scatterer side's near field is not needed with the impedance boundary (k_local_rows)
     const int nsides = h->ibc ? 1 : 2;
     // k_near_w over the right-hand sides rhs_base .. nr - 1 in blocks of rb
@@ -3890,7 +4000,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
         };
         if (h->near_cache64) launch_d(k_near_d<true>);
         else launch_d(k_near_d<false>);
-        k_near_finish<<<dim3(nblk(6 * N, 192), (unsigned)nr), 192, 0, s>>>(N, nr, nsp, p2, h->nbox, h->node_leaf, h->dom, h->perm,
+        k_near_finish<<<dim3(nblk(24 * N, 192), (unsigned)nr), 192, 0, s>>>(N, nr, nsp, p2, h->nbox, h->node_leaf, h->dom, h->perm,
                                                                           Bl2p, D, h->Mself, x, h->near_part, y);
     } else if (nr >= 4) {  // the allocation-free product
         constexpr int RBLK = 2;

@@ -35,7 +35,7 @@ def rel(a, b):
 
 # one and several tiles of 80 columns, windows of unequal width, ragged column counts
 @pytest.mark.parametrize("p", [4, 6, 8, 10])
-@pytest.mark.parametrize("n_rhs", [1, 2, 5, 17, 33])
+@pytest.mark.parametrize("n_rhs", [1, 2, 5, 16, 17, 33])
 def test_matches_dense_form(p, n_rhs):
     a, d = handles("torus", p, leaf_size=16)  # levels 2 to 4
     x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=p + n_rhs)).cuda()
