@@ -159,7 +159,8 @@ fmbem_status fmbem_batch_create(fmbem *const *handles, int32_t n_problems, int64
             }
         for (int32_t i = 0; i < n_problems; ++i) {
             const fmbem *h = b->hs[i];
-            for (int64_t lf = 0; lf < h->lev[h->lmax].n; ++lf) add(i, BK_NEAR, 0, (int32_t)lf, 0, 0);
+            for (int64_t lf = 0; lf < h->lev[h->lmax].n; ++lf)
+                for (int64_t r = 0; r < nr; ++r) add(i, BK_NEAR, 0, (int32_t)lf, 0, (int16_t)r);
         }
         b->n_items = (int64_t)items.size();
         for (fmbem *h : b->hs) {

@@ -459,7 +459,7 @@ __global__ void k_p2m_gemm(const int32_t *leaf_box, int64_t N, int64_t nr, int p
 // acc[cc] += sum_c T[c][r] X[cc][c] for the thread's output row r; X in shared memory
 template <typename R, int CC>
 __device__ __forceinline__ void apply_T(const cx<R> *__restrict__ T, const cx<R> *X, int p2, int r, int ncol, cx<R> *acc) {
-#pragma unroll 4
+#pragma unroll 8
     for (int c = 0; c < p2; ++c) {
         cx<R> t = T[(int64_t)c * p2 + r];
 #pragma unroll
@@ -506,7 +506,7 @@ __global__ void k_m2m(int64_t par_off, int l, int lmax, int64_t nr, int p2, int6
 }
 
 // M2L + L2L (Eq. 2.21): D(l,q) = R|R D(parent) + sum_{FF(l,q)} S|R C(source)
-template <typename R>
+template <typename R, int G>
 __device__ __forceinline__ void down_body(int64_t off, int l, int lmax, int64_t nr, int p2, int64_t nbox,
                                           const int32_t *parent, const uint64_t *key, const int32_t *ff_start,
                                           const int32_t *ff_src, const int16_t *ff_off, const cx<R> *Tm2l,
@@ -517,16 +517,20 @@ __device__ __forceinline__ void down_body(int64_t off, int l, int lmax, int64_t 
     int d = by;
     int col0 = bz * CC;
     int ncol = min(CC, (int)(3 * nr) - col0);
-    int r = threadIdx.x;
-    cx<R> acc[CC];
-    for (int cc = 0; cc < CC; ++cc) acc[cc] = {0, 0};
+    // the block's threads: rows_pad rows x column groups of NC columns
+    const int rows_pad = G == 1 ? blockDim.x : blockDim.x / G;
+    const int r = threadIdx.x % rows_pad, cg = threadIdx.x / rows_pad;
+    constexpr int NC = CC / G;
+    const int c0 = cg * NC;
+    cx<R> acc[NC];
+    for (int cc = 0; cc < NC; ++cc) acc[cc] = {0, 0};
     if (l >= 3) {
         int64_t P = parent[g];
         for (int e = threadIdx.x; e < ncol * p2; e += blockDim.x)
             X[e] = D[(((int64_t)d * nbox + P) * 3 * nr + col0 + e / p2) * p2 + e % p2];
         __syncthreads();
         int o = (int)(key[g] & 7);
-        if (r < p2) apply_T<R, CC>(Tll + oct_matrix(d, l, o, lmax) * p2 * p2, X, p2, r, ncol, acc);
+        if (r < p2) apply_T<R, NC>(Tll + oct_matrix(d, l, o, lmax) * p2 * p2, X + c0 * p2, p2, r, ncol - c0, acc);
     }
     for (int e0 = ff_start[g]; e0 < ff_start[g + 1]; ++e0) {
         __syncthreads();
@@ -534,16 +538,17 @@ __device__ __forceinline__ void down_body(int64_t off, int l, int lmax, int64_t 
         for (int e = threadIdx.x; e < ncol * p2; e += blockDim.x)
             X[e] = C[(((int64_t)d * nbox + src) * 3 * nr + col0 + e / p2) * p2 + e % p2];
         __syncthreads();
-        if (r < p2) apply_T<R, CC>(Tm2l + m2l_matrix(d, l, ff_off[e0], lmax) * p2 * p2, X, p2, r, ncol, acc);
+        if (r < p2) apply_T<R, NC>(Tm2l + m2l_matrix(d, l, ff_off[e0], lmax) * p2 * p2, X + c0 * p2, p2, r, ncol - c0, acc);
     }
     if (r < p2)
-        for (int cc = 0; cc < ncol; ++cc) D[(((int64_t)d * nbox + g) * 3 * nr + col0 + cc) * p2 + r] = acc[cc];
+        for (int cc = 0; cc < NC; ++cc)
+            if (c0 + cc < ncol) D[(((int64_t)d * nbox + g) * 3 * nr + col0 + c0 + cc) * p2 + r] = acc[cc];
 }
 template <typename R>
 __global__ void k_down(int64_t off, int l, int lmax, int64_t nr, int p2, int64_t nbox, const int32_t *parent,
                        const uint64_t *key, const int32_t *ff_start, const int32_t *ff_src, const int16_t *ff_off,
                        const cx<R> *Tm2l, const cx<R> *Tll, const cx<R> *C, cx<R> *D) {
-    down_body<R>(off, l, lmax, nr, p2, nbox, parent, key, ff_start, ff_src, ff_off, Tm2l, Tll, C, D, blockIdx.x,
+    down_body<R, 1>(off, l, lmax, nr, p2, nbox, parent, key, ff_start, ff_src, ff_off, Tm2l, Tll, C, D, blockIdx.x,
                  blockIdx.y, blockIdx.z);
 }
 
@@ -1285,7 +1290,7 @@ __device__ __forceinline__ void near_body(int64_t g, int64_t N, int64_t nr, int 
                                           const int32_t *dom, const int32_t *perm, const cx<R> *dens,
                                           const DomainConsts *dc, const cx<R> *Bl2p, const cx<R> *D, const c64 *Mself,
                                           const c64 *x, c64 *y, const int64_t *cache_base, const V4<R> *cache,
-                                          bool side1, int64_t bx) {
+                                          bool side1, int64_t bx, int64_t r0, int64_t r1) {
     __shared__ NearSmem<R> S;
     __shared__ int rng_beg[32], rng_cum[33];
     SrcTile<R> &T = S.tile;
@@ -1303,7 +1308,7 @@ __device__ __forceinline__ void near_body(int64_t g, int64_t N, int64_t nr, int 
     __syncthreads();
     const int nsrc = rng_cum[nnb];
     const int t0 = nbeg[g], t1 = nend[g];
-    for (int64_t r = 0; r < nr; ++r) {
+    for (int64_t r = r0; r < r1; ++r) {
         for (int tb = t0; tb < t1; tb += 128) {
             const int nt = min(128, t1 - tb);
             const int nsl = 128 / nt;
@@ -1428,7 +1433,7 @@ __global__ void __launch_bounds__(128) k_near(const int32_t *leaf_box, int64_t N
                                               const c64 *x, c64 *y, const int64_t *cache_base,
                                               const V4<R> *cache, bool side1) {
     near_body<R, DOUBLE_FLOAT>(leaf_box[blockIdx.x], N, nr, p2, nbox, nbeg, nend, nbr_start, nbr_idx, pos_hi, pos_lo, nrm, dom,
-                               perm, dens, dc, Bl2p, D, Mself, x, y, cache_base, cache, side1, blockIdx.x);
+                               perm, dens, dc, Bl2p, D, Mself, x, y, cache_base, cache, side1, blockIdx.x, 0, nr);
 }
 
 // ---------------------------------------------------------------- near field for blocks of RHS
@@ -2992,8 +2997,12 @@ __device__ bool batch_wait(const unsigned *c, unsigned target, uint64_t wait_ns,
     }
 }
 
+// Five blocks per SM (the items wait on loads of translation matrices and sources; 12 particles of 1000 to
+// 8000 nodes, 4 right-hand sides: four blocks 4.33 ms with eight loads in flight per thread, five 4.01, six
+// 4.03; with four loads in flight 4.65, 4.33, 4.19).  Translation items split their six columns over the
+// block's two halves where p^2 <= 64, and near items are one right-hand side of a leaf: 5.61 ms without.
 template <typename R>
-__global__ void __launch_bounds__(128) k_batch(const BatchProblem *probs, const BatchItem *items, int64_t n_items,
+__global__ void __launch_bounds__(128, 5) k_batch(const BatchProblem *probs, const BatchItem *items, int64_t n_items,
                                                int64_t nr, unsigned long long *next, unsigned *cnt,
                                                const unsigned *tgt, int *err, uint64_t wait_ns, int stall_problem) {
     __shared__ int64_t s_it;
@@ -3042,16 +3051,22 @@ __global__ void __launch_bounds__(128) k_batch(const BatchProblem *probs, const 
                                 (const cx<R> *)P.Tmm, (cx<R> *)P.C, w.a, w.b, w.c);
                 break;
             case BK_DOWN:
-                down_body<R>(P.lev_off[w.level], w.level, lmax, nr, P.p2, P.nbox, P.parent, P.key, P.ff_start,
-                             P.ff_src, P.ff_off, (const cx<R> *)P.Tm2l, (const cx<R> *)P.Tll, (const cx<R> *)P.C,
-                             (cx<R> *)P.D, w.a, w.b, w.c);
+                // p^2 <= 64: the block's 128 threads are 64 rows x two groups of three columns
+                if (P.p2 <= 64)
+                    down_body<R, 2>(P.lev_off[w.level], w.level, lmax, nr, P.p2, P.nbox, P.parent, P.key, P.ff_start,
+                                    P.ff_src, P.ff_off, (const cx<R> *)P.Tm2l, (const cx<R> *)P.Tll,
+                                    (const cx<R> *)P.C, (cx<R> *)P.D, w.a, w.b, w.c);
+                else
+                    down_body<R, 1>(P.lev_off[w.level], w.level, lmax, nr, P.p2, P.nbox, P.parent, P.key, P.ff_start,
+                                    P.ff_src, P.ff_off, (const cx<R> *)P.Tm2l, (const cx<R> *)P.Tll,
+                                    (const cx<R> *)P.C, (cx<R> *)P.D, w.a, w.b, w.c);
                 break;
             default:
                 near_body<R, sizeof(R) == 4>(P.lev_off[lmax] + w.a, P.N, nr, P.p2, P.nbox, P.nbeg, P.nend, P.nbr_start,
                                              P.nbr_idx, (const R *)P.pos_hi, (const R *)P.pos_lo, (const R *)P.nrm,
                                              P.dom, P.perm, (const cx<R> *)P.dens, (const DomainConsts *)P.dc,
                                              (const cx<R> *)P.Bl2p, (const cx<R> *)P.D, P.Mself, P.x, P.y, nullptr,
-                                             nullptr, true, w.a);
+                                             nullptr, true, w.a, w.c, w.c + 1);
                 break;
         }
         __syncthreads();
