@@ -374,8 +374,10 @@ void run_m2l_ofs(fmbem *h, const float *C, float *Y, int64_t nr, cudaStream_t s,
 bool m2l_oz_supported(const fmbem *h);
 void build_oz_tables(fmbem *h, cudaStream_t s);
 int64_t oz_y_dom(const fmbem *h, int W);
+template <typename R>
 size_t oz_digit_bytes(const fmbem *h, int W);
-void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s);
+template <typename R>
+void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W, cudaStream_t s);
 void check_oz_err(fmbem *h, cudaStream_t s);
 void pack_rot_tables(fmbem *h, cudaStream_t s);
 void pack_rot_tables_mm(fmbem *h, cudaStream_t s);

@@ -3424,16 +3424,23 @@ static size_t ofs_ybuf_need(const fmbem *h, int64_t nr) {
     return sizeof(float) * (size_t)(h->Jf + 1) * (ofs_y_dom(h, nr) + (size_t)ne * 3 * nr * 2 * h->p2);
 }
 
-// FP64 M2L on the tensor cores (m2l_oz.cu): columns per window.  All levels' pair results of a window
-// are kept (its products run in one launch), so the window is narrowed until they take at most 8 GB;
-// at most as many columns as the per-target reduction has threads for, in whole right-hand sides.
+// BF16x3 with few columns: the offset-stationary M2L
+static bool ofs_applies(const fmbem *h, int64_t nr, int tensor_mode) {
+    return tensor_mode == 2 && h->Aofs != nullptr && h->chunk_pairs != nullptr && 3 * nr <= 24;
+}
+// M2L on the tensor cores in 8-bit digits (m2l_oz.cu): FP64, and single precision where no BF16x3 or TF32
+// form runs.  Columns per window: all levels' pair results of a window are kept (its products run in one
+// launch), so the window is narrowed until they take at most 8 GB; at most as many columns as the
+// per-target reduction has threads for, in whole right-hand sides.
 // 0: not used (its images were not built, or the caller asked for a translation form).
-static int oz_window(const fmbem *h, int64_t nr) {
-    if (h->oz_img == nullptr) return 0;
+template <typename R>
+static int oz_window(const fmbem *h, int64_t nr, int tensor_mode) {
+    if (h->oz_img == nullptr || ofs_applies(h, nr, tensor_mode)) return 0;
+    if (tensor_mode && h->Atc != nullptr && 3 * nr >= 48) return 0;
     const int rows_pad = ((h->p2 + 31) / 32) * 32;
     int64_t most = std::min<int64_t>(48, 3 * (1024 / rows_pad));
     if (h->R_D64 != nullptr) most = std::min<int64_t>(most, 24);  // L2L in rotation form beside it
-    const int64_t per_col = (int64_t)sizeof(c64) * (h->Jf + 1) * std::max<int64_t>(h->n_ff, 1) * h->p2;
+    const int64_t per_col = (int64_t)sizeof(cx<R>) * (h->Jf + 1) * std::max<int64_t>(h->n_ff, 1) * h->p2;
     most = std::max<int64_t>(3, std::min(most, (int64_t(8) << 30) / per_col) / 3 * 3);
     const int64_t windows = (3 * nr + most - 1) / most, W = 3 * ((nr + windows - 1) / windows);
     // its row and result indices are 32-bit
@@ -3441,16 +3448,18 @@ static int oz_window(const fmbem *h, int64_t nr) {
     return (int)W;
 }
 // bytes of a window's pair results, then one level's rotation-form L2L entries
+template <typename R>
 static size_t oz_ybuf_need(const fmbem *h, int W) {
     int64_t ne = 0;
     for (int l = 2; l <= h->lmax; ++l)
         if (!h->h_rmm_first.empty()) ne = std::max(ne, h->h_rmm_first[l + 1] - h->h_rmm_first[l]);
-    return sizeof(c64) * (size_t)(h->Jf + 1) * (size_t)(std::max<int64_t>(h->n_ff, 1) + ne) * (size_t)W * h->p2;
+    return sizeof(cx<R>) * (size_t)(h->Jf + 1) * (size_t)(std::max<int64_t>(h->n_ff, 1) + ne) * (size_t)W * h->p2;
 }
 // the scratch of a window exists
+template <typename R>
 static bool oz_ready(const fmbem *h, int W) {
-    return W > 0 && h->oz_dig != nullptr && h->oz_dig_bytes >= oz_digit_bytes(h, W) && h->ybuf != nullptr &&
-           h->ybuf_bytes >= oz_ybuf_need(h, W);
+    return W > 0 && h->oz_dig != nullptr && h->oz_dig_bytes >= oz_digit_bytes<R>(h, W) && h->ybuf != nullptr &&
+           h->ybuf_bytes >= oz_ybuf_need<R>(h, W);
 }
 
 // source splits per item of k_near_d: about sixteen units for each of the 608 warp schedulers, no more than
@@ -3501,18 +3510,21 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
     // one column window of the FP64 rotation form for more columns); sized by the columns of
     // this call, so that a few-column call after a many-column one still takes the chunked path
     const bool many = rot_many_path(h, nr, precision == FMBEM_FP64);
-    const int ozw = precision == FMBEM_FP64 && pair_results ? oz_window(h, nr) : 0;
-    if (ozw > 0 && h->oz_dig_bytes < oz_digit_bytes(h, ozw)) {
+    const int mode = precision == FMBEM_BF16X3 ? 2 : precision == FMBEM_TF32 ? 1 : 0;
+    const bool dbl = precision == FMBEM_FP64;
+    const int ozw = !pair_results ? 0 : dbl ? oz_window<double>(h, nr, 0) : oz_window<float>(h, nr, mode);
+    const size_t dig = dbl ? oz_digit_bytes<double>(h, ozw) : oz_digit_bytes<float>(h, ozw);
+    if (ozw > 0 && h->oz_dig_bytes < dig) {
         if (h->oz_dig) dev_free(h, h->oz_dig);
         h->oz_dig = nullptr;
         h->oz_dig_bytes = 0;
-        h->oz_dig = dev_alloc(h, oz_digit_bytes(h, ozw));
-        h->oz_dig_bytes = oz_digit_bytes(h, ozw);
+        h->oz_dig = dev_alloc(h, dig);
+        h->oz_dig_bytes = dig;
     }
     if (pair_results && (3 * nr <= 24 || many || ozw > 0)) {
         size_t need = 3 * nr <= 24 || many ? ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb) : 0;
-        if (ozw > 0) need = std::max(need, oz_ybuf_need(h, ozw));
-        if (precision == FMBEM_BF16X3 && h->Aofs != nullptr && 3 * nr <= 24) need = std::max(need, ofs_ybuf_need(h, nr));
+        if (ozw > 0) need = std::max(need, dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw));
+        if (ofs_applies(h, nr, mode)) need = std::max(need, ofs_ybuf_need(h, nr));
         if (h->ybuf == nullptr || h->ybuf_bytes < need) {
             if (h->ybuf) dev_free(h, h->ybuf);
             h->ybuf = nullptr;
@@ -3653,9 +3665,9 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
     constexpr int MAXC = 24;
     // FP64 with more than MAXC columns and rotation tables: the rotation form in column windows
     const bool rot_many = rot_many_path(h, nr, !f32);
-    // FP64 on the tensor cores, any number of columns in windows
-    const int ozw = f32 ? 0 : oz_window(h, nr);
-    const bool oz = oz_ready(h, ozw);
+    // in digits on the tensor cores, any number of columns in windows
+    const int ozw = oz_window<R>(h, nr, tensor_mode);
+    const bool oz = oz_ready<R>(h, ozw);
     const int ncol = oz ? ozw : rot_many ? rot_many_cols(h) : (int)std::min<int64_t>(3 * nr, MAXC);
     const size_t tbytes = sizeof(cx<R>) * p2 * p2;
     const size_t budget = 200 * 1024;
@@ -3695,8 +3707,7 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
         // (all levels and domains in one launch first: the S|R products read only C; the pair
         // results of every level then wait in Y[d][CSR position], and the rotation form's L2L
         // results go after them)
-        const bool ofs = tensor_mode == 2 && f32 && h->Aofs != nullptr && h->chunk_pairs != nullptr && 3 * nr <= MAXC &&
-                         h->ybuf_bytes >= ofs_ybuf_need(h, nr);
+        const bool ofs = f32 && ofs_applies(h, nr, tensor_mode) && h->ybuf_bytes >= ofs_ybuf_need(h, nr);
         // With a second stream the coarse levels' M2L (levels 2..l_max-1) runs first; then, while
         // the leaf level's M2L occupies all but OFS_AUX_SMS SMs, the second stream runs those
         // levels' L2L + reductions and the leaf level's L2L, which are latency-bound chains of
@@ -3720,8 +3731,7 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
         // results at Y + d * ystr, its rotation-form L2L entries after every domain's pair results
         for (int col0 = 0; col0 < 3 * nr; col0 += ncol) {
             const int nc = (int)std::min<int64_t>(ncol, 3 * nr - col0);
-            if constexpr (sizeof(R) == 8)
-                if (oz) run_m2l_oz(h, C, Y, nr, col0, nc, s);
+            if (oz) run_m2l_oz<R>(h, C, Y, nr, col0, nc, s);
             for (int l = 2; l <= lmax; ++l) {
                 const LevelInfo &Lv = h->lev[l];
                 const int64_t c0 = h->h_chunk_first[l], nch = h->h_chunk_first[l + 1] - c0;

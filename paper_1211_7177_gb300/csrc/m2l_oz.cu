@@ -1,4 +1,4 @@
-// m2l_oz.cu -- the FP64 M2L (S|R part of Eq. 2.21) on the GB300 tensor cores.
+// m2l_oz.cu -- the FP64 and FP32 M2L (S|R part of Eq. 2.21) on the GB300 tensor cores.
 //
 // GB300 runs FP64 at about 1/60 of its FP32 rate, and the double-precision M2L on the FP64 pipe was
 // bound by it (the folded rotation form 88 % busy at p = 10, the dense many-column form at p = 8).
@@ -18,9 +18,16 @@
 // precision (rms relative error, torus of 3840 nodes): p = 8 8e-17 and p = 10 3e-16, where the FP64 sums
 // of the dense form have 5e-16 and the rotation form 1e-8 (a seven-digit form had 6e-16 and 1.5e-15).
 //
+// A single-precision product takes the first four digits of the same images and four digits of its sources
+// (2^-31 of the largest entry), ten products in four exact accumulators, added once in FP32: more exact than
+// the FP32 sums it replaces (product errors against FP64, torus of 9216 nodes: p = 8, 16 right-hand sides
+// 5.1e-7 with the dense sums, 1.3e-7; p = 10, 3 right-hand sides 1.2e-7 with the rotation form, 1.0e-7), and
+// faster at every size (a whole product: sphere of 642 nodes 135 -> 104 us, 40962 nodes p = 10 1.69 -> 1.03 ms,
+// torus of 9216 nodes with 16 right-hand sides 8.3 -> 2.4 ms).
+//
 // The FF pairs of one level and offset share a matrix; their columns (W per pair) follow one another
-// and are cut into tiles of OZ_N = 80, the N of the MMAs (six accumulators of 80 columns fill tensor
-// memory); the matrix rows are its M = 128 (one row tile for p <= 8, two for p = 10).  The results go to
+// and are cut into tiles of N columns, the N of the MMAs (FP64: 80, six accumulators of 80 columns fill tensor
+// memory; FP32: 128, four accumulators); the matrix rows are its M = 128 (one row tile for p <= 8, two for p = 10).  The results go to
 // Y[pair][column], which k_l2l_reduce sums per target.
 #include <algorithm>
 #include <string>
@@ -31,19 +38,34 @@
 namespace {
 
 constexpr int OZ_S = 8;      // digits per double
-constexpr int OZ_N = 80;     // pair columns per tile
-constexpr int OZ_ACC = 6;    // accumulators: d = 0, 1, 2, 3, 4 and 5..7
 constexpr int OZ_SLOTS = 4;  // operand ring: one K block of 16 each
 constexpr int OZ_FILL = 3;   // producer warps
 constexpr int OZ_EPI = 16;   // epilogue warps
 constexpr int OZ_NONFINITE = 1 << 20;  // exponent marking a column or row with an Inf or a NaN
-constexpr uint32_t OZ_A_BYTES = OZ_S * TC_M * 32u, OZ_B_BYTES = OZ_S * OZ_N * 32u;
-constexpr uint32_t OZ_SLOT_BYTES = OZ_A_BYTES + OZ_B_BYTES;
-constexpr int OZ_ROW = OZ_S * 32;  // bytes of a source column's digits in one K block
+constexpr uint32_t OZ_A_BYTES = OZ_S * TC_M * 32u;  // the matrix digits of one K block
+template <typename R>
+struct Oz;
+template <>
+struct Oz<double> {
+    static constexpr int S = OZ_S;  // digits
+    static constexpr int N = 80;    // pair columns per tile
+    static constexpr int ACC = 6;   // accumulators: d = 0, 1, 2, 3, 4 and 5..7
+};
+template <>
+struct Oz<float> {
+    static constexpr int S = 4, N = 128, ACC = 4;  // d = 0..3
+};
+template <typename R>
+constexpr uint32_t oz_a_bytes = Oz<R>::S * TC_M * 32u;
+template <typename R>
+constexpr uint32_t oz_slot_bytes = oz_a_bytes<R> + Oz<R>::S * Oz<R>::N * 32u;
+template <typename R>
+constexpr int oz_row = Oz<R>::S * 32;  // bytes of a source column's digits in one K block
 constexpr int OZ_MAX_LEVELS = 12;
 constexpr int OZ_THREADS = 32 * (OZ_FILL + 1 + OZ_EPI);
-static_assert(OZ_SLOTS == 4 && OZ_FILL == 3 && OZ_EPI == 16 && OZ_ACC * OZ_N <= 512 && OZ_S == 8,
-              "ring arithmetic, tensor-memory lanes of the epilogue warps, tensor memory, digit arithmetic");
+static_assert(OZ_SLOTS == 4 && OZ_FILL == 3 && OZ_EPI == 16 && OZ_S == 8 && Oz<double>::ACC * Oz<double>::N <= 512 &&
+                  Oz<float>::ACC * Oz<float>::N <= 512,
+              "ring arithmetic, tensor-memory lanes of the epilogue warps, digit arithmetic, tensor memory");
 
 // byte offset of the 16-byte chunk c (0, 1) of a row in the 32-byte-swizzled K-major layout
 __host__ __device__ __forceinline__ uint32_t sw32_chunk(int row, int c) {
@@ -73,7 +95,28 @@ __device__ __forceinline__ int oz_exp2(double a, double b) {
     return e - 1022;
 }
 
-// the digits of x 2^shift (|x 2^shift| < 1), each as the bf16 bits of digit 2^(-7 - 8 i)
+__device__ __forceinline__ int oz_exp2(float a, float b) {
+    const int ea = (__float_as_int(a) >> 23) & 0xff, eb = (__float_as_int(b) >> 23) & 0xff;
+    const int e = max(ea, eb);
+    if (e == 0xff) return OZ_NONFINITE;
+    if (e == 0) return a == 0.f && b == 0.f ? -OZ_NONFINITE : -126;
+    return e - 126;
+}
+
+// the digits of x 2^shift (|x 2^shift| < 1), each as the bf16 bits of digit 2^(-7 - 8 i); a float has
+// 24 bits, so that 2^31 times it is an int
+__device__ __forceinline__ void oz_digits(float x, int shift, uint16_t *out) {
+    constexpr int S = Oz<float>::S;
+    int m = __float2int_rn(ldexpf(x, shift + 8 * S - 1));
+#pragma unroll
+    for (int i = S - 1; i >= 0; --i) {
+        const int dgt = i > 0 ? (int)(int8_t)(m & 0xff) : m;
+        // (m - dgt may pass 2^31 - 1 by less than 2^7: the last digits' carry into the first)
+        if (i > 0) m = (m >> 8) + (dgt < 0 ? 1 : 0);
+        const float f = (float)dgt * __int_as_float((127 - 7 - 8 * i) << 23);
+        out[i] = (uint16_t)(__float_as_uint(f) >> 16);
+    }
+}
 __device__ __forceinline__ void oz_digits(double x, int shift, uint16_t *out) {
     long long m = __double2ll_rn(ldexp(x, shift + 8 * OZ_S - 1));
 #pragma unroll
@@ -172,9 +215,10 @@ __global__ void __launch_bounds__(256) k_oz_images(const c64 *T, int p, int lmax
 }
 
 // digits of the multipole expansions, columns col0 .. col0 + W - 1 of every box of levels >= 2: a warp
-// per (domain, box, column) row; row (d nbox + box) W + c holds per K block eight digit rows of 32
+// per (domain, box, column) row; row (d nbox + box) W + c holds per K block its digit rows of 32
 // bytes, and ec its exponent
-__global__ void __launch_bounds__(256) k_oz_split(const c64 *C, const OzLevels L, int64_t nbox, int64_t ncols, int col0,
+template <typename R>
+__global__ void __launch_bounds__(256) k_oz_split(const cx<R> *C, const OzLevels L, int64_t nbox, int64_t ncols, int col0,
                                                   int W, int ndom, int p, int kblocks, const int *bal, unsigned char *out,
                                                   int *ec) {
     const int lane = threadIdx.x & 31, p2 = p * p;
@@ -187,14 +231,14 @@ __global__ void __launch_bounds__(256) k_oz_split(const c64 *C, const OzLevels L
     int l = 2;
     while (l < L.lmax && L.off[l + 1] <= b) ++l;
     const int *s = bal + (d * (L.lmax - 1) + l - 2) * p;
-    const c64 *x = C + (((int64_t)d * nbox + b) * ncols + col0 + c) * p2;
+    const cx<R> *x = C + (((int64_t)d * nbox + b) * ncols + col0 + c) * p2;
     constexpr int Q = 4;  // p^2 <= 100 coefficients over 32 lanes
-    c64 v[Q];
+    cx<R> v[Q];
     int sc[Q], e = -OZ_NONFINITE;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
         const int q = lane + 32 * k;
-        v[k] = q < p2 ? x[q] : c64{0.0, 0.0};
+        v[k] = q < p2 ? x[q] : cx<R>{R(0), R(0)};
         sc[k] = q < p2 ? s[oz_degree(q)] : 0;
         const int y = oz_exp2(v[k].re, v[k].im);
         e = max(e, abs(y) == OZ_NONFINITE ? y : y - sc[k]);
@@ -204,17 +248,18 @@ __global__ void __launch_bounds__(256) k_oz_split(const c64 *C, const OzLevels L
     if (e < -OZ_NONFINITE / 2 || bad) e = 0;
     const int64_t row = ((int64_t)d * nbox + b) * W + c;
     if (lane == 0) ec[row] = bad ? OZ_NONFINITE : e;
-    unsigned char *o = out + row * (int64_t)kblocks * OZ_ROW;
+    constexpr int S = Oz<R>::S;
+    unsigned char *o = out + row * (int64_t)kblocks * oz_row<R>;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
         const int q = lane + 32 * k;
         if (q >= kblocks * 8) break;
-        uint16_t a[OZ_S], b2[OZ_S];
-        oz_digits(bad ? 0.0 : v[k].re, -sc[k] - e, a);
-        oz_digits(bad ? 0.0 : v[k].im, -sc[k] - e, b2);
-        unsigned char *w = o + (q >> 3) * OZ_ROW + (q & 7) * 4;
+        uint16_t a[S], b2[S];
+        oz_digits(bad ? R(0) : v[k].re, -sc[k] - e, a);
+        oz_digits(bad ? R(0) : v[k].im, -sc[k] - e, b2);
+        unsigned char *w = o + (q >> 3) * oz_row<R> + (q & 7) * 4;
 #pragma unroll
-        for (int j = 0; j < OZ_S; ++j) *reinterpret_cast<uint32_t *>(w + j * 32) = a[j] | (uint32_t)b2[j] << 16;
+        for (int j = 0; j < S; ++j) *reinterpret_cast<uint32_t *>(w + j * 32) = a[j] | (uint32_t)b2[j] << 16;
     }
 }
 
@@ -223,7 +268,10 @@ struct OzP {
     int W, p2, kblocks;  // columns per pair of this window, K blocks of 16
     int lmax, ndom, mt, ngroup;
 };
-__host__ __device__ __forceinline__ int oz_tiles(int64_t pairs, int W) { return (int)((pairs * W + OZ_N - 1) / OZ_N); }
+template <typename R>
+__host__ __device__ __forceinline__ int oz_tiles(int64_t pairs, int W) {
+    return (int)((pairs * W + Oz<R>::N - 1) / Oz<R>::N);
+}
 
 // unit v of a launch (row tile fastest, so that concurrent CTAs share source digits, then the tiles of
 // a group, which share a matrix): domain, row tile, group (level, offset) and its columns
@@ -232,6 +280,7 @@ struct OzTile {
     int64_t pair0;       // first pair (pair_e position) of the group
     int col0;            // first column within the group
 };
+template <typename R>
 __device__ __forceinline__ OzTile oz_tile(const OzP &P, int v, int ntile, const int *first, const int32_t *group) {
     OzTile t;
     t.mt = v % P.mt;
@@ -246,8 +295,8 @@ __device__ __forceinline__ OzTile oz_tile(const OzP &P, int v, int ntile, const 
     }
     t.g = lo;
     t.pair0 = group[lo];
-    t.col0 = (v - first[lo]) * OZ_N;
-    t.n = (int)min((int64_t)OZ_N, (int64_t)(group[lo + 1] - t.pair0) * P.W - t.col0);
+    t.col0 = (v - first[lo]) * Oz<R>::N;
+    t.n = (int)min((int64_t)Oz<R>::N, (int64_t)(group[lo + 1] - t.pair0) * P.W - t.col0);
     return t;
 }
 
@@ -283,21 +332,31 @@ __device__ __forceinline__ double oz_compose(float s, float w, float r, int k) {
     return eh == 0 ? 0.0 : __longlong_as_double(mag | (long long)(b & 0x80000000) << 32);
 }
 
+// x 2^k as a float (NaN where k holds the mark OZ_NONFINITE)
+__device__ __forceinline__ float oz_scale(float x, int k) {
+    if (k > OZ_NONFINITE / 2) return __int_as_float(0x7fc00000);
+    const int h = min(max(k >> 1, -126), 126), g = min(max(k - h, -126), 126);
+    return x * __int_as_float((127 + h) << 23) * __int_as_float((127 + g) << 23);
+}
+
 // Persistent, one CTA per SM (20 warps, five to a scheduler).  Warps 0-2 fill the ring, each every third K
 // block of the CTA's sequence of tiles (the digit image by bulk copy, the gathered source digits by 16-byte
 // cp.async), the pairs of their next tile already on the way; warp 3 issues the MMAs; warps 4-19 empty the
 // accumulators (three floats per result in registers), free tensor memory for the next tile, and then
 // compose the doubles and store them beside that tile's MMAs (eight epilogue warps with twice the columns,
 // and twice the unrolled code, took longer over it than the MMAs).
+template <typename R>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_m2l_oz(const OzP P, const int32_t *__restrict__ group, const int2 *__restrict__ pairs,
              const unsigned char *__restrict__ Cdig, const int *__restrict__ ec, const unsigned char *__restrict__ img,
-             const int *__restrict__ er, double *Y, int *err, int *err_host) {
+             const int *__restrict__ er, R *Y, int *err, int *err_host) {
+    constexpr int S = Oz<R>::S, N = Oz<R>::N, ACC = Oz<R>::ACC;
+    constexpr uint32_t A_BYTES = oz_a_bytes<R>;
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t full[OZ_SLOTS], empty[OZ_SLOTS], done, tfree, fin;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    __shared__ int rowid[OZ_FILL][OZ_N];  // per producer warp: digit row of each pair column (-1: none)
+    __shared__ int rowid[OZ_FILL][N];  // per producer warp: digit row of each pair column (-1: none)
     __shared__ int s_part[OZ_THREADS / 32];
     __shared__ int first[(OZ_MAX_LEVELS - 2) * 316 + 1];  // tiles before each group
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -325,7 +384,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const int per = (P.ngroup + OZ_THREADS - 1) / OZ_THREADS, g0 = min(threadIdx.x * per, P.ngroup);
         const int g1 = min(g0 + per, P.ngroup);
         int sum = 0;
-        for (int g = g0; g < g1; ++g) sum += oz_tiles(group[g + 1] - group[g], P.W);
+        for (int g = g0; g < g1; ++g) sum += oz_tiles<R>(group[g + 1] - group[g], P.W);
         int inc = sum;
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, inc, o);
@@ -337,7 +396,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         for (int w = 0; w < warp; ++w) at += s_part[w];
         for (int g = g0; g < g1; ++g) {
             first[g] = at;
-            at += oz_tiles(group[g + 1] - group[g], P.W);
+            at += oz_tiles<R>(group[g + 1] - group[g], P.W);
         }
         if (g0 < g1 && g1 == P.ngroup) first[P.ngroup] = at;
     }
@@ -349,18 +408,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
     if (warp < OZ_FILL) {
         // ------------------------------------------------------------------ producers
-        // source boxes of a tile's columns lane, lane + 32, lane + 64
+        // source boxes of a tile's columns lane, lane + 32, ..
+        constexpr int NSRC = (N + 31) / 32;
         auto sources = [&](const OzTile &t, int *src) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
+            for (int k = 0; k < NSRC; ++k) {
                 const int m = lane + 32 * k;
                 src[k] = m < t.n ? pairs[t.pair0 + (t.col0 + m) / P.W].x : -1;
             }
         };
-        int src[3];
+        int src[NSRC];
         OzTile t;
         if ((int)blockIdx.x < nunit) {
-            t = oz_tile(P, blockIdx.x, ntile, first, group);
+            t = oz_tile<R>(P, blockIdx.x, ntile, first, group);
             sources(t, src);
         }
         int u = 0, turn = 0, last = -1;  // K blocks of the CTA's sequence, u mod OZ_FILL, this warp's last
@@ -368,15 +428,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         for (int v = blockIdx.x; v < nunit && !stop; v += gridDim.x) {
             __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
+            for (int k = 0; k < NSRC; ++k) {
                 const int m = lane + 32 * k, c = (t.col0 + m) % P.W;
-                if (m < OZ_N)
+                if (m < N)
                     rowid[warp][m] = src[k] >= 0 ? (int)(((int64_t)t.d * P.nbox + src[k]) * P.W + c) : -1;
             }
             __syncwarp();
             const OzTile cur = t;
             if (v + (int)gridDim.x < nunit) {
-                t = oz_tile(P, v + gridDim.x, ntile, first, group);
+                t = oz_tile<R>(P, v + gridDim.x, ntile, first, group);
                 sources(t, src);
             }
             const int n_pad = (cur.n + 15) & ~15;
@@ -385,7 +445,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             for (int kb = 0; kb < P.kblocks; ++kb, ++u, turn = turn == OZ_FILL - 1 ? 0 : turn + 1) {
                 if (turn != warp) continue;
                 const int slot = u & 3;
-                const uint32_t sA = sbase + (uint32_t)slot * OZ_SLOT_BYTES, sB = sA + OZ_A_BYTES;
+                const uint32_t sA = sbase + (uint32_t)slot * oz_slot_bytes<R>, sB = sA + A_BYTES;
                 bool ok = u < OZ_SLOTS || mbar_wait(&empty[slot], (uint32_t)((u >> 2) - 1) & 1u);
                 ok = __all_sync(0xffffffffu, ok && !s_abort);
                 if (!ok) {
@@ -394,20 +454,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     break;
                 }
                 if (lane == 0) {
-                    mbar_arrive_expect_tx(&full[slot], OZ_A_BYTES);
-                    bulk_load(sA, A + (int64_t)kb * OZ_A_BYTES, OZ_A_BYTES, &full[slot]);
+                    mbar_arrive_expect_tx(&full[slot], A_BYTES);
+                    bulk_load(sA, A + (int64_t)kb * OZ_A_BYTES, A_BYTES, &full[slot]);
                 }
-                // a column's 256 bytes of digits: 16 lanes each, eight columns a lane in one go
-                const int part = lane & 15, dg = part >> 1, ch = part & 1;
-                const unsigned char *src0 = Cdig + (int64_t)kb * OZ_ROW + part * 16;
-                const uint32_t dst0 = sB + (uint32_t)dg * (OZ_N * 32u), stride = (uint32_t)P.kblocks * OZ_ROW;
-                for (int m0 = lane >> 4; m0 < n_pad; m0 += 16) {
-                    int row[8];
+                // a column's 32 S bytes of digits: 2 S lanes each, S columns a lane in one go
+                constexpr int CPW = 16 / S;  // columns of the warp at once
+                const int part = lane & (2 * S - 1), dg = part >> 1, ch = part & 1;
+                const unsigned char *src0 = Cdig + (int64_t)kb * oz_row<R> + part * 16;
+                const uint32_t dst0 = sB + (uint32_t)dg * (N * 32u), stride = (uint32_t)P.kblocks * oz_row<R>;
+                for (int m0 = lane / (2 * S); m0 < n_pad; m0 += 16) {
+                    int row[S];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) row[k] = rowid[warp][m0 + 2 * k];
+                    for (int k = 0; k < S; ++k) row[k] = rowid[warp][m0 + CPW * k];
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + sw32_chunk(m0 + 2 * k, ch)),
+                    for (int k = 0; k < S; ++k)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst0 + sw32_chunk(m0 + CPW * k, ch)),
                                      "l"(src0 + (uint64_t)(uint32_t)max(row[k], 0) * stride), "r"(row[k] >= 0 ? 16 : 0)
                                      : "memory");
                 }
@@ -429,7 +490,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         bool ok = true;
         int u = 0, nt = 0;
         for (int v = blockIdx.x; v < nunit && ok && !s_abort; v += gridDim.x) {
-            const OzTile t = oz_tile(P, v, ntile, first, group);
+            const OzTile t = oz_tile<R>(P, v, ntile, first, group);
             const uint32_t idesc = idesc_bf16((t.n + 15) & ~15);
             if (nt > 0) ok = __all_sync(0xffffffffu, mbar_wait(&tfree, (uint32_t)(nt - 1) & 1u));
             if (!ok) break;
@@ -439,21 +500,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)(u >> 2) & 1u));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t sA = sbase + (uint32_t)s * OZ_SLOT_BYTES;
-                const uint64_t da = smem_desc_sw32(sA), db = smem_desc_sw32(sA + OZ_A_BYTES);
+                const uint32_t sA = sbase + (uint32_t)s * oz_slot_bytes<R>;
+                const uint64_t da = smem_desc_sw32(sA), db = smem_desc_sw32(sA + A_BYTES);
                 // a digit of the matrix against every digit it meets, held in the collector after the
                 // first; the smallest products first, so that the shared accumulator loses least
 #pragma unroll
-                for (int i = 0; i < OZ_S; ++i)
+                for (int i = 0; i < S; ++i)
 #pragma unroll
-                    for (int j = OZ_S - 1 - i; j >= 0; --j) {
+                    for (int j = S - 1 - i; j >= 0; --j) {
                         const int dd = i + j;
-                        const uint32_t acc = tmem + (uint32_t)((dd < OZ_ACC ? dd : OZ_ACC - 1) * OZ_N);
-                        const bool head = i == 0 && (dd < OZ_ACC - 1 || dd == OZ_S - 1);
-                        const uint64_t a = da + (uint64_t)((i * (TC_M * 32)) >> 4), b = db + (uint64_t)((j * (OZ_N * 32)) >> 4);
+                        const uint32_t acc = tmem + (uint32_t)((dd < ACC ? dd : ACC - 1) * N);
+                        const bool head = i == 0 && (dd < ACC - 1 || dd == S - 1);
+                        const uint64_t a = da + (uint64_t)((i * (TC_M * 32)) >> 4), b = db + (uint64_t)((j * (N * 32)) >> 4);
                         const uint32_t add = head && kb == 0 ? 0u : 1u;
-                        if (i == OZ_S - 1) mma_bf16_if<0>(leader, acc, a, b, idesc, add);
-                        else if (j == OZ_S - 1 - i) mma_bf16_if<1>(leader, acc, a, b, idesc, add);
+                        if (i == S - 1) mma_bf16_if<0>(leader, acc, a, b, idesc, add);
+                        else if (j == S - 1 - i) mma_bf16_if<1>(leader, acc, a, b, idesc, add);
                         else if (j > 0) mma_bf16_if<2>(leader, acc, a, b, idesc, add);
                         else mma_bf16_if<3>(leader, acc, a, b, idesc, add);
                     }
@@ -474,15 +535,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // ------------------------------------------------------------------ epilogue warps 4..19
         // warp: accumulator lanes 32 (warp mod 4) .., columns 16 b + 4 sub + j (b < NG, j < 4)
         const int quarter = warp & 3, sub = (warp - 4) >> 2;
-        constexpr int NG = OZ_N / 16;
+        constexpr int NG = N / 16;
+        static_assert(4 * NG <= 32, "a lane per column of the warp");
         int nt = 0;
         for (int v = blockIdx.x; v < nunit; v += gridDim.x) {
-            const OzTile t = oz_tile(P, v, ntile, first, group);
+            const OzTile t = oz_tile<R>(P, v, ntile, first, group);
             const int64_t mat = (int64_t)t.d * (P.lmax - 1) * 316 + t.g;
-            const int R = t.mt * TC_M + quarter * 32 + lane;
-            const bool rows = t.mt * TC_M + quarter * 32 < 2 * P.p2, row_ok = R < 2 * P.p2;
-            const int eR = row_ok ? er[mat * P.p2 + (R >> 1)] : 0;
-            // lane i knows column i of this warp's 20: its row of Y and its exponent
+            const int rr = t.mt * TC_M + quarter * 32 + lane;
+            const bool rows = t.mt * TC_M + quarter * 32 < 2 * P.p2, row_ok = rr < 2 * P.p2;
+            const int eR = row_ok ? er[mat * P.p2 + (rr >> 1)] : 0;
+            // lane i knows column i of this warp's 4 NG: its row of Y and its exponent
             const int m = 16 * (lane >> 2) + 4 * sub + (lane & 3);
             int yr = -1, ex = 0;
             if (m < t.n && lane < 4 * NG) {
@@ -500,14 +562,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             ++nt;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int ng = rows ? (t.n - 4 * sub + 15) / 16 : 0;  // this warp's column groups in use
-            float hi[4 * NG], mi[4 * NG], lo[4 * NG];
+            constexpr bool DBL = sizeof(R) == 8;
+            float hi[4 * NG], mi[DBL ? 4 * NG : 1], lo[DBL ? 4 * NG : 1];
 #pragma unroll
             for (int b = 0; b < NG; ++b) {
                 if (b < ng) {
-                    uint32_t a[OZ_ACC][4];
+                    uint32_t a[ACC][4];
 #pragma unroll
-                    for (int k = 0; k < OZ_ACC; ++k) {
-                        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(k * OZ_N + 16 * b + 4 * sub);
+                    for (int k = 0; k < ACC; ++k) {
+                        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(k * N + 16 * b + 4 * sub);
                         asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                                      : "=r"(a[k][0]), "=r"(a[k][1]), "=r"(a[k][2]), "=r"(a[k][3])
                                      : "r"(ta));
@@ -515,23 +578,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float d0 = __uint_as_float(a[0][j]), d1 = __uint_as_float(a[1][j]);
-                        const float d3 = __uint_as_float(a[3][j]);
-                        const float s = d0 + d1, sb = s - d0;                         // s + e = d0 + d1
-                        const float e = (d0 - (s - sb)) + (d1 - sb);
-                        const float l = e + __uint_as_float(a[2][j]);                 // exact: within 24 bits
-                        const float m = l + d3, mb = m - l;                           // m + .. = l + d3
-                        const float x = ((l - (m - mb)) + (d3 - mb)) + __uint_as_float(a[4][j]);  // exact
-                        const float w = m + x, wb = w - m;                            // w + .. = m + x
-                        hi[4 * b + j] = s;
-                        mi[4 * b + j] = w;
-                        lo[4 * b + j] = ((m - (w - wb)) + (x - wb)) + __uint_as_float(a[5][j]);
+                        if constexpr (!DBL) {  // the smallest first
+                            hi[4 * b + j] = __uint_as_float(a[0][j]) + (__uint_as_float(a[1][j]) +
+                                            (__uint_as_float(a[2][j]) + __uint_as_float(a[3][j])));
+                        } else {
+                            const float d0 = __uint_as_float(a[0][j]), d1 = __uint_as_float(a[1][j]);
+                            const float d3 = __uint_as_float(a[3][j]);
+                            const float s = d0 + d1, sb = s - d0;                         // s + e = d0 + d1
+                            const float e = (d0 - (s - sb)) + (d1 - sb);
+                            const float l = e + __uint_as_float(a[2][j]);                 // exact: within 24 bits
+                            const float m = l + d3, mb = m - l;                           // m + .. = l + d3
+                            const float x = ((l - (m - mb)) + (d3 - mb)) + __uint_as_float(a[4][j]);  // exact
+                            const float w = m + x, wb = w - m;                            // w + .. = m + x
+                            hi[4 * b + j] = s;
+                            mi[4 * b + j] = w;
+                            lo[4 * b + j] = ((m - (w - wb)) + (x - wb)) + __uint_as_float(a[5][j]);
+                        }
                     }
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tfree)) : "memory");
-            double *Yd = Y + (int64_t)t.d * P.y_dom + R;
+            R *Yd = Y + (int64_t)t.d * P.y_dom + rr;
 #pragma unroll
             for (int b = 0; b < NG; ++b) {
                 if (b < ng) {
@@ -540,7 +608,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         const int i = 4 * b + j;
                         const int o = __shfl_sync(0xffffffffu, yr, i);
                         const int k = __shfl_sync(0xffffffffu, ex, i) + eR;
-                        const double x = oz_compose(hi[i], mi[i], lo[i], k);
+                        R x;
+                        if constexpr (DBL) x = oz_compose(hi[i], mi[i], lo[i], k);
+                        else x = oz_scale(hi[i], k);
                         if (row_ok && o >= 0) Yd[(int64_t)o * (2 * P.p2)] = x;
                     }
                 }
@@ -599,16 +669,20 @@ void build_oz_tables(fmbem *h, cudaStream_t s) {
     CKL("k_oz_images");
 }
 
-// doubles of Y per domain for a window of W columns, and bytes of the window's digits and exponents
+// real numbers of Y per domain for a window of W columns, and bytes of the window's digits and exponents
 int64_t oz_y_dom(const fmbem *h, int W) { return h->n_ff * W * 2 * h->p2; }
+template <typename R>
 size_t oz_digit_bytes(const fmbem *h, int W) {
     const size_t rows = (size_t)(h->Jf + 1) * h->nbox * W;
-    return rows * oz_kblocks(h->p2) * OZ_ROW + rows * sizeof(int);
+    return rows * oz_kblocks(h->p2) * oz_row<R> + rows * sizeof(int);
 }
+template size_t oz_digit_bytes<double>(const fmbem *, int);
+template size_t oz_digit_bytes<float>(const fmbem *, int);
 
 // the S|R products of every level and domain for columns col0 .. col0 + W - 1 of C (3 n_rhs columns)
 // into Y[d][CSR position][W][p^2] (domains oz_y_dom apart)
-void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s) {
+template <typename R>
+void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W, cudaStream_t s) {
     if (h->n_ff <= 0) return;
     const int p2 = h->p2, kb = oz_kblocks(p2), ndom = h->Jf + 1;
     OzLevels L{};
@@ -617,8 +691,8 @@ void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cud
     L.off[h->lmax + 1] = h->nbox;
     const int64_t rows = (int64_t)ndom * (h->nbox - L.off[2]) * W;
     unsigned char *dig = (unsigned char *)h->oz_dig;
-    int *ec = (int *)(dig + (size_t)ndom * h->nbox * W * kb * OZ_ROW);
-    k_oz_split<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(C, L, h->nbox, 3 * nr, col0, W, ndom, h->p, kb, h->oz_bal, dig, ec);
+    int *ec = (int *)(dig + (size_t)ndom * h->nbox * W * kb * oz_row<R>);
+    k_oz_split<R><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(C, L, h->nbox, 3 * nr, col0, W, ndom, h->p, kb, h->oz_bal, dig, ec);
     CKL("k_oz_split");
     OzP P{};
     P.nbox = h->nbox;
@@ -631,25 +705,27 @@ void run_m2l_oz(fmbem *h, const c64 *C, c64 *Y, int64_t nr, int col0, int W, cud
     P.ngroup = (h->lmax - 1) * 316;
     P.y_dom = oz_y_dom(h, W);
     int64_t tiles = 0;
-    for (int g = 0; g < P.ngroup; ++g) tiles += oz_tiles(h->h_group_beg[g + 1] - h->h_group_beg[g], W);
-    const size_t smem = OZ_SLOTS * (size_t)OZ_SLOT_BYTES + 1024;
-    CK(cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    for (int g = 0; g < P.ngroup; ++g) tiles += oz_tiles<R>(h->h_group_beg[g + 1] - h->h_group_beg[g], W);
+    const size_t smem = OZ_SLOTS * (size_t)oz_slot_bytes<R> + 1024;
+    CK(cudaFuncSetAttribute(k_m2l_oz<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int dev = 0, nsm = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     // an odd grid: a CTA then alternates between the row tiles, of which the second is the shorter
     const int64_t grid = std::min<int64_t>(tiles * ndom * P.mt, (nsm - 1) | 1);
     if (grid <= 0) return;
-    k_m2l_oz<<<(unsigned)grid, OZ_THREADS, smem, s>>>(P, h->oz_group, (const int2 *)h->oz_pairs, dig, ec,
-                                                      (const unsigned char *)h->oz_img, h->oz_er, (double *)Y, h->tc_err,
-                                                      h->oz_err_host);
+    k_m2l_oz<R><<<(unsigned)grid, OZ_THREADS, smem, s>>>(P, h->oz_group, (const int2 *)h->oz_pairs, dig, ec,
+                                                         (const unsigned char *)h->oz_img, h->oz_er, (R *)Y, h->tc_err,
+                                                         h->oz_err_host);
     CKL("k_m2l_oz");
 }
+template void run_m2l_oz<double>(fmbem *, const c64 *, c64 *, int64_t, int, int, cudaStream_t);
+template void run_m2l_oz<float>(fmbem *, const c32 *, c32 *, int64_t, int, int, cudaStream_t);
 
-// a wait of the FP64 tensor-core M2L that ran out on an earlier product of this handle
+// a wait of this M2L that ran out on an earlier product of this handle
 void check_oz_err(fmbem *h, cudaStream_t s) {
     if (h->oz_err_host == nullptr || *(volatile int *)h->oz_err_host == 0) return;
     *(volatile int *)h->oz_err_host = 0;
     CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
-    throw fmbem_error{FMBEM_ERR_DEVICE_TIMEOUT, "tensor-core M2L (FP64): an mbarrier wait timed out"};
+    throw fmbem_error{FMBEM_ERR_DEVICE_TIMEOUT, "tensor-core M2L (8-bit digits): an mbarrier wait timed out"};
 }
