@@ -75,70 +75,39 @@ __global__ void k_prep(int64_t N, int64_t nr, const c64 *x, const int32_t *perm,
     prep_body<R>(N, nr, x, perm, nrm, w, dom, dc, dens, blockIdx.x, blockIdx.y, sj, am);
 }
 
-// The single-precision densities straight into the node-major layout below (k_dens_node_major's
-// densS), for 32 k right-hand sides whose every consumer reads that layout (k_near_r, and P2M on
-// the tensor cores, which forms the scatterer side from v_1 = v_0 + s n, q_1 = -gamma_j q_0):
-// block = 8 nodes x 32 right-hand sides, lane = right-hand side, so that each warp stores one
-// node's 2 KB row whole; arithmetic as in prep_body<float>
-__global__ void __launch_bounds__(256) k_prep_node_major(int64_t N, int64_t nr, const c64 *x, const int32_t *perm,
+// The single-precision densities of four or more right-hand sides, node-major within blocks of 32 (the last
+// block as wide as what is left), for k_near_r and P2M on the tensor cores: densS[block][node][right-hand
+// side][4 float4] = (a, m_x), (m_y, m_z), (q_x, q_y), (q_z, s) of the background side, with a = n . v_0,
+// m = v_0 x n (the only forms in which those read v_0) and s = n . (v_1 - v_0) the scatterer side's jump
+// along the normal (v_1 = v_0 + s n, q_1 = -gamma_j q_0; see k_near_ws).  Thread per (node, right-hand
+// side), a block's right-hand sides next to each other, so that each warp stores whole rows; arithmetic as
+// in prep_body<float>.  Right-hand sides r0 .. r0 + n - 1, grid (.., blocks).
+__global__ void __launch_bounds__(256) k_prep_node_major(int64_t N, int64_t r0, int64_t n, const c64 *x, const int32_t *perm,
                                                          const double *nrm, const double *w, const int32_t *dom,
                                                          const DomainConsts *dc, float4 *densS) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), rb = blockIdx.y;
+    const int64_t rb = blockIdx.y, t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int width = (int)min((int64_t)32, n - 32 * rb);
+    const int64_t i = t / width;
     if (i >= N) return;
-    const int64_t r = rb * 32 + lane;
-    const c64 *xi = x + (r * N + perm[i]) * 6;
-    const float n[3] = {(float)nrm[3 * i], (float)nrm[3 * i + 1], (float)nrm[3 * i + 2]};
+    const int rl = (int)(t - i * width);
+    const c64 *xi = x + ((r0 + 32 * rb + rl) * N + perm[i]) * 6;
+    const float nn[3] = {(float)nrm[3 * i], (float)nrm[3 * i + 1], (float)nrm[3 * i + 2]};
     const float wi = (float)w[i];
     const cx<float> Phi[3] = {to<float>(xi[0]), to<float>(xi[1]), to<float>(xi[2])};
     const cx<float> Psi[3] = {to<float>(xi[3]), to<float>(xi[4]), to<float>(xi[5])};
-    const cx<float> nP = n[0] * Phi[0] + n[1] * Phi[1] + n[2] * Phi[2];
-    const cx<float> tn = to<float>(dc[dom[i]].t) * nP;
+    const cx<float> tn = to<float>(dc[dom[i]].t) * (nn[0] * Phi[0] + nn[1] * Phi[1] + nn[2] * Phi[2]);
     cx<float> v[3], q[3];
     for (int c = 0; c < 3; ++c) {
         v[c] = wi * Phi[c];
         q[c] = (-wi) * Psi[c];
     }
-    const cx<float> sj = wi * tn;  // n . (v_1 - v_0)
-    float4 *o = densS + ((rb * N + i) * 32 + lane) * 4;
-    o[0] = make_float4(v[0].re, v[0].im, v[1].re, v[1].im);
-    o[1] = make_float4(v[2].re, v[2].im, q[0].re, q[0].im);
-    o[2] = make_float4(q[1].re, q[1].im, q[2].re, q[2].im);
-    o[3] = make_float4(sj.re, sj.im, 0.f, 0.f);
-}
-
-// The single-precision densities node-major within blocks of 32 right-hand sides, for the
-// lane-per-RHS near field (a source's 32 right-hand sides are contiguous):
-// densS[block][node][32][4 float4] = (v0x, v0y), (v0z, q0x), (q0y, q0z), (s, 0) of the background
-// side, with s = n . (v_1 - v_0) the scatterer side's jump along the normal (v_1 = v_0 + s n, see
-// k_near_ws); grid (node tiles of 16, block), 32 x 16 entries through shared memory, written in
-// whole rows.
-__global__ void __launch_bounds__(256) k_dens_node_major(int64_t N, int64_t nr, const float4 *dens, const float4 *rec,
-                                                         float4 *densS) {
-    __shared__ float4 t[32][16 * 4 + 1];
-    const int64_t i0 = (int64_t)blockIdx.x * 16, rb = blockIdx.y;
-    const int ni = (int)min((int64_t)16, N - i0);
-    for (int e = threadIdx.x; e < 32 * 16; e += blockDim.x) {  // (right-hand side rl, node il)
-        const int rl = e / 16, il = e - rl * 16;
-        if (il < ni) {
-            const int64_t i = i0 + il;
-            const float4 *a = dens + ((rb * 32 + rl) * N + i) * 3;         // background side
-            const float4 *b = dens + ((nr + rb * 32 + rl) * N + i) * 3;    // scatterer side
-            const float4 a0 = a[0], a1 = a[1], b0 = b[0], b1 = b[1];
-            const float4 n1 = rec[3 * i + 1], n2 = rec[3 * i + 2];        // n = (n1.w, n2.x, n2.y)
-            const float sre = n1.w * (b0.x - a0.x) + n2.x * (b0.z - a0.z) + n2.y * (b1.x - a1.x);
-            const float sim = n1.w * (b0.y - a0.y) + n2.x * (b0.w - a0.w) + n2.y * (b1.y - a1.y);
-            t[rl][il * 4] = a0;
-            t[rl][il * 4 + 1] = a1;
-            t[rl][il * 4 + 2] = a[2];
-            t[rl][il * 4 + 3] = make_float4(sre, sim, 0.f, 0.f);
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 16 * 128; e += blockDim.x) {  // node il: 32 right-hand sides x 4 float4
-        const int il = e / 128, k = e - il * 128, rl = k / 4, c = k - rl * 4;
-        if (il < ni) densS[(rb * N + i0 + il) * 128 + k] = t[rl][il * 4 + c];
-    }
+    const cx<float> a = nn[0] * v[0] + nn[1] * v[1] + nn[2] * v[2], sj = wi * tn;
+    const cx<float> m[3] = {nn[2] * v[1] - nn[1] * v[2], nn[0] * v[2] - nn[2] * v[0], nn[1] * v[0] - nn[0] * v[1]};
+    float4 *o = densS + (rb * N * 32 + i * width + rl) * 4;
+    o[0] = make_float4(a.re, a.im, m[0].re, m[0].im);
+    o[1] = make_float4(m[1].re, m[1].im, m[2].re, m[2].im);
+    o[2] = make_float4(q[0].re, q[0].im, q[1].re, q[1].im);
+    o[3] = make_float4(q[2].re, q[2].im, sj.re, sj.im);
 }
 
 // ---------------------------------------------------------------- P2M (Eqs. 2.18-2.19)
@@ -1631,31 +1600,6 @@ __global__ void __launch_bounds__(128) k_near_rb(const int32_t *leaf_box, int64_
 }
 
 // ---------------------------------------------------------------- warp-independent near field
-// Steps 4-5 for many right-hand sides in single precision.  One warp owns one work item: a group
-// of tg target nodes of one leaf, split over nsl source slices (tg * nsl <= 32 lanes, nsl a power
-// of two; lane = target + tg * slice), for one side (domain 0, or the target's own scatterer) and
-// one block of RB right-hand sides.  The items are built once per tree (near_work_items) so that
-// leaves of every size keep most lanes busy.
-// - Near field: the warp streams the sources of the leaf's Neighbor list through two warp-private
-//   shared-memory tiles of NW_TS sources; while it computes on one, asynchronous copies (cp.async,
-//   16 bytes each: the 48-byte source record and the RB x 48 bytes of densities) fill the other,
-//   and the warp synchronises only itself.  Per (source, target) pair it evaluates the kernel
-//   scalars once and applies them to the RB right-hand sides.
-// - Far field (L2P, Eq. 2.23 first term): the leaf's local expansions of the block's 3 RB columns
-//   are staged in the same shared memory (in chunks of coefficients), and each slice adds the
-//   coefficients q = slice (mod nsl) of B_l2p[a][q] D[col][q] to its partial sums.
-// - The slices are summed by a fixed shuffle tree; the slice-0 lane of each target adds the side's
-//   rows of the analytic self block (App. B) applied to x in double precision and stores the
-//   side's three result rows.
-constexpr int NW_TS = 16;    // sources per tile
-static_assert(NW_TS == 16, "k_near_w stages a tile with two half-warps of 16 lanes");
-constexpr int NW_WARPS = 4;  // warps per block, one per SM sub-partition; each fetches its own units
-template <int RB>
-struct WarpTile {
-    float4 geo[3][NW_TS];     // source record: position hi + scatterer id bits, position lo + n_x, n_y n_z
-    float4 dv[RB][3][NW_TS];  // densities (v0, v1), (v2, q0), (q1, q2) of the side, per RHS
-};
-
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
@@ -1663,213 +1607,6 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-template <int RB>
-__global__ void __launch_bounds__(32 * NW_WARPS, 4) k_near_w(
-    const int32_t *leaf_box, const int4 *__restrict__ items, int n_items, int n_units, int *next_unit, int64_t N, int64_t nr,
-    int64_t rhs_base, int nsides,
-    const int32_t *nbeg, const int32_t *nend, const int32_t *nbr_start, const int32_t *nbr_idx,
-    const float4 *__restrict__ rec, const cx<float> *dens, const DomainConsts *dc, const int32_t *perm, int p2,
-    int64_t nbox, const cx<float> *__restrict__ Bl2p, const cx<float> *__restrict__ D,
-    const c64 *__restrict__ Mself, const c64 *__restrict__ x, c64 *y) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int rng_beg[NW_WARPS][32], rng_cum[NW_WARPS][33];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpTile<RB> *T = reinterpret_cast<WarpTile<RB> *>(smem_raw) + 2 * warp;  // two buffers per warp
-    int *rb_ = rng_beg[warp], *rc_ = rng_cum[warp];
-    // persistent warps: each takes the next unit (slab of side and RHS block, item) until none is
-    // left; units run slab by slab, so that a slab's densities stay in L2, and within a slab
-    // longest item first
-    for (;;) {
-        int unit = 0;
-        if (lane == 0) unit = atomicAdd(next_unit, 1);
-        unit = __shfl_sync(0xffffffffu, unit, 0);
-        if (unit >= n_units) break;
-        const int yslab = unit / n_items, item_id = unit - yslab * n_items;
-        __syncwarp();  // the previous unit's shared-memory reads are done
-        const int4 it = items[item_id];
-        const int leaf = it.x, tg = it.z, nsl = it.w;
-        const int64_t g = leaf_box[leaf];
-        // the Neighbor leaves' node ranges and their running sum (a Neighbor list has at most 27 entries)
-        const int nb0 = nbr_start[leaf], nnb = nbr_start[leaf + 1] - nb0;
-        {
-            int beg = 0, cnt = 0;
-            if (lane < nnb) {
-                const int b = nbr_idx[nb0 + lane];
-                beg = nbeg[b];
-                cnt = nend[b] - beg;
-            }
-            int incl = cnt;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            if (lane < nnb) { rb_[lane] = beg; rc_[lane] = incl - cnt; }
-            if (lane == nnb - 1) rc_[nnb] = incl;
-        }
-        // slabs (RHS block, side); with the impedance boundary only the background side (k_local_rows
-        // writes the scatterer rows)
-        const int side = yslab % nsides;
-        const int64_t rb0 = rhs_base + (int64_t)(yslab / nsides) * RB;
-        const int nrb = (int)min((int64_t)RB, nr - rb0);
-        // densities of the RHS past the block's end stay zero in both tiles
-        for (int e = nrb * 3 * NW_TS + lane; e < RB * 3 * NW_TS; e += 32) {
-            (&T[0].dv[0][0][0])[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            (&T[1].dv[0][0][0])[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncwarp();
-        const int nsrc = rc_[nnb];
-        const int ti = lane % tg, sl = lane / tg;
-        const bool busy = sl < nsl;
-        const int a = nbeg[g] + it.y + ti;  // lanes past tg * nsl shadow a valid target and never store
-        const float sgn = side == 0 ? -1.f : 1.f;  // domain 0 sees the scatterer normal reversed
-        const float4 ra = rec[3 * a], rla = rec[3 * a + 1];
-        const int adom = __float_as_int(ra.w);
-        const cx<float> k = to<float>(dc[side == 0 ? 0 : adom].k);
-        const cx<float> *dside = dens + (side * nr + rb0) * N * 6;
-        // stage the tile of sources s0 .. s0 + NW_TS - 1 into buffer B: lane j (and j + 16) stages
-        // source j, the lower half the record and the first RB/2 right-hand sides' densities, the upper
-        // half the other RB/2; a lane's sources advance monotonically, so it follows its Neighbor range
-        const int j = lane & (NW_TS - 1), hh = lane >> 4;
-        const int64_t rstride = N * 6;
-        int qcur = 0;
-        auto stage = [&](WarpTile<RB> &B, int s0) {
-            const int e = s0 + j;
-            if (e < nsrc) {
-                while (rc_[qcur + 1] <= e) ++qcur;
-                const int64_t i = rb_[qcur] + (e - rc_[qcur]);
-                if (hh == 0) {
-#pragma unroll
-                    for (int part = 0; part < 3; ++part) cp_async16(&B.geo[part][j], rec + 3 * i + part);
-                }
-                const cx<float> *src = dside + hh * (RB / 2) * rstride + 6 * i;
-#pragma unroll
-                for (int k = 0; k < RB / 2; ++k) {
-                    if (hh * (RB / 2) + k < nrb) {
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) cp_async16(&B.dv[hh * (RB / 2) + k][c][j], src + k * rstride + 2 * c);
-                    }
-                }
-            }
-            cp_async_commit();
-        };
-        cx<float> acc[RB][3];
-#pragma unroll
-        for (int rr = 0; rr < RB; ++rr)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[rr][c] = {0, 0};
-        const int ntile = (nsrc + NW_TS - 1) / NW_TS;
-        stage(T[0], 0);
-        for (int t = 0; t < ntile; ++t) {
-            if (t + 1 < ntile) stage(T[(t + 1) & 1], (t + 1) * NW_TS);
-            else cp_async_commit();  // an empty group keeps "all but the newest group done" meaning tile t
-            cp_async_wait1();
-            __syncwarp();
-            const WarpTile<RB> &B = T[t & 1];
-            const int ns = busy ? min(NW_TS, nsrc - t * NW_TS) : 0;
-            for (int u = sl; u < ns; u += nsl) {
-                const float4 pa = B.geo[0][u], pb = B.geo[1][u], pc = B.geo[2][u];
-                if (side == 1 && __float_as_int(pa.w) != adom) continue;  // a scatterer's sum runs over its own nodes
-                const float rv3[3] = {(pa.x - ra.x) + (pb.x - rla.x), (pa.y - ra.y) + (pb.y - rla.y),
-                                      (pa.z - ra.z) + (pb.z - rla.z)};
-                const float R2 = rv3[0] * rv3[0] + rv3[1] * rv3[1] + rv3[2] * rv3[2];
-                const float inv = R2 > 0.f ? rsqrt_(R2) : 0.f;  // the node itself drops out
-                const float Rr = R2 * inv;
-                const float nn[3] = {sgn * pb.w, sgn * pc.x, sgn * pc.y};
-                const float nrv = nn[0] * rv3[0] + nn[1] * rv3[1] + nn[2] * rv3[2];
-                const float w[3] = {nn[1] * rv3[2] - nn[2] * rv3[1], nn[2] * rv3[0] - nn[0] * rv3[2],
-                                    nn[0] * rv3[1] - nn[1] * rv3[0]};
-                cx<float> gs, cs;
-                pair_scalars<float>(inv, Rr, k, gs, cs);
-#pragma unroll
-                for (int rr = 0; rr < RB; ++rr) {
-                    const float4 a0 = B.dv[rr][0][u], a1 = B.dv[rr][1][u], a2 = B.dv[rr][2][u];
-                    const cx<float> v[3] = {{a0.x, a0.y}, {a0.z, a0.w}, {a1.x, a1.y}};
-                    const cx<float> qv[3] = {{a1.z, a1.w}, {a2.x, a2.y}, {a2.z, a2.w}};
-                    cross_apply<float>(w, nrv, gs, cs, v, qv, acc[rr]);
-                }
-            }
-            __syncwarp();  // the next stage overwrites this buffer
-        }
-        // far field: the local expansions of this side's domain at the leaf, for the block's columns
-        // 3 rb0 .. 3 (rb0 + nrb) - 1, staged through the tiles' shared memory in chunks of qc
-        // coefficients; on the scatterer side the warp's targets may lie in several scatterers, which
-        // are taken in turn
-        {
-            cx<float> *Ds = reinterpret_cast<cx<float> *>(T);
-            const int qc = min(p2, (int)(2 * sizeof(WarpTile<RB>) / sizeof(cx<float>)) / (3 * RB));
-            const int ncol = 3 * nrb;
-            const int64_t ncols = 3 * nr;
-            const int mydom = side == 0 ? 0 : adom;
-            const cx<float> *Ba = Bl2p + ((int64_t)side * N + a) * p2;
-            unsigned pending = 0xffffffffu;
-            while (pending) {
-                const int d = __shfl_sync(0xffffffffu, mydom, __ffs(pending) - 1);
-                const bool mine = mydom == d;
-                pending &= ~__ballot_sync(0xffffffffu, mine);
-                const cx<float> *Dg = D + ((int64_t)d * nbox + g) * ncols * p2 + 3 * rb0 * p2;
-                for (int q0 = 0; q0 < p2; q0 += qc) {
-                    const int qn = min(qc, p2 - q0);
-                    __syncwarp();
-                    for (int e = lane; e < ncol * qn; e += 32) {
-                        const int col = e / qn, qq = e - col * qn;
-                        Ds[col * qc + qq] = Dg[(int64_t)col * p2 + q0 + qq];
-                    }
-                    __syncwarp();
-                    if (busy && mine) {
-                        cx<float> bn = Ba[q0 + min(sl, qn - 1)];  // the next coefficient's load is in flight
-                        for (int qq = sl; qq < qn; qq += nsl) {
-                            const cx<float> bq = bn;
-                            if (qq + nsl < qn) bn = Ba[q0 + qq + nsl];
-#pragma unroll
-                            for (int rr = 0; rr < RB; ++rr) {
-                                if (rr < nrb) {
-#pragma unroll
-                                    for (int c = 0; c < 3; ++c) cfma(acc[rr][c], bq, Ds[(3 * rr + c) * qc + qq]);
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        // sum the slices of each target: lane ti + tg * sl, fixed tree over sl
-        for (int off = nsl >> 1; off >= 1; off >>= 1) {
-#pragma unroll
-            for (int rr = 0; rr < RB; ++rr)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float re = __shfl_down_sync(0xffffffffu, acc[rr][c].re, off * tg);
-                    const float im = __shfl_down_sync(0xffffffffu, acc[rr][c].im, off * tg);
-                    if (sl < off) { acc[rr][c].re += re; acc[rr][c].im += im; }
-                }
-        }
-        // the near + far sums of the slice-0 lanes go to shared memory (the tiles are free), and the
-        // whole warp adds the side's rows of the self block (its Psi columns are diagonal) in double
-        // precision and stores them, one (target, RHS, component) per lane and pass
-        cx<float> *Ys = reinterpret_cast<cx<float> *>(T);  // [target][RB][3]
-        __syncwarp();
-        if (sl == 0) {
-#pragma unroll
-            for (int rr = 0; rr < RB; ++rr)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) Ys[(ti * RB + rr) * 3 + c] = acc[rr][c];
-        }
-        __syncwarp();
-        for (int o = lane; o < tg * 3 * nrb; o += 32) {
-            const int t = o / (3 * nrb), rem = o - t * 3 * nrb, rr = rem / 3, c = rem - 3 * rr;
-            const int64_t u = perm[nbeg[g] + it.y + t];
-            const c64 *M = Mself + 36 * u + 18 * side + 6 * c;
-            const c64 *xa = x + ((rb0 + rr) * N + u) * 6;
-            const cx<float> f = Ys[(t * RB + rr) * 3 + c];
-            c64 v = {(double)f.re, (double)f.im};
-            cfma(v, M[0], xa[0]);
-            cfma(v, M[1], xa[1]);
-            cfma(v, M[2], xa[2]);
-            cfma(v, M[3 + c], xa[3 + c]);
-            y[((rb0 + rr) * N + u) * 6 + 3 * side + c] = v;
-        }
-    }
-}
 
 // The near field in double precision, any number of right-hand sides, both sides of every pair in one
 // pass.  Bound by the FP64 pipe (a warp instruction keeps a quarter of an SM busy for 64 cycles), so what
@@ -2068,9 +1805,11 @@ __global__ void __launch_bounds__(192) k_near_finish(int64_t N, int64_t nr, int 
 // the background's bracket is -U (it sees the normal -n) and the scatterer side's is U + s r,
 // since (n x r) x n + (n . r) n = r for a unit n.  So the geometry and U are evaluated once per
 // pair, and only the scalars g, c of grad'g = c r once per wavenumber.
-// The sources go through two warp-private tiles of NS_TS (one per lane, cp.async) as in
-// k_near_w; then the far field (L2P, Eq. 2.23 first term) and the rows of the analytic self block
-// (App. B) of both sides, as in k_near_w's epilogue.
+// A unit's lanes are tg targets x nsl source slices (near_work_items).  The sources go through two
+// warp-private tiles of NS_TS (one per lane): while the warp computes on one, asynchronous copies fill the
+// other, and the warp synchronises only itself.  Then the far field (L2P, Eq. 2.23 first term; the leaf's
+// local expansions staged in the same shared memory, each slice adding its coefficients), the sum of the
+// slices by a fixed shuffle tree, and the rows of the analytic self block (App. B) in double precision.
 constexpr int NS_TS = 32;    // sources per tile, one staged by each lane
 constexpr int NS_WARPS = 4;  // warps per block; each fetches its own units
 struct SideTile {
@@ -2302,36 +2041,45 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
     y[(r * N + u) * 6 + row] = v;
 }
 
-// Steps 4-5 for 32 or more right-hand sides in single precision, one lane per right-hand side,
-// both sides of every pair in one pass (the relations of k_near_ws: v_1 = v_0 + s n,
-// q_1 = -gamma_j q_0).  A warp owns one unit: a group of at most NR_TT targets of one leaf and a
-// block of 32 right-hand sides.  The sources of the leaf's Neighbor list go by in tiles of 32:
-// - pair phase: lane l takes source l of the tile and evaluates, against every target of the
-//   group, w = n x r, n.r and r, the background's scalars (-c_0, g_0) and the scatterer side's
-//   (c_1, -gamma_j g_1; zero where the source lies in another scatterer or past the list's end)
-//   into shared memory;
-// - right-hand-side phase: every lane reads its own (v_0, q_0, s) of each source (node-major copy
-//   k_dens_node_major; the next source's loads in flight while the current one is applied) and, per
-//   target, U = w x v_0 + (n.r) v_0 once, then acc_0 += -c_0 U + g_0 q_0 and
-//   acc_1 += c_1 (U + s r) - gamma_j g_1 q_0; a pair's scalars serve 32 right-hand sides.
+// Steps 4-5 for four or more right-hand sides in single precision, both sides of every pair in one pass
+// (the relations of k_near_ws: v_1 = v_0 + s n, q_1 = -gamma_j q_0).  A warp owns one unit: a group of at
+// most NR_TT targets of one leaf and a slab of W right-hand sides, its lanes being W right-hand sides x
+// 32 / W slices of the sources.  The sources of the leaf's Neighbor list go by in tiles of 32:
+// - pair phase: lane l takes source l of the tile and evaluates, against every target of the group, r, the
+//   background's scalars (-c_0, g_0) and the scatterer side's (c_1, -gamma_j g_1; zero where the source
+//   lies in another scatterer or past the list's end) into shared memory;
+// - right-hand-side phase: every lane reads its own (a, m, q_0, s) of each source (k_prep_node_major; the
+//   next source's loads in flight while the current one is applied) and, per target, U = a r + r x m once
+//   (a = n . v_0, m = v_0 x n), then acc_0 += -c_0 U + g_0 q_0 and acc_1 += c_1 (U + s r) - gamma_j g_1 q_0;
+//   a pair's scalars serve W right-hand sides.
 // Then L2P (Eq. 2.23 first term) of both sides from the lane's three columns of the leaf's local
 // expansions, and the rows of the analytic self block (App. B) in double precision; each lane
 // stores its right-hand side's rows.  With the impedance boundary (side1 false) the background
 // side only (k_local_rows writes the scatterer rows).
+// Bound by the FP32 pipe: 72 operations per pair and right-hand side beside three 16-byte words of scalars
+// from shared memory (four with w = n x r and n . r among them: 65536 nodes x 128 13.4 ms, now 13.2).  With
+// fewer than 32 right-hand sides, W lanes of right-hand sides keep the eight targets of every source they
+// load, where lanes of (targets x slices) per side and eight right-hand sides, the pair scalars formed for
+// each, took three times as long (21973 nodes x 8: 1.5 -> 0.49 ms); as W lanes x subsets of the targets, a
+// source's loads served two targets: 1.2 ms, and the sums over all sources in one lane were twice as inexact.
+// At the end each slice holds the sums of its own targets, so that the FP64 rows are formed once per target.
 constexpr int NR_TT = 8;   // targets per unit
 constexpr int NR_WARPS = 4;
 struct RhsTile {
-    float4 ps[NR_TT][32][4];  // (w, n.r), (-c_0, g_0), (c_1, -gamma g_1), (r, 0) per target and source
+    // (r_x, r_y, -c_0), (r_z, 0, g_0), (c_1, -gamma g_1) per target and source
+    float4 ps[NR_TT][32 * 3 + 1];
     float4 tp[NR_TT][2];      // target position hi + scatterer id bits, position lo
     float4 tk[NR_TT];         // the target's scatterer wavenumber k_j and -gamma_j
 };
 
+template <int W>
 __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
     const int32_t *leaf_box, const int4 *__restrict__ groups, int n_groups, int n_units, int *next_unit, int64_t N,
     int64_t nr, bool side1, const int32_t *nbeg, const int32_t *nend, const int32_t *nbr_start,
     const int32_t *nbr_idx, const float4 *__restrict__ rec, const float4 *densS, const DomainConsts *dc,
     const int32_t *perm, int p2, int64_t nbox, const cx<float> *__restrict__ Bl2p, const cx<float> *__restrict__ D,
-    const c64 *__restrict__ Mself, const c64 *__restrict__ x, c64 *y, int slab0, int slab_lf) {
+    const c64 *__restrict__ Mself, const c64 *__restrict__ x, c64 *y, int slab0, int slab_lf, int64_t r0, int width) {
+    constexpr int NSL = 32 / W;  // source slices
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int rng_beg[NR_WARPS][32], rng_cum[NR_WARPS][33];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2343,10 +2091,13 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
         if (lane == 0) unit = atomicAdd(next_unit, 1);
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= n_units) break;
-        // slabs of 32 right-hand sides from slab0 on; the launch's last one (slab_lf) takes its
+        // slabs of W right-hand sides from slab0 on; the launch's last one (slab_lf) takes its
         // groups longest first
         const int slab = slab0 + unit / n_groups, grp = unit - (slab - slab0) * n_groups;
-        const int64_t r = (int64_t)slab * 32 + lane;  // this lane's right-hand side
+        // this lane's right-hand side (the last one where the block has none for it: nothing is stored then)
+        const int rw = W == 32 ? lane : min(slab * W + lane % W, width - 1), sl = lane / W;
+        const bool stores = W == 32 || slab * W + lane % W < width;
+        const int64_t r = W == 32 ? (int64_t)slab * 32 + lane : r0 + rw;
         __syncwarp();  // the previous unit's shared-memory reads are done
         const int4 gi = groups[slab == slab_lf ? n_groups + grp : grp];
         const int leaf = gi.x, ntg = gi.z;
@@ -2379,8 +2130,9 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
         }
         __syncwarp();
         const int nsrc = rc_[nnb];
-        // node-major (v_0, q_0, s) of this lane's right-hand side: source i at dl + 128 i
-        const float4 *dl = densS + ((int64_t)slab * N * 32 + lane) * 4;
+        // node-major (a, m, q_0, s) of this lane's right-hand side: source i at dl + st i
+        const int64_t st = W == 32 ? 128 : 4 * width;
+        const float4 *dl = densS + (W == 32 ? (int64_t)slab * N * 128 : 0) + 4 * rw;
         cx<float> acc0[NR_TT][3], acc1[NR_TT][3];
 #pragma unroll
         for (int t = 0; t < NR_TT; ++t)
@@ -2396,9 +2148,8 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                 while (rc_[qcur + 1] <= e) ++qcur;
                 i = rb_[qcur] + (e - rc_[qcur]);
             }
-            const float4 pa = rec[3 * i], pb = rec[3 * i + 1], pc = rec[3 * i + 2];
+            const float4 pa = rec[3 * i], pb = rec[3 * i + 1];
             const int sdom = __float_as_int(pa.w);
-            const float nn[3] = {pb.w, pc.x, pc.y};
 #pragma unroll
             for (int t = 0; t < NR_TT; ++t) {
                 if (t < ntg) {
@@ -2408,7 +2159,6 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     const float R2 = rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
                     const float inv = R2 > 0.f ? rsqrt_(R2) : 0.f;  // the node itself drops out
                     const float Rr = R2 * inv;
-                    const float nrv = nn[0] * rv[0] + nn[1] * rv[1] + nn[2] * rv[2];
                     cx<float> g0, c0, g1 = {0, 0}, c1 = {0, 0};
                     pair_scalars<float>(inv, Rr, k0, g0, c0);
                     if (!valid) g0 = c0 = cx<float>{0.f, 0.f};
@@ -2417,52 +2167,54 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                         pair_scalars<float>(inv, Rr, cx<float>{tk.x, tk.y}, g1, c1);
                         g1 = cx<float>{tk.z, tk.w} * g1;  // -gamma_j g_1: q_1 = -gamma_j q_0
                     }
-                    S.ps[t][lane][0] = make_float4(nn[1] * rv[2] - nn[2] * rv[1], nn[2] * rv[0] - nn[0] * rv[2],
-                                                   nn[0] * rv[1] - nn[1] * rv[0], nrv);
-                    S.ps[t][lane][1] = make_float4(-c0.re, -c0.im, g0.re, g0.im);
-                    S.ps[t][lane][2] = make_float4(c1.re, c1.im, g1.re, g1.im);
-                    S.ps[t][lane][3] = make_float4(rv[0], rv[1], rv[2], 0.f);
+                    S.ps[t][3 * lane] = make_float4(rv[0], rv[1], -c0.re, -c0.im);
+                    S.ps[t][3 * lane + 1] = make_float4(rv[2], 0.f, g0.re, g0.im);
+                    S.ps[t][3 * lane + 2] = make_float4(c1.re, c1.im, g1.re, g1.im);
                 }
             }
             __syncwarp();
             // right-hand-side phase
-            const int nsv = min(32, nsrc - s0);
-            int ic = __shfl_sync(0xffffffffu, i, 0);
-            float4 d0 = dl[128 * (int64_t)ic], d1 = dl[128 * (int64_t)ic + 1], d2 = dl[128 * (int64_t)ic + 2],
-                   d3 = dl[128 * (int64_t)ic + 3];
-            for (int sv = 0; sv < nsv; ++sv) {
+            // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero)
+            const int nsv = min(32, (nsrc - s0 + NSL - 1) / NSL * NSL);
+            int ic = __shfl_sync(0xffffffffu, i, sl);
+            float4 d0 = dl[st * ic], d1 = dl[st * ic + 1], d2 = dl[st * ic + 2], d3 = dl[st * ic + 3];
+            for (int v0 = 0; v0 < nsv; v0 += NSL) {
+                const int sv = v0 + sl;
                 float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
-                const int in = __shfl_sync(0xffffffffu, i, (sv + 1) & 31);
-                if (sv + 1 < nsv) {
-                    n0 = dl[128 * (int64_t)in];
-                    n1 = dl[128 * (int64_t)in + 1];
-                    n2 = dl[128 * (int64_t)in + 2];
-                    n3 = dl[128 * (int64_t)in + 3];
+                const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
+                if (v0 + NSL < nsv) {
+                    n0 = dl[st * in];
+                    n1 = dl[st * in + 1];
+                    n2 = dl[st * in + 2];
+                    n3 = dl[st * in + 3];
                 }
-                const cx<float> v[3] = {{d0.x, d0.y}, {d0.z, d0.w}, {d1.x, d1.y}};
-                const cx<float> q[3] = {{d1.z, d1.w}, {d2.x, d2.y}, {d2.z, d2.w}};
-                const cx<float> sj = {d3.x, d3.y};
+                const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
+                const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
+                const float2 sj = {d3.z, d3.w};
 #pragma unroll
                 for (int t = 0; t < NR_TT; ++t) {
                     if (t < ntg) {
-                        const float4 p0 = S.ps[t][sv][0], p1 = S.ps[t][sv][1];
-                        const float w[3] = {p0.x, p0.y, p0.z};
-                        const cx<float> U[3] = {w[1] * v[2] - w[2] * v[1] + p0.w * v[0],
-                                                w[2] * v[0] - w[0] * v[2] + p0.w * v[1],
-                                                w[0] * v[1] - w[1] * v[0] + p0.w * v[2]};
-                        const cx<float> mc0 = {p1.x, p1.y}, g0 = {p1.z, p1.w};
+                        const float4 p0 = S.ps[t][3 * sv], p1 = S.ps[t][3 * sv + 1];
+                        const float rx = p0.x, ry = p0.y, rz = p1.x;
+                        // U = a r + r x m
+                        cx<float> U[3] = {{fmaf(A.x, rx, fmaf(ry, m2.x, -rz * m1.x)), fmaf(A.y, rx, fmaf(ry, m2.y, -rz * m1.y))},
+                                          {fmaf(A.x, ry, fmaf(rz, m0.x, -rx * m2.x)), fmaf(A.y, ry, fmaf(rz, m0.y, -rx * m2.y))},
+                                          {fmaf(A.x, rz, fmaf(rx, m1.x, -ry * m0.x)), fmaf(A.y, rz, fmaf(rx, m1.y, -ry * m0.y))}};
+                        const cx<float> mc0 = {p0.z, p0.w}, g0 = {p1.z, p1.w};
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
                             cfma(acc0[t][c], mc0, U[c]);
                             cfma(acc0[t][c], g0, q[c]);
                         }
                         if (side1) {
-                            const float4 p2v = S.ps[t][sv][2], p3 = S.ps[t][sv][3];
+                            const float4 p2v = S.ps[t][3 * sv + 2];
                             const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
-                            const float rr[3] = {p3.x, p3.y, p3.z};
+                            U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};
+                            U[1] = {fmaf(sj.x, ry, U[1].re), fmaf(sj.y, ry, U[1].im)};
+                            U[2] = {fmaf(sj.x, rz, U[2].re), fmaf(sj.y, rz, U[2].im)};
 #pragma unroll
                             for (int c = 0; c < 3; ++c) {
-                                cfma(acc1[t][c], c1, U[c] + rr[c] * sj);
+                                cfma(acc1[t][c], c1, U[c]);
                                 cfma(acc1[t][c], g1, q[c]);
                             }
                         }
@@ -2477,7 +2229,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
         // in turn); the targets' L2P rows are staged in the scalars' shared memory, chunks of qc
         // coefficients, and the lane's expansion coefficients are loaded two coefficients ahead
         auto l2p = [&](int side, cx<float>(&acc)[NR_TT][3]) {
-            cx<float> *Bs = reinterpret_cast<cx<float> *>(&S.ps[0][0][0]);
+            cx<float> *Bs = reinterpret_cast<cx<float> *>(&S.ps[0][0]);
             constexpr int BS_CAP = (int)(sizeof(S.ps) / sizeof(cx<float>));
             const int qc = min(p2, BS_CAP / NR_TT);
             const int64_t ncols = 3 * nr;
@@ -2497,18 +2249,18 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                         Bs[t * qc + qq] = Bl2p[((int64_t)side * N + tbase + t) * p2 + q0 + qq];
                     }
                     __syncwarp();
-                    cx<float> e1[3], e2[3];
+                    cx<float> e1[3], e2[3];  // the slices take every NSL-th coefficient
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
-                        e1[c] = Dr[c * p2 + q0];
-                        e2[c] = Dr[c * p2 + q0 + min(1, qn - 1)];
+                        e1[c] = Dr[c * p2 + q0 + min(sl, qn - 1)];
+                        e2[c] = Dr[c * p2 + q0 + min(sl + NSL, qn - 1)];
                     }
-                    for (int qq = 0; qq < qn; ++qq) {
+                    for (int qq = sl; qq < qn; qq += NSL) {
                         const cx<float> dq[3] = {e1[0], e1[1], e1[2]};
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
                             e1[c] = e2[c];
-                            if (qq + 2 < qn) e2[c] = Dr[c * p2 + q0 + qq + 2];
+                            if (qq + 2 * NSL < qn) e2[c] = Dr[c * p2 + q0 + qq + 2 * NSL];
                         }
 #pragma unroll
                         for (int t = 0; t < NR_TT; ++t) {
@@ -2524,10 +2276,33 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
         };
         l2p(0, acc0);
         if (side1) l2p(1, acc1);
+        // the slices' sums; slice sl keeps the targets NSL k + sl
+#pragma unroll
+        for (int t = 0; t < NR_TT; ++t)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int o = 16; o >= W; o >>= 1) {
+                    acc0[t][c].re += __shfl_xor_sync(0xffffffffu, acc0[t][c].re, o);
+                    acc0[t][c].im += __shfl_xor_sync(0xffffffffu, acc0[t][c].im, o);
+                    acc1[t][c].re += __shfl_xor_sync(0xffffffffu, acc1[t][c].re, o);
+                    acc1[t][c].im += __shfl_xor_sync(0xffffffffu, acc1[t][c].im, o);
+                }
+        constexpr int NT = NR_TT / NSL;
+#pragma unroll
+        for (int k = 0; k < NT; ++k)
+#pragma unroll
+            for (int m = 1; m < NSL; ++m)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    if (sl == m) acc0[NSL * k][c] = acc0[NSL * k + m][c];
+                    if (sl == m) acc1[NSL * k][c] = acc1[NSL * k + m][c];
+                }
         // the rows of the self block (Psi columns diagonal) in double precision, stored
 #pragma unroll
-        for (int t = 0; t < NR_TT; ++t) {
-            if (t < ntg) {
+        for (int k = 0; k < NT; ++k) {
+            const int t = NSL * k + sl;
+            if (t < ntg && stores) {
                 const int64_t u = perm[tbase + t];
                 const c64 *xa = x + (r * N + u) * 6;
                 c64 *ya = y + (r * N + u) * 6;
@@ -2538,7 +2313,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     const c64 *M = Mself + 36 * u + 18 * side;
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
-                        const cx<float> a = side == 0 ? acc0[t][c] : acc1[t][c];
+                        const cx<float> a = side == 0 ? acc0[NSL * k][c] : acc1[NSL * k][c];
                         c64 v = {(double)a.re, (double)a.im};
                         cfma(v, M[6 * c], x0);
                         cfma(v, M[6 * c + 1], x1);
@@ -3206,7 +2981,7 @@ void build_near_cache(fmbem *h, cudaStream_t s) {
     CK(cudaStreamSynchronize(s));
 }
 
-// warp work items of the near field (see k_near_w): per leaf of nt targets, the layout of W
+// warp work items of the near field (see k_near_ws): per leaf of nt targets, the layout of W
 // warps x (tg targets x nsl slices) with the least lane time W / nsl, tg = ceil(nt / W) <= 32,
 // nsl the largest power of two with tg * nsl <= 32, up to 8 warps per leaf
 void near_work_items(fmbem *h, cudaStream_t s) {
@@ -3845,7 +3620,7 @@ static void clear_unused_domains(fmbem *h, int64_t nr, size_t real_bytes, cudaSt
 
 template <typename R>
 static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t s, const DomainConsts *dc,
-                        int tensor_mode = 0) {
+                        int tensor_mode = 0, bool noalloc = false) {
     const int64_t N = h->N;
     const int p2 = h->p2, J = h->Jf;  // multipole passes over domains 0..Jf
     const bool f32 = sizeof(R) == 4;
@@ -3858,40 +3633,33 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
 
-    // single precision with 32 or more right-hand sides: a node-major copy of the background
-    // densities and the normal jumps for k_near_r in the half of the density buffer that double
-    // precision would use (64 bytes per node and RHS, within its 96)
-    const int64_t nrT = f32 ? (nr / 32) * 32 : 0;
-    cx<R> *densT = nrT > 0 ? dens + 2 * nr * N * 6 : nullptr;
-    // and with fewer than 4, the normal jump s of the densities (k_near_ws) in the same place
+    // single precision with four or more right-hand sides: node-major densities for k_near_r in the half of
+    // the density buffer that double precision would use (64 bytes per node and right-hand side of 96)
+    cx<R> *densT = f32 && nr >= 4 ? dens + 2 * nr * N * 6 : nullptr;
+    // and with fewer, the normal jump s of the densities (k_near_ws) in the same place
     cx<R> *sj = f32 && nr < 4 ? dens + 2 * nr * N * 6 : nullptr;
     if (h->ibc) clear_unused_domains(h, nr, sizeof(R), s);
     // BF16x3 with many columns: P2M and M2M on the tensor cores as well (their products then leave
     // C split for M2L); otherwise on the CUDA cores
     const bool tc_up = f32 && tensor_mode == 2 && h->Mmbf != nullptr && 3 * nr >= 48;
-    const bool tc_p2m = tc_up && p2m_tc_supported(h, nr);
-    // whole blocks of 32 right-hand sides with P2M on the tensor cores: every consumer reads the
-    // node-major densities, which are then the only ones formed
-    const bool node_major_only = tc_p2m && nrT == nr;
-    if (node_major_only) {
-        k_prep_node_major<<<dim3((unsigned)((N + 7) / 8), (unsigned)(nr / 32)), 256, 0, s>>>(
-            N, nr, x, h->perm, h->nrm, h->w, h->dom, dc, (float4 *)densT);
+    const bool tc_p2m = tc_up && p2m_tc_supported(h, nr);  // reads the node-major densities: the only ones formed
+    // (the static array has no such half for fewer than 32: they are formed after P2M, in another place)
+    const bool prep_first = densT != nullptr && !(noalloc && nr < 32);
+    auto prep_node_major = [&](int64_t r0, int64_t n, cx<R> *out) {
+        k_prep_node_major<<<dim3((unsigned)((N * std::min<int64_t>(n, 32) + 255) / 256), (unsigned)((n + 31) / 32)), 256, 0, s>>>(
+            N, r0, n, x, h->perm, h->nrm, h->w, h->dom, dc, (float4 *)out);
         CKL("k_prep_node_major");
-    } else {
+    };
+    if (prep_first) prep_node_major(0, nr, densT);
+    if (!tc_p2m) {
         k_prep<R><<<dim3(nblk(N, 128), (unsigned)nr), 128, 0, s>>>(N, nr, x, h->perm, h->nrm, h->w, h->dom, dc, dens,
                                                                     sj, f32 ? nullptr : (cx<R> *)h->near_am);
         CKL("k_prep");
-        if (densT != nullptr) {
-            k_dens_node_major<<<dim3((unsigned)((N + 15) / 16), (unsigned)(nrT / 32)), 256, 0, s>>>(
-                N, nr, (const float4 *)dens, h->src_rec, (float4 *)densT);
-            CKL("k_dens_node_major");
-        }
     }
     const int tbc = std::min(256, ((p2 + 31) / 32) * 32);
     constexpr int P2M_RB = sizeof(R) == 4 ? 8 : 4;
     if (tc_p2m) {
-        run_p2m_tc(h, (const float *)dens, node_major_only ? (const float4 *)densT : nullptr, (const float *)Bp2m,
-                   (float *)C, nr, s);
+        run_p2m_tc(h, (const float4 *)densT, (const float *)Bp2m, (float *)C, nr, s);
     } else if (nr >= 16) {
         constexpr int MT = p2m_mt<R>(), PT = p2m_pt<R>();
         const int nthr = ((p2 + 2 * PT - 1) / (2 * PT)) * (MT / 4);
@@ -3929,43 +3697,31 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     // precision, the cache holds them in double
     // the scatterer side's near field is not needed with the impedance boundary (k_local_rows)
     const int nsides = h->ibc ? 1 : 2;
-    // k_near_w over the right-hand sides rhs_base .. nr - 1 in blocks of rb
-    auto launch_w = [&](auto kern, int rb, size_t tile_bytes, int64_t rhs_base) {
-        if (h->near_items == nullptr) throw fmbem_error{FMBEM_ERR_CUDA, "near-field work items were not built"};
-        const size_t smw = 2 * tile_bytes * NW_WARPS;  // two tiles per warp
-        const int64_t units = (int64_t)h->n_near_items * nsides * ((nr - rhs_base + rb - 1) / rb);
-        if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
-        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
-        int per_sm = 0;
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW_WARPS, smw));
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((units + NW_WARPS - 1) / NW_WARPS,
-                                                                    (int64_t)std::max(per_sm, 1) * nsm));
-        CK(cudaMemsetAsync(h->near_next, 0, sizeof(int), s));
-        kern<<<(unsigned)grid, 32 * NW_WARPS, smw, s>>>(
-            h->leaf_box, h->near_items, h->n_near_items, (int)units, h->near_next, N, nr, rhs_base, nsides, h->box_nbeg,
-            h->box_nend, h->nbr_start, h->nbr_idx, h->src_rec, (const cx<float> *)dens, dc, h->perm, p2, h->nbox,
-            (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y);
-        CKL("k_near_w");
-    };
-    // k_near_r over the right-hand sides 32 slab0 .. 32 (slab0 + nslab) - 1
-    auto launch_r = [&](int64_t slab0, int64_t nslab) {
+    // k_near_r<W> over the slabs slab0 .. slab0 + nslab - 1 of W right-hand sides: whole blocks of 32 from
+    // densT, or the width right-hand sides from r0 on whose node-major densities are at dn
+    auto launch_r = [&](auto kern, int64_t slab0, int64_t nslab, const cx<R> *dn, int64_t r0, int width) {
         const int64_t units = (int64_t)h->n_near_groups * nslab;
         if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
         const size_t smr = sizeof(RhsTile) * NR_WARPS;
-        CK(cudaFuncSetAttribute(k_near_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr));
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr));
         int per_sm = 0;
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_near_r, 32 * NR_WARPS, smr));
+        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NR_WARPS, smr));
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((units + NR_WARPS - 1) / NR_WARPS,
                                                                     (int64_t)std::max(per_sm, 1) * nsm));
         CK(cudaMemsetAsync(h->near_next, 0, sizeof(int), s));
-        k_near_r<<<(unsigned)grid, 32 * NR_WARPS, smr, s>>>(
+        kern<<<(unsigned)grid, 32 * NR_WARPS, smr, s>>>(
             h->leaf_box, h->near_groups, h->n_near_groups, (int)units, h->near_next, N, nr, nsides == 2, h->box_nbeg,
-            h->box_nend, h->nbr_start, h->nbr_idx, h->src_rec, (const float4 *)densT, dc, h->perm, p2, h->nbox,
-            (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y, (int)slab0, (int)(slab0 + nslab - 1));
+            h->box_nend, h->nbr_start, h->nbr_idx, h->src_rec, (const float4 *)dn, dc, h->perm, p2, h->nbox,
+            (const cx<float> *)Bl2p, (const cx<float> *)D, h->Mself, x, y, (int)slab0, (int)(slab0 + nslab - 1), r0, width);
         CKL("k_near_r");
     };
+    // fewer than 32 right-hand sides: 4 or 8 per slab, the warp's lanes divided among the sources
+    auto launch_rest = [&](const cx<R> *dn, int64_t r0, int width) {
+        if (width <= 4) launch_r(k_near_r<4>, 0, 1, dn, r0, width);
+        else launch_r(k_near_r<8>, 0, (width + 7) / 8, dn, r0, width);
+    };
     if constexpr (sizeof(R) == 4) {
-        if (nr >= 4) {  // whole blocks of 32 right-hand sides one per lane, the rest by k_near_w
+        if (nr >= 4) {  // whole blocks of 32 right-hand sides one per lane, then the rest
             const int64_t nblk = nr / 32, rest = nr - 32 * nblk;
             // a host-buffer product (fmbem_matvec_host) whose rows are final after the near field:
             // one launch per slab, each slab's rows copied back beside the next slab's launch
@@ -3974,7 +3730,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                                   nblk <= (int64_t)(sizeof(io.ev) / sizeof(io.ev[0]));
             if (per_slab) {
                 for (int64_t b = 0; b < nblk; ++b) {
-                    launch_r(b, 1);
+                    launch_r(k_near_r<32>, b, 1, densT, 0, 32);
                     CK(cudaEventRecord(io.ev[b], s));
                     CK(cudaStreamWaitEvent(io.down, io.ev[b], 0));
                     const int64_t off = b * 32 * N * 6;
@@ -3983,10 +3739,20 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                 }
                 io.copied = true;
             } else if (nblk > 0) {
-                launch_r(0, nblk);
+                launch_r(k_near_r<32>, 0, nblk, densT, 0, 32);
             }
-            if (rest >= 8) launch_w(k_near_w<8>, 8, sizeof(WarpTile<8>), 32 * nblk);
-            else if (rest > 0) launch_w(k_near_w<4>, 4, sizeof(WarpTile<4>), 32 * nblk);
+            if (rest > 0 && prep_first) {
+                launch_rest(densT + nblk * N * 256, 32 * nblk, (int)rest);
+            } else if (rest > 0) {
+                // the scatterer side's densities are no longer needed: their place holds 48 bytes per node
+                // and right-hand side, so three quarters of the right-hand sides at a time
+                cx<R> *dn = dens + nr * N * 6;
+                for (int64_t q0 = 0, cap = 3 * nr / 4; q0 < nr; q0 += cap) {
+                    const int64_t n = std::min(cap, nr - q0);
+                    prep_node_major(q0, n, dn);
+                    launch_rest(dn, q0, (int)n);
+                }
+            }
         } else {  // few right-hand sides: both sides of a pair in one pass, one unit per item and RHS
             if (h->near_items == nullptr) throw fmbem_error{FMBEM_ERR_CUDA, "near-field work items were not built"};
             const int nsp = h->near_part != nullptr ? near_ws_splits(h, nr) : 1;
@@ -4235,7 +4001,7 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     h->oz_dig = nullptr;  // no digits in the static array: the FP64 pipe's translations,
     h->near_am = h->near_part = nullptr;  // and no partial sums: a block per leaf (FP64), whole items (FP32)
     try {
-        matvec_impl<R>(h, x, y, nr, s, (const DomainConsts *)h->dcons);
+        matvec_impl<R>(h, x, y, nr, s, (const DomainConsts *)h->dcons, 0, true);
     } catch (...) {
         restore();
         throw;

@@ -356,8 +356,8 @@ __device__ __forceinline__ void split8_bf16(const float *v, uint4 &hi, uint4 &lo
 
 __global__ void __launch_bounds__(P2M_TC_THREADS, 2)
     k_p2m_tc(const P2mTc P, const int32_t *__restrict__ leaf_box, const int32_t *__restrict__ nbeg,
-             const int32_t *__restrict__ nend, const int32_t *__restrict__ dom, const float *__restrict__ nrm,
-             const float2 *__restrict__ dens, const float4 *__restrict__ densS, const c64 *__restrict__ dcons,
+             const int32_t *__restrict__ nend, const int32_t *__restrict__ dom, const float4 *__restrict__ densS,
+             const c64 *__restrict__ dcons,
              const float2 *__restrict__ Bp2m, float *C, __nv_bfloat16 *Ch, __nv_bfloat16 *Cl, int *err) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t empty[P2M_TC_STAGES], done;
@@ -408,16 +408,14 @@ __global__ void __launch_bounds__(P2M_TC_THREADS, 2)
     const int il_b = threadIdx.x & 3, rl = threadIdx.x >> 2;
     const bool b_item = rl < P.nt / 3 && 3 * rl < nh;
     const int64_t r_b = col0 / 3 + rl;
-    // densS (node-major densities [block of 32 RHS][node][RHS][(v_0, q_0, s) as 4 float4]) when
-    // given, else dens [side][RHS][node][(v, q)]: the scatterer side from v_1 = v_0 + s n and
-    // q_1 = -gamma_d q_0
-    const cx<float> gam = d > 0 && densS ? to<float>(dcons[3 * d + 2]) : cx<float>{0.f, 0.f};
+    // densS: node-major densities (a, m, q_0, s) (k_prep_node_major); the scatterer side has a + s, m and
+    // -gamma_d q_0
+    const int width = (int)min((int64_t)32, P.nr - (r_b & ~(int64_t)31));  // of r_b's block
+    const cx<float> gam = d > 0 ? to<float>(dcons[3 * d + 2]) : cx<float>{0.f, 0.f};
     struct In {
         float2 a[2][4];  // B_k(i, q0), B_k(i, q0 + 32)
         int dom_a, dom_b;
-        float2 b[6];     // the densities (v, q) of node il_b, right-hand side r_b
-        float2 sj;       // with densS: s = n . (v_1 - v_0)
-        float n[3];
+        float4 b[4];     // the densities of node il_b, right-hand side r_b
     };
     auto load = [&](In &x, int kb) {
         const int ia = i0 + 4 * kb + il_a, ibn = i0 + 4 * kb + il_b;
@@ -438,23 +436,9 @@ __global__ void __launch_bounds__(P2M_TC_THREADS, 2)
         }
         if (b_item && ibn < i1) {
             x.dom_b = dom[ibn];
-            if (densS) {
-                const float4 *o = densS + (((r_b >> 5) * P.N + ibn) * 32 + (r_b & 31)) * 4;
-                const float4 o0 = o[0], o1 = o[1], o2 = o[2], o3 = o[3];
-                x.b[0] = make_float2(o0.x, o0.y);
-                x.b[1] = make_float2(o0.z, o0.w);
-                x.b[2] = make_float2(o1.x, o1.y);
-                x.b[3] = make_float2(o1.z, o1.w);
-                x.b[4] = make_float2(o2.x, o2.y);
-                x.b[5] = make_float2(o2.z, o2.w);
-                x.sj = make_float2(o3.x, o3.y);
-            } else {
-                const float2 *dn = dens + (((int64_t)side * P.nr + r_b) * P.N + ibn) * 6;
+            const float4 *o = densS + ((r_b >> 5) * P.N * 32 + (int64_t)ibn * width + (r_b & 31)) * 4;
 #pragma unroll
-                for (int c = 0; c < 6; ++c) x.b[c] = dn[c];
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) x.n[c] = nrm[3 * ibn + c];
+            for (int c = 0; c < 4; ++c) x.b[c] = o[c];
         }
     };
     In cur, nxt;
@@ -496,34 +480,27 @@ __global__ void __launch_bounds__(P2M_TC_THREADS, 2)
         if (rl < P.nt / 3) {
             float w[3][8];
             if (cur.dom_b >= 0 && (d == 0 || cur.dom_b == d)) {
-                float2 v[6];
+                // W_k(c) = +-((v_c n_k - n_c v_k) + (n.v) delta_ck): m's components off the diagonal
+                float2 a = {cur.b[0].x, cur.b[0].y};
+                const float2 m[3] = {{cur.b[0].z, cur.b[0].w}, {cur.b[1].x, cur.b[1].y}, {cur.b[1].z, cur.b[1].w}};
+                float2 q[3] = {{cur.b[2].x, cur.b[2].y}, {cur.b[2].z, cur.b[2].w}, {cur.b[3].x, cur.b[3].y}};
+                if (d > 0) {
+                    a.x += cur.b[3].z;
+                    a.y += cur.b[3].w;
 #pragma unroll
-                for (int c = 0; c < 6; ++c) v[c] = cur.b[c];
-                if (densS && d > 0) {  // scatterer side from the background's
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        v[c].x += cur.sj.x * cur.n[c];
-                        v[c].y += cur.sj.y * cur.n[c];
-                        const float2 q0 = cur.b[3 + c];
-                        v[3 + c] = make_float2(-(gam.re * q0.x - gam.im * q0.y), -(gam.re * q0.y + gam.im * q0.x));
-                    }
+                    for (int c = 0; c < 3; ++c)
+                        q[c] = make_float2(-(gam.re * q[c].x - gam.im * q[c].y), -(gam.re * q[c].y + gam.im * q[c].x));
                 }
-                const float n[3] = {sg * cur.n[0], sg * cur.n[1], sg * cur.n[2]};
-                const float nvr = n[0] * v[0].x + n[1] * v[1].x + n[2] * v[2].x;
-                const float nvi = n[0] * v[0].y + n[1] * v[1].y + n[2] * v[2].y;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    w[c][0] = v[3 + c].x;
-                    w[c][1] = v[3 + c].y;
+                    w[c][0] = q[c].x;
+                    w[c][1] = q[c].y;
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
-                        float tr = n[k] * v[c].x - n[c] * v[k].x, ti = n[k] * v[c].y - n[c] * v[k].y;
-                        if (k == c) {
-                            tr += nvr;
-                            ti += nvi;
-                        }
-                        w[c][2 + 2 * k] = tr;
-                        w[c][3 + 2 * k] = ti;
+                        const float s1 = k == c || k == (c + 1) % 3 ? sg : -sg;
+                        const float2 t = k == c ? a : m[3 - c - k];
+                        w[c][2 + 2 * k] = s1 * t.x;
+                        w[c][3 + 2 * k] = s1 * t.y;
                     }
                 }
             } else {
@@ -1065,12 +1042,10 @@ void run_m2m_tc(fmbem *h, float *C, int64_t nr, cudaStream_t s, bool leaves_spli
 
 // P2M of the leaves on the tensor cores (k_p2m_tc): BF16x3, 2 p^2 <= 128, 16 or more right-hand
 // sides; the second half of C receives the bf16 hi / lo split of the leaves' expansions (run_m2m_tc
-// with leaves_split).  The densities come from dens, or from the node-major densS when it is given
-// (whole blocks of 32 right-hand sides, dens then unused)
+// with leaves_split).  densS: the node-major densities of k_prep_node_major
 bool p2m_tc_supported(const fmbem *h, int64_t nr) { return 2 * h->p2 <= TC_M && nr >= 16; }
 
-void run_p2m_tc(fmbem *h, const float *dens, const float4 *densS, const float *Bp2m, float *C, int64_t nr,
-                cudaStream_t s) {
+void run_p2m_tc(fmbem *h, const float4 *densS, const float *Bp2m, float *C, int64_t nr, cudaStream_t s) {
     if (!p2m_tc_supported(h, nr)) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "tensor-core P2M: unsupported shape"};
     if (!h->tc_err) throw fmbem_error{FMBEM_ERR_CUDA, "tensor-core P2M: the error flag was not allocated"};
     const int64_t ncols = 3 * nr;
@@ -1089,8 +1064,8 @@ void run_p2m_tc(fmbem *h, const float *dens, const float4 *densS, const float *B
     const P2mTc P{h->N, nr, h->nbox, h->p2, (int)ncols, nt, ntile, tcols};
     const dim3 grid((unsigned)(h->n_leaves * ntile), (unsigned)(h->Jf + 1));
     // the FP32 copy of the leaves' expansions is not written: M2M and M2L read the split
-    k_p2m_tc<<<grid, P2M_TC_THREADS, smem, s>>>(P, h->leaf_box, h->box_nbeg, h->box_nend, h->dom, h->nrm_f,
-                                                (const float2 *)dens, densS, (const c64 *)h->dcons,
+    k_p2m_tc<<<grid, P2M_TC_THREADS, smem, s>>>(P, h->leaf_box, h->box_nbeg, h->box_nend, h->dom, densS,
+                                                (const c64 *)h->dcons,
                                                 (const float2 *)Bp2m, nullptr, Chi, Clo, h->tc_err);
     CKL("k_p2m_tc");
 }
