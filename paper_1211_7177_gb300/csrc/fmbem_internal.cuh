@@ -207,6 +207,12 @@ struct fmbem {
     int *oz_er = nullptr, *oz_bal = nullptr;
     void *oz_pairs = nullptr;        // int2 [n_ff]: (source box, CSR position) in pair_e order
     int32_t *oz_group = nullptr;     // device copy of h_group_beg
+    // and those of S|S and R|R (child levels 3..): groups by (level, octant), (source box, entry of the level)
+    void *oz_oimg[2] = {nullptr, nullptr};
+    int *oz_oer[2] = {nullptr, nullptr};
+    int32_t *oz_ogroup = nullptr;
+    std::vector<int32_t> h_oz_ogroup;
+    void *oz_up = nullptr, *oz_down = nullptr;
     void *oz_dig = nullptr;
     size_t oz_dig_bytes = 0;
     int *oz_err_host = nullptr;
@@ -377,6 +383,7 @@ template <typename R>
 size_t oz_digit_bytes(const fmbem *h, int W);
 template <typename R>
 void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W, cudaStream_t s);
+void run_oct_oz(fmbem *h, bool up, int l, const c64 *X, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s);
 void check_oz_err(fmbem *h, cudaStream_t s);
 void pack_rot_tables(fmbem *h, cudaStream_t s);
 void pack_rot_tables_mm(fmbem *h, cudaStream_t s);

@@ -3184,7 +3184,7 @@ static bool rot_many_path(const fmbem *h, int64_t nr, bool fp64) {
 static size_t ybuf_need(const fmbem *h, int64_t ncol, size_t elem) {
     int64_t mp = 1;
     for (int l = 2; l <= h->lmax; ++l) {
-        const int64_t ne = h->h_rmm_first.empty() ? 0 : h->h_rmm_first[l + 1] - h->h_rmm_first[l];
+        const int64_t ne = h->R_D64 == nullptr ? 0 : h->h_rmm_first[l + 1] - h->h_rmm_first[l];
         mp = std::max(mp, h->h_pair_first[l + 1] - h->h_pair_first[l] + ne);
     }
     return elem * (size_t)(h->Jf + 1) * (size_t)mp * (size_t)ncol * h->p2;
@@ -3195,7 +3195,7 @@ static size_t ybuf_need(const fmbem *h, int64_t ncol, size_t elem) {
 static size_t ofs_ybuf_need(const fmbem *h, int64_t nr) {
     int64_t ne = 1;
     for (int l = 2; l <= h->lmax; ++l)
-        if (!h->h_rmm_first.empty()) ne = std::max(ne, h->h_rmm_first[l + 1] - h->h_rmm_first[l]);
+        if (h->R_D64 != nullptr) ne = std::max(ne, h->h_rmm_first[l + 1] - h->h_rmm_first[l]);
     return sizeof(float) * (size_t)(h->Jf + 1) * (ofs_y_dom(h, nr) + (size_t)ne * 3 * nr * 2 * h->p2);
 }
 
@@ -3214,7 +3214,6 @@ static int oz_window(const fmbem *h, int64_t nr, int tensor_mode) {
     if (tensor_mode && h->Atc != nullptr && 3 * nr >= 48) return 0;
     const int rows_pad = ((h->p2 + 31) / 32) * 32;
     int64_t most = std::min<int64_t>(48, 3 * (1024 / rows_pad));
-    if (h->R_D64 != nullptr) most = std::min<int64_t>(most, 24);  // L2L in rotation form beside it
     const int64_t per_col = (int64_t)sizeof(cx<R>) * (h->Jf + 1) * std::max<int64_t>(h->n_ff, 1) * h->p2;
     most = std::max<int64_t>(3, std::min(most, (int64_t(8) << 30) / per_col) / 3 * 3);
     const int64_t windows = (3 * nr + most - 1) / most, W = 3 * ((nr + windows - 1) / windows);
@@ -3222,7 +3221,7 @@ static int oz_window(const fmbem *h, int64_t nr, int tensor_mode) {
     if ((h->Jf + 1) * h->nbox * W >= INT32_MAX || h->n_ff * W >= INT32_MAX) return 0;
     return (int)W;
 }
-// bytes of a window's pair results, then one level's rotation-form L2L entries
+// bytes of a window's pair results, then one level's L2L entries
 template <typename R>
 static size_t oz_ybuf_need(const fmbem *h, int W) {
     int64_t ne = 0;
@@ -3382,6 +3381,25 @@ static void upward_m2m(fmbem *h, int64_t nr, cudaStream_t s) {
     cx<R> *C = (cx<R> *)h->Cexp;
     const cx<R> *Tmm = f32 ? (const cx<R> *)h->T_mm32 : (const cx<R> *)h->T_mm64;
     const int rows_pad = ((p2 + 31) / 32) * 32;
+    // FP64 in digits on the tensor cores (m2l_oz.cu): every child's translation, then the sum per parent
+    if constexpr (sizeof(R) == 8) {
+        const int ozw = oz_window<R>(h, nr, 0);
+        if (oz_ready<R>(h, ozw)) {
+            cx<R> *Y = (cx<R> *)h->ybuf;
+            for (int col0 = 0; col0 < 3 * nr; col0 += ozw) {
+                const int nc = (int)std::min<int64_t>(ozw, 3 * nr - col0);
+                for (int l = lmax; l >= 3; --l) {
+                    const LevelInfo &P = h->lev[l - 1];
+                    run_oct_oz(h, true, l, C, Y, nr, col0, nc, s);
+                    k_mm_reduce<R><<<dim3((unsigned)P.n, (unsigned)(J + 1)), 128, 0, s>>>(
+                        P.off, 0, nr, p2, h->nbox, col0, nc, h->box_cbeg, h->box_cend, h->rmm_entry, h->h_rmm_first[l], Y, C,
+                        h->lev[l].n * nc * p2);
+                    CKL("k_mm_reduce");
+                }
+            }
+            return;
+        }
+    }
     // rotation form (p >= 9, few columns): the children of each level, by octant, translated to
     // their parents' centres (folded rotation, coaxial S|S, rotation back), then summed per parent
     const int ncol = (int)std::min<int64_t>(3 * nr, 24);
@@ -3476,7 +3494,7 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
         const cx<R> *RP = f32 ? (const cx<R> *)h->R_P32 : (const cx<R> *)h->R_P64;
         const cx<R> *RZ = f32 ? (const cx<R> *)h->R_Z32 : (const cx<R> *)h->R_Z64;
         const cx<R> *RZll = f32 ? (const cx<R> *)h->R_Zll32 : (const cx<R> *)h->R_Zll64;
-        const bool use_rot_mm = use_rot && h->rmm_chunk_beg != nullptr;
+        const bool use_rot_mm = use_rot && h->rmm_chunk_beg != nullptr && !(oz && !f32);
         cx<R> *Y = (cx<R> *)h->ybuf;
         // BF16x3 with few columns: the S|R products of each offset chunk on the tensor cores
         // (all levels and domains in one launch first: the S|R products read only C; the pair
@@ -3529,8 +3547,8 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                             h->pair_e, h->ff_src, Tm2l, C, Y, e_first, ystr);
                     CKL("k_m2l_chunks");
                 }
-                // L2L in rotation form: the children of level l, by octant, from their parents'
-                // local expansions
+                // L2L in rotation form or in digits: the children of level l, by octant, from their
+                // parents' local expansions
                 cx<R> *Yll = nullptr;
                 int64_t ll_first = 0;
                 const int64_t yll_str = nchild * nc * p2;
@@ -3543,6 +3561,13 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                                   h->rmm_chunk_cnt, h->rmm_chunk_ll, h->rmm_iota, h->rmm_par, h->rot_zero, 1, RD, RP,
                                   RZll, D, Yll, ll_first, yll_str);
                     CKL("k_m2l_rot (L2L)");
+                }
+                if constexpr (sizeof(R) == 8) {
+                    if (oz && l >= 3) {
+                        ll_first = h->h_rmm_first[l];
+                        Yll = Y + (J + 1) * ystr;
+                        run_oct_oz(h, false, l, D, Yll, nr, col0, nc, s);
+                    }
                 }
                 if (overlap && l == lmax) {  // join: the leaf level's reduction on the caller's stream
                     CK(cudaEventRecord(h->ev_join, h->aux_stream));

@@ -25,6 +25,12 @@
 // faster at every size (a whole product: sphere of 642 nodes 135 -> 104 us, 40962 nodes p = 10 1.69 -> 1.03 ms,
 // torus of 9216 nodes with 16 right-hand sides 8.3 -> 2.4 ms).
 //
+// S|S and R|R between levels run the same way in double precision: the children of a level grouped by octant
+// (torus of 9216 nodes, 16 right-hand sides, p = 8: M2M 2.18 and L2L 2.4 ms on the FP64 pipe, product 16.8 ms,
+// now 13.2; p = 10, three right-hand sides: in rotation form 6.19 ms and 5e-13 from the dense form, now 4.63 ms
+// and 2e-16).  In single precision the forms on the FP32 pipe are as fast (10242 nodes, p = 10: product 0.41
+// ms, 0.45 in digits; 9216 nodes, three right-hand sides: 1.28, 1.15) and stay.
+//
 // The FF pairs of one level and offset share a matrix; their columns (W per pair) follow one another
 // and are cut into tiles of N columns, the N of the MMAs (FP64: 80, six accumulators of 80 columns fill tensor
 // memory; FP32: 128, four accumulators); the matrix rows are its M = 128 (one row tile for p <= 8, two for p = 10).  The results go to
@@ -157,16 +163,24 @@ __device__ __forceinline__ int oz_degree(int q) {
     return n;
 }
 
-// digit images of the S|R matrices: block per matrix; per (row tile, K block) eight digit blocks of
-// 128 rows x 16 K in the 32-byte-swizzled K-major layout, real-form rows 2r + a as in m2l_tc.cu
-__global__ void __launch_bounds__(256) k_oz_images(const c64 *T, int p, int lmax, int mt, int kblocks, const int *bal,
-                                                   unsigned char *img, int *er) {
+// exponent by which the sources of degree n are scaled down: s_K for multipole expansions; for the local
+// expansions of R|R, which grow where the multipole ones shrink, the opposite, less the same n / 4
+__device__ __forceinline__ int oz_scale_of(const int *bal, int n, bool local) {
+    return local ? -bal[n] - n / 2 : bal[n];
+}
+
+// digit images of the matrices of one kind (per of them per domain and level l0 .. l0 + nlev - 1, T's set of a
+// domain having lmax + 1 levels; sources of level lsrc ..): block per matrix; per (row tile, K block) eight
+// digit blocks of 128 rows x 16 K in the 32-byte-swizzled K-major layout, real-form rows 2r + a as in m2l_tc.cu
+__global__ void __launch_bounds__(256) k_oz_images(const c64 *T, int p, int lmax, int per, int l0, int nlev, int lsrc, bool local,
+                                                   int mt, int kblocks, const int *bal, unsigned char *img, int *er) {
     const int64_t mat = blockIdx.x;
-    const int set = (int)(mat / 316), o = (int)(mat % 316), p2 = p * p;
-    const int d = set / (lmax - 1), l = 2 + set % (lmax - 1);
-    const c64 *M = T + m2l_matrix(d, l, o, lmax) * p2 * p2;
+    const int set = (int)(mat / per), o = (int)(mat % per), p2 = p * p;
+    const int d = set / nlev, l = set % nlev;
+    const c64 *M = T + (((int64_t)d * (lmax + 1) + l0 + l) * per + o) * p2 * p2;
+    bal += (d * (lmax - 1) + lsrc - 2 + l) * p;
     __shared__ int s_er[400], s_bal[400];
-    for (int c = threadIdx.x; c < p2; c += blockDim.x) s_bal[c] = bal[set * p + oz_degree(c)];
+    for (int c = threadIdx.x; c < p2; c += blockDim.x) s_bal[c] = oz_scale_of(bal, oz_degree(c), local);
     __syncthreads();
     for (int r = threadIdx.x; r < p2; r += blockDim.x) {
         int e = -OZ_NONFINITE;
@@ -214,19 +228,18 @@ __global__ void __launch_bounds__(256) k_oz_images(const c64 *T, int p, int lmax
     }
 }
 
-// digits of the multipole expansions, columns col0 .. col0 + W - 1 of every box of levels >= 2: a warp
+// digits of the expansions, columns col0 .. col0 + W - 1 of the boxes b0 .. b0 + nb - 1 (levels >= 2): a warp
 // per (domain, box, column) row; row (d nbox + box) W + c holds per K block its digit rows of 32
 // bytes, and ec its exponent
 template <typename R>
-__global__ void __launch_bounds__(256) k_oz_split(const cx<R> *C, const OzLevels L, int64_t nbox, int64_t ncols, int col0,
-                                                  int W, int ndom, int p, int kblocks, const int *bal, unsigned char *out,
-                                                  int *ec) {
+__global__ void __launch_bounds__(256) k_oz_split(const cx<R> *C, const OzLevels L, int64_t b0, int64_t nb, bool local,
+                                                  int64_t nbox, int64_t ncols, int col0, int W, int ndom, int p, int kblocks,
+                                                  const int *bal, unsigned char *out, int *ec) {
     const int lane = threadIdx.x & 31, p2 = p * p;
-    const int64_t nb = nbox - L.off[2];
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= (int64_t)ndom * nb * W) return;
     const int c = (int)(i % W);
-    const int64_t b = L.off[2] + (i / W) % nb;
+    const int64_t b = b0 + (i / W) % nb;
     const int d = (int)(i / W / nb);
     int l = 2;
     while (l < L.lmax && L.off[l + 1] <= b) ++l;
@@ -239,7 +252,7 @@ __global__ void __launch_bounds__(256) k_oz_split(const cx<R> *C, const OzLevels
     for (int k = 0; k < Q; ++k) {
         const int q = lane + 32 * k;
         v[k] = q < p2 ? x[q] : cx<R>{R(0), R(0)};
-        sc[k] = q < p2 ? s[oz_degree(q)] : 0;
+        sc[k] = q < p2 ? oz_scale_of(s, oz_degree(q), local) : 0;
         const int y = oz_exp2(v[k].re, v[k].im);
         e = max(e, abs(y) == OZ_NONFINITE ? y : y - sc[k]);
     }
@@ -265,8 +278,9 @@ __global__ void __launch_bounds__(256) k_oz_split(const cx<R> *C, const OzLevels
 
 struct OzP {
     int64_t nbox, y_dom;
-    int W, p2, kblocks;  // columns per pair of this window, K blocks of 16
-    int lmax, ndom, mt, ngroup;
+    int64_t mat_dom, mat0;  // matrices of a domain, and of its first group
+    int W, p2, kblocks;     // columns per pair of this window, K blocks of 16
+    int ndom, mt, ngroup;
 };
 template <typename R>
 __host__ __device__ __forceinline__ int oz_tiles(int64_t pairs, int W) {
@@ -440,7 +454,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 sources(t, src);
             }
             const int n_pad = (cur.n + 15) & ~15;
-            const int64_t mat = (int64_t)cur.d * (P.lmax - 1) * 316 + cur.g;
+            const int64_t mat = cur.d * P.mat_dom + P.mat0 + cur.g;
             const unsigned char *A = img + (mat * P.mt + cur.mt) * P.kblocks * (int64_t)OZ_A_BYTES;
             for (int kb = 0; kb < P.kblocks; ++kb, ++u, turn = turn == OZ_FILL - 1 ? 0 : turn + 1) {
                 if (turn != warp) continue;
@@ -540,7 +554,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         int nt = 0;
         for (int v = blockIdx.x; v < nunit; v += gridDim.x) {
             const OzTile t = oz_tile<R>(P, v, ntile, first, group);
-            const int64_t mat = (int64_t)t.d * (P.lmax - 1) * 316 + t.g;
+            const int64_t mat = t.d * P.mat_dom + P.mat0 + t.g;
             const int rr = t.mt * TC_M + quarter * 32 + lane;
             const bool rows = t.mt * TC_M + quarter * 32 < 2 * P.p2, row_ok = rr < 2 * P.p2;
             const int eR = row_ok ? er[mat * P.p2 + (rr >> 1)] : 0;
@@ -664,9 +678,45 @@ void build_oz_tables(fmbem *h, cudaStream_t s) {
     *h->oz_err_host = 0;
     k_oz_balance<<<dim3((unsigned)sets, (unsigned)h->p), 256, 0, s>>>(h->T_m2l64, h->p, h->lmax, h->oz_bal);
     CKL("k_oz_balance");
-    k_oz_images<<<(unsigned)nmat, 256, 0, s>>>(h->T_m2l64, h->p, h->lmax, mt, kb, h->oz_bal, (unsigned char *)h->oz_img,
-                                               h->oz_er);
+    k_oz_images<<<(unsigned)nmat, 256, 0, s>>>(h->T_m2l64, h->p, h->lmax, 316, 2, h->lmax - 1, 2, false, mt, kb, h->oz_bal,
+                                               (unsigned char *)h->oz_img, h->oz_er);
     CKL("k_oz_images");
+    if (h->lmax < 3) return;
+    // S|S and R|R between levels: the children of levels 3.. by octant (source and result rows per entry)
+    if (h->rmm_entry == nullptr) build_rot_mm_lists(h, s);
+    if (h->n_rmm == 0) return;
+    std::vector<int32_t> cnt((size_t)8 * (h->lmax - 2), 0), entry(h->nbox);
+    std::vector<uint64_t> key(h->nbox);
+    std::vector<int32_t> par(h->nbox);
+    CK(cudaMemcpyAsync(key.data(), h->box_key, sizeof(uint64_t) * h->nbox, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(par.data(), h->box_parent, sizeof(int32_t) * h->nbox, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(entry.data(), h->rmm_entry, sizeof(int32_t) * h->nbox, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    std::vector<int2> up(h->n_rmm), down(h->n_rmm);
+    for (int l = 3; l <= h->lmax; ++l)
+        for (int64_t g = h->lev[l].off; g < h->lev[l].off + h->lev[l].n; ++g) {
+            const int row = entry[g] - (int)h->h_rmm_first[l];
+            up[entry[g]] = make_int2((int)g, row);
+            down[entry[g]] = make_int2(par[g], row);
+            ++cnt[(size_t)(l - 3) * 8 + (key[g] & 7)];
+        }
+    h->h_oz_ogroup.assign(1, 0);
+    for (const int32_t c : cnt) h->h_oz_ogroup.push_back(h->h_oz_ogroup.back() + c);
+    h->oz_ogroup = (int32_t *)dev_alloc(h, sizeof(int32_t) * h->h_oz_ogroup.size());
+    h->oz_up = dev_alloc(h, sizeof(int2) * up.size());
+    h->oz_down = dev_alloc(h, sizeof(int2) * down.size());
+    CK(cudaMemcpyAsync(h->oz_ogroup, h->h_oz_ogroup.data(), sizeof(int32_t) * h->h_oz_ogroup.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(h->oz_up, up.data(), sizeof(int2) * up.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(h->oz_down, down.data(), sizeof(int2) * down.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaStreamSynchronize(s));
+    const int64_t noct = (int64_t)(h->Jf + 1) * (h->lmax - 2) * 8;
+    for (int k = 0; k < 2; ++k) {
+        h->oz_oer[k] = (int *)dev_alloc(h, sizeof(int) * noct * p2);
+        h->oz_oimg[k] = dev_alloc(h, noct * mt * kb * (int64_t)OZ_A_BYTES);
+        k_oz_images<<<(unsigned)noct, 256, 0, s>>>(k == 0 ? h->T_mm64 : h->T_ll64, h->p, h->lmax, 8, 3, h->lmax - 2, k == 0 ? 3 : 2,
+                                                   k == 1, mt, kb, h->oz_bal, (unsigned char *)h->oz_oimg[k], h->oz_oer[k]);
+        CKL("k_oz_images");
+    }
 }
 
 // real numbers of Y per domain for a window of W columns, and bytes of the window's digits and exponents
@@ -679,33 +729,36 @@ size_t oz_digit_bytes(const fmbem *h, int W) {
 template size_t oz_digit_bytes<double>(const fmbem *, int);
 template size_t oz_digit_bytes<float>(const fmbem *, int);
 
-// the S|R products of every level and domain for columns col0 .. col0 + W - 1 of C (3 n_rhs columns)
-// into Y[d][CSR position][W][p^2] (domains oz_y_dom apart)
+// the digits of the boxes b0 .. b0 + nb - 1 of X, then the products of the groups' matrices and pairs
 template <typename R>
-void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W, cudaStream_t s) {
-    if (h->n_ff <= 0) return;
+static void oz_products(fmbem *h, const cx<R> *X, int64_t b0, int64_t nb, bool local, cx<R> *Y, int64_t y_dom, int64_t nr,
+                        int col0, int W, int ngroup, const int32_t *h_group, const int32_t *group, const void *pairs,
+                        const void *img, const int *er, int64_t mat_dom, int64_t mat0, cudaStream_t s) {
     const int p2 = h->p2, kb = oz_kblocks(p2), ndom = h->Jf + 1;
+    OzP P{};
+    P.nbox = h->nbox;
+    P.y_dom = y_dom;
+    P.mat_dom = mat_dom;
+    P.mat0 = mat0;
+    P.W = W;
+    P.p2 = p2;
+    P.kblocks = kb;
+    P.ndom = ndom;
+    P.mt = oz_mt(p2);
+    P.ngroup = ngroup;
+    int64_t tiles = 0;
+    for (int g = 0; g < ngroup; ++g) tiles += oz_tiles<R>(h_group[g + 1] - h_group[g], W);
+    if (tiles == 0) return;
     OzLevels L{};
     L.lmax = h->lmax;
     for (int l = 2; l <= h->lmax; ++l) L.off[l] = h->lev[l].off;
     L.off[h->lmax + 1] = h->nbox;
-    const int64_t rows = (int64_t)ndom * (h->nbox - L.off[2]) * W;
+    const int64_t rows = (int64_t)ndom * nb * W;
     unsigned char *dig = (unsigned char *)h->oz_dig;
     int *ec = (int *)(dig + (size_t)ndom * h->nbox * W * kb * oz_row<R>);
-    k_oz_split<R><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(C, L, h->nbox, 3 * nr, col0, W, ndom, h->p, kb, h->oz_bal, dig, ec);
+    k_oz_split<R><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(X, L, b0, nb, local, h->nbox, 3 * nr, col0, W, ndom, h->p, kb,
+                                                             h->oz_bal, dig, ec);
     CKL("k_oz_split");
-    OzP P{};
-    P.nbox = h->nbox;
-    P.W = W;
-    P.p2 = p2;
-    P.kblocks = kb;
-    P.lmax = h->lmax;
-    P.ndom = ndom;
-    P.mt = oz_mt(p2);
-    P.ngroup = (h->lmax - 1) * 316;
-    P.y_dom = oz_y_dom(h, W);
-    int64_t tiles = 0;
-    for (int g = 0; g < P.ngroup; ++g) tiles += oz_tiles<R>(h->h_group_beg[g + 1] - h->h_group_beg[g], W);
     const size_t smem = OZ_SLOTS * (size_t)oz_slot_bytes<R> + 1024;
     CK(cudaFuncSetAttribute(k_m2l_oz<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int dev = 0, nsm = 0;
@@ -713,11 +766,27 @@ void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W,
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     // an odd grid: a CTA then alternates between the row tiles, of which the second is the shorter
     const int64_t grid = std::min<int64_t>(tiles * ndom * P.mt, (nsm - 1) | 1);
-    if (grid <= 0) return;
-    k_m2l_oz<R><<<(unsigned)grid, OZ_THREADS, smem, s>>>(P, h->oz_group, (const int2 *)h->oz_pairs, dig, ec,
-                                                         (const unsigned char *)h->oz_img, h->oz_er, (R *)Y, h->tc_err,
-                                                         h->oz_err_host);
+    k_m2l_oz<R><<<(unsigned)grid, OZ_THREADS, smem, s>>>(P, group, (const int2 *)pairs, dig, ec, (const unsigned char *)img, er,
+                                                         (R *)Y, h->tc_err, h->oz_err_host);
     CKL("k_m2l_oz");
+}
+
+// the S|R products of every level and domain for columns col0 .. col0 + W - 1 of C (3 n_rhs columns)
+// into Y[d][CSR position][W][p^2] (domains oz_y_dom apart)
+template <typename R>
+void run_m2l_oz(fmbem *h, const cx<R> *C, cx<R> *Y, int64_t nr, int col0, int W, cudaStream_t s) {
+    if (h->n_ff <= 0) return;
+    const int64_t b0 = h->lev[2].off;
+    oz_products<R>(h, C, b0, h->nbox - b0, false, Y, oz_y_dom(h, W), nr, col0, W, (h->lmax - 1) * 316, h->h_group_beg.data(),
+                   h->oz_group, h->oz_pairs, h->oz_img, h->oz_er, (int64_t)(h->lmax - 1) * 316, 0, s);
+}
+// the S|S products of the children of level l (up: X their multipole expansions) or the R|R products of their
+// parents' local expansions X, into Y[d][entry of the level][W][p^2] (domains n W p^2 complex values apart)
+void run_oct_oz(fmbem *h, bool up, int l, const c64 *X, c64 *Y, int64_t nr, int col0, int W, cudaStream_t s) {
+    const LevelInfo &S = h->lev[up ? l : l - 1];
+    oz_products<double>(h, X, S.off, S.n, !up, Y, h->lev[l].n * W * 2 * h->p2, nr, col0, W, 8, h->h_oz_ogroup.data() + (l - 3) * 8,
+                        h->oz_ogroup + (l - 3) * 8, up ? h->oz_up : h->oz_down, h->oz_oimg[up ? 0 : 1], h->oz_oer[up ? 0 : 1],
+                        (int64_t)(h->lmax - 2) * 8, (int64_t)(l - 3) * 8, s);
 }
 template void run_m2l_oz<double>(fmbem *, const c64 *, c64 *, int64_t, int, int, cudaStream_t);
 template void run_m2l_oz<float>(fmbem *, const c32 *, c32 *, int64_t, int, int, cudaStream_t);

@@ -4,9 +4,8 @@
 Tolerance.  Both forms translate with the same matrices; a pair result differs by the rounding of the
 dense form's sum of K = 2 p^2 <= 200 terms, at most about K 2^-53 of the terms' sum and 1e-15 of the
 result in the mean, and by the digits that are not multiplied, below 2^-62 of the largest terms.  A product adds
-the near field, which is the same, and up to 189 pairs per box: 1e-13 leaves two orders.  For p = 10 the
-automatic handle translates M2M and L2L in rotation form, whose factors are projected separately from the
-dense matrices (their quadrature agrees to about 1e-12): 1e-10."""
+the near field, which is the same, and up to 189 pairs per box: 1e-13 leaves two orders.  M2M and L2L
+between levels 2 to 4 are further such translations, at most four in a row."""
 import numpy as np
 import pytest
 
@@ -39,9 +38,8 @@ def rel(a, b):
 def test_matches_dense_form(p, n_rhs):
     a, d = handles("torus", p, leaf_size=16)  # levels 2 to 4
     x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=p + n_rhs)).cuda()
-    tol = 1e-13 if p <= 8 else 1e-10
-    assert rel(a.matvec(x), d.matvec(x)) < tol
-    assert rel(a.adjoint_matvec(x), d.adjoint_matvec(x)) < tol
+    assert rel(a.matvec(x), d.matvec(x)) < 1e-13
+    assert rel(a.adjoint_matvec(x), d.adjoint_matvec(x)) < 1e-13
 
 
 @pytest.mark.parametrize("mesh,opt", [("two", {}), ("two", dict(adaptive=1, leaf_size=12)),
