@@ -39,7 +39,9 @@ __device__ __forceinline__ cx<R> load_as(const T *p, int64_t i) {
 // partial[r][i][blk] = sum over the block's DOT_TB * MD_E elements of conj(V_i[r]) w[r] for
 // i = 0..nv-1 (V_i[r] at V + (i * nr + r) * n), in arithmetic R; the warps' sums are combined
 // in double precision.  The block keeps its slice of w in registers and walks the basis vectors
-// MD_G at a time, so w is read once and every basis vector once.
+// MD_G at a time, so w is read once and every basis vector once.  Where the slices of w are few, the groups of
+// MD_G vectors are split over grid.z as well (dot_splits): a group takes a block about 5 us, most of it the
+// FP64 sums over the warp, and 15 blocks (2562 nodes) took the groups one after the other.
 template <typename TV, typename TW, typename R, int MD_E>
 __global__ void __launch_bounds__(DOT_TB) k_multidot(const TV *V, int nv, const TW *w, int64_t n, int64_t nr,
                                                     c64 *partial) {
@@ -53,7 +55,7 @@ __global__ void __launch_bounds__(DOT_TB) k_multidot(const TV *V, int nv, const 
         const int64_t q = q0 + (int64_t)e * DOT_TB;
         wv[e] = q < n ? load_as<R>(w, r * n + q) : cx<R>{0, 0};
     }
-    for (int i0 = 0; i0 < nv; i0 += MD_G) {
+    for (int i0 = blockIdx.z * MD_G; i0 < nv; i0 += gridDim.z * MD_G) {
         R re[MD_G], im[MD_G];
 #pragma unroll
         for (int gI = 0; gI < MD_G; ++gI) {
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(DOT_TB) k_multidot2(const TV *V, int nv, const
         uv[e] = q < n ? load_as<R>(u, r * n + q) : cx<R>{0, 0};
         wv[e] = q < n ? load_as<R>(w, r * n + q) : cx<R>{0, 0};
     }
-    for (int i0 = 0; i0 < nv; i0 += G) {
+    for (int i0 = blockIdx.z * G; i0 < nv; i0 += gridDim.z * G) {
         R re[2 * G], im[2 * G];
 #pragma unroll
         for (int gI = 0; gI < G; ++gI) {
@@ -241,13 +243,19 @@ struct Work {
     void *dcoef;
     std::vector<c64> hres;
     std::vector<c32> hres32;
+    // grid.z of the reductions over groups of basis vectors: about six blocks for each of the 152 SMs
+    unsigned dot_splits(int groups) const {
+        const int64_t blocks = std::max<int64_t>(1, nblocks * nr);
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(groups, (6 * 152 + blocks - 1) / blocks));
+    }
     // dots[r][i] = <V_i[r], w[r]> for i < nv, arithmetic R
     template <typename R, typename TV, typename TW>
     void dots(const TV *V, int nv, const TW *w, std::vector<cd> &out) {
+        const dim3 grid(nblocks, (unsigned)nr, dot_splits((nv + MD_G - 1) / MD_G));
         if (md_e == MD_E_BIG)
-            k_multidot<TV, TW, R, MD_E_BIG><<<dim3(nblocks, (unsigned)nr), DOT_TB, 0, s>>>(V, nv, w, n, nr, partial);
+            k_multidot<TV, TW, R, MD_E_BIG><<<grid, DOT_TB, 0, s>>>(V, nv, w, n, nr, partial);
         else
-            k_multidot<TV, TW, R, MD_E_SMALL><<<dim3(nblocks, (unsigned)nr), DOT_TB, 0, s>>>(V, nv, w, n, nr, partial);
+            k_multidot<TV, TW, R, MD_E_SMALL><<<grid, DOT_TB, 0, s>>>(V, nv, w, n, nr, partial);
         CKL("k_multidot");
         const int64_t cnt = nr * nv;
         k_reduce_partials<<<nblk(cnt * 32, 256), 256, 0, s>>>(partial, nblocks, cnt, dres);
@@ -261,10 +269,11 @@ struct Work {
     // d1[r][i] = <V_i[r], u[r]>, d2[r][i] = <V_i[r], w[r]> for i < nv, in one pass over V
     template <typename R, typename TV>
     void dots2(const TV *V, int nv, const TV *u, const c64 *w, std::vector<cd> &d1, std::vector<cd> &d2) {
+        const dim3 grid(nblocks, (unsigned)nr, dot_splits((nv + MD_G / 2 - 1) / (MD_G / 2)));
         if (md_e == MD_E_BIG)
-            k_multidot2<TV, R, MD_E_BIG><<<dim3(nblocks, (unsigned)nr), DOT_TB, 0, s>>>(V, nv, u, w, n, nr, partial);
+            k_multidot2<TV, R, MD_E_BIG><<<grid, DOT_TB, 0, s>>>(V, nv, u, w, n, nr, partial);
         else
-            k_multidot2<TV, R, MD_E_SMALL><<<dim3(nblocks, (unsigned)nr), DOT_TB, 0, s>>>(V, nv, u, w, n, nr, partial);
+            k_multidot2<TV, R, MD_E_SMALL><<<grid, DOT_TB, 0, s>>>(V, nv, u, w, n, nr, partial);
         CKL("k_multidot2");
         const int64_t cnt = nr * 2 * nv;
         k_reduce_partials<<<nblk(cnt * 32, 256), 256, 0, s>>>(partial, nblocks, cnt, dres);
