@@ -2654,7 +2654,8 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
 
 // assembly of k_near_adj's partial sums: eight lanes per (node, right-hand side), four per side; each sums a
 // quarter of the far field (L2P of phi and grad phi) of its side's domain, then in double precision
-// u far + u near, T_d, the weights, and the transposed self block, a row of which each of six lanes takes
+// u far + u near, T_d, the weights, and the transposed self block, a lane per component of u and phi and then
+// per row (each lane with all six: single precision, 17026 nodes x 3 RHS 163 us, the FP64 pipe; now 100)
 template <typename R>
 __global__ void __launch_bounds__(128) k_near_adj_finish(
     int64_t N, int64_t nr, int nsp, int p2, int64_t nbox, const int32_t *__restrict__ node_leaf,
@@ -2690,7 +2691,9 @@ __global__ void __launch_bounds__(128) k_near_adj_finish(
     const R sg = side == 0 ? (R)-1 : (R)1;
     const R n1[3] = {sg * (R)nrm[3 * a], sg * (R)nrm[3 * a + 1], sg * (R)nrm[3 * a + 2]};
     const cx<R> div = fg[0][0] + fg[1][1] + fg[2][2];
-    c64 u[3], ph[3];
+    // (lane qpart < 3 of a side goes on with component qpart: FP64 instructions are what the rest costs)
+    c64 u = {0, 0}, ph = {0, 0};
+    const int cc = min(qpart, 2);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         cx<R> v = n1[c] * div;
@@ -2703,38 +2706,38 @@ __global__ void __launch_bounds__(128) k_near_adj_finish(
             fp[c].re += __shfl_xor_sync(0xffffffffu, fp[c].re, o);
             fp[c].im += __shfl_xor_sync(0xffffffffu, fp[c].im, o);
         }
-        u[c] = {(double)v.re, (double)v.im};
-        ph[c] = {(double)fp[c].re, (double)fp[c].im};
-    }
-    for (int s = 0; s < nsp; ++s) {
-        const cx<R> *P = part + ((s * nr + r) * N + a) * 12 + 6 * side;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            u[c] += c64{(double)P[c].re, (double)P[c].im};
-            ph[c] += c64{(double)P[3 + c].re, (double)P[3 + c].im};
+        if (cc == c) {
+            u = {(double)v.re, (double)v.im};
+            ph = {(double)fp[c].re, (double)fp[c].im};
         }
     }
-    if (side == 1) {  // T_j u = u + t_j n (n.u), n the scatterer normal
-        const double nb[3] = {nrm[3 * a], nrm[3 * a + 1], nrm[3 * a + 2]};
-        const c64 tn = dc[d].t * (nb[0] * u[0] + nb[1] * u[1] + nb[2] * u[2]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) u[c] += nb[c] * tn;
+    for (int s = 0; s < nsp; ++s) {
+        const cx<R> *P = part + ((s * nr + r) * N + a) * 12 + 6 * side + cc;
+        u += c64{(double)P[0].re, (double)P[0].im};
+        ph += c64{(double)P[3].re, (double)P[3].im};
     }
+    // T_j u = u + t_j n (n.u) on the scatterer side, n the scatterer normal
+    const double nb = qpart < 3 ? nrm[3 * a + cc] : 0.0;
+    c64 nu = nb * u;
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+        nu.re += __shfl_xor_sync(0xffffffffu, nu.re, o);
+        nu.im += __shfl_xor_sync(0xffffffffu, nu.im, o);
+    }
+    if (side == 1) u += nb * (dc[d].t * nu);
     const double wa = w[a];
-    const c64 sig = side == 0 ? c64{-1.0, 0.0} : dc[d].gamma;
-    c64 acc = {0, 0};  // row l8 of the result (l8 < 6)
-#pragma unroll
-    for (int row = 0; row < 6; ++row) {
-        c64 v = row < 3 ? wa * u[row % 3] : (sig * ph[row % 3]) * wa;
-        v.re += __shfl_xor_sync(0xffffffffu, v.re, 4);  // the other side
-        v.im += __shfl_xor_sync(0xffffffffu, v.im, 4);
-        if (row == l8) acc = v;
-    }
-    if (l8 < 6 && a_ < N) {
+    c64 vu = wa * u, vp = wa * ((side == 0 ? c64{-1.0, 0.0} : dc[d].gamma) * ph);
+    vu.re += __shfl_xor_sync(0xffffffffu, vu.re, 4);  // the other side
+    vu.im += __shfl_xor_sync(0xffffffffu, vu.im, 4);
+    vp.re += __shfl_xor_sync(0xffffffffu, vp.re, 4);
+    vp.im += __shfl_xor_sync(0xffffffffu, vp.im, 4);
+    c64 acc = side == 0 ? vu : vp;  // row 3 side + qpart of the result
+    const int row = 3 * side + qpart;
+    if (qpart < 3 && a_ < N) {
         const int64_t uu = perm[a];
         const c64 *M = Mself + 36 * uu, *xa = x + (r * N + uu) * 6;
-        for (int q = 0; q < 6; ++q) cfma(acc, M[q * 6 + l8], xa[q]);
-        y[(r * N + uu) * 6 + l8] = acc;
+        for (int q = 0; q < 6; ++q) cfma(acc, M[q * 6 + row], xa[q]);
+        y[(r * N + uu) * 6 + row] = acc;
     }
 }
 
