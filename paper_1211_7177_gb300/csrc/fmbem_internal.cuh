@@ -214,7 +214,7 @@ struct fmbem {
     std::vector<int32_t> h_oz_ogroup;
     void *oz_up = nullptr, *oz_down = nullptr;
     void *oz_dig = nullptr;
-    size_t oz_dig_bytes = 0;
+    size_t oz_dig_bytes = 0, oz_refused = ~size_t(0);
     int *oz_err_host = nullptr;
     bool m2l_rotation = false;
     int n_tlen = 0;

@@ -3255,7 +3255,8 @@ static int near_ws_splits(const fmbem *h, int64_t nr) {
     return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * 152 + units - 1) / units}));
 }
 // the near field's partial sums (rows complex values of a node, right-hand side and split), and per-source
-// vectors of the FP64 forward product
+// vectors of the FP64 forward product; without room for them the forward product takes the kernels of the
+// allocation-free one, and the transposed one fails
 static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, int rows, bool am) {
     const size_t npart = sizeof(c64) * rows * h->N * nr * nsp, nam = sizeof(c64) * 5 * h->N * nr;
     if (h->near_part_bytes < npart) {
@@ -3289,25 +3290,35 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
     const bool many = rot_many_path(h, nr, precision == FMBEM_FP64);
     const int mode = precision == FMBEM_BF16X3 ? 2 : precision == FMBEM_TF32 ? 1 : 0;
     const bool dbl = precision == FMBEM_FP64;
-    const int ozw = !pair_results ? 0 : dbl ? oz_window<double>(h, nr, 0) : oz_window<float>(h, nr, mode);
-    const size_t dig = dbl ? oz_digit_bytes<double>(h, ozw) : oz_digit_bytes<float>(h, ozw);
-    if (ozw > 0 && h->oz_dig_bytes < dig) {
-        if (h->oz_dig) dev_free(h, h->oz_dig);
-        h->oz_dig = nullptr;
-        h->oz_dig_bytes = 0;
-        h->oz_dig = dev_alloc(h, dig);
-        h->oz_dig_bytes = dig;
-    }
-    if (pair_results && (3 * nr <= 24 || many || ozw > 0)) {
-        size_t need = 3 * nr <= 24 || many ? ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb) : 0;
-        if (ozw > 0) need = std::max(need, dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw));
-        if (ofs_applies(h, nr, mode)) need = std::max(need, ofs_ybuf_need(h, nr));
-        if (h->ybuf == nullptr || h->ybuf_bytes < need) {
-            if (h->ybuf) dev_free(h, h->ybuf);
-            h->ybuf = nullptr;
-            h->ybuf = dev_alloc(h, need);
-            h->ybuf_bytes = need;
+    if (!pair_results) return;
+    auto grow = [&](void *&p, size_t &have, size_t need) {
+        if (p != nullptr && have >= need) return;
+        if (p) dev_free(h, p);
+        p = nullptr;
+        have = 0;
+        p = dev_alloc(h, need);
+        have = need;
+    };
+    const int ozw = dbl ? oz_window<double>(h, nr, 0) : oz_window<float>(h, nr, mode);
+    if (ozw > 0) {
+        // where the device has no room for the digits and a window's pair results (oz_refused: the least
+        // that was refused), the forms below remain
+        const size_t dig = dbl ? oz_digit_bytes<double>(h, ozw) : oz_digit_bytes<float>(h, ozw);
+        const size_t res = dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw);
+        if (dig + res < h->oz_refused) {
+            try {
+                grow(h->oz_dig, h->oz_dig_bytes, dig);
+                grow(h->ybuf, h->ybuf_bytes, res);
+            } catch (const fmbem_error &e) {
+                if (e.st != FMBEM_ERR_OOM) throw;
+                h->oz_refused = dig + res;
+            }
         }
+    }
+    if (3 * nr <= 24 || many) {
+        size_t need = ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb);
+        if (ofs_applies(h, nr, mode)) need = std::max(need, ofs_ybuf_need(h, nr));
+        grow(h->ybuf, h->ybuf_bytes, need);
     }
 }
 
@@ -3801,7 +3812,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                 k_near_sum<<<dim3(nblk(6 * N, 192), (unsigned)nr), 192, 0, s>>>(
                     N, nr, nsp, h->ibc ? 3 : 6, h->perm, (const cx<float> *)h->near_part, h->Mself, x, y);
         }
-    } else if (h->near_am != nullptr) {
+    } else if (h->near_am != nullptr && h->near_part != nullptr) {
         const int nsp = near_d_splits(h, nr);
         const int64_t units = (int64_t)h->n_near_ditems * nr * nsp;
         if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
@@ -3941,8 +3952,12 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
-    if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6, true);
-    else if (nr < 4) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
+    try {
+        if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6, true);
+        else if (nr < 4) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
+    } catch (const fmbem_error &e) {
+        if (e.st != FMBEM_ERR_OOM) throw;
+    }
     static_assert(sizeof(DomainConsts) == 3 * sizeof(c64), "layout");
     DomainConsts *dc = (DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {

@@ -1,0 +1,33 @@
+"""Products whose optional scratch (digits and pair results of the tensor-core M2L, the near field's partial
+sums) the device has no room for: the forms without it give the result, and nothing fails that needs no more
+than the densities and expansions.
+
+Tolerance: the two forms differ by the rounding of FP64 sums of some hundreds of terms, 1e-15 to 1e-14 (the
+tensor-core M2L against the dense one: 1e-13 is two orders above); FP32 2e-6 as for every such product."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import fmbem_inputs as fi  # noqa: E402
+import paper_1211_7177_gb300 as fm  # noqa: E402
+
+
+@pytest.mark.parametrize("n_rhs", [1, 9])
+@pytest.mark.parametrize("precision,tol", [(fm.FP64, 1e-13), (fm.FP32, 2e-6)])
+def test_without_room(n_rhs, precision, tol):
+    V, F, D = fi.torus(1.0, 0.25, 61, 19)
+    lib = fm.load_library()
+    a, b = [fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j], [1.0, 1.0], 1.5, p=8, leaf_size=16) for _ in range(2)]
+    x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=n_rhs)).cuda()
+    b.matvec(x[:1], precision=fm.BF16X3)  # densities, expansions and pair results of one right-hand side
+    if n_rhs > 1:
+        b.matvec(x.repeat(2, 1, 1), precision=fm.BF16X3)  # and, without pair results, of eighteen
+    lib.fmbem_debug_set_device_budget(0)
+    try:
+        y = b.matvec(x, precision=precision)
+    finally:
+        lib.fmbem_debug_set_device_budget(-1)
+    z = a.matvec(x)
+    assert float((y - z).norm()) < tol * float(z.norm())
+    assert float((b.matvec(x, precision=precision) - z).norm()) < tol * float(z.norm())
