@@ -76,11 +76,12 @@ __global__ void k_prep(int64_t N, int64_t nr, const c64 *x, const int32_t *perm,
 }
 
 // The single-precision densities of four or more right-hand sides, node-major within blocks of 32 (the last
-// block as wide as what is left), for k_near_r and P2M on the tensor cores: densS[block][node][right-hand
-// side][4 float4] = (a, m_x), (m_y, m_z), (q_x, q_y), (q_z, s) of the background side, with a = n . v_0,
+// block as wide as what is left), for k_near_r and P2M on the tensor cores: densS[block][node][4 float4]
+// [right-hand side] = (a, m_x), (m_y, m_z), (q_x, q_y), (q_z, s) of the background side, with a = n . v_0,
 // m = v_0 x n (the only forms in which those read v_0) and s = n . (v_1 - v_0) the scatterer side's jump
 // along the normal (v_1 = v_0 + s n, q_1 = -gamma_j q_0; see k_near_ws).  Thread per (node, right-hand
-// side), a block's right-hand sides next to each other, so that each warp stores whole rows; arithmetic as
+// side), a block's right-hand sides next to each other, so that a warp stores and k_near_r loads 512 bytes in
+// a piece; arithmetic as
 // in prep_body<float>.  Right-hand sides r0 .. r0 + n - 1, grid (.., blocks).
 __global__ void __launch_bounds__(256) k_prep_node_major(int64_t N, int64_t r0, int64_t n, const c64 *x, const int32_t *perm,
                                                          const double *nrm, const double *w, const int32_t *dom,
@@ -103,11 +104,11 @@ __global__ void __launch_bounds__(256) k_prep_node_major(int64_t N, int64_t r0, 
     }
     const cx<float> a = nn[0] * v[0] + nn[1] * v[1] + nn[2] * v[2], sj = wi * tn;
     const cx<float> m[3] = {nn[2] * v[1] - nn[1] * v[2], nn[0] * v[2] - nn[2] * v[0], nn[1] * v[0] - nn[0] * v[1]};
-    float4 *o = densS + (rb * N * 32 + i * width + rl) * 4;
+    float4 *o = densS + (rb * N * 32 + i * width) * 4 + rl;
     o[0] = make_float4(a.re, a.im, m[0].re, m[0].im);
-    o[1] = make_float4(m[1].re, m[1].im, m[2].re, m[2].im);
-    o[2] = make_float4(q[0].re, q[0].im, q[1].re, q[1].im);
-    o[3] = make_float4(q[2].re, q[2].im, sj.re, sj.im);
+    o[width] = make_float4(m[1].re, m[1].im, m[2].re, m[2].im);
+    o[2 * width] = make_float4(q[0].re, q[0].im, q[1].re, q[1].im);
+    o[3 * width] = make_float4(q[2].re, q[2].im, sj.re, sj.im);
 }
 
 // ---------------------------------------------------------------- P2M (Eqs. 2.18-2.19)
@@ -2056,8 +2057,11 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
 // expansions, and the rows of the analytic self block (App. B) in double precision; each lane
 // stores its right-hand side's rows.  With the impedance boundary (side1 false) the background
 // side only (k_local_rows writes the scatterer rows).
-// Bound by the FP32 pipe: 72 operations per pair and right-hand side beside three 16-byte words of scalars
-// from shared memory (four with w = n x r and n . r among them: 65536 nodes x 128 13.4 ms, now 13.2).  With
+// Per pair and right-hand side 72 FP32 operations beside three 16-byte words of scalars from shared memory
+// (four with w = n x r and n . r among them: 65536 nodes x 128 13.4 ms, now 13.2; 12.9 with the densities of 32
+// right-hand sides in 512-byte pieces instead of 64 bytes apart).  Issue slots 61 % busy, FMA 46 %: three
+// warps of 168 registers per scheduler do not hide the latency; a body per target count without branches
+// took 24 ms (instruction cache).  With
 // fewer than 32 right-hand sides, W lanes of right-hand sides keep the eight targets of every source they
 // load, where lanes of (targets x slices) per side and eight right-hand sides, the pair scalars formed for
 // each, took three times as long (21973 nodes x 8: 1.5 -> 0.49 ms); as W lanes x subsets of the targets, a
@@ -2131,8 +2135,9 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
         __syncwarp();
         const int nsrc = rc_[nnb];
         // node-major (a, m, q_0, s) of this lane's right-hand side: source i at dl + st i
-        const int64_t st = W == 32 ? 128 : 4 * width;
-        const float4 *dl = densS + (W == 32 ? (int64_t)slab * N * 128 : 0) + 4 * rw;
+        const int wd = W == 32 ? 32 : width;
+        const int64_t st = 4 * wd;
+        const float4 *dl = densS + (W == 32 ? (int64_t)slab * N * 128 : 0) + rw;
         cx<float> acc0[NR_TT][3], acc1[NR_TT][3];
 #pragma unroll
         for (int t = 0; t < NR_TT; ++t)
@@ -2150,9 +2155,9 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             }
             const float4 pa = rec[3 * i], pb = rec[3 * i + 1];
             const int sdom = __float_as_int(pa.w);
-#pragma unroll
-            for (int t = 0; t < NR_TT; ++t) {
-                if (t < ntg) {
+#pragma unroll 2
+            for (int t = 0; t < ntg; ++t) {
+                {
                     const float4 ta = S.tp[t][0], tl = S.tp[t][1];
                     const float rv[3] = {(pa.x - ta.x) + (pb.x - tl.x), (pa.y - ta.y) + (pb.y - tl.y),
                                          (pa.z - ta.z) + (pb.z - tl.z)};
@@ -2177,16 +2182,16 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero)
             const int nsv = min(32, (nsrc - s0 + NSL - 1) / NSL * NSL);
             int ic = __shfl_sync(0xffffffffu, i, sl);
-            float4 d0 = dl[st * ic], d1 = dl[st * ic + 1], d2 = dl[st * ic + 2], d3 = dl[st * ic + 3];
+            float4 d0 = dl[st * ic], d1 = dl[st * ic + wd], d2 = dl[st * ic + 2 * wd], d3 = dl[st * ic + 3 * wd];
             for (int v0 = 0; v0 < nsv; v0 += NSL) {
                 const int sv = v0 + sl;
                 float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
                 const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
                 if (v0 + NSL < nsv) {
                     n0 = dl[st * in];
-                    n1 = dl[st * in + 1];
-                    n2 = dl[st * in + 2];
-                    n3 = dl[st * in + 3];
+                    n1 = dl[st * in + wd];
+                    n2 = dl[st * in + 2 * wd];
+                    n3 = dl[st * in + 3 * wd];
                 }
                 const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
                 const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};

@@ -436,9 +436,9 @@ __global__ void __launch_bounds__(P2M_TC_THREADS, 2)
         }
         if (b_item && ibn < i1) {
             x.dom_b = dom[ibn];
-            const float4 *o = densS + ((r_b >> 5) * P.N * 32 + (int64_t)ibn * width + (r_b & 31)) * 4;
+            const float4 *o = densS + ((r_b >> 5) * P.N * 32 + (int64_t)ibn * width) * 4 + (r_b & 31);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) x.b[c] = o[c];
+            for (int c = 0; c < 4; ++c) x.b[c] = o[c * width];
         }
     };
     In cur, nxt;
