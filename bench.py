@@ -66,11 +66,10 @@ UNIT = "points*RHS/s"
 # each transcendental = 1)
 NEAR_PAIR = 52
 NEAR_RHS = 78
-# FP64 with fewer than 4 right-hand sides reads g and c from the near-field cache built at create:
-# per pair only r, w = n x r and n.r remain (14 flops, shared by both domains), and the scatterer
-# domain's bracket is the background's plus s r (6 FFMA per RHS instead of u's 30 flops): per
-# (pair, domain) 7 + 69 per right-hand side, averaged over the two domains
-NEAR_PAIR_CACHED = 7
+# FP64 reads g and c from the near-field cache built at create, and forms the bracket U = a r + r x m from
+# the per-source a = n.v and m = v x n (30 flops per pair and RHS, shared by both domains; the scatterer's
+# is U + s r, 12 more): per (pair, domain) 1.5 for r + 69 per right-hand side, averaged over the two domains
+NEAR_PAIR_CACHED = 1.5
 NEAR_RHS_CACHED = 69
 PEAK_TFLOPS = {"fp64": 1.2, "fp32": 74.6}  # measured FMA throughput on GB300 (self-written probe)
 TF32_OVER_BF16 = 1.1 / 2.25  # nominal dense TF32 : BF16 tensor-core rate
@@ -238,9 +237,15 @@ class ClockSampler:
 
 
 # ------------------------------------------------------------------------------- GPU arm
+def digit_path(p):
+    """The FP64 and FP32 products translate in 8-bit digits on the tensor cores (even p in 4..10); otherwise
+    in rotation form or with dense matrices on the CUDA cores."""
+    return p % 2 == 0 and 4 <= p <= 10
+
+
 def m2l_flops_per_column(p, nr):
-    """Algorithmic real flops of one S|R translation of one column: dense p^2 x p^2 complex matrix
-    (8 p^4), or, in the rotation form the library uses for p >= 9 with at most 8 right-hand sides,
+    """Algorithmic real flops of one S|R translation of one column on the CUDA cores: dense p^2 x p^2 complex
+    matrix (8 p^4), or, in the rotation form the library uses for p >= 9 with at most 8 right-hand sides,
     an azimuthal phase and a fold into mirror-even/odd halves, a real polar rotation per degree on
     the folded halves (real x complex, 4 flops per entry), the complex coaxial S|R per order block,
     the folded polar rotation back, the unfold and a phase."""
@@ -271,6 +276,11 @@ def roofline(info, p, nr, n_dom, phases, precision, workload=None):
             form = "dense S|R on tcgen05 TF32"
             peak, src = tensor_peak_tf32()
         bound = "tensor"
+    elif digit_path(p):
+        per_col, bound = 8.0 * p ** 4, "tensor"
+        products = 36 if precision == "fp64" else 10
+        form = f"dense S|R on tcgen05 in exact 8-bit digits ({products} digit products)"
+        peak, src = tensor_peak_bf16(products, "digit products")
     else:
         per_col, form = m2l_flops_per_column(p, nr)
         peak, src, bound = alu_peak, alu_src, "alu"
@@ -280,12 +290,11 @@ def roofline(info, p, nr, n_dom, phases, precision, workload=None):
                           frac=ach / peak, ms=avg["m2l_l2l"], algorithmic_flops_per_launch=flops, peak_source=src,
                           traffic=phase_traffic(workload, precision, nr, "m2l_l2l"))
     # near field + L2P + self
-    cached = precision == "fp64" and nr < 4
+    cached = precision == "fp64"
     per_pair, per_rhs = (NEAR_PAIR_CACHED, NEAR_RHS_CACHED) if cached else (NEAR_PAIR, NEAR_RHS)
     flops = info["near_pairs"] * n_dom * (per_pair + per_rhs * nr)
     ach = flops / (avg["near_l2p_self"] * 1e-3) / 1e12
-    kern = ("k_near (pair-scalar cache)" if cached else "k_near_rb") if arith == "fp64" else \
-        ("k_near_ws" if nr < 4 else "k_near_r + k_near_w" if nr >= 32 else "k_near_w")
+    kern = "k_near_d, pair-scalar cache" if cached else "k_near_ws" if nr < 4 else "k_near_r"
     out["near_l2p_self"] = dict(kernel=f"near field + L2P + self ({kern})", bound="alu", achieved=ach, peak=alu_peak,
                                 unit="TFLOP/s", frac=ach / alu_peak, ms=avg["near_l2p_self"],
                                 algorithmic_flops_per_launch=flops, peak_source=alu_src,
@@ -306,29 +315,39 @@ def tensor_path(nr):
 def launches_per_matvec(lmax, nr, n_dom, precision, p, rotation):
     """Kernels per matvec of the main line's path, as the ncu launch lists under profiles/ show
     them (every domain of a level in one launch):
-    - tensor-core path (BF16x3 or TF32, 16 or more RHS, p <= 8): the densities (k_prep_node_major
-      for whole blocks of 32 RHS in BF16x3, else k_prep, plus k_dens_node_major when there are
-      32 or more), P2M (k_p2m_tc in BF16x3, k_p2m_gemm in TF32), M2M per level 3..l_max
+    - tensor-core path (BF16x3 or TF32, 16 or more RHS, p <= 8): k_prep_node_major (and k_prep in
+      TF32), P2M (k_p2m_tc in BF16x3, k_p2m_gemm in TF32), M2M per level 3..l_max
       (k_m2l_tc in BF16x3; k_m2m on the CUDA cores in TF32), k_round_tf32 (TF32), one k_m2l_tc per
-      level 2..l_max, and the near field (k_near_r per whole block launch, k_near_w for the rest);
-    - otherwise k_prep and P2M; M2M per level 3..l_max (the rotation form: k_m2l_rot* + k_mm_reduce;
-      dense: k_m2m); the downward pass: BF16x3 with at most 8 RHS: k_split_bf16, two k_m2l_ofs
-      launches and per level a k_l2l_reduce (with a rotation-form L2L on levels 3..l_max);
-      else per level a k_l2l_reduce after the M2L (k_m2l_rot* or k_m2l_chunks), with the L2L
-      translation as its own launch on levels 3..l_max in the rotation form; one near-field
-      kernel."""
-    near = 1
+      level 2..l_max, and the near field (k_near_r: one launch for whole blocks of 32 right-hand
+      sides, one for the rest);
+    - FP64 with even p in 4..10 (digits; windows of at most 48 columns, 24 for p = 10): k_prep and P2M; per
+      window and level 3..l_max M2M in three launches (k_oz_split, k_m2l_oz, k_mm_reduce); per window the
+      M2L in two, per level 2..l_max k_l2l_reduce, and on levels 3..l_max the L2L in two; k_near_d and
+      k_near_finish;
+    - otherwise k_prep (and k_prep_node_major for four or more right-hand sides) and P2M; M2M per level
+      3..l_max (the rotation form: k_m2l_rot* + k_mm_reduce; dense: k_m2m); the downward pass: k_l2l_reduce
+      per level after the M2L (BF16x3 with at most 8 RHS: k_split_bf16 and two k_m2l_ofs launches; FP32 with
+      even p in 4..10: k_oz_split and k_m2l_oz), with the L2L translation as its own launch on levels
+      3..l_max in the rotation form; the near field (k_near_ws; k_near_r as above)."""
+    near = (1 if nr >= 32 else 0) + (1 if nr % 32 else 0)
+    bf3 = precision == "bf16x3"
     if precision in ("bf16x3", "tf32") and tensor_path(nr) and p <= 8:
-        bf3 = precision == "bf16x3"
-        prep = 1 if (bf3 and nr % 32 == 0) else (2 if nr >= 32 else 1)
-        near = (1 if nr >= 32 else 0) + (1 if nr % 32 else 0)
-        return prep + 1 + (lmax - 2) + (0 if bf3 else 1) + (lmax - 1) + near
-    m2m = 2 * (lmax - 2) if rotation else (lmax - 2)
-    if precision == "bf16x3" and 3 * nr <= 24:
-        down = 1 + 2 + 1 + (2 if rotation else 1) * (lmax - 2)
+        return (1 if bf3 else 2) + 1 + (lmax - 2) + (0 if bf3 else 1) + (lmax - 1) + near
+    windows = -(-3 * nr // (48 if p <= 8 else 24))
+    if precision == "fp64" and digit_path(p):
+        return 2 + windows * (3 * (lmax - 2) + 2 + (lmax - 1) + 2 * (lmax - 2)) + 2
+    rot = rotation and 3 * nr <= 24
+    m2m = (2 if rot else 1) * (lmax - 2)
+    if precision == "fp64":  # odd p: the M2L of each level beside its reduction, k_near_d and k_near_finish
+        return 2 + m2m + 2 + (3 if rot else 2) * (lmax - 2) + 2
+    prep = 2 if nr >= 4 else 1
+    if bf3 and 3 * nr <= 24:
+        down = 3 + (lmax - 1) + (lmax - 2 if rot else 0)
+    elif digit_path(p):
+        down = windows * (2 + (lmax - 1)) + (lmax - 2 if rot else 0)
     else:
-        down = 2 + (3 if rotation else 2) * (lmax - 2)
-    return 2 + m2m + down + near
+        down = 2 + (3 if rot else 2) * (lmax - 2)
+    return prep + 1 + m2m + down + near
 
 
 def run_gradients(fd_check=False):
@@ -458,15 +477,19 @@ def gmres_roofline(N, iters, restart, ms_total, matvec_ms):
                 peak_source=f"HBM {hsrc} copy bandwidth; FP64 measured FMA throughput (self-written probe)")
 
 
-def tensor_peak_bf16x3():
-    """Effective tensor peak of the BF16x3 form: the measured cuBLAS BF16 burst rate over the three
-    bf16 products that carry one algorithmic product."""
+def tensor_peak_bf16(products, what):
+    """Effective tensor peak of a form that carries one algorithmic product in several bf16 products: the
+    measured cuBLAS BF16 burst rate over their count."""
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
             bf16, src = float(json.load(f)["bf16_tflops"]), "of measured"
     except (OSError, KeyError, ValueError):
         bf16, src = 1900.0, "of fallback"
-    return bf16 / 3, f"{src} BF16 GEMM burst rate / 3 (three bf16 products per algorithmic product)"
+    return bf16 / products, f"{src} BF16 GEMM burst rate / {products} ({what} per algorithmic product)"
+
+
+def tensor_peak_bf16x3():
+    return tensor_peak_bf16(3, "bf16 products")
 
 
 def phase_rooflines(info, p, nr, n_dom, N, phases, workload, form="bf16x3"):

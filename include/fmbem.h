@@ -124,17 +124,17 @@ typedef struct {
     int m2l_rotation;        /* S|R translations for few right-hand sides: 0 dense p^2 x p^2
                                 matrices, 1 rotation form (rotate to the translation axis, coaxial
                                 translation, rotate back; ~3.3 p^3 instead of p^4 operations),
-                                -1 automatic: FP64 S|R on the tensor cores in exact 8-bit digits
-                                where p is even in 4..10 and the digit images (32 to 43 bytes per matrix
-                                value) take at most an eighth of the free device memory, for any
-                                number of right-hand sides; otherwise, and for the remaining
-                                translations, rotation form for p >= 9 [-1]                     */
+                                -1 automatic: on the tensor cores in exact 8-bit digits (FP64: all
+                                translations, FP32: S|R) where p is even in 4..10 and the digit images
+                                (32 to 43 bytes per matrix value) take at most an eighth of the free
+                                device memory, for any number of right-hand sides; otherwise, and
+                                for the remaining translations, rotation form for p >= 9 [-1]   */
     int profile_phases;      /* non-zero: record CUDA events around the matvec phases so that
                                 fmbem_last_matvec_times can report them [0]                       */
     int near_cache;          /* near-field kernel scalars g, c of every (target, source, domain)
                                 pair, which depend on the geometry only, computed once at create
-                                in FP64 and read by the FP64 matvecs with fewer than 4 right-hand
-                                sides instead of evaluating exp, sincos and rsqrt per pair:
+                                in FP64 and read by the FP64 matvecs, forward and transposed,
+                                instead of evaluating exp, sincos and rsqrt per pair:
                                 0 off, 1 on, -1 automatic: on when the cache (32 bytes per pair and
                                 domain) takes at most a quarter of the free device memory [-1]    */
     int boundary;            /* fmbem_boundary: how the scatterers enter [PENETRABLE]             */

@@ -3959,7 +3959,7 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     ensure_scratch(h, nr, precision);
     try {
         if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6, true);
-        else if (nr < 4) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
+        else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
     } catch (const fmbem_error &e) {
         if (e.st != FMBEM_ERR_OOM) throw;
     }
