@@ -406,22 +406,22 @@ def run_gradients(fd_check=False):
 # records the SHA-256 prefixes of the kernel sources it was taken with, and the bench reports null
 # once a source has changed.
 TRAFFIC = {
-    ('silver_sphere_s7', 'fp64', 1, 'p2m'): dict(bytes=2213602816, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp64', 1, 'm2m'): dict(bytes=117071872, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp64', 1, 'm2l_l2l'): dict(bytes=5563075072, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp64', 1, 'near_l2p_self'): dict(bytes=6586166784, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp32', 1, 'p2m'): dict(bytes=1114655488, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp32', 1, 'm2m'): dict(bytes=58543872, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp32', 1, 'm2l_l2l'): dict(bytes=2677159680, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'fp32', 1, 'near_l2p_self'): dict(bytes=466040320, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'p2m'): dict(bytes=1114879744, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'm2m'): dict(bytes=58574080, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'm2l_l2l'): dict(bytes=3223854080, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'near_l2p_self'): dict(bytes=466579712, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('torus_512x128', 'bf16x3', 128, 'p2m'): dict(bytes=3513320192, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('torus_512x128', 'bf16x3', 128, 'm2m'): dict(bytes=1576227072, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('torus_512x128', 'bf16x3', 128, 'm2l_l2l'): dict(bytes=4913404416, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
-    ('torus_512x128', 'bf16x3', 128, 'near_l2p_self'): dict(bytes=4988141312, src={'fmm.cu': '4618eded26d502e7', 'm2l_tc.cu': 'b48e3b613c191a6f'}),
+    ('silver_sphere_s7', 'fp64', 1, 'p2m'): dict(bytes=2224433664, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp64', 1, 'm2m'): dict(bytes=357572608, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp64', 1, 'm2l_l2l'): dict(bytes=8746043648, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp64', 1, 'near_l2p_self'): dict(bytes=7813899008, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp32', 1, 'p2m'): dict(bytes=1114938624, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp32', 1, 'm2m'): dict(bytes=58539264, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp32', 1, 'm2l_l2l'): dict(bytes=4041595648, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'fp32', 1, 'near_l2p_self'): dict(bytes=467235840, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'p2m'): dict(bytes=1114957312, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'm2m'): dict(bytes=58548992, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'm2l_l2l'): dict(bytes=3212554496, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'near_l2p_self'): dict(bytes=466675712, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('torus_512x128', 'bf16x3', 128, 'p2m'): dict(bytes=3513552384, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('torus_512x128', 'bf16x3', 128, 'm2m'): dict(bytes=1576060928, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('torus_512x128', 'bf16x3', 128, 'm2l_l2l'): dict(bytes=4952579840, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
+    ('torus_512x128', 'bf16x3', 128, 'near_l2p_self'): dict(bytes=4967983104, src={'fmm.cu': 'bae6eea9d5ac4d6e', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '1a7b025595155f66'}),
 }
 
 
