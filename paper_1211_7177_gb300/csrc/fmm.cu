@@ -3280,6 +3280,13 @@ static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, int rows, bool am
     }
 }
 
+// they hold this call's: part of rows values for nsp splits, and the per-source vectors (am).  Both are looked at
+// before either is used: k_prep writes the vectors of every right-hand side
+static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, int rows, bool am) {
+    return h->near_part != nullptr && h->near_part_bytes >= sizeof(c64) * rows * h->N * nr * nsp &&
+           (!am || (h->near_am != nullptr && h->near_am_bytes >= sizeof(c64) * 5 * h->N * nr));
+}
+
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_results = true) {
     const size_t cb = sizeof(c64);
     if (h->scratch_rhs < nr) {
@@ -3695,9 +3702,10 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
         CKL("k_prep_node_major");
     };
     if (prep_first) prep_node_major(0, nr, densT);
+    const bool near_d = !f32 && near_scratch_holds(h, nr, near_d_splits(h, nr), 6, true);
     if (!tc_p2m) {
         k_prep<R><<<dim3(nblk(N, 128), (unsigned)nr), 128, 0, s>>>(N, nr, x, h->perm, h->nrm, h->w, h->dom, dc, dens,
-                                                                    sj, f32 ? nullptr : (cx<R> *)h->near_am);
+                                                                    sj, near_d ? (cx<R> *)h->near_am : nullptr);
         CKL("k_prep");
     }
     const int tbc = std::min(256, ((p2 + 31) / 32) * 32);
@@ -3799,7 +3807,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
             }
         } else {  // few right-hand sides: both sides of a pair in one pass, one unit per item and RHS
             if (h->near_items == nullptr) throw fmbem_error{FMBEM_ERR_CUDA, "near-field work items were not built"};
-            const int nsp = h->near_part != nullptr ? near_ws_splits(h, nr) : 1;
+            const int nsp = near_scratch_holds(h, nr, near_ws_splits(h, nr), 6, false) ? near_ws_splits(h, nr) : 1;
             const int64_t units = (int64_t)h->n_near_items * nr * nsp;
             if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
             int per_sm = 0;
@@ -3817,7 +3825,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                 k_near_sum<<<dim3(nblk(6 * N, 192), (unsigned)nr), 192, 0, s>>>(
                     N, nr, nsp, h->ibc ? 3 : 6, h->perm, (const cx<float> *)h->near_part, h->Mself, x, y);
         }
-    } else if (h->near_am != nullptr && h->near_part != nullptr) {
+    } else if (near_d) {
         const int nsp = near_d_splits(h, nr);
         const int64_t units = (int64_t)h->n_near_ditems * nr * nsp;
         if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};

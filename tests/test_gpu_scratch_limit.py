@@ -31,3 +31,23 @@ def test_without_room(n_rhs, precision, tol):
     z = a.matvec(x)
     assert float((y - z).norm()) < tol * float(z.norm())
     assert float((b.matvec(x, precision=precision) - z).norm()) < tol * float(z.norm())
+
+
+@pytest.mark.parametrize("room", [0, 1 << 18, 1 << 20, 1 << 22, 1 << 24])
+def test_without_room_after_fewer_right_hand_sides(room):
+    """A handle whose near-field scratch was sized by a product of one right-hand side, then one of nine with
+    no room, or room for a part, of what they want: each buffer holds the call's size or is not used."""
+    V, F, D = fi.torus(1.0, 0.25, 61, 19)
+    lib = fm.load_library()
+    a, b = [fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j], [1.0, 1.0], 1.5, p=8, leaf_size=16) for _ in range(2)]
+    x = torch.from_numpy(fi.random_complex((9, a.N, 6), seed=room)).cuda()
+    z = a.matvec(x)
+    b.matvec(x[:1])
+    b.matvec(x.repeat(2, 1, 1), precision=fm.BF16X3)  # densities and expansions of eighteen
+    lib.fmbem_debug_set_device_budget(room)
+    try:
+        y = b.matvec(x)
+    finally:
+        lib.fmbem_debug_set_device_budget(-1)
+    assert float((y - z).norm()) < 1e-13 * float(z.norm())
+    assert float((b.matvec(x, precision=fm.FP32) - z).norm()) < 2e-6 * float(z.norm())
