@@ -3290,7 +3290,12 @@ static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, int rows, bo
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_results = true) {
     const size_t cb = sizeof(c64);
     if (h->scratch_rhs < nr) {
-        if (h->dens) { dev_free(h, h->dens); dev_free(h, h->Cexp); dev_free(h, h->Dexp); }
+        // (a refused allocation leaves no freed buffer behind: the next call allocates what it needs)
+        h->scratch_rhs = 0;
+        for (void **p : {&h->dens, &h->Cexp, &h->Dexp}) {
+            dev_free(h, *p);
+            *p = nullptr;
+        }
         h->dens = dev_alloc(h, cb * 2 * nr * h->N * 6);
         h->Cexp = dev_alloc(h, cb * (size_t)(h->J + 1) * h->nbox * 3 * nr * h->p2);
         h->Dexp = dev_alloc(h, cb * (size_t)(h->J + 1) * h->nbox * 3 * nr * h->p2);

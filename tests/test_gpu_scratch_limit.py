@@ -51,3 +51,23 @@ def test_without_room_after_fewer_right_hand_sides(room):
         lib.fmbem_debug_set_device_budget(-1)
     assert float((y - z).norm()) < 1e-13 * float(z.norm())
     assert float((b.matvec(x, precision=fm.FP32) - z).norm()) < 2e-6 * float(z.norm())
+
+
+@pytest.mark.parametrize("call", ["matvec", "adjoint_matvec"])
+@pytest.mark.parametrize("room", [0, 9 * 1159 * 192, 9 * 1159 * 192 + (1 << 20)])
+def test_refused_product_leaves_the_handle_usable(call, room):
+    """No room (or room for the densities alone) for the expansions of more right-hand sides: that product is
+    refused, and the handle's next products, smaller and the same, give what they gave."""
+    V, F, D = fi.torus(1.0, 0.25, 61, 19)
+    lib = fm.load_library()
+    b = fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j], [1.0, 1.0], 1.5, p=8, leaf_size=16)
+    x = torch.from_numpy(fi.random_complex((9, b.N, 6), seed=3)).cuda()
+    y1 = getattr(b, call)(x[:1])
+    lib.fmbem_debug_set_device_budget(room)
+    try:
+        with pytest.raises(fm.FMBEMError):
+            getattr(b, call)(x)
+    finally:
+        lib.fmbem_debug_set_device_budget(-1)
+    assert torch.equal(getattr(b, call)(x[:1]), y1)
+    assert float((getattr(b, call)(x)[0] - y1[0]).norm()) < 1e-13 * float(y1.norm())
