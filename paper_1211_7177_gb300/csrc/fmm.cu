@@ -2496,7 +2496,9 @@ __global__ void k_p2m_adj(const int32_t *leaf_box, int64_t N, int64_t nr, int p2
 // are, per source and side, +-c B(x), B(x) = x x w - (n.r) x (the target sees -n on the background side), so
 // a pair keeps 3 + 3 sums per side instead of the 3 + 9 of phi and grad phi, and geometry, w and, in single
 // precision, the pair scalars of RB right-hand sides are formed once.  Partial sums (u near, phi near of both
-// sides) go to part[split][r][node][12]; k_near_adj_finish adds them, the far field and the self block.
+// sides) go to part[split][r][node][12]; k_near_adj_finish adds them, the far field and the self block.  Without
+// that scratch (part null, one split) u goes to the result's own rows and phi to the components 3 to 5 of the
+// densities (slots), which k_prep_adj leaves unused.
 // A block per leaf, right-hand side and side before, L2P by one thread per target: 17026 nodes x 3 RHS in
 // single precision 915 us, 10242 nodes in double 2865 us.
 template <typename R, int RB>
@@ -2511,7 +2513,7 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
     const int32_t *__restrict__ nbr_start, const int32_t *__restrict__ nbr_idx, const R *__restrict__ pos_hi,
     const R *__restrict__ pos_lo, const double *__restrict__ nrm, const int32_t *__restrict__ dom,
     const cx<R> *__restrict__ dens, const DomainConsts *dc, const int64_t *__restrict__ cache_base,
-    const V4<R> *__restrict__ cache, cx<R> *part) {
+    const V4<R> *__restrict__ cache, cx<R> *part, const int32_t *__restrict__ perm, cx<R> *slots, c64 *y) {
     constexpr bool LO = sizeof(R) == 4;  // double-float positions
     __shared__ AdjTile<R, RB> tiles[ND_WARPS];
     __shared__ int rng_beg[ND_WARPS][32], rng_cum[ND_WARPS][33];
@@ -2650,7 +2652,11 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
                     const int tt = o / HALF, j = o - tt * HALF;
                     cx<R> v = S[j * 32 + tt];
                     for (int k = 1; k < nsl; ++k) v += S[j * 32 + k * tg + tt];
-                    part[(((int64_t)sp * nr + r0 + rr) * N + t0 + it.y + tt) * 12 + h0 + j] = v;
+                    const int row = h0 + j, sd = row / 6, c = row % 6;
+                    const int64_t b = t0 + it.y + tt, r = r0 + rr;
+                    if (part) part[((sp * nr + r) * N + b) * 12 + row] = v;
+                    else if (c < 3) y[(r * N + perm[b]) * 6 + 3 * sd + c] = c64{(double)v.re, (double)v.im};
+                    else slots[((sd * nr + r) * N + b) * 6 + c] = v;
                 }
             }
         }
@@ -2667,7 +2673,7 @@ __global__ void __launch_bounds__(128) k_near_adj_finish(
     const double *__restrict__ nrm, const double *__restrict__ w, const int32_t *__restrict__ dom,
     const int32_t *__restrict__ perm, const DomainConsts *dc, const cx<R> *__restrict__ Bl2p,
     const cx<R> *__restrict__ Bl2pg, const cx<R> *__restrict__ D, const c64 *__restrict__ Mself,
-    const c64 *__restrict__ x, const cx<R> *__restrict__ part, c64 *y) {
+    const c64 *__restrict__ x, const cx<R> *__restrict__ part, const cx<R> *__restrict__ slots, c64 *y) {
     const int64_t a_ = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3, r = blockIdx.y;
     const int64_t a = min(a_, N - 1);  // whole groups of eight lanes stay for the shuffles
     const int l8 = threadIdx.x & 7, side = l8 >> 2, qpart = l8 & 3;
@@ -2716,10 +2722,16 @@ __global__ void __launch_bounds__(128) k_near_adj_finish(
             ph = {(double)fp[c].re, (double)fp[c].im};
         }
     }
-    for (int s = 0; s < nsp; ++s) {
-        const cx<R> *P = part + ((s * nr + r) * N + a) * 12 + 6 * side + cc;
-        u += c64{(double)P[0].re, (double)P[0].im};
-        ph += c64{(double)P[3].re, (double)P[3].im};
+    if (part) {
+        for (int s = 0; s < nsp; ++s) {
+            const cx<R> *P = part + ((s * nr + r) * N + a) * 12 + 6 * side + cc;
+            u += c64{(double)P[0].re, (double)P[0].im};
+            ph += c64{(double)P[3].re, (double)P[3].im};
+        }
+    } else if (a_ < N) {  // (read here, and written by this group of lanes after the shuffles below)
+        const cx<R> P = slots[((side * nr + r) * N + a) * 6 + 3 + cc];
+        u += y[(r * N + perm[a]) * 6 + 3 * side + cc];
+        ph += c64{(double)P.re, (double)P.im};
     }
     // T_j u = u + t_j n (n.u) on the scatterer side, n the scatterer normal
     const double nb = qpart < 3 ? nrm[3 * a + cc] : 0.0;
@@ -3259,11 +3271,11 @@ static int near_ws_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_items * nr);
     return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * 152 + units - 1) / units}));
 }
-// the near field's partial sums (rows complex values of a node, right-hand side and split), and per-source
-// vectors of the FP64 forward product; without room for them the forward product takes the kernels of the
-// allocation-free one, and the transposed one fails
-static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, int rows, bool am) {
-    const size_t npart = sizeof(c64) * rows * h->N * nr * nsp, nam = sizeof(c64) * 5 * h->N * nr;
+// the near field's partial sums (6 or 12 complex values of a node, right-hand side and split), and per-source
+// vectors of the FP64 forward product (row_bytes a node, right-hand side and split); without room for them the
+// forward product takes the kernels of the allocation-free one, and the transposed one keeps its sums in the result
+static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
+    const size_t npart = row_bytes * h->N * nr * nsp, nam = sizeof(c64) * 5 * h->N * nr;
     if (h->near_part_bytes < npart) {
         if (h->near_part) dev_free(h, h->near_part);
         h->near_part = nullptr;
@@ -3280,10 +3292,10 @@ static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, int rows, bool am
     }
 }
 
-// they hold this call's: part of rows values for nsp splits, and the per-source vectors (am).  Both are looked at
+// they hold this call's: the partial sums of nsp splits, and the per-source vectors (am).  Both are looked at
 // before either is used: k_prep writes the vectors of every right-hand side
-static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, int rows, bool am) {
-    return h->near_part != nullptr && h->near_part_bytes >= sizeof(c64) * rows * h->N * nr * nsp &&
+static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
+    return h->near_part != nullptr && h->near_part_bytes >= row_bytes * h->N * nr * nsp &&
            (!am || (h->near_am != nullptr && h->near_am_bytes >= sizeof(c64) * 5 * h->N * nr));
 }
 
@@ -3707,7 +3719,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
         CKL("k_prep_node_major");
     };
     if (prep_first) prep_node_major(0, nr, densT);
-    const bool near_d = !f32 && near_scratch_holds(h, nr, near_d_splits(h, nr), 6, true);
+    const bool near_d = !f32 && near_scratch_holds(h, nr, near_d_splits(h, nr), 6 * sizeof(c64), true);
     if (!tc_p2m) {
         k_prep<R><<<dim3(nblk(N, 128), (unsigned)nr), 128, 0, s>>>(N, nr, x, h->perm, h->nrm, h->w, h->dom, dc, dens,
                                                                     sj, near_d ? (cx<R> *)h->near_am : nullptr);
@@ -3812,7 +3824,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
             }
         } else {  // few right-hand sides: both sides of a pair in one pass, one unit per item and RHS
             if (h->near_items == nullptr) throw fmbem_error{FMBEM_ERR_CUDA, "near-field work items were not built"};
-            const int nsp = near_scratch_holds(h, nr, near_ws_splits(h, nr), 6, false) ? near_ws_splits(h, nr) : 1;
+            const int nsp = near_scratch_holds(h, nr, near_ws_splits(h, nr), 6 * sizeof(c32), false) ? near_ws_splits(h, nr) : 1;
             const int64_t units = (int64_t)h->n_near_items * nr * nsp;
             if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
             int per_sm = 0;
@@ -3902,7 +3914,9 @@ static void adjoint_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     auto launch_adj = [&](auto kern, int rb) {
         const int64_t nrb = (nr + rb - 1) / rb;
-        const int nsp = near_d_splits(h, nrb);
+        const bool held = near_scratch_holds(h, nr, near_d_splits(h, nrb), 12 * sizeof(cx<R>), false);
+        const int nsp = held ? near_d_splits(h, nrb) : 1;
+        cx<R> *part = held ? (cx<R> *)h->near_part : nullptr;
         const int64_t units = (int64_t)h->n_near_ditems * nrb * nsp;
         if (units >= INT32_MAX) throw fmbem_error{FMBEM_ERR_INVALID_ARGUMENT, "too many near-field work units"};
         int per_sm = 0;
@@ -3913,11 +3927,11 @@ static void adjoint_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_
         kern<<<(unsigned)grid, 32 * ND_WARPS, 0, s>>>(
             h->leaf_box, h->near_ditems, h->n_near_ditems, (int)units, nsp, (int)nrb, h->near_next, N, nr, h->box_nbeg,
             h->box_nend, h->nbr_start, h->nbr_idx, ph, pl, h->nrm, h->dom, dens, dc, h->near_base,
-            f32 ? nullptr : (const V4<R> *)h->near_cache64, (cx<R> *)h->near_part);
+            f32 ? nullptr : (const V4<R> *)h->near_cache64, part, h->perm, dens, y);
         CKL("k_near_adj");
         k_near_adj_finish<R><<<dim3(nblk(8 * N, 128), (unsigned)nr), 128, 0, s>>>(
             N, nr, nsp, p2, h->nbox, h->node_leaf, h->nrm, h->w, h->dom, h->perm, dc, Bl2p, Bl2pg, D, h->Mself, x,
-            (const cx<R> *)h->near_part, y);
+            part, dens, y);
     };
     if constexpr (sizeof(R) == 4) {  // three right-hand sides share the pair scalars
         if (nr == 1) launch_adj(k_near_adj<R, false, 1>, 1);
@@ -3954,7 +3968,13 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
-    ensure_near_scratch(h, nr, near_d_splits(h, precision == FMBEM_FP64 || nr == 1 ? nr : (nr + 2) / 3), 12, false);
+    try {
+        const bool dbl = precision == FMBEM_FP64;
+        ensure_near_scratch(h, nr, near_d_splits(h, dbl || nr == 1 ? nr : (nr + 2) / 3), 12 * (dbl ? sizeof(c64) : sizeof(c32)),
+                            false);
+    } catch (const fmbem_error &e) {
+        if (e.st != FMBEM_ERR_OOM) throw;
+    }
     const DomainConsts *dc = (const DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
         adjoint_impl<float>(h, x, y, nr, s, dc, precision == FMBEM_TF32 ? 1 : 2);
@@ -3971,8 +3991,8 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision);
     try {
-        if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6, true);
-        else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6, false);
+        if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6 * sizeof(c64), true);
+        else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6 * sizeof(c32), false);
     } catch (const fmbem_error &e) {
         if (e.st != FMBEM_ERR_OOM) throw;
     }

@@ -71,3 +71,33 @@ def test_refused_product_leaves_the_handle_usable(call, room):
         lib.fmbem_debug_set_device_budget(-1)
     assert torch.equal(getattr(b, call)(x[:1]), y1)
     assert float((getattr(b, call)(x)[0] - y1[0]).norm()) < 1e-13 * float(y1.norm())
+
+
+@pytest.mark.parametrize("mesh,opt", [("torus", {}), ("two", {}), ("two", dict(boundary=fm.IMPEDANCE)),
+                                      ("torus", dict(near_cache=0)), ("torus", dict(adaptive=1, leaf_size=12))])
+@pytest.mark.parametrize("n_rhs", [1, 2, 4, 9])
+@pytest.mark.parametrize("precision,tol", [(fm.FP64, 1e-13), (fm.FP32, 2e-6)])
+def test_transposed_without_room(mesh, opt, n_rhs, precision, tol):
+    """The transposed product without its partial sums: they go to the result and the densities' unused
+    components."""
+    if mesh == "torus":
+        V, F, D = fi.torus(1.0, 0.25, 61, 19)
+    else:
+        V, F, D = fi.torus_and_sphere(nu=60, nv=18, sphere_subdiv=2)[0]
+    eps, mu = [1.0, -8.5 + 0.3j, 2.25][: D.max() + 1], [1.0] * (D.max() + 1)
+    lib = fm.load_library()
+    a, b = [fm.FMBEM(V, F, D, eps, mu, 1.5, p=8, **opt) for _ in range(2)]
+    x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=n_rhs)).cuda()
+    x[0] *= 1e-3
+    z = a.adjoint_matvec(x)
+    b.matvec(x, precision=fm.FP32)  # densities and expansions
+    if 4 <= n_rhs <= 8:
+        b.matvec(x)  # and FP64 pair results
+    y = torch.full_like(x, float("nan"))
+    lib.fmbem_debug_set_device_budget(0)
+    try:
+        b.adjoint_matvec(x, y, precision=precision)
+    finally:
+        lib.fmbem_debug_set_device_budget(-1)
+    for r in range(n_rhs):
+        assert float((y[r] - z[r]).norm()) < tol * float(z[r].norm())
