@@ -260,8 +260,14 @@ fmbem_status fmbem_plane_wave_rhs(fmbem *h, int64_t n_rhs, const double *dir, co
  *   x_dev, y_dev  device [n_rhs][N][6] complex128 (user order); x is read, y written; they
  *                 must not overlap.
  *   precision     fmbem_precision of the passes (see above).
- * Scratch (expansion coefficients, source densities) is owned by the handle and grown on
- * demand, so the first call with a larger n_rhs allocates. */
+ * Scratch (expansion coefficients, source densities, and per form of the product digits, pair
+ * results and partial sums) is owned by the handle and grown on demand, so the first call of a kind,
+ * or with a larger n_rhs, allocates.
+ * Stream capture: FP64 and FP32 products (forward and transposed) can be recorded into a CUDA graph
+ * after one product of as many right-hand sides (of the same precision for more than eight); a form
+ * whose scratch does not exist yet is then replaced by one without (the results differ by
+ * rounding).  The graph stays valid until a call on the handle with more right-hand sides than any
+ * before it, or fmbem_destroy. */
 fmbem_status fmbem_matvec(fmbem *h, const void *x_dev, void *y_dev, int64_t n_rhs, int precision, void *stream);
 
 /* The same product with x and y in HOST memory, the copies included: the right-hand sides are

@@ -164,7 +164,7 @@ fmbem_status fmbem_batch_create(fmbem *const *handles, int32_t n_problems, int64
         }
         b->n_items = (int64_t)items.size();
         for (fmbem *h : b->hs) {
-            batch_ensure_scratch(h, nr, precision);
+            batch_ensure_scratch(h, nr, precision, 0);
             b->p2max = std::max(b->p2max, h->p2);
         }
         b->hp.resize(n_problems);
@@ -204,7 +204,7 @@ fmbem_status fmbem_batch_matvec(fmbem_batch *b, const void *const *x_dev, void *
     try {
         // a handle used alone in between may have regrown its scratch: take its pointers now
         for (int32_t i = 0; i < n; ++i) {
-            batch_ensure_scratch(b->hs[i], b->nr, b->precision);
+            batch_ensure_scratch(b->hs[i], b->nr, b->precision, s);
             b->hp[i] = batch_problem(b->hs[i]);
             b->hp[i].x = (const c64 *)x_dev[i];
             b->hp[i].y = (c64 *)y_dev[i];

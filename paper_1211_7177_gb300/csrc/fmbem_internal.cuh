@@ -155,7 +155,7 @@ struct fmbem {
     int4 *near_ditems = nullptr;  // items of the double-precision near field (k_near_d): leaf, target offset, tg, nsl
     int n_near_ditems = 0;
     int64_t near_tiles_max = 0;   // 32-source tiles of the longest source list
-    c64 *near_am = nullptr, *near_part = nullptr;  // its per-source vectors and partial sums (scratch)
+    void *near_am = nullptr, *near_part = nullptr;  // its per-source vectors and partial sums (scratch)
     size_t near_am_bytes = 0, near_part_bytes = 0;
     int4 *near_groups = nullptr;  // target groups of the lane-per-RHS near field (leaf, target offset, count, -):
                                   // n_near_groups in leaf order, then the same sorted by pair work
@@ -243,6 +243,9 @@ struct fmbem {
 
     // scratch grown on demand
     int64_t scratch_rhs = 0;
+    bool capturing = false;        // this call is recorded into a CUDA graph: nothing can be allocated
+    bool graphs = false;           // a product of at most scratch_rhs right-hand sides was recorded
+    std::vector<void *> retired;   // scratch that such a graph may hold (grow_scratch)
     void *dens = nullptr;   // source densities
     void *Cexp = nullptr;   // multipole coefficients [J+1][nbox][3 n_rhs][p2]
     void *Dexp = nullptr;   // local coefficients
@@ -438,7 +441,7 @@ __host__ __device__ inline int batch_done_counter(int kind, int level, int lmax)
 void run_batch_kernel(int precision, const BatchProblem *probs, const BatchItem *items, int64_t n_items,
                       unsigned long long *next, unsigned *cnt, const unsigned *tgt, int *err, uint64_t wait_ns,
                       int stall_problem, int p2max, int64_t nr, cudaStream_t s);
-void batch_ensure_scratch(fmbem *h, int64_t nr, int precision);
+void batch_ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s);
 void build_near_singular(fmbem *h, const fmbem_mesh *mesh, cudaStream_t s);
 void apply_near_singular(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t s, bool transpose);
 void run_precond(fmbem *h, const c64 *v, c64 *z, int64_t n_rhs, cudaStream_t s);

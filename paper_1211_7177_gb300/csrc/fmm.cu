@@ -3228,6 +3228,7 @@ static bool ofs_applies(const fmbem *h, int64_t nr, int tensor_mode) {
 // launch), so the window is narrowed until they take at most 8 GB; at most as many columns as the
 // per-target reduction has threads for, in whole right-hand sides.
 // 0: not used (its images were not built, or the caller asked for a translation form).
+constexpr int64_t OZ_Y_BYTES = int64_t(8) << 30;
 template <typename R>
 static int oz_window(const fmbem *h, int64_t nr, int tensor_mode) {
     if (h->oz_img == nullptr || ofs_applies(h, nr, tensor_mode)) return 0;
@@ -3235,7 +3236,7 @@ static int oz_window(const fmbem *h, int64_t nr, int tensor_mode) {
     const int rows_pad = ((h->p2 + 31) / 32) * 32;
     int64_t most = std::min<int64_t>(48, 3 * (1024 / rows_pad));
     const int64_t per_col = (int64_t)sizeof(cx<R>) * (h->Jf + 1) * std::max<int64_t>(h->n_ff, 1) * h->p2;
-    most = std::max<int64_t>(3, std::min(most, (int64_t(8) << 30) / per_col) / 3 * 3);
+    most = std::max<int64_t>(3, std::min(most, OZ_Y_BYTES / per_col) / 3 * 3);
     const int64_t windows = (3 * nr + most - 1) / most, W = 3 * ((nr + windows - 1) / windows);
     // its row and result indices are 32-bit
     if ((h->Jf + 1) * h->nbox * W >= INT32_MAX || h->n_ff * W >= INT32_MAX) return 0;
@@ -3271,25 +3272,45 @@ static int near_ws_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_items * nr);
     return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * 152 + units - 1) / units}));
 }
+// Scratch that grows.  A CUDA graph captured from a product holds these buffers' addresses, so that one which is
+// outgrown after a capture stays allocated (retired) until a call with more right-hand sides than any before
+// replaces the densities and expansions, which every captured product reads as well, or the handle is
+// destroyed; it is then at least doubled, so that the retired ones take no more than the last.  A refused
+// allocation leaves the buffer as it was after a capture, and none otherwise.
+static const char *NO_ROOM_IN_CAPTURE =
+    "the product's scratch would have to grow during a stream capture: run one of as many right-hand sides before";
+static void grow_scratch(fmbem *h, void *&p, size_t &have, size_t need, size_t most = SIZE_MAX) {
+    if (p != nullptr && have >= need) return;
+    if (h->capturing) throw fmbem_error{FMBEM_ERR_OOM, NO_ROOM_IN_CAPTURE};
+    void *q = nullptr;
+    size_t size = need;
+    if (p != nullptr && h->graphs) {
+        const size_t twice = std::max(need, std::min(2 * have, most));
+        if (twice > need) try {
+                q = dev_alloc(h, twice);
+                size = twice;
+            } catch (const fmbem_error &e) {
+                if (e.st != FMBEM_ERR_OOM) throw;
+            }
+        if (q == nullptr) q = dev_alloc(h, need);
+        h->retired.push_back(p);
+    } else {
+        dev_free(h, p);
+        p = nullptr;
+        have = 0;
+        q = dev_alloc(h, need);
+    }
+    p = q;
+    have = size;
+}
+
 // the near field's partial sums (6 or 12 complex values of a node, right-hand side and split), and per-source
-// vectors of the FP64 forward product (row_bytes a node, right-hand side and split); without room for them the
-// forward product takes the kernels of the allocation-free one, and the transposed one keeps its sums in the result
+// vectors of the FP64 forward product (row_bytes a node, right-hand side and split); without room for them, or
+// where they would have to grow during a stream capture, the forward product takes the kernels of the
+// allocation-free one, and the transposed one keeps its sums in the result
 static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
-    const size_t npart = row_bytes * h->N * nr * nsp, nam = sizeof(c64) * 5 * h->N * nr;
-    if (h->near_part_bytes < npart) {
-        if (h->near_part) dev_free(h, h->near_part);
-        h->near_part = nullptr;
-        h->near_part_bytes = 0;
-        h->near_part = (c64 *)dev_alloc(h, npart);
-        h->near_part_bytes = npart;
-    }
-    if (am && h->near_am_bytes < nam) {
-        if (h->near_am) dev_free(h, h->near_am);
-        h->near_am = nullptr;
-        h->near_am_bytes = 0;
-        h->near_am = (c64 *)dev_alloc(h, nam);
-        h->near_am_bytes = nam;
-    }
+    grow_scratch(h, h->near_part, h->near_part_bytes, row_bytes * h->N * nr * nsp);
+    if (am) grow_scratch(h, h->near_am, h->near_am_bytes, sizeof(c64) * 5 * h->N * nr);
 }
 
 // they hold this call's: the partial sums of nsp splits, and the per-source vectors (am).  Both are looked at
@@ -3299,9 +3320,19 @@ static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, size_t row_b
            (!am || (h->near_am != nullptr && h->near_am_bytes >= sizeof(c64) * 5 * h->N * nr));
 }
 
-static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_results = true) {
+static void ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s, bool pair_results = true) {
     const size_t cb = sizeof(c64);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {  // (the legacy stream beside another one's capture)
+        cudaGetLastError();
+        cap = cudaStreamCaptureStatusNone;
+    }
+    h->capturing = cap != cudaStreamCaptureStatusNone;
     if (h->scratch_rhs < nr) {
+        if (h->capturing) throw fmbem_error{FMBEM_ERR_OOM, NO_ROOM_IN_CAPTURE};
+        for (void *p : h->retired) dev_free(h, p);
+        h->retired.clear();
+        h->graphs = false;
         // (a refused allocation leaves no freed buffer behind: the next call allocates what it needs)
         h->scratch_rhs = 0;
         for (void **p : {&h->dens, &h->Cexp, &h->Dexp}) {
@@ -3313,6 +3344,7 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
         h->Dexp = dev_alloc(h, cb * (size_t)(h->J + 1) * h->nbox * 3 * nr * h->p2);
         h->scratch_rhs = nr;
     }
+    h->graphs |= h->capturing;
     // per-pair M2L results of one level, one domain and up to 24 columns (chunked path only;
     // one column window of the FP64 rotation form for more columns); sized by the columns of
     // this call, so that a few-column call after a many-column one still takes the chunked path
@@ -3320,14 +3352,6 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
     const int mode = precision == FMBEM_BF16X3 ? 2 : precision == FMBEM_TF32 ? 1 : 0;
     const bool dbl = precision == FMBEM_FP64;
     if (!pair_results) return;
-    auto grow = [&](void *&p, size_t &have, size_t need) {
-        if (p != nullptr && have >= need) return;
-        if (p) dev_free(h, p);
-        p = nullptr;
-        have = 0;
-        p = dev_alloc(h, need);
-        have = need;
-    };
     const int ozw = dbl ? oz_window<double>(h, nr, 0) : oz_window<float>(h, nr, mode);
     if (ozw > 0) {
         // where the device has no room for the digits and a window's pair results (oz_refused: the least
@@ -3336,18 +3360,18 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, bool pair_result
         const size_t res = dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw);
         if (dig + res < h->oz_refused) {
             try {
-                grow(h->oz_dig, h->oz_dig_bytes, dig);
-                grow(h->ybuf, h->ybuf_bytes, res);
+                grow_scratch(h, h->oz_dig, h->oz_dig_bytes, dig);
+                grow_scratch(h, h->ybuf, h->ybuf_bytes, res, OZ_Y_BYTES);
             } catch (const fmbem_error &e) {
                 if (e.st != FMBEM_ERR_OOM) throw;
-                h->oz_refused = dig + res;
+                if (!h->capturing) h->oz_refused = dig + res;
             }
         }
     }
     if (3 * nr <= 24 || many) {
         size_t need = ybuf_need(h, many ? rot_many_cols(h) : 3 * nr, cb);
         if (ofs_applies(h, nr, mode)) need = std::max(need, ofs_ybuf_need(h, nr));
-        grow(h->ybuf, h->ybuf_bytes, need);
+        grow_scratch(h, h->ybuf, h->ybuf_bytes, need, OZ_Y_BYTES);
     }
 }
 
@@ -3854,14 +3878,14 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
             CK(cudaMemsetAsync(h->near_next, 0, sizeof(int), s));
             kern<<<(unsigned)grid, 32 * ND_WARPS, 0, s>>>(
                 h->leaf_box, h->near_ditems, h->n_near_ditems, (int)units, nsp, h->near_next, N, nr, h->box_nbeg,
-                h->box_nend, h->nbr_start, h->nbr_idx, h->pos, h->dom, dens, h->near_am, dc, h->near_base,
-                (const V4<double> *)h->near_cache64, h->near_part, !h->ibc);
+                h->box_nend, h->nbr_start, h->nbr_idx, h->pos, h->dom, dens, (const c64 *)h->near_am, dc, h->near_base,
+                (const V4<double> *)h->near_cache64, (c64 *)h->near_part, !h->ibc);
             CKL("k_near_d");
         };
         if (h->near_cache64) launch_d(k_near_d<true>);
         else launch_d(k_near_d<false>);
         k_near_finish<<<dim3(nblk(24 * N, 192), (unsigned)nr), 192, 0, s>>>(N, nr, nsp, p2, h->nbox, h->node_leaf, h->dom, h->perm,
-                                                                          Bl2p, D, h->Mself, x, h->near_part, y);
+                                                                          Bl2p, D, h->Mself, x, (const c64 *)h->near_part, y);
     } else if (nr >= 4) {  // the allocation-free product
         constexpr int RBLK = 2;
         const size_t smn = sizeof(NearSmemRB<R, RBLK>);
@@ -3967,7 +3991,7 @@ static void check_fp32_only(const fmbem *h, int precision) {
 void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaStream_t s) {
     check_fp32_only(h, precision);
     check_oz_err(h, s);
-    ensure_scratch(h, nr, precision);
+    ensure_scratch(h, nr, precision, s);
     try {
         const bool dbl = precision == FMBEM_FP64;
         ensure_near_scratch(h, nr, near_d_splits(h, dbl || nr == 1 ? nr : (nr + 2) / 3), 12 * (dbl ? sizeof(c64) : sizeof(c32)),
@@ -3989,7 +4013,7 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
 void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaStream_t s) {
     check_fp32_only(h, precision);
     check_oz_err(h, s);
-    ensure_scratch(h, nr, precision);
+    ensure_scratch(h, nr, precision, s);
     try {
         if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6 * sizeof(c64), true);
         else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6 * sizeof(c32), false);
@@ -4067,7 +4091,7 @@ static void matvec_static_scratch(fmbem *h, const c64 *x, c64 *y, int64_t nr, cu
     // run the regular passes on pointers into the static array; the handle's own scratch
     // pointers are restored afterwards, so fmbem_matvec is unaffected
     void *sv_dens = h->dens, *sv_C = h->Cexp, *sv_D = h->Dexp, *sv_y = h->ybuf, *sv_dig = h->oz_dig;
-    c64 *sv_am = h->near_am, *sv_part = h->near_part;
+    void *sv_am = h->near_am, *sv_part = h->near_part;
     const size_t sv_yb = h->ybuf_bytes;
     auto restore = [&] {
         h->dens = sv_dens; h->Cexp = sv_C; h->Dexp = sv_D; h->ybuf = sv_y; h->ybuf_bytes = sv_yb; h->oz_dig = sv_dig;
@@ -4120,4 +4144,4 @@ void run_batch_kernel(int precision, const BatchProblem *probs, const BatchItem 
 
 // scratch of a handle for an n_rhs product in the given precision (batch.cu): densities and
 // expansions only, the batch's dense translation items keep no per-pair results
-void batch_ensure_scratch(fmbem *h, int64_t nr, int precision) { ensure_scratch(h, nr, precision, false); }
+void batch_ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s) { ensure_scratch(h, nr, precision, s, false); }
