@@ -17,9 +17,7 @@ std::string cuda_msg(cudaError_t e, const char *what) {
 // negative: unlimited
 static std::atomic<int64_t> g_device_budget{-1};
 
-void *dev_alloc(fmbem *h, size_t bytes) {
-    void *p = nullptr;
-    if (bytes == 0) bytes = 16;
+static void charge_budget(size_t bytes) {
     for (int64_t left = g_device_budget.load(); left >= 0;) {
         if ((int64_t)bytes > left)
             throw fmbem_error{FMBEM_ERR_OOM, "device allocation of " + std::to_string(bytes) +
@@ -27,6 +25,12 @@ void *dev_alloc(fmbem *h, size_t bytes) {
                                                  " bytes left"};
         if (g_device_budget.compare_exchange_weak(left, left - (int64_t)bytes)) break;
     }
+}
+
+void *dev_alloc(fmbem *h, size_t bytes) {
+    void *p = nullptr;
+    if (bytes == 0) bytes = 16;
+    charge_budget(bytes);
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -44,6 +48,31 @@ void dev_free(fmbem *h, void *p) {
         h->allocations.pop_back();
     }
     cudaFree(p);
+}
+
+void dev_replace(fmbem *h, void *&p, size_t &have, size_t need) {
+    if (need > have) charge_budget(need - have);
+    const size_t old = have;
+    cudaFree(p);
+    have = 0;
+    cudaError_t e = cudaErrorMemoryAllocation;
+    void *q = nullptr;
+    for (const size_t size : {need, old}) {
+        const cudaError_t r = cudaMalloc(&q, size);
+        if (r == cudaSuccess) {
+            have = size;
+            break;
+        }
+        cudaGetLastError();
+        q = nullptr;
+        e = r;
+    }
+    auto it = std::find(h->allocations.begin(), h->allocations.end(), p);
+    if (q != nullptr) *it = q;
+    else h->allocations.erase(it);
+    p = q;
+    if (have != need)
+        throw fmbem_error{FMBEM_ERR_OOM, "cudaMalloc of " + std::to_string(need) + " bytes failed: " + cudaGetErrorString(e)};
 }
 
 static void free_all(fmbem *h) {

@@ -322,6 +322,10 @@ __host__ __device__ __forceinline__ int m2l_offset_code(int dx, int dy, int dz) 
 std::string cuda_msg(cudaError_t e, const char *what);
 void *dev_alloc(fmbem *h, size_t bytes);  // records the allocation; throws std::bad_alloc on failure
 void dev_free(fmbem *h, void *p);
+// an allocation of have bytes replaced by one of need bytes, its contents lost: freed first, so that the two need not
+// fit together, and allocated again as it was where the new size is refused (FMBEM_ERR_OOM; p is null, have 0,
+// where even that is)
+void dev_replace(fmbem *h, void *&p, size_t &have, size_t need);
 
 struct fmbem_error {
     fmbem_status st;

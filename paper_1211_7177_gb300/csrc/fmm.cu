@@ -3276,7 +3276,7 @@ static int near_ws_splits(const fmbem *h, int64_t nr) {
 // outgrown after a capture stays allocated (retired) until a call with more right-hand sides than any before
 // replaces the densities and expansions, which every captured product reads as well, or the handle is
 // destroyed; it is then at least doubled, so that the retired ones take no more than the last.  A refused
-// allocation leaves the buffer as it was after a capture, and none otherwise.
+// allocation leaves a buffer of the size that it had.
 static const char *NO_ROOM_IN_CAPTURE =
     "the product's scratch would have to grow during a stream capture: run one of as many right-hand sides before";
 static void grow_scratch(fmbem *h, void *&p, size_t &have, size_t need, size_t most = SIZE_MAX) {
@@ -3294,10 +3294,10 @@ static void grow_scratch(fmbem *h, void *&p, size_t &have, size_t need, size_t m
             }
         if (q == nullptr) q = dev_alloc(h, need);
         h->retired.push_back(p);
+    } else if (p != nullptr) {
+        dev_replace(h, p, have, need);
+        return;
     } else {
-        dev_free(h, p);
-        p = nullptr;
-        have = 0;
         q = dev_alloc(h, need);
     }
     p = q;
@@ -3355,16 +3355,37 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s, 
     const int ozw = dbl ? oz_window<double>(h, nr, 0) : oz_window<float>(h, nr, mode);
     if (ozw > 0) {
         // where the device has no room for the digits and a window's pair results (oz_refused: the least
-        // that was refused), the forms below remain
+        // that was refused, tried again when the device reports as much free), the forms below remain, and
+        // the digits are given back to them
         const size_t dig = dbl ? oz_digit_bytes<double>(h, ozw) : oz_digit_bytes<float>(h, ozw);
         const size_t res = dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw);
-        if (dig + res < h->oz_refused) {
+        bool room = !h->capturing && (h->oz_dig_bytes < dig || h->ybuf_bytes < res);
+        if (room && dig + res >= h->oz_refused) {
+            size_t free_b = 0, total_b = 0;
+            room = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b >= dig + res;
+        }
+        if (room) {
+            void *dig0 = h->oz_dig;
+            const size_t have0 = h->oz_dig_bytes, kept = h->retired.size();
             try {
                 grow_scratch(h, h->oz_dig, h->oz_dig_bytes, dig);
                 grow_scratch(h, h->ybuf, h->ybuf_bytes, res, OZ_Y_BYTES);
+                h->oz_refused = ~size_t(0);
             } catch (const fmbem_error &e) {
                 if (e.st != FMBEM_ERR_OOM) throw;
-                if (!h->capturing) h->oz_refused = dig + res;
+                h->oz_refused = std::min(h->oz_refused, dig + res);
+                if (h->retired.size() > kept) {  // a graph may hold the digits that these replaced
+                    dev_free(h, h->oz_dig);
+                    h->oz_dig = dig0;
+                    h->oz_dig_bytes = have0;
+                    h->retired.resize(kept);
+                } else if (have0 > 0 && h->oz_dig_bytes > have0) {
+                    dev_replace(h, h->oz_dig, h->oz_dig_bytes, have0);
+                } else if (have0 == 0) {
+                    dev_free(h, h->oz_dig);
+                    h->oz_dig = nullptr;
+                    h->oz_dig_bytes = 0;
+                }
             }
         }
     }

@@ -101,3 +101,40 @@ def test_transposed_without_room(mesh, opt, n_rhs, precision, tol):
         lib.fmbem_debug_set_device_budget(-1)
     for r in range(n_rhs):
         assert float((y[r] - z[r]).norm()) < tol * float(z[r].norm())
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("n_rhs", [1, 3, 9])
+@pytest.mark.parametrize("call", ["matvec", "adjoint_matvec"])
+def test_part_of_the_room(call, n_rhs, captured):
+    """Room for some of the optional scratch only, in steps of two: every product runs, in some form, and once
+    there is room again in its usual one (the same bits as a handle that never lacked it)."""
+    V, F, D = fi.torus(1.0, 0.25, 61, 19)
+    lib = fm.load_library()
+    a = fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j], [1.0, 1.0], 1.5, p=8, leaf_size=16)
+    x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=n_rhs)).cuda()
+    z = getattr(a, call)(x)
+    for k in range(14, 29, 2):
+        b = fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j], [1.0, 1.0], 1.5, p=8, leaf_size=16)
+        y32 = b.matvec(x, precision=fm.FP32)
+        if captured:
+            out = torch.zeros_like(x)
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                b.matvec(x, out, precision=fm.FP32)
+        lib.fmbem_debug_set_device_budget(1 << k)
+        try:
+            y, again = getattr(b, call)(x), getattr(b, call)(x)
+            short = b.matvec(x, precision=fm.FP32)
+        finally:
+            lib.fmbem_debug_set_device_budget(-1)
+        assert torch.equal(short, y32)
+        for v in (y, again):
+            assert float((v - z).norm()) < 1e-13 * float(z.norm())
+        assert torch.equal(getattr(b, call)(x), z)
+        if captured:
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, y32)
+        b.close()
