@@ -2070,7 +2070,7 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
 constexpr int NR_TT = 8;   // targets per unit
 constexpr int NR_WARPS = 4;
 struct RhsTile {
-    // (r_x, r_y, -c_0), (r_z, 0, g_0), (c_1, -gamma g_1) per target and source
+    // (r_x, r_y, -c_0), (r_z, 1 in the target's scatterer, g_0), (c_1, -gamma g_1) per target and source
     float4 ps[NR_TT][32 * 3 + 1];
     float4 tp[NR_TT][2];      // target position hi + scatterer id bits, position lo
     float4 tk[NR_TT];         // the target's scatterer wavenumber k_j and -gamma_j
@@ -2167,22 +2167,25 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     cx<float> g0, c0, g1 = {0, 0}, c1 = {0, 0};
                     pair_scalars<float>(inv, Rr, k0, g0, c0);
                     if (!valid) g0 = c0 = cx<float>{0.f, 0.f};
-                    if (side1 && valid && sdom == __float_as_int(ta.w)) {
+                    const bool own = side1 && valid && sdom == __float_as_int(ta.w);
+                    if (own) {
                         const float4 tk = S.tk[t];
                         pair_scalars<float>(inv, Rr, cx<float>{tk.x, tk.y}, g1, c1);
                         g1 = cx<float>{tk.z, tk.w} * g1;  // -gamma_j g_1: q_1 = -gamma_j q_0
                     }
                     S.ps[t][3 * lane] = make_float4(rv[0], rv[1], -c0.re, -c0.im);
-                    S.ps[t][3 * lane + 1] = make_float4(rv[2], 0.f, g0.re, g0.im);
+                    S.ps[t][3 * lane + 1] = make_float4(rv[2], own ? 1.f : 0.f, g0.re, g0.im);
                     S.ps[t][3 * lane + 2] = make_float4(c1.re, c1.im, g1.re, g1.im);
                 }
             }
             __syncwarp();
             // right-hand-side phase
-            // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero)
+            // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero, and
+            // so are the densities, which need not be finite where they are stored)
             const int nsv = min(32, (nsrc - s0 + NSL - 1) / NSL * NSL);
             int ic = __shfl_sync(0xffffffffu, i, sl);
             float4 d0 = dl[st * ic], d1 = dl[st * ic + wd], d2 = dl[st * ic + 2 * wd], d3 = dl[st * ic + 3 * wd];
+            if (W < 32 && sl >= nsrc - s0) d0 = d1 = d2 = d3 = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int v0 = 0; v0 < nsv; v0 += NSL) {
                 const int sv = v0 + sl;
                 float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
@@ -2192,6 +2195,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     n1 = dl[st * in + wd];
                     n2 = dl[st * in + 2 * wd];
                     n3 = dl[st * in + 3 * wd];
+                    if (W < 32 && sv + NSL >= nsrc - s0) n0 = n1 = n2 = n3 = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
                 const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
                 const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
@@ -2211,7 +2215,9 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                             cfma(acc0[t][c], mc0, U[c]);
                             cfma(acc0[t][c], g0, q[c]);
                         }
-                        if (side1) {
+                        // (a source of another scatterer is left out where it need not be finite: a block of 32
+                        // multiplies it by zero scalars)
+                        if (side1 && (W == 32 || p1.y != 0.f)) {
                             const float4 p2v = S.ps[t][3 * sv + 2];
                             const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
                             U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};

@@ -49,3 +49,20 @@ def test_static_scratch(n_rhs):
     x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=n_rhs)).cuda()
     y = fm.fmbem_matvec_noalloc(a.h, x, torch.empty_like(x), fm.FP32)
     check(y, a.matvec(x), 2e-6)
+
+
+@pytest.mark.parametrize("n_rhs", [1, 3, 4, 5, 8, 9, 12, 20, 31])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_nonfinite_unknowns_of_another_scatterer(bad, n_rhs):
+    """The scatterer rows (3 to 5) of a node sum over its own scatterer: non-finite unknowns of the other one
+    leave them as they are, in every form of the near field below 32 right-hand sides."""
+    V, F, D = fi.merge_meshes(fi.torus(1.0, 0.25, 60, 18, domain=1), fi.icosphere(2, 0.1, (1.0, 0.0, 0.37), domain=2))
+    a = fm.FMBEM(V, F, D, [1.0, -8.5 + 0.3j, 2.25], [1.0] * 3, 1.5, p=8, leaf_size=40)
+    other = torch.zeros(a.N, dtype=torch.bool, device="cuda")
+    other[torch.from_numpy(F[D == 2].ravel()).long().cuda()] = True
+    x = torch.from_numpy(fi.random_complex((n_rhs, a.N, 6), seed=n_rhs)).cuda()
+    x[:, other] = 0
+    z = a.matvec(x, precision=fm.FP32)
+    x[:, other] = bad
+    y = a.matvec(x, precision=fm.FP32)
+    assert torch.equal(y[:, ~other, 3:], z[:, ~other, 3:])
