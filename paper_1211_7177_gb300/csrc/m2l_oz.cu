@@ -503,7 +503,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
         bool ok = true;
         int u = 0, nt = 0;
-        for (int v = blockIdx.x; v < nunit && ok && !s_abort; v += gridDim.x) {
+        for (int v = blockIdx.x; v < nunit && ok; v += gridDim.x) {
+            // (one answer for the whole warp: the flag may be raised between two lanes' reads of it)
+            if (__any_sync(0xffffffffu, s_abort)) break;
             const OzTile t = oz_tile<R>(P, v, ntile, first, group);
             const uint32_t idesc = idesc_bf16((t.n + 15) & ~15);
             if (nt > 0) ok = __all_sync(0xffffffffu, mbar_wait(&tfree, (uint32_t)(nt - 1) & 1u));
