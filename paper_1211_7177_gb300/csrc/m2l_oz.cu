@@ -419,6 +419,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
     const int ntile = first[P.ngroup], nunit = ntile * P.ndom * P.mt;
+    int last = -1;  // a producer warp's last K block
 
     if (warp < OZ_FILL) {
         // ------------------------------------------------------------------ producers
@@ -437,7 +438,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             t = oz_tile<R>(P, blockIdx.x, ntile, first, group);
             sources(t, src);
         }
-        int u = 0, turn = 0, last = -1;  // K blocks of the CTA's sequence, u mod OZ_FILL, this warp's last
+        int u = 0, turn = 0;  // K blocks of the CTA's sequence, u mod OZ_FILL
         bool stop = false;
         for (int v = blockIdx.x; v < nunit && !stop; v += gridDim.x) {
             __syncwarp();
@@ -492,8 +493,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 last = u;
             }
         }
-        // after an abort: wait (bounded) for this warp's last bulk copy
-        if (lane == 0 && s_abort && last >= 0 && !mbar_wait(&full[last & 3], (uint32_t)(last >> 2) & 1u)) give_up();
     } else if (warp == OZ_FILL) {
         // ------------------------------------------------------------------ MMA issuer
         // the whole warp runs the loop, so that descriptors stay in uniform registers (issued by one
@@ -635,6 +634,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
     __syncwarp();
     __syncthreads();
+    // After an abort (which any warp may have raised, also after the producers were through) no bulk copy may be in
+    // flight when the CTA ends: wait (bounded) for each producer warp's last two.  Those before them have landed, as
+    // the last one's slot was free only after the MMAs of the K block OZ_SLOTS earlier.
+    if (warp < OZ_FILL && lane == 0 && s_abort)
+        for (int u = max(last - OZ_FILL, last % OZ_FILL); u >= 0 && u <= last; u += OZ_FILL)
+            if (!mbar_wait(&full[u & 3], (uint32_t)(u >> 2) & 1u)) give_up();
     if (threadIdx.x == 0 && !mbar_wait(&fin, 0)) give_up();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
