@@ -192,6 +192,11 @@ void fmbem_debug_set_device_budget(int64_t bytes);
 
 typedef struct fmbem fmbem;  /* opaque handle */
 
+/* Fault injection for tests of the tensor-core kernels' bounded waits: leaves the handle as if a wait of an
+ * earlier kernel of its next product had run out, so that the product's tensor-core kernels give up
+ * at once and it reports FMBEM_ERR_DEVICE_TIMEOUT. */
+fmbem_status fmbem_debug_raise_wait_timeout(fmbem *h);
+
 /* Builds everything that depends on geometry and frequency, Sections 2.1-2.2 and Appendices
  * B-C: nodes, weights and normals (Eq. 2.8); the self-patch integrals of Appendix B (Eqs.
  * B.2-B.9) on a planar patch around each node -- the triangle itself for CENTROID nodes, the

@@ -71,6 +71,7 @@ def load_library(build_if_missing: bool = True):
     sig = {
         "fmbem_default_options": (None, [ctypes.POINTER(Options)]),
         "fmbem_debug_set_device_budget": (None, [i64]),
+        "fmbem_debug_raise_wait_timeout": (i32, [P]),
         "fmbem_create": (i32, [ctypes.POINTER(Mesh), P, P, dbl, ctypes.POINTER(Options), P, ctypes.POINTER(P)]),
         "fmbem_destroy": (None, [P]),
         "fmbem_last_error": (ctypes.c_char_p, [P]),

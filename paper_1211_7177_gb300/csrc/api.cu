@@ -137,6 +137,17 @@ extern "C" {
 
 void fmbem_debug_set_device_budget(int64_t bytes) { g_device_budget.store(bytes < 0 ? -1 : bytes); }
 
+fmbem_status fmbem_debug_raise_wait_timeout(fmbem *h) {
+    if (!h) return FMBEM_ERR_INVALID_ARGUMENT;
+    return guarded(h, [&] {
+        for (fmbem *q : {h, h->eps_plus, h->eps_minus})
+            if (q && q->tc_err) {
+                const int one = 1;
+                CK(cudaMemcpy(q->tc_err, &one, sizeof(int), cudaMemcpyHostToDevice));
+            }
+    });
+}
+
 void fmbem_default_options(fmbem_options *o) {
     if (!o) return;
     o->node_mode = FMBEM_NODES_VERTEX;

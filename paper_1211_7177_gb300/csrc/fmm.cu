@@ -4004,6 +4004,7 @@ static void check_tc_err(fmbem *h, cudaStream_t s) {
     CK(cudaStreamSynchronize(s));
     if (e) {
         CK(cudaMemsetAsync(h->tc_err, 0, sizeof(int), s));
+        if (h->oz_err_host) *(volatile int *)h->oz_err_host = 0;  // raised by the same wait: reported here
         throw fmbem_error{FMBEM_ERR_DEVICE_TIMEOUT, "tensor-core M2L: an mbarrier wait timed out"};
     }
 }
