@@ -55,7 +55,10 @@ typedef enum {
     FMBEM_ERR_DEVICE_TIMEOUT = 7    /* a bounded wait inside a kernel ran out (a pipeline stage
                                        or a work item never became ready); the kernel stopped,
                                        released what it held and returned, the context stays
-                                       usable and the call's outputs are undefined              */
+                                       usable and the call's outputs are undefined.  FP64 and FP32
+                                       products do not wait for the device: all rows of such a
+                                       product become NaN, and a later call on the handle returns
+                                       this status instead of starting                          */
 } fmbem_status;
 
 typedef enum { FMBEM_NODES_VERTEX = 0, FMBEM_NODES_CENTROID = 1 } fmbem_node_mode;

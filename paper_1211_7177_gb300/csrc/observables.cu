@@ -730,6 +730,7 @@ void run_near_field_fmm(fmbem *h, const c64 *x, int64_t nr, int64_t n_pts, const
         CK(cudaMemcpyAsync(E_host, dE, sizeof(c64) * 3 * n_pts * nr, cudaMemcpyDeviceToHost, s));
         if (dH) CK(cudaMemcpyAsync(H_host, dH, sizeof(c64) * 3 * n_pts * nr, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        check_oz_err(h, s);  // a wait of the product that ran out
     } catch (...) {
         cleanup();
         throw;
@@ -1010,6 +1011,13 @@ void run_eps_sensitivity(fmbem *h, int j, const c64 *x, const c64 *lam, int64_t 
         CKL("k_bilinear");
         CK(cudaMemcpyAsync(out_host, dout, sizeof(c64) * nr, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        bool out = false;  // a wait of either product that ran out: both flags are reset, one error reported
+        for (fmbem *q : {h->eps_plus, h->eps_minus}) try {
+                check_oz_err(q, s);
+            } catch (const fmbem_error &) {
+                out = true;
+            }
+        if (out) throw fmbem_error{FMBEM_ERR_DEVICE_TIMEOUT, "perturbed operator: a wait of a tensor-core kernel ran out"};
     } catch (...) {
         cleanup();
         throw;

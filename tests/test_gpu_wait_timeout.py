@@ -50,3 +50,24 @@ def test_solve(opt):
         h.solve(b, tol=1e-4)
     assert e.value.status == TIMEOUT
     assert torch.equal(h.solve(b, tol=1e-4)[0], x)
+
+
+def test_calls_that_return_host_results():
+    """They wait for their products and report what happened to them."""
+    h = handle()
+    x = torch.from_numpy(fi.random_complex((1, h.N, 6), seed=1)).cuda()
+    pts = [[0.0, 0.0, 2.0], [2.0, 0.5, 0.0]]
+    calls = [lambda: h.near_field(x, pts, fmm=True), lambda: h.eps_sensitivity(1, x, x)]
+    for call in calls:
+        want = torch.as_tensor(call())
+        raise_timeout(h)
+        with pytest.raises(fm.FMBEMError) as e:
+            call()
+        assert e.value.status == TIMEOUT
+        assert torch.equal(torch.as_tensor(call()), want)
+        # (the flag that the other call's handles had: theirs is not this one's)
+        for other in calls:
+            try:
+                other()
+            except fm.FMBEMError as e2:
+                assert other is not call and e2.status == TIMEOUT
