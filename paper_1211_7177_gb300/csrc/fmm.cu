@@ -959,7 +959,8 @@ __global__ void __launch_bounds__(32 * ROTC_WARPS) k_m2l_rot_cols(
 // Threads: rows_pad x ct column groups x NG pair groups; a thread owns columns cid * L2L_CPT .. + L2L_CPT - 1
 // and, with few columns, a quarter of the pairs (and of the dense R|R's inputs), the quarters added in order
 // through shared memory: a box has up to 189 pairs, whose results one thread read one after the other (FP64,
-// 642 nodes: 32 us for one level of 56 boxes).
+// 642 nodes: 32 us for one level of 56 boxes).  Column groups beyond 1024 threads (p >= 12 and 7 or more
+// right-hand sides) go to grid.z.
 constexpr int L2L_CPT = 3;
 constexpr int L2L_GROUPS = 4;
 template <typename R, int NG>
@@ -978,15 +979,17 @@ __global__ void __launch_bounds__(1024)
     const int nt = rows_pad * ct, grp = NG == 1 ? 0 : threadIdx.x / nt;
     const int r = threadIdx.x % rows_pad, cid = (NG == 1 ? threadIdx.x : threadIdx.x % nt) / rows_pad;
     const cx<R> *T = nullptr;
+    // the block's columns (all of them where they are few)
+    const int cb = NG == 1 ? blockIdx.z * ct * L2L_CPT : 0, ncb = NG == 1 ? min(ncol - cb, ct * L2L_CPT) : ncol;
     if (l >= 3 && Yll == nullptr) {
         const int64_t P = parent[g];
-        for (int e = threadIdx.x; e < ncol * p2; e += blockDim.x)
-            X[e] = D[(((int64_t)d * nbox + P) * 3 * nr + col0 + e / p2) * p2 + e % p2];
+        for (int e = threadIdx.x; e < ncb * p2; e += blockDim.x)
+            X[e] = D[(((int64_t)d * nbox + P) * 3 * nr + col0 + cb + e / p2) * p2 + e % p2];
         T = Tll + oct_matrix(d, l, (int)(key[g] & 7), lmax) * p2 * p2;
         __syncthreads();
     }
     // this thread's columns c0 .. c0 + L2L_CPT - 1: one read of T per row k feeds all of them
-    const int c0 = cid * L2L_CPT;
+    const int c0 = cb + cid * L2L_CPT;
     cx<R> sum[L2L_CPT];
 #pragma unroll
     for (int j = 0; j < L2L_CPT; ++j) sum[j] = {0, 0};
@@ -998,7 +1001,7 @@ __global__ void __launch_bounds__(1024)
                 const cx<R> t = T[(int64_t)k * p2 + r];
 #pragma unroll
                 for (int j = 0; j < L2L_CPT; ++j)
-                    if (c0 + j < ncol) cfma(sum[j], t, X[(c0 + j) * p2 + k]);
+                    if (c0 + j < ncol) cfma(sum[j], t, X[(c0 - cb + j) * p2 + k]);
             }
         if (l >= 3 && Yll != nullptr && grp == 0) {  // R|R already applied in rotation form, per child entry
             const cx<R> *yl = Yll + ((int64_t)(ll_entry[g] - ll_first) * ncol) * p2 + r;
@@ -1025,7 +1028,7 @@ __global__ void __launch_bounds__(1024)
         }
     }
     if (NG > 1) {
-        cx<R> *S = X + (T ? ncol * p2 : 0);  // [group][L2L_CPT][rows_pad ct]
+        cx<R> *S = X + (T ? ncb * p2 : 0);  // [group][L2L_CPT][rows_pad ct]
         if (grp > 0)
 #pragma unroll
             for (int j = 0; j < L2L_CPT; ++j) S[((grp - 1) * L2L_CPT + j) * nt + threadIdx.x % nt] = sum[j];
@@ -3668,13 +3671,13 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                     CK(cudaStreamWaitEvent(s, h->ev_join, 0));
                 }
                 cudaStream_t sr = overlap && l < lmax ? h->aux_stream : s;  // this level's reduction
-                const int ct = (nc + L2L_CPT - 1) / L2L_CPT;
+                const int groups = (nc + L2L_CPT - 1) / L2L_CPT, ct = std::min(groups, 1024 / rows_pad);
                 // pair groups where the boxes do not fill the chip (3384 boxes in two domains, FP64: 690 us with
                 // one group, 1016 with four), and none on the few SMs that the BF16x3 overlap leaves
                 const bool one = Lv.n * (J + 1) >= 512 || (overlap && l < lmax) || rows_pad * ct * L2L_GROUPS > 512;
-                const size_t smr = sizeof(cx<R>) * ((l >= 3 && Yll == nullptr ? (size_t)nc * p2 : 0) +
+                const size_t smr = sizeof(cx<R>) * ((l >= 3 && Yll == nullptr ? (size_t)std::min(nc, ct * L2L_CPT) * p2 : 0) +
                                                     (one ? 0 : (size_t)(L2L_GROUPS - 1) * L2L_CPT * rows_pad * ct));
-                const dim3 rgrid((unsigned)Lv.n, (unsigned)(J + 1));
+                const dim3 rgrid((unsigned)Lv.n, (unsigned)(J + 1), (unsigned)((groups + ct - 1) / ct));
                 if (one)
                     k_l2l_reduce<R, 1><<<rgrid, rows_pad * ct, smr, sr>>>(
                         Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent, h->box_key, h->ff_start,
