@@ -2503,7 +2503,9 @@ __global__ void k_p2m_adj(const int32_t *leaf_box, int64_t N, int64_t nr, int p2
 // The transposed near field by warps, both sides of every pair in one pass (the units, slices and splits of
 // k_near_d).  With w = r x n, r = s_a - s_b and n the target's normal, the three gradient terms of u above
 // are, per source and side, +-c B(x), B(x) = x x w - (n.r) x (the target sees -n on the background side), so
-// a pair keeps 3 + 3 sums per side instead of the 3 + 9 of phi and grad phi, and geometry, w and, in single
+// a pair keeps 3 + 3 sums per side instead of the 3 + 9 of phi and grad phi (in single precision u is then summed
+// from rounded c B, where u used to be formed in double from the nine rounded sums: error of a product against FP64
+// 1.8e-7 -> 1.3e-7, the nine sums being larger than u), and geometry, w and, in single
 // precision, the pair scalars of RB right-hand sides are formed once.  Partial sums (u near, phi near of both
 // sides) go to part[split][r][node][12]; k_near_adj_finish adds them, the far field and the self block.  Without
 // that scratch (part null, one split) u goes to the result's own rows and phi to the components 3 to 5 of the
@@ -2673,9 +2675,10 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
 }
 
 // assembly of k_near_adj's partial sums: eight lanes per (node, right-hand side), four per side; each sums a
-// quarter of the far field (L2P of phi and grad phi) of its side's domain, then in double precision
-// u far + u near, T_d, the weights, and the transposed self block, a lane per component of u and phi and then
-// per row (each lane with all six: single precision, 17026 nodes x 3 RHS 163 us, the FP64 pipe; now 100)
+// quarter of the far field (L2P of phi and grad phi) of its side's domain in the working precision, then in double
+// precision u far from grad phi, u far + u near, T_d, the weights, and the transposed self block, a lane per
+// component of u and phi and then per row (each lane with all six: single precision, 17026 nodes x 3 RHS 163 us,
+// the FP64 pipe; now 100)
 template <typename R>
 __global__ void __launch_bounds__(128) k_near_adj_finish(
     int64_t N, int64_t nr, int nsp, int p2, int64_t nbox, const int32_t *__restrict__ node_leaf,
@@ -2707,29 +2710,49 @@ __global__ void __launch_bounds__(128) k_near_adj_finish(
             cfma(fg[2][c], dq, gz);
         }
     }
-    // the far u of this quarter (linear in grad phi), then phi and u summed over the quarters
-    const R sg = side == 0 ? (R)-1 : (R)1;
-    const R n1[3] = {sg * (R)nrm[3 * a], sg * (R)nrm[3 * a + 1], sg * (R)nrm[3 * a + 2]};
-    const cx<R> div = fg[0][0] + fg[1][1] + fg[2][2];
-    // (lane qpart < 3 of a side goes on with component qpart: FP64 instructions are what the rest costs)
-    c64 u = {0, 0}, ph = {0, 0};
-    const int cc = min(qpart, 2);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        cx<R> v = n1[c] * div;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v += n1[i] * (fg[i][c] - fg[c][i]);
+    // phi and u = n div + (n_i d_i) phi - n_i grad phi_i of the far field: in double from this quarter's sums, then
+    // summed over the quarters; in single precision the quarters are summed first, and u is formed from them in double
+    const auto quarters = [](cx<R> &v) {
 #pragma unroll
         for (int o = 2; o > 0; o >>= 1) {
             v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
             v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
-            fp[c].re += __shfl_xor_sync(0xffffffffu, fp[c].re, o);
-            fp[c].im += __shfl_xor_sync(0xffffffffu, fp[c].im, o);
         }
-        if (cc == c) {
-            u = {(double)v.re, (double)v.im};
-            ph = {(double)fp[c].re, (double)fp[c].im};
+    };
+    // (lane qpart < 3 of a side goes on with component cc = qpart: FP64 instructions are what the rest costs)
+    const int cc = min(qpart, 2);
+    c64 u = {0, 0}, ph = {0, 0};
+    if constexpr (sizeof(R) == 8) {
+        const R sg = side == 0 ? (R)-1 : (R)1;
+        const R n1[3] = {sg * (R)nrm[3 * a], sg * (R)nrm[3 * a + 1], sg * (R)nrm[3 * a + 2]};
+        const cx<R> div = fg[0][0] + fg[1][1] + fg[2][2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            cx<R> v = n1[c] * div;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) v += n1[i] * (fg[i][c] - fg[c][i]);
+            quarters(v);
+            quarters(fp[c]);
+            if (cc == c) {
+                u = v;
+                ph = fp[c];
+            }
         }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            quarters(fp[c]);
+#pragma unroll
+            for (int kk = 0; kk < 3; ++kk) quarters(fg[kk][c]);
+        }
+        const auto wide = [](cx<R> v) { return c64{(double)v.re, (double)v.im}; };
+        const auto pick = [=](cx<R> v0, cx<R> v1, cx<R> v2) { return wide(cc == 0 ? v0 : cc == 1 ? v1 : v2); };
+        const int ci = (cc + 1) % 3, cj = (cc + 2) % 3;
+        ph = pick(fp[0], fp[1], fp[2]);
+        u = nrm[3 * a + cc] * (wide(fg[0][0]) + wide(fg[1][1]) + wide(fg[2][2]));
+        u += nrm[3 * a + ci] * (pick(fg[1][0], fg[2][1], fg[0][2]) - pick(fg[0][1], fg[1][2], fg[2][0]));
+        u += nrm[3 * a + cj] * (pick(fg[2][0], fg[0][1], fg[1][2]) - pick(fg[0][2], fg[1][0], fg[2][1]));
+        if (side == 0) u = -u;
     }
     if (part) {
         for (int s = 0; s < nsp; ++s) {
