@@ -2508,7 +2508,7 @@ __global__ void k_p2m_adj(const int32_t *leaf_box, int64_t N, int64_t nr, int p2
 // 1.8e-7 -> 1.3e-7, the nine sums being larger than u), and geometry, w and, in single
 // precision, the pair scalars of RB right-hand sides are formed once.  Partial sums (u near, phi near of both
 // sides) go to part[split][r][node][12]; k_near_adj_finish adds them, the far field and the self block.  Without
-// that scratch (part null, one split) u goes to the result's own rows and phi to the components 3 to 5 of the
+// that scratch (PART false, one split) u goes to the result's own rows and phi to the components 3 to 5 of the
 // densities (slots), which k_prep_adj leaves unused.
 // A block per leaf, right-hand side and side before, L2P by one thread per target: 17026 nodes x 3 RHS in
 // single precision 915 us, 10242 nodes in double 2865 us.
@@ -2517,7 +2517,7 @@ struct AdjTile {  // 32 sources: position (high part) and scatterer, low part, x
     V4<R> pa[32], pb[32];
     V2<R> x[RB][2][3][32];
 };
-template <typename R, bool CACHED, int RB>
+template <typename R, bool CACHED, int RB, bool PART>
 __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
     const int32_t *__restrict__ leaf_box, const int4 *__restrict__ items, int n_items, int n_units, int nsp, int nrb,
     int *next_unit, int64_t N, int64_t nr, const int32_t *__restrict__ nbeg, const int32_t *__restrict__ nend,
@@ -2663,11 +2663,14 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
                     const int tt = o / HALF, j = o - tt * HALF;
                     cx<R> v = S[j * 32 + tt];
                     for (int k = 1; k < nsl; ++k) v += S[j * 32 + k * tg + tt];
-                    const int row = h0 + j, sd = row / 6, c = row % 6;
-                    const int64_t b = t0 + it.y + tt, r = r0 + rr;
-                    if (part) part[((sp * nr + r) * N + b) * 12 + row] = v;
-                    else if (c < 3) y[(r * N + perm[b]) * 6 + 3 * sd + c] = c64{(double)v.re, (double)v.im};
-                    else slots[((sd * nr + r) * N + b) * 6 + c] = v;
+                    if constexpr (PART) {
+                        part[(((int64_t)sp * nr + r0 + rr) * N + t0 + it.y + tt) * 12 + h0 + j] = v;
+                    } else {
+                        const int row = h0 + j, sd = row / 6, c = row % 6;
+                        const int64_t b = t0 + it.y + tt, r = r0 + rr;
+                        if (c < 3) y[(r * N + perm[b]) * 6 + 3 * sd + c] = c64{(double)v.re, (double)v.im};
+                        else slots[((sd * nr + r) * N + b) * 6 + c] = v;
+                    }
                 }
             }
         }
@@ -3989,9 +3992,10 @@ static void adjoint_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_
     int dev = 0, nsm = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    auto launch_adj = [&](auto kern, int rb) {
-        const int64_t nrb = (nr + rb - 1) / rb;
-        const bool held = near_scratch_holds(h, nr, near_d_splits(h, nrb), 12 * sizeof(cx<R>), false);
+    const int rb = f32 && nr > 1 ? 3 : 1;  // right-hand sides that share the pair scalars in single precision
+    const int64_t nrb = (nr + rb - 1) / rb;
+    const bool held = near_scratch_holds(h, nr, near_d_splits(h, nrb), 12 * sizeof(cx<R>), false);
+    auto launch_adj = [&](auto kern) {
         const int nsp = held ? near_d_splits(h, nrb) : 1;
         cx<R> *part = held ? (cx<R> *)h->near_part : nullptr;
         const int64_t units = (int64_t)h->n_near_ditems * nrb * nsp;
@@ -4010,14 +4014,18 @@ static void adjoint_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_
             N, nr, nsp, p2, h->nbox, h->node_leaf, h->nrm, h->w, h->dom, h->perm, dc, Bl2p, Bl2pg, D, h->Mself, x,
             part, dens, y);
     };
-    if constexpr (sizeof(R) == 4) {  // three right-hand sides share the pair scalars
-        if (nr == 1) launch_adj(k_near_adj<R, false, 1>, 1);
-        else launch_adj(k_near_adj<R, false, 3>, 3);
-    } else if (h->near_cache64) {
-        launch_adj(k_near_adj<R, true, 1>, 1);
-    } else {
-        launch_adj(k_near_adj<R, false, 1>, 1);
-    }
+    auto with_scratch = [&](auto PART) {
+        if constexpr (sizeof(R) == 4) {
+            if (rb == 1) launch_adj(k_near_adj<R, false, 1, PART.value>);
+            else launch_adj(k_near_adj<R, false, 3, PART.value>);
+        } else if (h->near_cache64) {
+            launch_adj(k_near_adj<R, true, 1, PART.value>);
+        } else {
+            launch_adj(k_near_adj<R, false, 1, PART.value>);
+        }
+    };
+    if (held) with_scratch(std::true_type{});
+    else with_scratch(std::false_type{});
     CKL("k_near_adj");
     apply_near_singular(h, x, y, nr, s, true);  // transposed near-singular pair corrections (option)
 }
