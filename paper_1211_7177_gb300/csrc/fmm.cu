@@ -2158,6 +2158,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             }
             const float4 pa = rec[3 * i], pb = rec[3 * i + 1];
             const int sdom = __float_as_int(pa.w);
+            bool foreign = false;  // a source that some target's scatterer side leaves out
 #pragma unroll 2
             for (int t = 0; t < ntg; ++t) {
                 {
@@ -2171,6 +2172,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     pair_scalars<float>(inv, Rr, k0, g0, c0);
                     if (!valid) g0 = c0 = cx<float>{0.f, 0.f};
                     const bool own = side1 && valid && sdom == __float_as_int(ta.w);
+                    foreign |= sdom != __float_as_int(ta.w);
                     if (own) {
                         const float4 tk = S.tk[t];
                         pair_scalars<float>(inv, Rr, cx<float>{tk.x, tk.y}, g1, c1);
@@ -2183,59 +2185,61 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             }
             __syncwarp();
             // right-hand-side phase
-            // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero, and
-            // so are the densities, which need not be finite where they are stored)
+            // (W < 32: slices of a quarter or an eighth of the tile; past the list's end the scalars are zero)
             const int nsv = min(32, (nsrc - s0 + NSL - 1) / NSL * NSL);
             int ic = __shfl_sync(0xffffffffu, i, sl);
             float4 d0 = dl[st * ic], d1 = dl[st * ic + wd], d2 = dl[st * ic + 2 * wd], d3 = dl[st * ic + 3 * wd];
-            if (W < 32 && sl >= nsrc - s0) d0 = d1 = d2 = d3 = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int v0 = 0; v0 < nsv; v0 += NSL) {
-                const int sv = v0 + sl;
-                float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
-                const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
-                if (v0 + NSL < nsv) {
-                    n0 = dl[st * in];
-                    n1 = dl[st * in + wd];
-                    n2 = dl[st * in + 2 * wd];
-                    n3 = dl[st * in + 3 * wd];
-                    if (W < 32 && sv + NSL >= nsrc - s0) n0 = n1 = n2 = n3 = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
-                const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
-                const float2 sj = {d3.z, d3.w};
+            // PICK: sources of another scatterer are left out of the scatterer side, where they need not be finite;
+            // without, they are multiplied by zero scalars (blocks of 32 always do).  A loop of its own, as the branch
+            // per source and target made the slabs of eight 10 % slower where one scatterer needs no branch
+            auto rhs_phase = [&](auto PICK) {
+                for (int v0 = 0; v0 < nsv; v0 += NSL) {
+                    const int sv = v0 + sl;
+                    float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
+                    const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
+                    if (v0 + NSL < nsv) {
+                        n0 = dl[st * in];
+                        n1 = dl[st * in + wd];
+                        n2 = dl[st * in + 2 * wd];
+                        n3 = dl[st * in + 3 * wd];
+                    }
+                    const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
+                    const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
+                    const float2 sj = {d3.z, d3.w};
 #pragma unroll
-                for (int t = 0; t < NR_TT; ++t) {
-                    if (t < ntg) {
-                        const float4 p0 = S.ps[t][3 * sv], p1 = S.ps[t][3 * sv + 1];
-                        const float rx = p0.x, ry = p0.y, rz = p1.x;
-                        // U = a r + r x m
-                        cx<float> U[3] = {{fmaf(A.x, rx, fmaf(ry, m2.x, -rz * m1.x)), fmaf(A.y, rx, fmaf(ry, m2.y, -rz * m1.y))},
-                                          {fmaf(A.x, ry, fmaf(rz, m0.x, -rx * m2.x)), fmaf(A.y, ry, fmaf(rz, m0.y, -rx * m2.y))},
-                                          {fmaf(A.x, rz, fmaf(rx, m1.x, -ry * m0.x)), fmaf(A.y, rz, fmaf(rx, m1.y, -ry * m0.y))}};
-                        const cx<float> mc0 = {p0.z, p0.w}, g0 = {p1.z, p1.w};
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            cfma(acc0[t][c], mc0, U[c]);
-                            cfma(acc0[t][c], g0, q[c]);
-                        }
-                        // (a source of another scatterer is left out where it need not be finite: a block of 32
-                        // multiplies it by zero scalars)
-                        if (side1 && (W == 32 || p1.y != 0.f)) {
-                            const float4 p2v = S.ps[t][3 * sv + 2];
-                            const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
-                            U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};
-                            U[1] = {fmaf(sj.x, ry, U[1].re), fmaf(sj.y, ry, U[1].im)};
-                            U[2] = {fmaf(sj.x, rz, U[2].re), fmaf(sj.y, rz, U[2].im)};
+                    for (int t = 0; t < NR_TT; ++t) {
+                        if (t < ntg) {
+                            const float4 p0 = S.ps[t][3 * sv], p1 = S.ps[t][3 * sv + 1];
+                            const float rx = p0.x, ry = p0.y, rz = p1.x;
+                            // U = a r + r x m
+                            cx<float> U[3] = {{fmaf(A.x, rx, fmaf(ry, m2.x, -rz * m1.x)), fmaf(A.y, rx, fmaf(ry, m2.y, -rz * m1.y))},
+                                              {fmaf(A.x, ry, fmaf(rz, m0.x, -rx * m2.x)), fmaf(A.y, ry, fmaf(rz, m0.y, -rx * m2.y))},
+                                              {fmaf(A.x, rz, fmaf(rx, m1.x, -ry * m0.x)), fmaf(A.y, rz, fmaf(rx, m1.y, -ry * m0.y))}};
+                            const cx<float> mc0 = {p0.z, p0.w}, g0 = {p1.z, p1.w};
 #pragma unroll
                             for (int c = 0; c < 3; ++c) {
-                                cfma(acc1[t][c], c1, U[c]);
-                                cfma(acc1[t][c], g1, q[c]);
+                                cfma(acc0[t][c], mc0, U[c]);
+                                cfma(acc0[t][c], g0, q[c]);
+                            }
+                            if (side1 && (!PICK.value || p1.y != 0.f)) {
+                                const float4 p2v = S.ps[t][3 * sv + 2];
+                                const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
+                                U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};
+                                U[1] = {fmaf(sj.x, ry, U[1].re), fmaf(sj.y, ry, U[1].im)};
+                                U[2] = {fmaf(sj.x, rz, U[2].re), fmaf(sj.y, rz, U[2].im)};
+#pragma unroll
+                                for (int c = 0; c < 3; ++c) {
+                                    cfma(acc1[t][c], c1, U[c]);
+                                    cfma(acc1[t][c], g1, q[c]);
+                                }
                             }
                         }
                     }
+                    d0 = n0; d1 = n1; d2 = n2; d3 = n3;
                 }
-                d0 = n0; d1 = n1; d2 = n2; d3 = n3;
-            }
+            };
+            if (W < 32 && side1 && __any_sync(0xffffffffu, foreign)) rhs_phase(std::true_type{});
+            else rhs_phase(std::false_type{});
             __syncwarp();  // the next tile's pair phase overwrites the scalars
         }
         // far field of each side: this lane's three columns of the leaf's local expansion of the
