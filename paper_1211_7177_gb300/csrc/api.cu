@@ -252,6 +252,9 @@ fmbem_status fmbem_create(const fmbem_mesh *mesh, const fmbem_c64 *eps, const fm
             h->m2l_rotation = o.m2l_rotation == 1 || (o.m2l_rotation == -1 && h->p >= 9);
         }
         build_tables(h, s);
+        int dev = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, dev));
         near_work_items(h, s);
         std::vector<c64> dc(3 * (h->J + 1));
         for (int d = 0; d <= h->J; ++d) {

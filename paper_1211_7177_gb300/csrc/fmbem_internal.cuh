@@ -242,6 +242,7 @@ struct fmbem {
     int64_t n_rmm = 0;
 
     // scratch grown on demand
+    int nsm = 0;  // SMs of the device that the handle was created on
     int64_t scratch_rhs = 0;
     bool capturing = false;        // this call is recorded into a CUDA graph: nothing can be allocated
     bool graphs = false;           // a product of at most scratch_rhs right-hand sides was recorded

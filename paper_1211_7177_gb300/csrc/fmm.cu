@@ -3296,20 +3296,20 @@ static bool oz_ready(const fmbem *h, int W) {
            h->ybuf_bytes >= oz_ybuf_need<R>(h, W);
 }
 
-// source splits per item of k_near_d: about sixteen units for each of the 608 warp schedulers, no more than
+// source splits per item of k_near_d: about sixteen units for each warp scheduler (four per SM), no more than
 // the longest source list has tiles, 32 at most (the partial sums' buffer).  The four warps of a scheduler
 // share its FP64 pipe and end together, so with five units each some got eight (2562 nodes: 520-930 us with
 // at most eight splits)
 static int near_d_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_ditems * nr);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({32, h->near_tiles_max, (16 * 608 + units - 1) / units}));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({32, h->near_tiles_max, (16 * 4 * h->nsm + units - 1) / units}));
 }
 // and per item of k_near_ws (single precision, 1-3 right-hand sides): about four units for each of the 24
 // warps an SM holds.  A unit is latency-bound (a pair takes about 400 cycles of its warp), so with one unit
 // per item 10242 nodes (1450 units) took 215 us, ten times the arithmetic's time
 static int near_ws_splits(const fmbem *h, int64_t nr) {
     const int64_t units = std::max<int64_t>(1, (int64_t)h->n_near_items * nr);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * 152 + units - 1) / units}));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({16, h->near_tiles_max, (4 * 24 * h->nsm + units - 1) / units}));
 }
 // Scratch that grows.  A CUDA graph captured from a product holds these buffers' addresses, so that one which is
 // outgrown after a capture stays allocated (retired) until a call with more right-hand sides than any before

@@ -243,10 +243,10 @@ struct Work {
     void *dcoef;
     std::vector<c64> hres;
     std::vector<c32> hres32;
-    // grid.z of the reductions over groups of basis vectors: about six blocks for each of the 152 SMs
+    // grid.z of the reductions over groups of basis vectors: about six blocks for each SM
     unsigned dot_splits(int groups) const {
         const int64_t blocks = std::max<int64_t>(1, nblocks * nr);
-        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(groups, (6 * 152 + blocks - 1) / blocks));
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>(groups, (6 * h->nsm + blocks - 1) / blocks));
     }
     // dots[r][i] = <V_i[r], w[r]> for i < nv, arithmetic R
     template <typename R, typename TV, typename TW>
