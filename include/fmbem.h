@@ -129,9 +129,14 @@ typedef struct {
                                 translation, rotate back; ~3.3 p^3 instead of p^4 operations),
                                 -1 automatic: on the tensor cores in exact 8-bit digits (FP64: all
                                 translations, FP32: S|R) where p is even in 4..10 and the digit images
-                                (32 to 43 bytes per matrix value) take at most an eighth of the free
-                                device memory, for any number of right-hand sides; otherwise, and
-                                for the remaining translations, rotation form for p >= 9 [-1]   */
+                                (per real number of the matrices 128 bytes at p = 4, 63 at p = 6, 32 at
+                                p = 8, 43 at p = 10: rows are padded to 128) take at most an eighth of
+                                the free device memory at create, for any number of right-hand sides;
+                                otherwise, and for the remaining translations, rotation form for
+                                p >= 9.  The images, and up to 8 GB of pair results kept from the first
+                                such product on, are the price of the digits, and which form runs, and
+                                so the last bits of a result, depends on the free memory; 0 and 1 do
+                                without both [-1]                                                */
     int profile_phases;      /* non-zero: record CUDA events around the matvec phases so that
                                 fmbem_last_matvec_times can report them [0]                       */
     int near_cache;          /* near-field kernel scalars g, c of every (target, source, domain)
@@ -545,8 +550,11 @@ fmbem_status fmbem_precond_apply(fmbem *h, const void *v_dev, void *z_dev, int64
  * capture), code whose device memory is owned by a framework allocator, or callbacks that must
  * not trigger the implicit device synchronisation of cudaMalloc/cudaFree.  The paper has no
  * counterpart; this is a library-level variant of fmbem_matvec.
- * Same arguments, layouts, kernels and results as fmbem_matvec, except that precision must be
- * FMBEM_FP64 or FMBEM_FP32 (FMBEM_TF32 is refused with FMBEM_ERR_INVALID_ARGUMENT).  The scratch
+ * Same arguments and layouts as fmbem_matvec, and its results up to rounding, except that precision
+ * must be FMBEM_FP64 or FMBEM_FP32 (FMBEM_TF32 is refused with FMBEM_ERR_INVALID_ARGUMENT).  It runs the
+ * forms that need no more scratch than is listed here: the translations in rotation form or dense on
+ * the CUDA cores (not in digits), the FP64 near field by a block per leaf, the FP32 one without source
+ * splits (and below 32 right-hand sides in two parts).  The scratch
  * (source densities, expansion coefficients, per-pair M2L results) lives in one file-scope device array
  * of 32 MiB that every GPU loading the library holds until the process exits; no cudaMalloc,
  * cudaFree or allocating library routine is called.  Problems whose scratch for the given n_rhs
@@ -565,7 +573,7 @@ fmbem_status fmbem_matvec_noalloc(fmbem *h, const void *x_dev, void *y_dev, int6
  * of every problem -- source densities per (node block, right-hand side), P2M per (leaf, domain,
  * right-hand side), M2M per (parent box, domain, column chunk) level by level upwards, M2L + L2L
  * per (box, domain, column chunk) level by level downwards (dense S|S, S|R, R|R), near field +
- * L2P + self per leaf -- in stage order, with the number of items of every stage of every
+ * L2P + self per (leaf, right-hand side) -- in stage order, with the number of items of every stage of every
  * problem.  Each fmbem_batch_matvec is one launch of as many 128-thread blocks as can be
  * resident; a block takes the next item from a device queue counter, waits (bounded spin) until
  * the stages its item reads are complete for its problem, runs it and counts it complete.  Items

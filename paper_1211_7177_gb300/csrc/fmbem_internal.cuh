@@ -116,7 +116,7 @@ struct fmbem {
     double *pos = nullptr, *nrm = nullptr, *w = nullptr;  // [N][3], [N][3], [N]
     int32_t *dom = nullptr;                                // [N]
     float *pos_hi = nullptr, *pos_lo = nullptr, *nrm_f = nullptr;  // [N][3]
-    float4 *src_rec = nullptr;  // [N][3]: position hi + scatterer id, position lo + n_x, n_y n_z (k_near_w)
+    float4 *src_rec = nullptr;  // [N][3]: position hi + scatterer id, position lo + n_x, n_y n_z (k_near_ws, k_near_r)
     // self blocks (user order): M = A_self [N][6][6], LU factors and pivots
     c64 *Mself = nullptr, *Mlu = nullptr;
     int8_t *piv = nullptr;

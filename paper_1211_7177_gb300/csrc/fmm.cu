@@ -4103,10 +4103,12 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
 // Allocation-free matvec.  Some callers cannot allocate device memory at the time they need a
 // product: code running inside a CUDA stream capture (where cudaMalloc is not allowed), code
 // under a framework allocator that owns all device memory, or callbacks that must not block
-// on an implicit device synchronisation.  fmbem_matvec_noalloc runs the same kernels as
+// on an implicit device synchronisation.  fmbem_matvec_noalloc runs the passes of
 // fmbem_matvec, but takes its scratch (source densities, multipole and local coefficients,
 // per-pair M2L results) from the file-scope device array below instead of the handle's
-// grow-on-demand buffers, so it never calls cudaMalloc or cudaFree.
+// grow-on-demand buffers, so it never calls cudaMalloc or cudaFree.  The optional scratch has no place
+// there: the translations run without digits, the FP64 near field by a block per leaf (k_near, k_near_rb), the
+// FP32 one without source splits.
 //
 // The array is STATIC_SCRATCH_BYTES (32 MiB) on every GPU that loads the library and stays
 // resident until the process exits.  All calls share it and it keeps the last call's contents:

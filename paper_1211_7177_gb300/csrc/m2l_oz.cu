@@ -18,6 +18,12 @@
 // precision (rms relative error, torus of 3840 nodes): p = 8 8e-17 and p = 10 3e-16, where the FP64 sums
 // of the dense form have 5e-16 and the rotation form 1e-8 (a seven-digit form had 6e-16 and 1.5e-15).
 //
+// The digits are fixed-point: an entry is held to 2^-63 of the largest balanced one of its matrix row or source
+// column, and the products with i + j > 7 are left out.  An FP64 entry more than 2^-10 below the largest has fewer
+// bits than a double (a single-precision one more than 2^-7 below, with four digits: 2^-31), so that the error is
+// small against the norm of a row's products, not against each of them.  The balance by degree keeps the
+// entries that matter within that range.
+//
 // A single-precision product takes the first four digits of the same images and four digits of its sources
 // (2^-31 of the largest entry), ten products in four exact accumulators, added once in FP32: more exact than
 // the FP32 sums it replaces (product errors against FP64, torus of 9216 nodes: p = 8, 16 right-hand sides
@@ -659,8 +665,9 @@ int oz_mt(int p2) { return (2 * p2 + TC_M - 1) / TC_M; }
 
 }  // namespace
 
-// even p in 4..10: K = 2 p^2 <= 200 keeps the digit sums exact, and a K block of 16 ends at a whole
-// coefficient
+// even p in 4..10: K = 2 p^2 <= 200 keeps the digit sums exact (a diagonal of five products of at most 2^14 units
+// per K, 2 p^2 5 2^14 < 2^24).  Odd p would be as exact (images and digits are padded with zeros to whole K
+// blocks); they have not been measured and keep the rotation and dense forms
 bool m2l_oz_supported(const fmbem *h) {
     return h->p >= 4 && h->p <= 10 && h->p % 2 == 0 && h->lmax >= 2 && h->lmax < OZ_MAX_LEVELS && !h->opt.fp32_only;
 }
