@@ -543,7 +543,7 @@ def run_batched(args, world, flush):
     V, F, D = wl["mesh"]()
     t0 = time.perf_counter()
     g = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf, profile_phases=1,
-                 m2l_rotation=1, gmres_restart=restart)
+                 gmres_restart=restart)
     torch.cuda.synchronize()
     setup_s = time.perf_counter() - t0
     info = g.tree_info()
@@ -615,7 +615,7 @@ def run_batched(args, world, flush):
     solve = {}
     if not args.no_solve:
         # plain: FP64 GMRES(100) on one right-hand side
-        gp = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf, m2l_rotation=1,
+        gp = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf,
                       gmres_restart=restart)
         b1 = b[:1].contiguous()
         xs1 = torch.zeros_like(b1)
@@ -638,7 +638,7 @@ def run_batched(args, world, flush):
         # and the outer loop takes a single FP64 product (128 columns of FP64 FMM cost about as
         # much as 80 inner iterations)
         itol = 2.5e-5
-        gb = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf, m2l_rotation=1,
+        gb = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf,
                       gmres_restart=restart, solve_precision=fm.BF16X3, inner_tol=itol, outer_precision=fm.FP64)
         xs = torch.zeros_like(b)
         gb.solve(b, xs, tol=1e-4, max_iter=2)  # warm-up
@@ -914,7 +914,7 @@ def run_ours(args):
             # above the floor its input rounding sets), true residual with the FP64 operator and
             # FP64 vectors
             h2 = fm.FMBEM(V, F, D, wl["eps"], wl["mu"], wl["k0"], p=p, leaf_size=args.leaf, gmres_restart=args.restart,
-                          solve_precision=sp, inner_tol=itol, outer_precision=fm.FP64, m2l_rotation=1 if nr > 8 else -1)
+                          solve_precision=sp, inner_tol=itol, outer_precision=fm.FP64)
             xs = torch.zeros_like(b)
             h2.solve(b, xs, tol=1e-4, max_iter=1000)  # warm-up (allocates the Krylov basis)
             xs.zero_()
