@@ -2062,12 +2062,12 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
 // side only (k_local_rows writes the scatterer rows).
 // Per pair and right-hand side 72 FP32 operations beside three 16-byte words of scalars from shared memory
 // (four with w = n x r and n . r among them: 65536 nodes x 128 13.4 ms, now 13.2; 12.9 with the densities of 32
-// right-hand sides in 512-byte pieces instead of 64 bytes apart).  Issue slots 61 % busy, FMA 46 %: three
-// warps of 168 registers per scheduler do not hide the latency; a body per target count without branches
-// took 24 ms (instruction cache).  With
-// fewer than 32 right-hand sides, W lanes of right-hand sides keep the eight targets of every source they
+// right-hand sides in 512-byte pieces instead of 64 bytes apart).  Issue slots 60 % busy, FMA 49 % of the active
+// cycles (65536 nodes, 32 right-hand sides): three warps of 168 registers per scheduler do not hide the latency;
+// a body per target count without branches took 24 ms (instruction cache).
+// With fewer than 32 right-hand sides, W lanes of right-hand sides keep the eight targets of every source they
 // load, where lanes of (targets x slices) per side and eight right-hand sides, the pair scalars formed for
-// each, took three times as long (21973 nodes x 8: 1.5 -> 0.49 ms); as W lanes x subsets of the targets, a
+// each, took three times as long (21973 nodes x 8: 1.5 -> 0.50 ms); as W lanes x subsets of the targets, a
 // source's loads served two targets: 1.2 ms, and the sums over all sources in one lane were twice as inexact.
 // At the end each slice holds the sums of its own targets, so that the FP64 rows are formed once per target.
 constexpr int NR_TT = 8;   // targets per unit
@@ -2191,7 +2191,7 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             float4 d0 = dl[st * ic], d1 = dl[st * ic + wd], d2 = dl[st * ic + 2 * wd], d3 = dl[st * ic + 3 * wd];
             // PICK: sources of another scatterer are left out of the scatterer side, where they need not be finite;
             // without, they are multiplied by zero scalars (blocks of 32 always do).  A loop of its own, as the branch
-            // per source and target made the slabs of eight 10 % slower where one scatterer needs no branch
+            // per source and target made the slabs of eight 6 % slower where one scatterer needs no branch
             auto rhs_phase = [&](auto PICK) {
                 for (int v0 = 0; v0 < nsv; v0 += NSL) {
                     const int sv = v0 + sl;
@@ -2685,7 +2685,7 @@ __global__ void __launch_bounds__(32 * ND_WARPS, 4) k_near_adj(
 // quarter of the far field (L2P of phi and grad phi) of its side's domain in the working precision, then in double
 // precision u far from grad phi, u far + u near, T_d, the weights, and the transposed self block, a lane per
 // component of u and phi and then per row (each lane with all six: single precision, 17026 nodes x 3 RHS 163 us,
-// the FP64 pipe; now 100)
+// the FP64 pipe; now 106, of which forming the far field's u in double is 6)
 template <typename R>
 __global__ void __launch_bounds__(128) k_near_adj_finish(
     int64_t N, int64_t nr, int nsp, int p2, int64_t nbox, const int32_t *__restrict__ node_leaf,
