@@ -156,7 +156,7 @@ struct fmbem {
     int n_near_ditems = 0;
     int64_t near_tiles_max = 0;   // 32-source tiles of the longest source list
     void *near_am = nullptr, *near_part = nullptr;  // its per-source vectors and partial sums (scratch)
-    size_t near_am_bytes = 0, near_part_bytes = 0;
+    size_t near_am_bytes = 0, near_part_bytes = 0, near_refused = ~size_t(0);
     int4 *near_groups = nullptr;  // target groups of the lane-per-RHS near field (leaf, target offset, count, -):
                                   // n_near_groups in leaf order, then the same sorted by pair work
     int n_near_groups = 0;

@@ -3343,20 +3343,36 @@ static void grow_scratch(fmbem *h, void *&p, size_t &have, size_t need, size_t m
     have = size;
 }
 
-// the near field's partial sums (6 or 12 complex values of a node, right-hand side and split), and per-source
-// vectors of the FP64 forward product (row_bytes a node, right-hand side and split); without room for them, or
-// where they would have to grow during a stream capture, the forward product takes the kernels of the
-// allocation-free one, and the transposed one keeps its sums in the result
-static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
-    grow_scratch(h, h->near_part, h->near_part_bytes, row_bytes * h->N * nr * nsp);
-    if (am) grow_scratch(h, h->near_am, h->near_am_bytes, sizeof(c64) * 5 * h->N * nr);
+// whether optional scratch of need bytes is worth asking for: after a refusal (of at least refused bytes) only where
+// the device reports as much free again
+static bool room_for(size_t need, size_t refused) {
+    size_t free_b = 0, total_b = 0;
+    return need < refused || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b >= need);
 }
 
-// they hold this call's: the partial sums of nsp splits, and the per-source vectors (am).  Both are looked at
-// before either is used: k_prep writes the vectors of every right-hand side
+// the scratch of the near field (see ensure_near_scratch) holds this call's: the partial sums of nsp splits, and the
+// per-source vectors (am).  Both are looked at before either is used: k_prep writes the vectors of every
+// right-hand side
 static bool near_scratch_holds(const fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
     return h->near_part != nullptr && h->near_part_bytes >= row_bytes * h->N * nr * nsp &&
            (!am || (h->near_am != nullptr && h->near_am_bytes >= sizeof(c64) * 5 * h->N * nr));
+}
+
+// the near field's partial sums (6 or 12 complex values of a node, right-hand side and split: row_bytes), and
+// per-source vectors of the FP64 forward product; without room for them, or where they would have to grow during a
+// stream capture, the forward product takes the kernels of the allocation-free one, and the transposed one keeps
+// its sums in the result
+static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, size_t row_bytes, bool am) {
+    const size_t part = row_bytes * h->N * nr * nsp, vec = am ? sizeof(c64) * 5 * h->N * nr : 0;
+    if (h->capturing || near_scratch_holds(h, nr, nsp, row_bytes, am) || !room_for(part + vec, h->near_refused)) return;
+    try {
+        grow_scratch(h, h->near_part, h->near_part_bytes, part);
+        if (am) grow_scratch(h, h->near_am, h->near_am_bytes, vec);
+        h->near_refused = ~size_t(0);
+    } catch (const fmbem_error &e) {
+        if (e.st != FMBEM_ERR_OOM) throw;
+        h->near_refused = std::min(h->near_refused, part + vec);
+    }
 }
 
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s, bool pair_results = true) {
@@ -3398,12 +3414,7 @@ static void ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s, 
         // the digits are given back to them
         const size_t dig = dbl ? oz_digit_bytes<double>(h, ozw) : oz_digit_bytes<float>(h, ozw);
         const size_t res = dbl ? oz_ybuf_need<double>(h, ozw) : oz_ybuf_need<float>(h, ozw);
-        bool room = !h->capturing && (h->oz_dig_bytes < dig || h->ybuf_bytes < res);
-        if (room && dig + res >= h->oz_refused) {
-            size_t free_b = 0, total_b = 0;
-            room = cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b >= dig + res;
-        }
-        if (room) {
+        if (!h->capturing && (h->oz_dig_bytes < dig || h->ybuf_bytes < res) && room_for(dig + res, h->oz_refused)) {
             void *dig0 = h->oz_dig;
             const size_t have0 = h->oz_dig_bytes, kept = h->retired.size();
             try {
@@ -4058,13 +4069,9 @@ void run_adjoint_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precisio
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision, s);
-    try {
-        const bool dbl = precision == FMBEM_FP64;
-        ensure_near_scratch(h, nr, near_d_splits(h, dbl || nr == 1 ? nr : (nr + 2) / 3), 12 * (dbl ? sizeof(c64) : sizeof(c32)),
-                            false);
-    } catch (const fmbem_error &e) {
-        if (e.st != FMBEM_ERR_OOM) throw;
-    }
+    const bool dbl = precision == FMBEM_FP64;
+    ensure_near_scratch(h, nr, near_d_splits(h, dbl || nr == 1 ? nr : (nr + 2) / 3), 12 * (dbl ? sizeof(c64) : sizeof(c32)),
+                        false);
     const DomainConsts *dc = (const DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
         adjoint_impl<float>(h, x, y, nr, s, dc, precision == FMBEM_TF32 ? 1 : 2);
@@ -4080,12 +4087,8 @@ void run_matvec(fmbem *h, const c64 *x, c64 *y, int64_t nr, int precision, cudaS
     check_fp32_only(h, precision);
     check_oz_err(h, s);
     ensure_scratch(h, nr, precision, s);
-    try {
-        if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6 * sizeof(c64), true);
-        else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6 * sizeof(c32), false);
-    } catch (const fmbem_error &e) {
-        if (e.st != FMBEM_ERR_OOM) throw;
-    }
+    if (precision == FMBEM_FP64) ensure_near_scratch(h, nr, near_d_splits(h, nr), 6 * sizeof(c64), true);
+    else if (nr < 4 && near_ws_splits(h, nr) > 1) ensure_near_scratch(h, nr, near_ws_splits(h, nr), 6 * sizeof(c32), false);
     static_assert(sizeof(DomainConsts) == 3 * sizeof(c64), "layout");
     DomainConsts *dc = (DomainConsts *)h->dcons;
     if (precision == FMBEM_TF32 || precision == FMBEM_BF16X3) {
