@@ -959,11 +959,12 @@ __global__ void __launch_bounds__(32 * ROTC_WARPS) k_m2l_rot_cols(
 // Threads: rows_pad x ct column groups x NG pair groups; a thread owns columns cid * L2L_CPT .. + L2L_CPT - 1
 // and, with few columns, a quarter of the pairs (and of the dense R|R's inputs), the quarters added in order
 // through shared memory: a box has up to 189 pairs, whose results one thread read one after the other (FP64,
-// 642 nodes: 32 us for one level of 56 boxes).  Column groups beyond 1024 threads (p >= 12 and 7 or more
-// right-hand sides) go to grid.z.
+// 642 nodes: 32 us for one level of 56 boxes).  WIDE: column groups beyond 1024 threads (p >= 12 and 7 or more
+// right-hand sides) go to grid.z; elsewhere the registers of that cost a block per SM (93600 nodes x 9 RHS, FP32:
+// 0.78 -> 1.06 ms).
 constexpr int L2L_CPT = 3;
 constexpr int L2L_GROUPS = 4;
-template <typename R, int NG>
+template <typename R, int NG, bool WIDE>
 __global__ void __launch_bounds__(1024)
     k_l2l_reduce(int64_t off, int l, int lmax, int d0, int64_t nr, int p2, int64_t nbox, int col0, int ncol, int ct,
                              int rows_pad, const int32_t *parent, const uint64_t *key, const int32_t *ff_start,
@@ -979,8 +980,7 @@ __global__ void __launch_bounds__(1024)
     const int nt = rows_pad * ct, grp = NG == 1 ? 0 : threadIdx.x / nt;
     const int r = threadIdx.x % rows_pad, cid = (NG == 1 ? threadIdx.x : threadIdx.x % nt) / rows_pad;
     const cx<R> *T = nullptr;
-    // the block's columns (all of them where they are few)
-    const int cb = NG == 1 ? blockIdx.z * ct * L2L_CPT : 0, ncb = NG == 1 ? min(ncol - cb, ct * L2L_CPT) : ncol;
+    const int cb = WIDE ? blockIdx.z * ct * L2L_CPT : 0, ncb = WIDE ? min(ncol - cb, ct * L2L_CPT) : ncol;  // its columns
     if (l >= 3 && Yll == nullptr) {
         const int64_t P = parent[g];
         for (int e = threadIdx.x; e < ncb * p2; e += blockDim.x)
@@ -3719,14 +3719,14 @@ static void downward_pass(fmbem *h, int64_t nr, cudaStream_t s, int tensor_mode,
                 const size_t smr = sizeof(cx<R>) * ((l >= 3 && Yll == nullptr ? (size_t)std::min(nc, ct * L2L_CPT) * p2 : 0) +
                                                     (one ? 0 : (size_t)(L2L_GROUPS - 1) * L2L_CPT * rows_pad * ct));
                 const dim3 rgrid((unsigned)Lv.n, (unsigned)(J + 1), (unsigned)((groups + ct - 1) / ct));
-                if (one)
-                    k_l2l_reduce<R, 1><<<rgrid, rows_pad * ct, smr, sr>>>(
-                        Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent, h->box_key, h->ff_start,
-                        Tll, Y, e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
-                else
-                    k_l2l_reduce<R, L2L_GROUPS><<<rgrid, rows_pad * ct * L2L_GROUPS, smr, sr>>>(
-                        Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent, h->box_key, h->ff_start,
-                        Tll, Y, e_first, D, Yll, h->rmm_entry, ll_first, ystr, yll_str, oz ? h->tc_err : nullptr);
+                auto reduce = [&](auto kern, int nt) {
+                    kern<<<rgrid, nt, smr, sr>>>(Lv.off, l, lmax, 0, nr, p2, h->nbox, col0, nc, ct, rows_pad, h->box_parent,
+                                                 h->box_key, h->ff_start, Tll, Y, e_first, D, Yll, h->rmm_entry, ll_first, ystr,
+                                                 yll_str, oz ? h->tc_err : nullptr);
+                };
+                if (!one) reduce(k_l2l_reduce<R, L2L_GROUPS, false>, rows_pad * ct * L2L_GROUPS);
+                else if (ct < groups) reduce(k_l2l_reduce<R, 1, true>, rows_pad * ct);
+                else reduce(k_l2l_reduce<R, 1, false>, rows_pad * ct);
                 CKL("k_l2l_reduce");
             }
         }
