@@ -2070,16 +2070,19 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
 // each, took three times as long (21973 nodes x 8: 1.5 -> 0.50 ms); as W lanes x subsets of the targets, a
 // source's loads served two targets: 1.2 ms, and the sums over all sources in one lane were twice as inexact.
 // At the end each slice holds the sums of its own targets, so that the FP64 rows are formed once per target.
+// PICK (fewer than 32 right-hand sides, several scatterers): sources of another scatterer are left out of the
+// scatterer side, where they need not be finite; without it they are multiplied by zero scalars, as blocks of 32
+// always do.  The branch per source and target costs 6 % (93600 nodes x 9 RHS 3.47 -> 3.69 ms).
 constexpr int NR_TT = 8;   // targets per unit
 constexpr int NR_WARPS = 4;
 struct RhsTile {
-    // (r_x, r_y, -c_0), (r_z, 1 in the target's scatterer, g_0), (c_1, -gamma g_1) per target and source
+    // (r_x, r_y, -c_0), (r_z, PICK: 1 in the target's scatterer, g_0), (c_1, -gamma g_1) per target and source
     float4 ps[NR_TT][32 * 3 + 1];
     float4 tp[NR_TT][2];      // target position hi + scatterer id bits, position lo
     float4 tk[NR_TT];         // the target's scatterer wavenumber k_j and -gamma_j
 };
 
-template <int W>
+template <int W, bool PICK>
 __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
     const int32_t *leaf_box, const int4 *__restrict__ groups, int n_groups, int n_units, int *next_unit, int64_t N,
     int64_t nr, bool side1, const int32_t *nbeg, const int32_t *nend, const int32_t *nbr_start,
@@ -2158,7 +2161,6 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             }
             const float4 pa = rec[3 * i], pb = rec[3 * i + 1];
             const int sdom = __float_as_int(pa.w);
-            bool foreign = false;  // a source that some target's scatterer side leaves out
 #pragma unroll 2
             for (int t = 0; t < ntg; ++t) {
                 {
@@ -2172,14 +2174,13 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
                     pair_scalars<float>(inv, Rr, k0, g0, c0);
                     if (!valid) g0 = c0 = cx<float>{0.f, 0.f};
                     const bool own = side1 && valid && sdom == __float_as_int(ta.w);
-                    foreign |= sdom != __float_as_int(ta.w);
                     if (own) {
                         const float4 tk = S.tk[t];
                         pair_scalars<float>(inv, Rr, cx<float>{tk.x, tk.y}, g1, c1);
                         g1 = cx<float>{tk.z, tk.w} * g1;  // -gamma_j g_1: q_1 = -gamma_j q_0
                     }
                     S.ps[t][3 * lane] = make_float4(rv[0], rv[1], -c0.re, -c0.im);
-                    S.ps[t][3 * lane + 1] = make_float4(rv[2], own ? 1.f : 0.f, g0.re, g0.im);
+                    S.ps[t][3 * lane + 1] = make_float4(rv[2], PICK && own ? 1.f : 0.f, g0.re, g0.im);
                     S.ps[t][3 * lane + 2] = make_float4(c1.re, c1.im, g1.re, g1.im);
                 }
             }
@@ -2189,57 +2190,50 @@ __global__ void __launch_bounds__(32 * NR_WARPS, 3) k_near_r(
             const int nsv = min(32, (nsrc - s0 + NSL - 1) / NSL * NSL);
             int ic = __shfl_sync(0xffffffffu, i, sl);
             float4 d0 = dl[st * ic], d1 = dl[st * ic + wd], d2 = dl[st * ic + 2 * wd], d3 = dl[st * ic + 3 * wd];
-            // PICK: sources of another scatterer are left out of the scatterer side, where they need not be finite;
-            // without, they are multiplied by zero scalars (blocks of 32 always do).  A loop of its own, as the branch
-            // per source and target made the slabs of eight 6 % slower where one scatterer needs no branch
-            auto rhs_phase = [&](auto PICK) {
-                for (int v0 = 0; v0 < nsv; v0 += NSL) {
-                    const int sv = v0 + sl;
-                    float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
-                    const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
-                    if (v0 + NSL < nsv) {
-                        n0 = dl[st * in];
-                        n1 = dl[st * in + wd];
-                        n2 = dl[st * in + 2 * wd];
-                        n3 = dl[st * in + 3 * wd];
-                    }
-                    const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
-                    const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
-                    const float2 sj = {d3.z, d3.w};
+            for (int v0 = 0; v0 < nsv; v0 += NSL) {
+                const int sv = v0 + sl;
+                float4 n0 = d0, n1 = d1, n2 = d2, n3 = d3;
+                const int in = __shfl_sync(0xffffffffu, i, (sv + NSL) & 31);
+                if (v0 + NSL < nsv) {
+                    n0 = dl[st * in];
+                    n1 = dl[st * in + wd];
+                    n2 = dl[st * in + 2 * wd];
+                    n3 = dl[st * in + 3 * wd];
+                }
+                const float2 A = {d0.x, d0.y}, m0 = {d0.z, d0.w}, m1 = {d1.x, d1.y}, m2 = {d1.z, d1.w};
+                const cx<float> q[3] = {{d2.x, d2.y}, {d2.z, d2.w}, {d3.x, d3.y}};
+                const float2 sj = {d3.z, d3.w};
 #pragma unroll
-                    for (int t = 0; t < NR_TT; ++t) {
-                        if (t < ntg) {
-                            const float4 p0 = S.ps[t][3 * sv], p1 = S.ps[t][3 * sv + 1];
-                            const float rx = p0.x, ry = p0.y, rz = p1.x;
-                            // U = a r + r x m
-                            cx<float> U[3] = {{fmaf(A.x, rx, fmaf(ry, m2.x, -rz * m1.x)), fmaf(A.y, rx, fmaf(ry, m2.y, -rz * m1.y))},
-                                              {fmaf(A.x, ry, fmaf(rz, m0.x, -rx * m2.x)), fmaf(A.y, ry, fmaf(rz, m0.y, -rx * m2.y))},
-                                              {fmaf(A.x, rz, fmaf(rx, m1.x, -ry * m0.x)), fmaf(A.y, rz, fmaf(rx, m1.y, -ry * m0.y))}};
-                            const cx<float> mc0 = {p0.z, p0.w}, g0 = {p1.z, p1.w};
+                for (int t = 0; t < NR_TT; ++t) {
+                    if (t < ntg) {
+                        const float4 p0 = S.ps[t][3 * sv], p1 = S.ps[t][3 * sv + 1];
+                        const float rx = p0.x, ry = p0.y, rz = p1.x;
+                        // U = a r + r x m
+                        cx<float> U[3] = {{fmaf(A.x, rx, fmaf(ry, m2.x, -rz * m1.x)), fmaf(A.y, rx, fmaf(ry, m2.y, -rz * m1.y))},
+                                          {fmaf(A.x, ry, fmaf(rz, m0.x, -rx * m2.x)), fmaf(A.y, ry, fmaf(rz, m0.y, -rx * m2.y))},
+                                          {fmaf(A.x, rz, fmaf(rx, m1.x, -ry * m0.x)), fmaf(A.y, rz, fmaf(rx, m1.y, -ry * m0.y))}};
+                        const cx<float> mc0 = {p0.z, p0.w}, g0 = {p1.z, p1.w};
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            cfma(acc0[t][c], mc0, U[c]);
+                            cfma(acc0[t][c], g0, q[c]);
+                        }
+                        if (side1 && (!PICK || p1.y != 0.f)) {
+                            const float4 p2v = S.ps[t][3 * sv + 2];
+                            const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
+                            U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};
+                            U[1] = {fmaf(sj.x, ry, U[1].re), fmaf(sj.y, ry, U[1].im)};
+                            U[2] = {fmaf(sj.x, rz, U[2].re), fmaf(sj.y, rz, U[2].im)};
 #pragma unroll
                             for (int c = 0; c < 3; ++c) {
-                                cfma(acc0[t][c], mc0, U[c]);
-                                cfma(acc0[t][c], g0, q[c]);
-                            }
-                            if (side1 && (!PICK.value || p1.y != 0.f)) {
-                                const float4 p2v = S.ps[t][3 * sv + 2];
-                                const cx<float> c1 = {p2v.x, p2v.y}, g1 = {p2v.z, p2v.w};
-                                U[0] = {fmaf(sj.x, rx, U[0].re), fmaf(sj.y, rx, U[0].im)};
-                                U[1] = {fmaf(sj.x, ry, U[1].re), fmaf(sj.y, ry, U[1].im)};
-                                U[2] = {fmaf(sj.x, rz, U[2].re), fmaf(sj.y, rz, U[2].im)};
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    cfma(acc1[t][c], c1, U[c]);
-                                    cfma(acc1[t][c], g1, q[c]);
-                                }
+                                cfma(acc1[t][c], c1, U[c]);
+                                cfma(acc1[t][c], g1, q[c]);
                             }
                         }
                     }
-                    d0 = n0; d1 = n1; d2 = n2; d3 = n3;
                 }
-            };
-            if (W < 32 && side1 && __any_sync(0xffffffffu, foreign)) rhs_phase(std::true_type{});
-            else rhs_phase(std::false_type{});
+                d0 = n0; d1 = n1; d2 = n2; d3 = n3;
+            }
             __syncwarp();  // the next tile's pair phase overwrites the scalars
         }
         // far field of each side: this lane's three columns of the leaf's local expansion of the
@@ -3881,8 +3875,12 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
     };
     // fewer than 32 right-hand sides: 4 or 8 per slab, the warp's lanes divided among the sources
     auto launch_rest = [&](const cx<R> *dn, int64_t r0, int width) {
-        if (width <= 4) launch_r(k_near_r<4>, 0, 1, dn, r0, width);
-        else launch_r(k_near_r<8>, 0, (width + 7) / 8, dn, r0, width);
+        auto launch = [&](auto PICK) {
+            if (width <= 4) launch_r(k_near_r<4, PICK.value>, 0, 1, dn, r0, width);
+            else launch_r(k_near_r<8, PICK.value>, 0, (width + 7) / 8, dn, r0, width);
+        };
+        if (h->J > 1 && nsides == 2) launch(std::true_type{});
+        else launch(std::false_type{});
     };
     if constexpr (sizeof(R) == 4) {
         if (nr >= 4) {  // whole blocks of 32 right-hand sides one per lane, then the rest
@@ -3894,7 +3892,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                                   nblk <= (int64_t)(sizeof(io.ev) / sizeof(io.ev[0]));
             if (per_slab) {
                 for (int64_t b = 0; b < nblk; ++b) {
-                    launch_r(k_near_r<32>, b, 1, densT, 0, 32);
+                    launch_r(k_near_r<32, false>, b, 1, densT, 0, 32);
                     CK(cudaEventRecord(io.ev[b], s));
                     CK(cudaStreamWaitEvent(io.down, io.ev[b], 0));
                     const int64_t off = b * 32 * N * 6;
@@ -3903,7 +3901,7 @@ static void matvec_impl(fmbem *h, const c64 *x, c64 *y, int64_t nr, cudaStream_t
                 }
                 io.copied = true;
             } else if (nblk > 0) {
-                launch_r(k_near_r<32>, 0, nblk, densT, 0, 32);
+                launch_r(k_near_r<32, false>, 0, nblk, densT, 0, 32);
             }
             if (rest > 0 && prep_first) {
                 launch_rest(densT + nblk * N * 256, 32 * nblk, (int)rest);
