@@ -3371,11 +3371,9 @@ static void ensure_near_scratch(fmbem *h, int64_t nr, int nsp, size_t row_bytes,
 
 static void ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s, bool pair_results = true) {
     const size_t cb = sizeof(c64);
+    // (the legacy stream cannot be captured; asking about it costs 1 to 2 us)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {  // (the legacy stream beside another one's capture)
-        cudaGetLastError();
-        cap = cudaStreamCaptureStatusNone;
-    }
+    if (s != nullptr && s != cudaStreamLegacy) CK(cudaStreamIsCapturing(s, &cap));
     h->capturing = cap != cudaStreamCaptureStatusNone;
     if (h->scratch_rhs < nr) {
         if (h->capturing) throw fmbem_error{FMBEM_ERR_OOM, NO_ROOM_IN_CAPTURE};
@@ -4213,4 +4211,6 @@ void run_batch_kernel(int precision, const BatchProblem *probs, const BatchItem 
 
 // scratch of a handle for an n_rhs product in the given precision (batch.cu): densities and
 // expansions only, the batch's dense translation items keep no per-pair results
-void batch_ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s) { ensure_scratch(h, nr, precision, s, false); }
+void batch_ensure_scratch(fmbem *h, int64_t nr, int precision, cudaStream_t s) {
+    if (h->scratch_rhs < nr) ensure_scratch(h, nr, precision, s, false);
+}
