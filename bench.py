@@ -406,22 +406,22 @@ def run_gradients(fd_check=False):
 # records the SHA-256 prefixes of the kernel sources it was taken with, and the bench reports null
 # once a source has changed.
 TRAFFIC = {
-    ('silver_sphere_s7', 'fp64', 1, 'p2m'): dict(bytes=2225861632, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp64', 1, 'm2m'): dict(bytes=357696256, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp64', 1, 'm2l_l2l'): dict(bytes=8744454400, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp64', 1, 'near_l2p_self'): dict(bytes=7818759680, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp32', 1, 'p2m'): dict(bytes=1114935808, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp32', 1, 'm2m'): dict(bytes=58539008, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp32', 1, 'm2l_l2l'): dict(bytes=4030363648, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'fp32', 1, 'near_l2p_self'): dict(bytes=467260416, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'p2m'): dict(bytes=1114789120, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'm2m'): dict(bytes=58546176, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'm2l_l2l'): dict(bytes=3199853312, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('silver_sphere_s7', 'bf16x3', 1, 'near_l2p_self'): dict(bytes=467227904, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('torus_512x128', 'bf16x3', 128, 'p2m'): dict(bytes=3513123584, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('torus_512x128', 'bf16x3', 128, 'm2m'): dict(bytes=1576411136, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('torus_512x128', 'bf16x3', 128, 'm2l_l2l'): dict(bytes=4959117056, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
-    ('torus_512x128', 'bf16x3', 128, 'near_l2p_self'): dict(bytes=4956057600, src={'fmm.cu': '6bad18b3f655403b', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp64', 1, 'p2m'): dict(bytes=2225393152, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp64', 1, 'm2m'): dict(bytes=357817088, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp64', 1, 'm2l_l2l'): dict(bytes=8780792576, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp64', 1, 'near_l2p_self'): dict(bytes=7830456576, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp32', 1, 'p2m'): dict(bytes=1114828288, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp32', 1, 'm2m'): dict(bytes=58538496, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp32', 1, 'm2l_l2l'): dict(bytes=4048004352, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'fp32', 1, 'near_l2p_self'): dict(bytes=467411456, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'p2m'): dict(bytes=1114830080, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'm2m'): dict(bytes=58541056, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'm2l_l2l'): dict(bytes=3211651072, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('silver_sphere_s7', 'bf16x3', 1, 'near_l2p_self'): dict(bytes=467339776, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('torus_512x128', 'bf16x3', 128, 'p2m'): dict(bytes=3513459712, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('torus_512x128', 'bf16x3', 128, 'm2m'): dict(bytes=1576210176, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('torus_512x128', 'bf16x3', 128, 'm2l_l2l'): dict(bytes=4955230208, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
+    ('torus_512x128', 'bf16x3', 128, 'near_l2p_self'): dict(bytes=4958862336, src={'fmm.cu': 'e3bd4f9073dd5eb6', 'm2l_tc.cu': '04f3a37fe229d9f7', 'm2l_oz.cu': '36c44f03ddfd8810'}),
 }
 
 

@@ -2067,7 +2067,7 @@ __global__ void __launch_bounds__(192) k_near_sum(int64_t N, int64_t nr, int nsp
 // a body per target count without branches took 24 ms (instruction cache).
 // With fewer than 32 right-hand sides, W lanes of right-hand sides keep the eight targets of every source they
 // load, where lanes of (targets x slices) per side and eight right-hand sides, the pair scalars formed for
-// each, took three times as long (21973 nodes x 8: 1.5 -> 0.50 ms); as W lanes x subsets of the targets, a
+// each, took three times as long (21973 nodes x 8: 1.5 -> 0.49 ms); as W lanes x subsets of the targets, a
 // source's loads served two targets: 1.2 ms, and the sums over all sources in one lane were twice as inexact.
 // At the end each slice holds the sums of its own targets, so that the FP64 rows are formed once per target.
 // PICK (fewer than 32 right-hand sides, several scatterers): sources of another scatterer are left out of the
